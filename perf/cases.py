@@ -230,3 +230,56 @@ def run(st):
     call = g.verify_step_host_gqa if grouped else g.verify_step_host
     call(kc, vc, k=st["k"], scale=SCALE, h_outs=st["h_out"], **st["h_in"])
     return [st["h_out"], st["caches"]]
+
+
+# ------------------------------------------------------------------------------------------------ the same in 64 bits
+def _attention(q, K, V, row0, ctx, n, parent):
+    """Nodes 0..n-1 of one sequence over its ctx prefix rows and, of its tree rows, a node's ancestors and itself."""
+    sees = torch.zeros(n, n, dtype=torch.bool)
+    for i in range(n):
+        if i:
+            sees[i] = sees[parent[i]]
+        sees[i, i] = True
+    sees = torch.cat([torch.ones(n, ctx, dtype=torch.bool), sees], 1).to(q.device)
+    group = q.shape[1] // K.shape[1]
+    out = torch.empty(n, q.shape[1], D, dtype=torch.float64, device=q.device)
+    for hk in range(K.shape[1]):
+        keys, values = (t[row0:row0 + ctx + n, hk].double() for t in (K, V))
+        for h in range(hk * group, (hk + 1) * group):
+            p = (SCALE * (q[:n, h].double() @ keys.T)).masked_fill_(~sees, -math.inf)
+            out[:, h] = torch.softmax(p, 1) @ values
+    return out
+
+
+def exact(c, seed):
+    """The attention's output, the k largest logits of each row, the rows' log-sum-exp and the table's scores."""
+    st = prepare(c, seed)
+    k, V = c["k"], c["V"]
+    logits = (st["h_in"]["h_logits"].cuda() if c["op"] == "host" else st["logits"]).double()
+    ids = torch.sort(logits, dim=1, descending=True, stable=True)[1][:, :k] if c["op"] in ("cycle", "prefill") else None
+    top = torch.topk(logits, k, dim=1)[0]
+    lse = torch.logsumexp(logits, 1)
+    if c["op"] == "prefill":
+        tokens, nodes = st["row_tok"].tolist(), [c["B"]]
+    else:
+        ctx, nodes = _shapes(c)
+        tokens, parent, offsets = st["tok"].view(-1).tolist(), st["parent"].tolist(), st["row_off"].tolist()
+        out = torch.zeros(c["layers"], c["S"], c["B"], c["H"], D, dtype=torch.float64, device="cuda")
+        for layer in range(c["layers"]):
+            q, K, Vc = st["layers"][layer][:3]
+            for s, n in enumerate(nodes):
+                if n:
+                    out[layer, s, :n] = _attention(q[s], K, Vc, offsets[s], ctx[s], n, parent[s])
+    if c["op"] == "model":
+        return [out, None, None, top, None, None, None, None, None]
+    live = torch.tensor([i < n for n in nodes for i in range(c["B"])], device="cuda")   # nothing is written of other rows
+    top, lse = top * live[:, None], lse * live
+    if c["op"] in ("step", "host"):
+        return [dict(out=out[0], topk_vals=top), None]
+    scores = torch.zeros(V, k, dtype=torch.float64, device="cuda")
+    for row, token in enumerate(tokens):                       # of several rows with one token the last one stands
+        if live[row] and 0 <= token < V:
+            scores[token] = torch.exp(logits[row, ids[row]] - lse[row])
+    if c["op"] == "prefill":
+        return [[None, None, top, lse], None, scores]
+    return [dict(out=out[0], topk_vals=top, row_lse=lse), None, None, scores]
