@@ -17,15 +17,21 @@ harvest_scatter_kernel(const int32_t* __restrict__ row_tok, int rows, int table_
                        float* __restrict__ adj_scores) {
     const int lane = threadIdx.x & 31;
     const int r = blockIdx.x * (kScatterThreads / 32) + (threadIdx.x >> 5);
+    // row_tok[] is an input of the call: the top-k kernel in front lets this one start only after its own wait, so the
+    // decision is taken while that kernel still runs (it is a scan of up to `rows` tokens, 47 loads a lane for 1500 rows)
+    int tok = -1;
+    bool write = false;
+    if (r < rows) {
+        tok = row_tok[r];
+        if (tok >= 0 && tok < table_rows) {                  // else not a table row: skipped
+            bool later = false;                              // does a later row carry the same token?
+            for (int j = r + 1 + lane; j < rows; j += 32) later |= (row_tok[j] == tok);
+            write = !__any_sync(0xFFFFFFFFu, later);
+        }
+    }
     pdl_wait();
     pdl_trigger();
-    if (r >= rows) return;
-    const int tok = row_tok[r];
-    if (tok < 0 || tok >= table_rows) return;              // not a table row: skipped
-    bool later = false;                                      // does a later row carry the same token?
-    for (int j = r + 1 + lane; j < rows; j += 32) later |= (row_tok[j] == tok);
-    if (__any_sync(0xFFFFFFFFu, later)) return;
-    if (lane < k) {
+    if (write && lane < k) {
         adj_ids[(size_t)tok * k + lane] = ids[(size_t)r * k + lane];
         adj_scores[(size_t)tok * k + lane] = expf(vals[(size_t)r * k + lane] - row_lse[r]);
     }

@@ -1,36 +1,61 @@
 // Per-node argmax and top-k over bf16 logits (Algorithm 3 step 2; batched top-K harvest of App. C.1).
 //
-// A row is cut into chunks of 32768 elements; the (row, chunk) items, in row-major order, are dealt in contiguous
-// ranges to a persistent grid of one 1024-thread CTA per SM.  One thread streams the CTA's items into a ring of
-// three 64 KB shared-memory stages with bulk asynchronous copies (cp.async.bulk, mbarrier completion), so HBM keeps
-// streaming while the CTA selects; every thread then takes 32 values of the current item into registers.
-// The exact order is carried by 32-bit keys
+// A row is cut into equal chunks of at most 32768 elements; the (row, chunk) items, in row-major order, are dealt in
+// contiguous ranges to a persistent grid of one CTA per SM.  The exact order is carried by 32-bit keys
 //     (order-preserving 16-bit image of the bf16 value) << 16 | (0xFFFF - index_in_chunk)
-// so "largest key" is "largest value, lowest index on ties", all keys are distinct, and a key carries its own
-// index.  Building a key costs several instructions per element, so keys are built only for candidates: packed-bf16
-// maxima give every thread's maximum, one redux.sync gives every warp's maximum, and T = the k-th largest of the 32
-// warp maxima is a threshold with at least k elements at or above it -- hence every one of the chunk's k best is
-// >= T.  Only the elements >= T (about ten of 32768) become keys, and one warp ranks them.  Selections among up
-// to 32 distinct keys are done by rank counting (every lane counts the keys above its own: independent compares
-// instead of k dependent warp-wide reduction rounds).  Chunks with more than
-// 1024 elements at or above T (a constant row) take an exact slow path over all keys.  The chunks of a row are merged
-// by the CTA as it walks them; a row whose chunks are spread over several CTAs is finished by the last of those CTAs
-// to arrive (arrival counter, no spinning).  Every mbarrier wait is bounded: when one runs out the CTA reports
-// GOOSE_ST_TIMEOUT, drains its own copies in flight (bounded again) and returns.
+// so "largest key" is "largest value, lowest index on ties", all keys are distinct, and a key carries its own index.
+// Building a key costs several instructions per element, so keys are built only for candidates: elements not below T, the
+// k-th largest of the 32 half-warp maxima of an item (at least k elements are >= T, hence the chunk's k best are among
+// them; about ten of 32768 qualify).  Roles, coupled by mbarriers alone (no CTA-wide barrier):
+//   control warp (1)     streams the items into a ring of three 64 KB shared-memory stages with bulk asynchronous copies
+//                        (cp.async.bulk), ranks an item's candidates, merges the chunks of a row, writes the results
+//   data warps (16)      64 values per thread into registers: thread maxima with packed-bf16 max, half-warp maxima with
+//                        redux.sync.  With the log-sum-exp they also sum the exponentials relative to the warp's largest
+//                        value so far, eight elements at a time behind their load, so that one warp's exponentials cover
+//                        another's loads and maxima
+//   collector warps (4)  T by rank counting (every lane counts the keys above its own: independent compares instead of k
+//                        dependent reduction rounds); the threads whose maximum is >= T; keys of their elements >= T
+// What bounds it: the stream (64 KB an item and SM: 1.47 us at the copy peak) and, with the log-sum-exp, the 32768
+// exponentials of an item (2048 cycles of the special-function units).  The selection is a chain of some 500 dependent
+// instructions on few warps (2000 to 4000 cycles by a clock trace); behind CTA-wide barriers, with every warp waiting for
+// it, it was a third to half of an item's time.  Call times, one set of
+// 1024-thread CTAs with three barriers an item -> these roles: 1500 x 32000 25.9 -> 19.2 us, with log-sum-exp and scatter
+// 45.8 -> 26.6; 1024 x 32000 22.0 -> 14.5; 128 x 128256 11.7 -> 9.4; 480 x 32000 with counts and log-sum-exp 18.8 -> 12.7;
+// one item a CTA (80 x 32000) 4.0 as before.  Measured and dropped: one barrier an item (23.1 and 40.8 us for 1500 rows),
+// eight warps for the maxima and eight for the exponentials (39.4: two warps a scheduler do not fill the special-function
+// units), a running maximum updated at every sweep (33.4: a redux.sync and a branch every eight elements).
+// A quarter with many candidates (ties, as in a constant row) is cut with the k-th largest thread maximum instead and
+// takes only the first k of the elements equal to it, so the list is bounded whatever the row holds.
+// A row whose chunks are spread over several CTAs is finished by the last of those CTAs to arrive (arrival counter, no
+// spinning).  Every mbarrier wait is bounded: when one runs out the CTA reports GOOSE_ST_TIMEOUT, drains its own copies in
+// flight (bounded again) and returns.
 #include <mutex>
 
 #include "goose_internal.cuh"
 
 namespace goose {
 
-constexpr int kTopkThreads = 1024;
-constexpr int kTopkPerThread = 32;                          // 4 x 128-bit shared-memory loads
-constexpr int kTopkChunk = kTopkThreads * kTopkPerThread;    // 32768 elements
+constexpr int kTopkDataWarps = 16;
+constexpr int kTopkCollectWarps = 4;
+constexpr int kTopkDataThreads = kTopkDataWarps * 32;
+constexpr int kTopkThreads = kTopkDataThreads + kTopkCollectWarps * 32 + 32;   // 16 + 4 + 1 warps
+constexpr int kTopkPerThread = 64;                           // of a data thread: 8 x 128-bit shared-memory loads
+constexpr int kTopkChunk = kTopkDataThreads * kTopkPerThread;   // 32768 elements
+constexpr int kTopkSweep = kTopkDataThreads * 8;             // elements that the data threads load at once
 constexpr int kTopkMaxChunks = GOOSE_MAX_V / kTopkChunk;     // 8
 constexpr int kTopkStages = 3;
 constexpr int kTopkStageBytes = kTopkChunk * 2;              // 64 KB
-constexpr int kTopkSmem = kTopkStages * kTopkStageBytes;     // dynamic shared memory of the kernel
+// what an item hands from role to role lives in slot (item & 3): a slot comes back into use only after the control warp
+// has finished its last item, because that warp issues item j + 4 behind finishing item j
+constexpr int kTopkSlots = 4;
+// a collector adds at most kTopkQuickList keys, or cuts with the k-th largest thread maximum T': fewer than k threads hold
+// elements > T', 64 each, and of the elements equal to T' every collector takes at most k
+constexpr int kTopkQuickList = 128;
+constexpr int kTopkListCap = kMaxK * kTopkPerThread + kTopkCollectWarps * kMaxK + (kTopkCollectWarps - 1) * kTopkQuickList;
+constexpr int kTopkSmem = kTopkStages * kTopkStageBytes + kTopkSlots * kTopkListCap * 4;   // dynamic shared memory
 constexpr long long kTopkWaitCycles = 2000000000ll;          // bound of every wait: about one second of SM clock
+constexpr float kTopkLog2e = 1.4426950408889634f;
+constexpr uint32_t kImageNegInf = 0x007Fu;                   // sortable16 of -inf
 
 typedef unsigned long long u64;
 
@@ -45,11 +70,15 @@ __device__ __forceinline__ float value_of_sortable16(uint32_t s) {
     return __uint_as_float(bits << 16);
 }
 
-constexpr int kTopkListCap = 1024;                           // candidate list of the fast path
-
 __device__ __forceinline__ uint32_t bits_of_sortable16(uint32_t s) {
     return (s & 0x8000u) ? (s ^ 0x8000u) : (~s & 0xFFFFu);
 }
+__device__ __forceinline__ float topk_ex2(float x) {         // 2^x; results below 2^-126 are 0
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float float_of_sortable16(uint32_t s) { return __uint_as_float(bits_of_sortable16(s) << 16); }
 __device__ __forceinline__ __nv_bfloat162 as_bf162(uint32_t w) { return *reinterpret_cast<__nv_bfloat162*>(&w); }
 __device__ __forceinline__ uint32_t as_u32(__nv_bfloat162 v) { return *reinterpret_cast<uint32_t*>(&v); }
 
@@ -64,33 +93,82 @@ __device__ __forceinline__ u64 warp_max_u64(u64 v) {
 
 namespace {
 __device__ __forceinline__ uint32_t topk_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void topk_mbar_init(u64* bar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(topk_smem_u32(bar)), "r"(count));
+}
+__device__ __forceinline__ void topk_mbar_arrive(u64* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(topk_smem_u32(bar)) : "memory");
+}
+// bit e of the result: element e of the eight in w is >= (or, with kStrict, >) the value in both halves of t (a NaN passes)
+template <bool kStrict>
+__device__ __forceinline__ uint32_t topk_above(const uint4& w, __nv_bfloat162 t) {
+    const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+    uint32_t m = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const uint32_t c = kStrict ? __hgtu2_mask(as_bf162(x[q]), t) : __hgeu2_mask(as_bf162(x[q]), t);
+        m |= ((c & 1u) | ((c >> 15) & 2u)) << (2 * q);
+    }
+    return m;
+}
+
+// a walk over the rows that exist: rows of the call, or with node counts the rows of nodes that exist, numbered densely
+template <bool COUNTS>
+struct RowCursor {
+    long long row, chunk;      // current item: dense row number and chunk in it
+    long long mem;             // the row's place in memory
+    int s, left;               // its sequence, and the existing rows of that sequence from this one on
+    __device__ __forceinline__ void seek(long long w, int chunks, const int32_t* n_nodes, int S, int B) {
+        row = w / chunks; chunk = w - row * chunks;
+        mem = row; s = 0; left = 0;
+        if (COUNTS) {
+            long long r = row;
+            for (; s < S; ++s) {
+                const int n = nodes_of(n_nodes, s, B);
+                if (r < n) { mem = (long long)s * B + r; left = n - (int)r; return; }
+                r -= n;
+            }
+            mem = 0;                                         // behind the last row (a CTA without items): not used
+        }
+    }
+    __device__ __forceinline__ void next(int chunks, const int32_t* n_nodes, int S, int B) {
+        if (++chunk < chunks) return;
+        chunk = 0; ++row; ++mem;
+        if (COUNTS && --left == 0) {
+            do ++s; while (s < S && (left = nodes_of(n_nodes, s, B)) == 0);
+            mem = (long long)s * B;
+        }
+    }
+};
 }  // namespace
 
-// LSE = true additionally returns the row's log-sum-exp (for the softmax scores of the harvest): the second
-// pass sums exp(x - chunk max) over every element, chunks are merged like split softmax partials.
+// LSE = true additionally returns the row's log-sum-exp (for the softmax scores of the harvest): the data warps sum
+// exp(x - chunk max) over every element, chunks are merged like split softmax partials.
 // COUNTS = false is the instantiation for n_nodes == NULL (the item list is known before the dependency wait)
-template <int KCAP, bool LSE, bool COUNTS>
+template <bool LSE, bool COUNTS>
 __global__ void __launch_bounds__(kTopkThreads, 1)
 node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, int V, int64_t ldl, int k, int chunks,
-                 u64* __restrict__ ws_cand, int32_t* __restrict__ row_counters,
+                 int chunk_elems, u64* __restrict__ ws_cand, int32_t* __restrict__ row_counters,
                  int32_t* __restrict__ argmax, int32_t* __restrict__ ids, float* __restrict__ vals,
                  float* __restrict__ row_lse, float2* __restrict__ ws_lse, int32_t* __restrict__ status,
                  int inputs_ready, const int32_t* __restrict__ n_nodes, int S, int B) {
-    extern __shared__ __align__(128) unsigned char s_stage[];   // kTopkStages x 64 KB
-    __shared__ u64 s_full[kTopkStages];
-    __shared__ float s_sum[32];
-    __shared__ __align__(16) uint32_t s_wmax[32];        // warp maxima as distinct keys: value image << 5 | 31 - warp
+    extern __shared__ __align__(128) unsigned char s_stage[];   // kTopkStages x 64 KB, then the candidate lists
+    __shared__ u64 s_full[kTopkStages];                  // the stage holds its item
+    __shared__ u64 s_max_done[kTopkSlots], s_list_done[kTopkSlots];
+    __shared__ __align__(16) uint32_t s_gmax[kTopkSlots][32];   // half-warp maxima as distinct keys: value image << 5 | 31 - index
+    __shared__ __align__(16) unsigned short s_tmax[kTopkStages][kTopkDataThreads];   // thread maxima (value images)
+    __shared__ float s_sum[kTopkSlots][kTopkDataWarps];   // sums of exponentials, and the images of what they are relative to
+    __shared__ uint32_t s_sum_max[kTopkSlots][kTopkDataWarps];
+    __shared__ int s_count[kTopkSlots];                  // length of the candidate list
+    __shared__ unsigned short s_hold[kTopkCollectWarps][16];
     __shared__ __align__(16) uint32_t s_sel[32];         // rank-ordered keys of a selection
     __shared__ __align__(16) u64 s_m64[32];              // candidates of a 64-bit merge
     __shared__ u64 s_run[kMaxK];
-    __shared__ uint32_t s_thresh, s_cmax;
-    __shared__ uint32_t s_cand[32 * KCAP];               // slow path: per-warp winners (exact keys)
-    __shared__ __align__(16) uint32_t s_list[kTopkListCap];   // fast path: keys of all elements >= threshold; entries
-                                                         // 0..31 are zero between items
-    __shared__ u64 s_merge[kTopkMaxChunks * KCAP];
-    __shared__ int s_count;                              // length of s_list
+    __shared__ u64 s_merge[kTopkMaxChunks * kMaxK];
     __shared__ int s_last;
     __shared__ volatile int s_abort;
+    uint32_t* const s_lists = reinterpret_cast<uint32_t*>(s_stage + kTopkStages * kTopkStageBytes);   // candidates' keys;
+                                                         // entries 0..31 of a list are zero between items
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = gridDim.x;
@@ -98,12 +176,17 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
     long long items = items_all;
     long long w_begin = items * blockIdx.x / G, w_end = items * (blockIdx.x + 1) / G;   // final when !COUNTS
     if (tid == 0) {
-        for (int i = 0; i < kTopkStages; ++i)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(topk_smem_u32(&s_full[i])));
-        s_count = 0; s_abort = 0;
+        for (int i = 0; i < kTopkStages; ++i) topk_mbar_init(&s_full[i], 1);
+        for (int i = 0; i < kTopkSlots; ++i) {
+            topk_mbar_init(&s_max_done[i], kTopkDataWarps);
+            topk_mbar_init(&s_list_done[i], kTopkCollectWarps);
+            s_count[i] = 0;
+        }
+        s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (tid < 32) s_list[tid] = 0;
+    if (tid < 32)
+        for (int i = 0; i < kTopkSlots; ++i) s_lists[i * kTopkListCap + tid] = 0;
     __syncthreads();
     // inputs_ready: the caller guarantees that the logits were complete before the preceding kernel in the stream
     // started (the whole-step call: that kernel is the attention kernel, which neither reads nor writes them).  The
@@ -114,108 +197,316 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
     pdl_trigger();
     // Per-sequence node counts (n_nodes != NULL; rows = S * B, row s * B + i belongs to node i of sequence s): rows of
     // nodes that do not exist are left out of the item list, so their logits are never read.  The list then runs over
-    // the rows that exist, numbered densely ("row" below; the cross-CTA scratch is indexed by it), and row_of() gives
-    // the row in memory.  n_nodes[] is an input like the logits: it may be read ahead of the dependency wait.
+    // the rows that exist, numbered densely (the cross-CTA scratch is indexed by that number).  n_nodes[] is an input
+    // like the logits: it may be read ahead of the dependency wait.
     if (COUNTS && n_nodes) {
         long long live = 0;
         for (int s = 0; s < S; ++s) live += nodes_of(n_nodes, s, B);
         items = live * chunks;
         w_begin = items * blockIdx.x / G; w_end = items * (blockIdx.x + 1) / G;
     }
-    auto row_of = [&](long long r) -> long long {
-        if constexpr (!COUNTS) {
-            return r;
-        } else {
-            if (!n_nodes) return r;
-            for (int s = 0; s < S; ++s) {
-                const int n = nodes_of(n_nodes, s, B);
-                if (r < n) return (long long)s * B + r;
-                r -= n;
-            }
-            return 0;                                    // not reached: r is below the number of live rows
-        }
-    };
     const int n_local = (int)(w_end - w_begin);
 
-    const unsigned short* lg = reinterpret_cast<const unsigned short*>(logits);
-    // thread 0: stream item j of this CTA into stage j % kTopkStages (the copy is rounded up to 16 bytes, which
-    // stays inside the row because ldl is a multiple of 8 elements)
-    auto issue = [&](int j) {
-        const long long w = w_begin + j;
-        const long long row = w / chunks;
-        const int base = (int)(w - row * chunks) * kTopkChunk;
-        const int n_valid = min(kTopkChunk, V - base);
-        const uint32_t bytes = ((uint32_t)n_valid * 2u + 15u) & ~15u;
-        u64* bar = &s_full[j % kTopkStages];
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(topk_smem_u32(bar)), "r"(bytes) : "memory");
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(topk_smem_u32(s_stage + (j % kTopkStages) * kTopkStageBytes)),
-                       "l"(lg + (size_t)row_of(row) * ldl + base), "r"(bytes), "r"(topk_smem_u32(bar)) : "memory");
+    // bounded wait for item j's hand-over in its slot; a wait that runs out raises the CTA's abort flag, which ends the
+    // waits of all other warps
+    auto slot_wait = [&](u64* bars, int j) -> bool {
+        if (mbar_wait_bounded(&bars[j % kTopkSlots], (uint32_t)(j / kTopkSlots) & 1u, kTopkWaitCycles, &s_abort) == 0) return true;
+        s_abort = 1;
+        return false;
     };
-    int issued = 0;
-    if (tid == 0)
-        for (; issued < n_local && issued < kTopkStages; ++issued) issue(issued);
 
-    long long row = w_begin / chunks;
-    int chunk = (int)(w_begin - row * chunks);
-    // warp 0: the current row's k best over the chunks walked so far (lane r: r-th 64-bit key
-    // value image << 32 | ~global index; 0 = none) and its running log-sum-exp parts
+    if (warp < kTopkDataWarps) {
+        // ================================================================================ data warps
+        int chunk = (int)(w_begin % chunks);
+        for (int j = 0; j < n_local; ++j) {
+            const int st = j % kTopkStages, slot = j % kTopkSlots;
+            const unsigned char* sp = s_stage + st * kTopkStageBytes;
+            const int n_valid = min(chunk_elems, V - chunk * chunk_elems);
+            if (mbar_wait_bounded(&s_full[st], (uint32_t)(j / kTopkStages) & 1u, kTopkWaitCycles, &s_abort) != 0) {
+                s_abort = 1;
+                break;
+            }
+            // thread tid's 64 values: element (it, e) sits at chunk offset it * 4096 + tid * 8 + e; elements past the
+            // chunk's end read as -inf
+            auto trim = [&](uint4& w, int it) {
+                const int off0 = it * kTopkSweep + tid * 8;
+                if (off0 + 8 > n_valid) {
+                    uint32_t y[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const uint32_t lo = (off0 + 2 * q < n_valid) ? (y[q] & 0xFFFFu) : 0xFF80u;
+                        const uint32_t hi = (off0 + 2 * q + 1 < n_valid) ? (y[q] >> 16) : 0xFF80u;
+                        y[q] = lo | (hi << 16);
+                    }
+                    w = make_uint4(y[0], y[1], y[2], y[3]);
+                }
+            };
+            auto load = [&](int it) { return *reinterpret_cast<const uint4*>(sp + (size_t)(it * kTopkSweep + tid * 8) * 2); };
+            auto load_trimmed = [&](int it) {
+                uint4 w = load(it);
+                trim(w, it);
+                return w;
+            };
+            auto max8 = [&](const uint4& w) { return __hmax2(__hmax2(as_bf162(w.x), as_bf162(w.y)), __hmax2(as_bf162(w.z), as_bf162(w.w))); };
+            auto image_max = [&](__nv_bfloat162 m) -> uint32_t {     // value image of the larger half
+                const uint32_t lo = sortable16(as_u32(m) & 0xFFFFu), hi = sortable16(as_u32(m) >> 16);
+                return lo > hi ? lo : hi;
+            };
+            __nv_bfloat162 m2;
+            if (LSE) {
+                // sum of exp(x - c), c = the largest value of the warp's first sweep; the control warp weights the sum with
+                // the c it was taken with.  Elements past the end: 0.  Later sweeps may hold larger values: only where one
+                // is above c by more than 44 (2^64) is the sum taken again.  (Two lanes of packed fp32 arithmetic an
+                // instruction: the issue slots, not the special-function units, would be the limit otherwise.)
+                auto add8 = [&](const uint4& w, u64 (&es)[2], float c) {
+                    const u64 l2 = pack_f32x2(kTopkLog2e, kTopkLog2e), c2 = pack_f32x2(-c, -c);
+                    const uint32_t y[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 t = unpack_f32x2(mul_f32x2(add_f32x2(pack_f32x2(__uint_as_float(y[q] << 16), __uint_as_float(y[q] & 0xFFFF0000u)), c2), l2));
+                        es[q & 1] = add_f32x2(es[q & 1], pack_f32x2(topk_ex2(t.x), topk_ex2(t.y)));
+                    }
+                };
+                const uint4 w0 = load_trimmed(0);
+                m2 = max8(w0);
+                uint32_t sum_max = __reduce_max_sync(0xFFFFFFFFu, image_max(m2));
+                u64 es[2] = {0, 0};
+                float c = sum_max == kImageNegInf ? 0.f : float_of_sortable16(sum_max);
+                add8(w0, es, c);
+#pragma unroll
+                for (int it = 1; it < 8; ++it) {
+                    const uint4 w = load_trimmed(it);
+                    m2 = __hmax2(m2, max8(w));
+                    add8(w, es, c);
+                }
+                const uint32_t wmax = __reduce_max_sync(0xFFFFFFFFu, image_max(m2));
+                if (wmax != kImageNegInf && (sum_max == kImageNegInf || float_of_sortable16(wmax) - c > 44.f)) {
+                    sum_max = wmax;
+                    c = float_of_sortable16(wmax);
+                    es[0] = es[1] = 0;
+                    for (int it = 0; it < 8; ++it) add8(load_trimmed(it), es, c);
+                }
+                const float2 e2 = unpack_f32x2(add_f32x2(es[0], es[1]));
+                float sum = e2.x + e2.y;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+                if (lane == 0) { s_sum[slot][warp] = sum; s_sum_max[slot][warp] = sum_max; }
+            } else {
+                uint4 x[8];                                  // all loads first: nothing else hides their latency here
+#pragma unroll
+                for (int it = 0; it < 8; ++it) x[it] = load(it);
+                if (n_valid < kTopkChunk) {
+#pragma unroll
+                    for (int it = 0; it < 8; ++it) trim(x[it], it);
+                }
+                m2 = max8(x[0]);
+#pragma unroll
+                for (int it = 1; it < 8; ++it) m2 = __hmax2(m2, max8(x[it]));
+            }
+            const uint32_t tmax = image_max(m2);             // this thread's maximum
+            s_tmax[st][tid] = (unsigned short)tmax;
+            const uint32_t h0 = __reduce_max_sync(0xFFFFFFFFu, lane < 16 ? tmax : 0u);
+            const uint32_t h1 = __reduce_max_sync(0xFFFFFFFFu, lane < 16 ? 0u : tmax);
+            if (lane < 2) s_gmax[slot][2 * warp + lane] = ((lane ? h1 : h0) << 5) | (uint32_t)(31 - 2 * warp - lane);
+            __syncwarp();
+            if (lane == 0) topk_mbar_arrive(&s_max_done[slot]);
+            if (++chunk == chunks) chunk = 0;
+        }
+        if (!waited) pdl_wait();                             // completion of this grid implies that of the preceding one
+        return;
+    }
+
+    if (warp < kTopkDataWarps + kTopkCollectWarps) {
+        // ================================================================================ collector warps
+        const int c = warp - kTopkDataWarps;                 // looks after the data threads 128 c .. 128 c + 127
+        int chunk = (int)(w_begin % chunks);
+        for (int j = 0; j < n_local; ++j) {
+            const int st = j % kTopkStages, slot = j % kTopkSlots;
+            const unsigned short* sp = reinterpret_cast<const unsigned short*>(s_stage + st * kTopkStageBytes);
+            const int n_valid = min(chunk_elems, V - chunk * chunk_elems);
+            if (!slot_wait(s_max_done, j)) break;
+            // T: lane l counts the half-warp maxima above the l-th (distinct keys); rank k-1 holds T
+            const uint32_t v = s_gmax[slot][lane];
+            const uint2 t4 = *reinterpret_cast<const uint2*>(&s_tmax[st][128 * c + 4 * lane]);   // four threads' maxima
+            int rank = 0;
+#pragma unroll
+            for (int i = 0; i < 32; i += 4) {
+                const uint4 w4 = *reinterpret_cast<const uint4*>(&s_gmax[slot][i]);
+                rank += (w4.x > v) + (w4.y > v) + (w4.z > v) + (w4.w > v);
+            }
+            const uint32_t thr = __shfl_sync(0xFFFFFFFFu, v >> 5, __ffs(__ballot_sync(0xFFFFFFFFu, rank == k - 1)) - 1);
+            // the threads that hold an element >= T: those whose maximum is (about ten of the item's 512)
+            const uint32_t below = (1u << lane) - 1u;
+            const uint32_t tm[4] = {t4.x & 0xFFFFu, t4.x >> 16, t4.y & 0xFFFFu, t4.y >> 16};
+            int n_hold = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t b = __ballot_sync(0xFFFFFFFFu, tm[i] >= thr);
+                const int at = n_hold + __popc(b & below);
+                if (tm[i] >= thr && at < 16) s_hold[c][at] = (unsigned short)(128 * c + 4 * lane + i);
+                n_hold += __popc(b);
+            }
+            __syncwarp();
+            auto append = [&](uint32_t mask, int off) {      // keys of the elements off + (bits of mask)
+                int at = mask ? atomicAdd(&s_count[slot], __popc(mask)) : 0;
+                while (mask) {
+                    const int o = off + __ffs(mask) - 1;
+                    mask &= mask - 1;
+                    if (at < kTopkListCap) s_lists[slot * kTopkListCap + at] = (sortable16(sp[o]) << 16) | (0xFFFFu - (uint32_t)o);
+                    ++at;
+                }
+            };
+            auto valid_mask = [&](int off) -> uint32_t {     // which of the eight elements from off on exist
+                const int n = n_valid - off;
+                return n >= 8 ? 0xFFu : n > 0 ? (1u << n) - 1u : 0u;
+            };
+            bool quick = n_hold <= 16;
+            if (quick) {
+                // four holders a round, eight lanes each: lane = (holder, sweep), eight elements per lane
+                const __nv_bfloat162 t2 = as_bf162(bits_of_sortable16(thr) * 0x10001u);
+                uint32_t masks = 0;
+                for (int r = 0; 4 * r < n_hold; ++r) {
+                    const int hi = 4 * r + (lane >> 3);
+                    if (hi < n_hold) {
+                        const int off = (lane & 7) * kTopkSweep + (int)s_hold[c][hi] * 8;
+                        masks |= (topk_above<false>(*reinterpret_cast<const uint4*>(sp + off), t2) & valid_mask(off)) << (8 * r);
+                    }
+                }
+                quick = __reduce_add_sync(0xFFFFFFFFu, __popc(masks)) <= kTopkQuickList;
+                if (quick)
+                    for (int r = 0; 4 * r < n_hold; ++r) {
+                        const int hi = 4 * r + (lane >> 3);
+                        const uint32_t m = (masks >> (8 * r)) & 0xFFu;
+                        if (m) append(m, (lane & 7) * kTopkSweep + (int)s_hold[c][hi] * 8);
+                    }
+            }
+            if (!quick) {
+                // many candidates: T' = the k-th largest thread maximum (bisection over the 16-bit images), then this
+                // quarter's elements in index order, all > T' and the first k of those equal to it
+                const uint4* tp = reinterpret_cast<const uint4*>(&s_tmax[st][16 * lane]);
+                const uint4 ta = tp[0], tb = tp[1];
+                const uint32_t tw[8] = {ta.x, ta.y, ta.z, ta.w, tb.x, tb.y, tb.z, tb.w};
+                uint32_t cut = 0;
+                for (int b = 15; b >= 0; --b) {
+                    const uint32_t cand = cut | (1u << b);
+                    uint32_t n = 0;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) n += ((tw[q] & 0xFFFFu) >= cand) + ((tw[q] >> 16) >= cand);
+                    if (__reduce_add_sync(0xFFFFFFFFu, n) >= (uint32_t)k) cut = cand;
+                }
+                const __nv_bfloat162 t2 = as_bf162(bits_of_sortable16(cut) * 0x10001u);
+                int eq_left = k;
+                for (int step = 0; step < 32; ++step) {
+                    const int off = (step >> 2) * kTopkSweep + c * 1024 + (step & 3) * 256 + lane * 8;
+                    const uint4 w4 = *reinterpret_cast<const uint4*>(sp + off);
+                    const uint32_t valid = valid_mask(off);
+                    const uint32_t gt = topk_above<true>(w4, t2) & valid;
+                    uint32_t eq = topk_above<false>(w4, t2) & valid & ~gt;
+                    if (eq_left > 0 && __any_sync(0xFFFFFFFFu, eq != 0)) {
+                        int upto = __popc(eq);               // inclusive prefix over the lanes
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const int u = __shfl_up_sync(0xFFFFFFFFu, upto, o);
+                            if (lane >= o) upto += u;
+                        }
+                        int mine = min(__popc(eq), max(0, eq_left - (upto - __popc(eq))));
+                        uint32_t keep = 0;
+                        for (; mine > 0; --mine) { keep |= eq & -eq; eq &= eq - 1; }
+                        eq_left -= __shfl_sync(0xFFFFFFFFu, upto, 31);
+                        append(gt | keep, off);
+                    } else {
+                        append(gt, off);
+                    }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) topk_mbar_arrive(&s_list_done[slot]);
+            if (++chunk == chunks) chunk = 0;
+        }
+        if (!waited) pdl_wait();
+        return;
+    }
+
+    // ==================================================================================== control warp
+    const unsigned short* lg = reinterpret_cast<const unsigned short*>(logits);
+    RowCursor<COUNTS> in, cur;                               // the next item to stream, the item being finished
+    in.seek(w_begin, chunks, n_nodes, S, B);
+    cur = in;
+    // stream the next item into stage `issued` % kTopkStages (the copy is rounded up to 16 bytes, which stays inside the
+    // row because ldl is a multiple of 8 elements)
+    int issued = 0;
+    auto issue = [&]() {
+        const int base = (int)in.chunk * chunk_elems;
+        const uint32_t bytes = ((uint32_t)min(chunk_elems, V - base) * 2u + 15u) & ~15u;
+        const int st = issued % kTopkStages;
+        if (lane == 0) {
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(topk_smem_u32(&s_full[st])), "r"(bytes) : "memory");
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(topk_smem_u32(s_stage + st * kTopkStageBytes)), "l"(lg + (size_t)in.mem * ldl + base), "r"(bytes),
+                           "r"(topk_smem_u32(&s_full[st])) : "memory");
+        }
+        in.next(chunks, n_nodes, S, B);
+        ++issued;
+    };
+    while (issued < n_local && issued < kTopkStages) issue();
+
+    // the current row's k best over the chunks walked so far (lane r: r-th 64-bit key value image << 32 | ~global index;
+    // 0 = none) and its running log-sum-exp parts
     u64 run = 0;
     float run_m = -INFINITY, run_s = 0.f;
     bool part_starts_row = false;
-    // the item whose candidate list is complete but not yet ranked (warp 0 ranks it while warp 1 finds the next
-    // item's threshold): its row, chunk, chunk maximum, and the slow path's result if that path had to run
-    long long pend_row = 0;
-    int pend_chunk = -1, pend_j = 0;
-    uint32_t pend_cmax_s = 0, pend_mine = 0;
-    bool pend_has_mine = false;
 
-    // warp 0: rank the pending item's candidates, merge them into the row's list, write what is complete
-    auto finish_pending = [&]() {
-        if (!waited) { pdl_wait(); waited = true; }      // warp 0 does every global write of the CTA
-        const int n_list = s_count;
-        uint32_t mine = pend_mine;                       // lane r: the chunk's r-th winner
-        if (!pend_has_mine) {
-            if (n_list <= 32) {
-                // entries n_list..31 are zero: lane l ranks key l among the (distinct) keys
-                const uint32_t c = s_list[lane];
-                int rank = 0;
+    // rank the candidates of item i, merge them into the row's list, write what is complete
+    auto finish_item = [&](int i) {
+        const int p = i % kTopkSlots;
+        uint32_t* list = s_lists + p * kTopkListCap;
+        const int n_list = min(s_count[p], kTopkListCap);
+        uint32_t mine = 0;                               // lane r: the chunk's r-th winner
+        if (n_list <= 32) {
+            // entries n_list..31 are zero: lane l ranks key l among the (distinct) keys
+            const uint32_t c = list[lane];
+            int rank = 0;
 #pragma unroll
-                for (int i = 0; i < 32; i += 4) {
-                    const uint4 w4 = *reinterpret_cast<const uint4*>(&s_list[i]);
-                    rank += (w4.x > c) + (w4.y > c) + (w4.z > c) + (w4.w > c);
-                }
+            for (int q = 0; q < 32; q += 4) {
+                const uint4 w4 = *reinterpret_cast<const uint4*>(&list[q]);
+                rank += (w4.x > c) + (w4.y > c) + (w4.z > c) + (w4.w > c);
+            }
+            __syncwarp();
+            if (c != 0) s_sel[rank] = c;
+            __syncwarp();
+            mine = lane < min(k, n_list) ? s_sel[lane] : 0u;
+        } else {
+            for (int r = 0; r < k; ++r) {
+                uint32_t m = 0;
+                for (int q = lane; q < n_list; q += 32) m = list[q] > m ? list[q] : m;
+                const uint32_t w = __reduce_max_sync(0xFFFFFFFFu, m);
+                if (lane == r) mine = w;
+                if (w != 0)
+                    for (int q = lane; q < n_list; q += 32)
+                        if (list[q] == w) list[q] = 0;
                 __syncwarp();
-                if (c != 0) s_sel[rank] = c;
-                __syncwarp();
-                mine = lane < min(k, n_list) ? s_sel[lane] : 0u;
-            } else {
-                for (int r = 0; r < k; ++r) {
-                    uint32_t m = 0;
-                    for (int i = lane; i < n_list; i += 32) m = s_list[i] > m ? s_list[i] : m;
-                    const uint32_t w = __reduce_max_sync(0xFFFFFFFFu, m);
-                    if (lane == r) mine = w;
-                    if (w != 0)
-                        for (int i = lane; i < n_list; i += 32)
-                            if (s_list[i] == w) s_list[i] = 0;
-                    __syncwarp();
-                }
             }
         }
         __syncwarp();
-        s_list[lane] = 0;                                // entries 0..31 are zero between items
-        if (lane == 0) s_count = 0;
+        list[lane] = 0;                                  // entries 0..31 are zero between items
+        if (lane == 0) s_count[p] = 0;
 
-        const int base = pend_chunk * kTopkChunk;
+        const long long row = cur.row;
+        const int chunk = (int)cur.chunk, base = chunk * chunk_elems;
+        const size_t out_row = (size_t)cur.mem;
+        cur.next(chunks, n_nodes, S, B);
         float csum = 0.f;
-        const float cmax = LSE ? __uint_as_float(bits_of_sortable16(pend_cmax_s) << 16) : 0.f;
+        const float cmax = LSE ? float_of_sortable16(__reduce_max_sync(0xFFFFFFFFu, s_gmax[p][lane]) >> 5) : 0.f;
         if (LSE) {
-            csum = s_sum[lane];
+            // warp w's sum is relative to its c_w: weight exp(c_w - cmax)
+            if (lane < kTopkDataWarps) {
+                const uint32_t m = s_sum_max[p][lane];
+                if (m != kImageNegInf) csum = s_sum[p][lane] * topk_ex2((float_of_sortable16(m) - cmax) * kTopkLog2e);   // else: -inf alone
+            }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) csum += __shfl_xor_sync(0xFFFFFFFFu, csum, o);
         }
         if (chunks == 1) {                               // the chunk is the row: write it out
-            const size_t out_row = (size_t)row_of(pend_row);
             if (lane < k) {
                 const int32_t id = (int32_t)(0xFFFFu - (mine & 0xFFFFu));
                 ids[out_row * k + lane] = id;
@@ -225,9 +516,9 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
             if (LSE && lane == 0) row_lse[out_row] = cmax + logf(csum);
             return;
         }
-        const bool part_begins = (pend_j == 0) || (pend_chunk == 0);
-        const bool part_ends = (pend_j == n_local - 1) || (pend_chunk == chunks - 1);
-        if (part_begins) part_starts_row = (pend_chunk == 0);
+        const bool part_begins = (i == 0) || (chunk == 0);
+        const bool part_ends = (i == n_local - 1) || (chunk == chunks - 1);
+        if (part_begins) part_starts_row = (chunk == 0);
         // this chunk's winners as 64-bit keys of the row
         const u64 ck = mine ? (((u64)(mine >> 16) << 32) | (u64)(0xFFFFFFFFu - (uint32_t)(base + (int)(0xFFFFu - (mine & 0xFFFFu))))) : 0ull;
         if (part_begins) {
@@ -243,8 +534,8 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
             __syncwarp();
             int rank = 0;
 #pragma unroll
-            for (int i = 0; i < 32; i += 2) {
-                const ulonglong2 w2 = *reinterpret_cast<const ulonglong2*>(&s_m64[i]);
+            for (int q = 0; q < 32; q += 2) {
+                const ulonglong2 w2 = *reinterpret_cast<const ulonglong2*>(&s_m64[q]);
                 rank += (w2.x > cand) + (w2.y > cand);
             }
             if (cand != 0 && rank < k) s_run[rank] = cand;
@@ -260,7 +551,7 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
         if (!part_ends) return;
         u64 win = run;
         float fin_m = run_m, fin_s = run_s;
-        if (!(part_starts_row && pend_chunk == chunks - 1)) {
+        if (!(part_starts_row && chunk == chunks - 1)) {
             // the row's chunks are spread over several CTAs: CTAs c_first..c_last each hold one part
             auto cta_of = [&](long long w) -> int {      // the CTA whose range contains item w
                 int c = (int)((w * G) / items);
@@ -268,21 +559,21 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
                 while (c > 0 && items * c / G > w) --c;
                 return c;
             };
-            const int c_first = cta_of(pend_row * chunks), c_last = cta_of(pend_row * chunks + chunks - 1);
+            const int c_first = cta_of(row * chunks), c_last = cta_of(row * chunks + chunks - 1);
             const int n_parts = c_last - c_first + 1, slot = (int)blockIdx.x - c_first;
-            u64* dst = ws_cand + ((size_t)pend_row * chunks + slot) * kMaxK;
+            u64* dst = ws_cand + ((size_t)row * chunks + slot) * kMaxK;
             if (lane < k) dst[lane] = run;
-            if (LSE && lane == 0) ws_lse[(size_t)pend_row * chunks + slot] = make_float2(run_m, run_s);
+            if (LSE && lane == 0) ws_lse[(size_t)row * chunks + slot] = make_float2(run_m, run_s);
             __threadfence();
             __syncwarp();
             if (lane == 0) {
-                const int old = atomicAdd(&row_counters[pend_row], 1);
+                const int old = atomicAdd(&row_counters[row], 1);
                 s_last = (old == n_parts - 1);
             }
             __syncwarp();
             if (!s_last) return;
             __threadfence();
-            const u64* src = ws_cand + (size_t)pend_row * chunks * kMaxK;
+            const u64* src = ws_cand + (size_t)row * chunks * kMaxK;
             const int n = n_parts * k;
             if (n <= 32) {
                 const u64 cand = lane < n ? __ldcg(src + (size_t)(lane / k) * kMaxK + (lane % k)) : 0ull;
@@ -291,8 +582,8 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
                 __syncwarp();
                 int rank = 0;
 #pragma unroll
-                for (int i = 0; i < 32; i += 2) {
-                    const ulonglong2 w2 = *reinterpret_cast<const ulonglong2*>(&s_m64[i]);
+                for (int q = 0; q < 32; q += 2) {
+                    const ulonglong2 w2 = *reinterpret_cast<const ulonglong2*>(&s_m64[q]);
                     rank += (w2.x > cand) + (w2.y > cand);
                 }
                 if (cand != 0 && rank < k) s_run[rank] = cand;
@@ -300,33 +591,32 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
                 win = lane < k ? s_run[lane] : 0ull;
                 __syncwarp();
             } else {
-                for (int i = lane; i < n; i += 32) s_merge[i] = __ldcg(src + (size_t)(i / k) * kMaxK + (i % k));
+                for (int q = lane; q < n; q += 32) s_merge[q] = __ldcg(src + (size_t)(q / k) * kMaxK + (q % k));
                 __syncwarp();
                 win = 0;
                 for (int r = 0; r < k; ++r) {
                     u64 m = 0;
-                    for (int i = lane; i < n; i += 32) m = s_merge[i] > m ? s_merge[i] : m;
+                    for (int q = lane; q < n; q += 32) m = s_merge[q] > m ? s_merge[q] : m;
                     const u64 w = warp_max_u64(m);
                     if (lane == r) win = w;
                     if (w != 0)
-                        for (int i = lane; i < n; i += 32)
-                            if (s_merge[i] == w) s_merge[i] = 0;
+                        for (int q = lane; q < n; q += 32)
+                            if (s_merge[q] == w) s_merge[q] = 0;
                     __syncwarp();
                 }
             }
-            if (lane == 0) row_counters[pend_row] = 0;   // ready for the next launch
+            if (lane == 0) row_counters[row] = 0;        // ready for the next launch
             if (LSE && lane == 0) {
                 float M = -INFINITY;
-                for (int c = 0; c < n_parts; ++c) M = fmaxf(M, __ldcg(&ws_lse[(size_t)pend_row * chunks + c]).x);
+                for (int c = 0; c < n_parts; ++c) M = fmaxf(M, __ldcg(&ws_lse[(size_t)row * chunks + c]).x);
                 float sum = 0.f;
                 for (int c = 0; c < n_parts; ++c) {
-                    const float2 ms = __ldcg(&ws_lse[(size_t)pend_row * chunks + c]);
+                    const float2 ms = __ldcg(&ws_lse[(size_t)row * chunks + c]);
                     sum += ms.y * expf(ms.x - M);
                 }
                 fin_m = M; fin_s = sum;
             }
         }
-        const size_t out_row = (size_t)row_of(pend_row);
         if (lane < k) {
             const int32_t id = (int32_t)(0xFFFFFFFFu - (uint32_t)(win & 0xFFFFFFFFull));
             ids[out_row * k + lane] = id;
@@ -337,205 +627,44 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
     };
 
     for (int j = 0; j < n_local; ++j) {
-        const int st = j % kTopkStages;
-        const int base = chunk * kTopkChunk;
-        const int n_valid = min(kTopkChunk, V - base);
-        const unsigned char* sp = s_stage + st * kTopkStageBytes;
-        // a wait that runs out raises the CTA's abort flag; everybody learns of it behind the next barrier
-        const bool have = mbar_wait_bounded(&s_full[st], (uint32_t)(j / kTopkStages) & 1u, kTopkWaitCycles, &s_abort) == 0;
-        if (!have) s_abort = 1;
-
-        // ---- phase 1: 32 values per thread into registers (element (it, e) of thread tid sits at chunk offset
-        //      it*8192 + tid*8 + e); elements past the row's end read as -inf; thread maximum with packed bf16 max
-        uint32_t x[16];
-        if (have) {
-#pragma unroll
-            for (int it = 0; it < 4; ++it) {
-                const uint4 v4 = *reinterpret_cast<const uint4*>(sp + (size_t)(it * (kTopkThreads * 8) + tid * 8) * 2);
-                x[4 * it] = v4.x; x[4 * it + 1] = v4.y; x[4 * it + 2] = v4.z; x[4 * it + 3] = v4.w;
-            }
-            if (n_valid < kTopkChunk) {
-#pragma unroll
-                for (int it = 0; it < 4; ++it) {
-                    const int off0 = it * (kTopkThreads * 8) + tid * 8;
-                    if (off0 + 8 > n_valid) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const uint32_t lo = (off0 + 2 * q < n_valid) ? (x[4 * it + q] & 0xFFFFu) : 0xFF80u;
-                            const uint32_t hi = (off0 + 2 * q + 1 < n_valid) ? (x[4 * it + q] >> 16) : 0xFF80u;
-                            x[4 * it + q] = lo | (hi << 16);
-                        }
-                    }
-                }
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < 16; ++q) x[q] = 0xFF80FF80u;
+        const bool have = slot_wait(s_list_done, j);     // (implies the maxima and sums: the collectors waited for them)
+        if (have && issued < n_local) {                  // nobody reads item j's stage any more
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            issue();
         }
-        __nv_bfloat162 m2 = __hmax2(as_bf162(x[0]), as_bf162(x[1]));
-#pragma unroll
-        for (int q = 2; q < 16; q += 2) m2 = __hmax2(m2, __hmax2(as_bf162(x[q]), as_bf162(x[q + 1])));
-        const uint32_t mw = as_u32(m2);
-        const uint32_t s_lo = sortable16(mw & 0xFFFFu), s_hi = sortable16(mw >> 16);
-        const uint32_t tmax = s_lo > s_hi ? s_lo : s_hi;   // this thread's maximum (16-bit value image)
-        const uint32_t wmax = __reduce_max_sync(0xFFFFFFFFu, tmax);
-        if (lane == 0) s_wmax[warp] = (wmax << 5) | (uint32_t)(31 - warp);
-        __syncthreads();
-        if (s_abort) {
-            // give up as one: report, wait (bounded) for this thread's copies still in flight, return
-            if (!waited) pdl_wait();                     // completion of this grid must imply that of the preceding one
-            if (tid == 0) {
+        if (!waited) { pdl_wait(); waited = true; }      // this warp does every global write of the CTA
+        if (!have) {
+            // give up: report, wait (bounded) for the copies still in flight, return
+            if (lane == 0) {
                 if (status) atomicOr(status, GOOSE_ST_TIMEOUT);
                 volatile int no_abort = 0;               // draining ignores the abort flag
                 for (int jj = j; jj < issued; ++jj)
                     mbar_wait_bounded(&s_full[jj % kTopkStages], (uint32_t)(jj / kTopkStages) & 1u, kTopkWaitCycles, &no_abort);
             }
-            return;
+            break;
         }
-
-        // ---- phase 2, two warps side by side.  Warp 1: T = the k-th largest warp maximum -- lane l counts the warp
-        //      maxima above warp l's (the keys are distinct), the lane of rank k-1 holds T.  The k largest warp
-        //      maxima are k different elements >= T, hence every one of the chunk's k best is >= T.
-        //      Warp 0: ranks the previous item's candidates.
-        if (warp == 1) {
-            const uint32_t mykey = s_wmax[lane];
-            int rank = 0;
-#pragma unroll
-            for (int i = 0; i < 32; i += 4) {
-                const uint4 w4 = *reinterpret_cast<const uint4*>(&s_wmax[i]);
-                rank += (w4.x > mykey) + (w4.y > mykey) + (w4.z > mykey) + (w4.w > mykey);
-            }
-            if (rank == k - 1) s_thresh = mykey >> 5;
-            if (rank == 0) s_cmax = mykey >> 5;          // the chunk's maximum
-        } else if (warp == 0 && pend_chunk >= 0) {
-            finish_pending();
-        }
-        __syncthreads();
-        const uint32_t thr_s = s_thresh, cmax_s = s_cmax;
-
-        // ---- phase 3: every element >= T becomes a full key (value image << 16 | 0xFFFF - index in chunk).
-        //      A thread holds such an element exactly when its maximum is >= T (about ten threads of the CTA); the
-        //      warp then looks at that thread's 32 elements together, one lane per element, in the stage.
-        float esum = 0.f;
-        const float cmax = LSE ? __uint_as_float(bits_of_sortable16(cmax_s) << 16) : 0.f;
-        if (LSE) {                                       // elements past the row's end are -inf: exp gives 0
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                esum += exp2f((__uint_as_float(x[q] << 16) - cmax) * 1.4426950408889634f);
-                esum += exp2f((__uint_as_float(x[q] & 0xFFFF0000u) - cmax) * 1.4426950408889634f);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) esum += __shfl_xor_sync(0xFFFFFFFFu, esum, o);
-            if (lane == 0) s_sum[warp] = esum;
-        }
-        uint32_t holders = __ballot_sync(0xFFFFFFFFu, tmax >= thr_s);
-        while (holders) {
-            const int src_tid = (warp << 5) + __ffs(holders) - 1;
-            holders &= holders - 1;
-            const int off = (lane >> 3) * (kTopkThreads * 8) + src_tid * 8 + (lane & 7);
-            const uint32_t sv = sortable16(reinterpret_cast<const unsigned short*>(sp)[off]);
-            const bool pass = off < n_valid && sv >= thr_s;
-            const uint32_t pm = __ballot_sync(0xFFFFFFFFu, pass);
-            int pos0 = 0;
-            if (lane == 0) pos0 = atomicAdd(&s_count, __popc(pm));
-            pos0 = __shfl_sync(0xFFFFFFFFu, pos0, 0);
-            if (pass) {
-                const int pos = pos0 + __popc(pm & ((1u << lane) - 1u));
-                if (pos < kTopkListCap) s_list[pos] = (sv << 16) | (0xFFFFu - (uint32_t)off);
-            }
-        }
-        __syncthreads();
-        // every thread is done with the stage: fetch the item three ahead into it
-        if (tid == 0 && issued < n_local) {
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            issue(issued);
-            ++issued;
-        }
-        pend_row = row; pend_chunk = chunk; pend_j = j; pend_cmax_s = cmax_s;
-        pend_has_mine = false; pend_mine = 0;
-
-        if (s_count > kTopkListCap) {
-            // ---- slow path (more than kTopkListCap elements tie at or above T, e.g. a constant row): exact rounds
-            //      on full keys, rebuilt from the registers whenever a lane needs its next best.
-            // largest key of this thread strictly below `bound` (all keys are distinct)
-            auto best_below = [&](uint32_t bound) -> uint32_t {
-                uint32_t nb = 0;
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    const int off = (q >> 2) * (kTopkThreads * 8) + tid * 8 + (q & 3) * 2;
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const uint32_t bits = e ? (x[q] >> 16) : (x[q] & 0xFFFFu);
-                        const uint32_t kk = (off + e < n_valid) ? ((sortable16(bits) << 16) | (0xFFFFu - (uint32_t)(off + e))) : 0u;
-                        nb = (kk < bound && kk > nb) ? kk : nb;
-                    }
-                }
-                return nb;
-            };
-            uint32_t best = best_below(0xFFFFFFFFu);
-            for (int r = 0; r < k; ++r) {
-                const uint32_t w = __reduce_max_sync(0xFFFFFFFFu, best);
-                if (lane == 0) s_cand[warp * KCAP + r] = w;
-                if (best == w && w != 0) best = best_below(w);
-            }
-            __syncthreads();
-            if (warp == 0) {
-                uint32_t c[KCAP];
-                uint32_t lm = 0;
-#pragma unroll
-                for (int i = 0; i < KCAP; ++i) {
-                    c[i] = (i < k) ? s_cand[lane * KCAP + i] : 0u;
-                    lm = c[i] > lm ? c[i] : lm;
-                }
-                for (int r = 0; r < k; ++r) {
-                    uint32_t w = __reduce_max_sync(0xFFFFFFFFu, lm);
-                    if (lane == r) pend_mine = w;
-                    if (lm == w && w != 0) {
-                        uint32_t nb = 0;
-#pragma unroll
-                        for (int i = 0; i < KCAP; ++i) {
-                            c[i] = (c[i] == w) ? 0u : c[i];
-                            nb = c[i] > nb ? c[i] : nb;
-                        }
-                        lm = nb;
-                    }
-                }
-            }
-            pend_has_mine = true;
-            __syncthreads();                             // s_cand is reused by the next slow item
-        }
-        if (++chunk == chunks) { chunk = 0; ++row; }
+        finish_item(j);
     }
-    if (warp == 0 && pend_chunk >= 0) finish_pending();  // the CTA's last item
-    if (!waited) pdl_wait();                             // a CTA without items, or the warps that wrote nothing
+    if (!waited) pdl_wait();                             // a CTA without items
 }
 
 namespace {
-template <int KCAP, bool LSE>
-cudaError_t launch_topk_inst(int grid, cudaStream_t st, const __nv_bfloat16* logits, long long items, int V, int64_t ldl,
-                             int k, int chunks, u64* ws, int32_t* counters, int32_t* argmax, int32_t* ids, float* vals,
-                             float* row_lse, float2* ws_lse, int32_t* status, int inputs_ready, const int32_t* n_nodes, int S,
-                             int B) {
-    return launch_pdl(n_nodes ? node_topk_kernel<KCAP, LSE, true> : node_topk_kernel<KCAP, LSE, false>, dim3(grid),
-                      dim3(kTopkThreads), kTopkSmem, st, logits, items, V, ldl, k,
-                      chunks, ws, counters, argmax, ids, vals, row_lse, ws_lse, status, inputs_ready, n_nodes, S, B);
-}
-
 cudaError_t launch_topk_any(int num_sms, cudaStream_t st, const __nv_bfloat16* logits, int rows, int V, int64_t ldl, int k,
                             u64* ws, int32_t* counters, int32_t* argmax, int32_t* ids, float* vals, float* row_lse,
                             float2* ws_lse, int32_t* status, int inputs_ready, const int32_t* n_nodes = nullptr, int B = 0) {
     const int S = (n_nodes && B > 0) ? rows / B : 0;
+    // equal chunks (a multiple of 8 elements: every copy starts on 16 bytes), so that no item is a remainder
     const int chunks = (V + kTopkChunk - 1) / kTopkChunk;
+    const int chunk_elems = ((V + chunks - 1) / chunks + 7) & ~7;
     const long long items = (long long)rows * chunks;
     // every CTA gets q = ceil(items / SMs) items or one fewer; using the fewest CTAs that q allows loses no time and
     // makes the ranges fall on row boundaries when q is a multiple of the chunks per row (no cross-CTA merges then)
     const long long q = (items + num_sms - 1) / num_sms;
     const int grid = (int)((items + q - 1) / q);
-    if (row_lse)
-        return k <= 8 ? launch_topk_inst<8, true>(grid, st, logits, items, V, ldl, k, chunks, ws, counters, argmax, ids, vals, row_lse, ws_lse, status, inputs_ready, n_nodes, S, B)
-                      : launch_topk_inst<16, true>(grid, st, logits, items, V, ldl, k, chunks, ws, counters, argmax, ids, vals, row_lse, ws_lse, status, inputs_ready, n_nodes, S, B);
-    return k <= 8 ? launch_topk_inst<8, false>(grid, st, logits, items, V, ldl, k, chunks, ws, counters, argmax, ids, vals, row_lse, ws_lse, status, inputs_ready, n_nodes, S, B)
-                  : launch_topk_inst<16, false>(grid, st, logits, items, V, ldl, k, chunks, ws, counters, argmax, ids, vals, row_lse, ws_lse, status, inputs_ready, n_nodes, S, B);
+    auto kernel = row_lse ? (n_nodes ? node_topk_kernel<true, true> : node_topk_kernel<true, false>)
+                          : (n_nodes ? node_topk_kernel<false, true> : node_topk_kernel<false, false>);
+    return launch_pdl(kernel, dim3(grid), dim3(kTopkThreads), kTopkSmem, st, logits, items, V, ldl, k, chunks, chunk_elems, ws,
+                      counters, argmax, ids, vals, row_lse, ws_lse, status, inputs_ready, n_nodes, S, B);
 }
 }  // namespace
 
@@ -546,10 +675,8 @@ cudaError_t init_topk_kernel() {
     auto opt_in = [&](const void* fn) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopkSmem);
     };
-    opt_in((const void*)node_topk_kernel<8, false, false>);  opt_in((const void*)node_topk_kernel<8, false, true>);
-    opt_in((const void*)node_topk_kernel<16, false, false>); opt_in((const void*)node_topk_kernel<16, false, true>);
-    opt_in((const void*)node_topk_kernel<8, true, false>);   opt_in((const void*)node_topk_kernel<8, true, true>);
-    opt_in((const void*)node_topk_kernel<16, true, false>);  opt_in((const void*)node_topk_kernel<16, true, true>);
+    opt_in((const void*)node_topk_kernel<false, false>);  opt_in((const void*)node_topk_kernel<false, true>);
+    opt_in((const void*)node_topk_kernel<true, false>);   opt_in((const void*)node_topk_kernel<true, true>);
     return e;
 }
 

@@ -1,0 +1,74 @@
+"""GPU parity of the top-k's candidate selection where it can go wrong: rows with many elements at or above the
+threshold, chunk lengths at the edges of a thread's, a sweep's and a chunk's share, masked rows, and row log-sum-exps whose
+largest value comes late, far above the first sweep's, or not at all.  Identifiers and values bit-exact against the oracle;
+the log-sum-exp against numpy in 64 bits: fp32 sums of at most 2^18 terms in chains of at most 64, then trees, hence
+|error| <= (64 + 20) 2^-24 + 2 ulp of ex2.approx (2^-22) = 6e-6, plus half an ulp of the largest |lse| here (2^-17)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2604_02047_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+NEG_INF, LOWEST = 0xFF80, 0xFF7F
+
+
+@pytest.fixture(scope="module")
+def goose():
+    from paper_2604_02047_b200 import binding, build
+    build.build()
+    g = binding.Goose(max_S=2, max_B=128, max_H=4)
+    yield g
+    g.close()
+
+
+def _rows(V, rng):
+    """bf16 bit patterns, one row per kind."""
+    bf = synth.f32_to_bf16_bits
+    noise = lambda: bf(rng.standard_normal(V).astype(np.float32))  # noqa: E731
+    rows = [noise(), np.full(V, bf(np.float32([2.5]))[0], np.uint16)]
+    rows += [bf(np.sort(rng.standard_normal(V)).astype(np.float32)), bf(-np.sort(rng.standard_normal(V)).astype(np.float32))]
+    rows.append(bf(rng.integers(0, 2, V).astype(np.float32)))                       # half the row ties at the top
+    for lo, n in ((V // 2, 1200), (0, 900), (max(0, V - 1500), 1500), (V // 3, 5000)):   # a band far above the rest
+        r = noise()
+        band = r[lo:lo + n]
+        band[:] = bf((50 + 4 * rng.standard_normal(len(band))).astype(np.float32))
+        rows.append(r)
+    for mask in (NEG_INF, LOWEST):
+        r = np.full(V, mask, np.uint16)                                             # all but a few masked; the last one too
+        keep = rng.choice(V, min(V, 5), replace=False)
+        r[keep] = bf(rng.standard_normal(len(keep)).astype(np.float32))
+        rows.append(r)
+        r = noise()
+        r[:V // 2] = mask
+        rows.append(r)
+    r = noise()
+    r[V - 1] = bf(np.float32([90.0]))[0]                                           # the largest comes last, far above
+    rows.append(r)
+    rows.append(bf((rng.standard_normal(V) * 1e4).astype(np.float32)))
+    return np.stack(rows)
+
+
+@pytest.mark.parametrize("k", [1, 8, 16])
+@pytest.mark.parametrize("V", [16, 248, 4096, 4104, 32000, 32768, 32776, 70008, 128256, 262144])
+def test_candidates_of_odd_rows(goose, oracle, V, k):
+    rng = np.random.default_rng([V, k])
+    bits = _rows(V, rng)
+    rows = len(bits)
+    x = torch.from_numpy(bits.view(np.int16)).view(torch.bfloat16).cuda()
+    ref_am, ref_ids, ref_vals = oracle.node_topk(bits, k)
+    am, ids, vals = goose.node_topk(x, k)
+    adj_ids = torch.zeros((rows, k), dtype=torch.int32, device="cuda")
+    adj_sc = torch.zeros((rows, k), dtype=torch.float32, device="cuda")
+    am2, ids2, vals2, lse = goose.harvest(x, k, torch.arange(rows, dtype=torch.int32, device="cuda"), adj_ids, adj_sc)
+    torch.cuda.synchronize()
+    for a, i, v in ((am, ids, vals), (am2, ids2, vals2)):
+        assert np.array_equal(i.cpu().numpy(), ref_ids) and np.array_equal(a.cpu().numpy(), ref_am)
+        assert np.array_equal(v.cpu().numpy().astype(np.float64), ref_vals)
+    wide = x.double().cpu().numpy()
+    top = wide.max(axis=1)
+    ref = top + np.log(np.exp(wide - top[:, None]).sum(axis=1))
+    got = lse.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(got - ref) <= 6e-6 + np.abs(ref) * 2.0 ** -23), (got - ref)
+    assert goose.last_status(2).tolist() == [0, 0]
