@@ -115,17 +115,17 @@ __device__ __forceinline__ uint32_t topk_above(const uint4& w, __nv_bfloat162 t)
 // a walk over the rows that exist: rows of the call, or with node counts the rows of nodes that exist, numbered densely
 template <bool COUNTS>
 struct RowCursor {
-    long long row, chunk;      // current item: dense row number and chunk in it
+    int row, chunk;            // current item: dense row number and chunk in it
     long long mem;             // the row's place in memory
     int s, left;               // its sequence, and the existing rows of that sequence from this one on
-    __device__ __forceinline__ void seek(long long w, int chunks, const int32_t* n_nodes, int S, int B) {
+    __device__ __forceinline__ void seek(int w, int chunks, const int32_t* n_nodes, int S, int B) {
         row = w / chunks; chunk = w - row * chunks;
         mem = row; s = 0; left = 0;
         if (COUNTS) {
-            long long r = row;
+            int r = row;
             for (; s < S; ++s) {
                 const int n = nodes_of(n_nodes, s, B);
-                if (r < n) { mem = (long long)s * B + r; left = n - (int)r; return; }
+                if (r < n) { mem = (long long)s * B + r; left = n - r; return; }
                 r -= n;
             }
             mem = 0;                                         // behind the last row (a CTA without items): not used
@@ -147,7 +147,7 @@ struct RowCursor {
 // COUNTS = false is the instantiation for n_nodes == NULL (the item list is known before the dependency wait)
 template <bool LSE, bool COUNTS>
 __global__ void __launch_bounds__(kTopkThreads, 1)
-node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, int V, int64_t ldl, int k, int chunks,
+node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V, int64_t ldl, int k, int chunks,
                  int chunk_elems, u64* __restrict__ ws_cand, int32_t* __restrict__ row_counters,
                  int32_t* __restrict__ argmax, int32_t* __restrict__ ids, float* __restrict__ vals,
                  float* __restrict__ row_lse, float2* __restrict__ ws_lse, int32_t* __restrict__ status,
@@ -173,21 +173,26 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = gridDim.x;
     if (!COUNTS) n_nodes = nullptr;
-    long long items = items_all;
-    long long w_begin = items * blockIdx.x / G, w_end = items * (blockIdx.x + 1) / G;   // final when !COUNTS
-    if (tid == 0) {
+    const bool control = warp == kTopkThreads / 32 - 1;
+    if (control && lane == 0) {
         for (int i = 0; i < kTopkStages; ++i) topk_mbar_init(&s_full[i], 1);
-        for (int i = 0; i < kTopkSlots; ++i) {
-            topk_mbar_init(&s_max_done[i], kTopkDataWarps);
-            topk_mbar_init(&s_list_done[i], kTopkCollectWarps);
-            s_count[i] = 0;
-        }
-        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (tid < kTopkSlots) {
+        topk_mbar_init(&s_max_done[tid], kTopkDataWarps);
+        topk_mbar_init(&s_list_done[tid], kTopkCollectWarps);
+        s_count[tid] = 0;
+        if (tid == 0) s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (tid < 32)
-        for (int i = 0; i < kTopkSlots; ++i) s_lists[i * kTopkListCap + tid] = 0;
-    __syncthreads();
+    if (warp == 1)
+        for (int i = 0; i < kTopkSlots; ++i) s_lists[i * kTopkListCap + lane] = 0;
+    // CTA c's items: the first `more` CTAs have per + 1 of them, the others per (32-bit arithmetic throughout: 64-bit
+    // divisions in front of the first copy and barrier set-up by one thread had cost 0.5 us a call)
+    int items = items_all, per = items_all / G, more = items_all - per * G;   // final when !COUNTS
+    auto cta_start = [&](int c) { return c * per + min(c, more); };
+    auto cta_of = [&](int w) { return w < more * (per + 1) ? w / (per + 1) : more + (w - more * (per + 1)) / per; };
     // inputs_ready: the caller guarantees that the logits were complete before the preceding kernel in the stream
     // started (the whole-step call: that kernel is the attention kernel, which neither reads nor writes them).  The
     // CTA then streams and selects at once and only waits for the preceding kernel before its first write to global
@@ -200,12 +205,37 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
     // the rows that exist, numbered densely (the cross-CTA scratch is indexed by that number).  n_nodes[] is an input
     // like the logits: it may be read ahead of the dependency wait.
     if (COUNTS && n_nodes) {
-        long long live = 0;
+        int live = 0;
         for (int s = 0; s < S; ++s) live += nodes_of(n_nodes, s, B);
         items = live * chunks;
-        w_begin = items * blockIdx.x / G; w_end = items * (blockIdx.x + 1) / G;
+        per = items / G; more = items - per * G;
     }
-    const int n_local = (int)(w_end - w_begin);
+    const int w_begin = cta_start(blockIdx.x), n_local = cta_start(blockIdx.x + 1) - w_begin;
+
+    // control warp: the next item to stream; its first copies leave before the rest of the CTA is set up
+    const unsigned short* lg = reinterpret_cast<const unsigned short*>(logits);
+    RowCursor<COUNTS> in{};
+    int issued = 0;
+    // stream the next item into stage `issued` % kTopkStages (the copy is rounded up to 16 bytes, which stays inside the
+    // row because ldl is a multiple of 8 elements)
+    auto issue = [&]() {
+        const int base = in.chunk * chunk_elems;
+        const uint32_t bytes = ((uint32_t)min(chunk_elems, V - base) * 2u + 15u) & ~15u;
+        const int st = issued % kTopkStages;
+        if (lane == 0) {
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(topk_smem_u32(&s_full[st])), "r"(bytes) : "memory");
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(topk_smem_u32(s_stage + st * kTopkStageBytes)), "l"(lg + (size_t)in.mem * ldl + base), "r"(bytes),
+                           "r"(topk_smem_u32(&s_full[st])) : "memory");
+        }
+        in.next(chunks, n_nodes, S, B);
+        ++issued;
+    };
+    if (control) {
+        in.seek(w_begin, chunks, n_nodes, S, B);
+        while (issued < n_local && issued < kTopkStages) issue();
+    }
+    __syncthreads();
 
     // bounded wait for item j's hand-over in its slot; a wait that runs out raises the CTA's abort flag, which ends the
     // waits of all other warps
@@ -217,7 +247,7 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
 
     if (warp < kTopkDataWarps) {
         // ================================================================================ data warps
-        int chunk = (int)(w_begin % chunks);
+        int chunk = w_begin % chunks;
         for (int j = 0; j < n_local; ++j) {
             const int st = j % kTopkStages, slot = j % kTopkSlots;
             const unsigned char* sp = s_stage + st * kTopkStageBytes;
@@ -319,7 +349,7 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
     if (warp < kTopkDataWarps + kTopkCollectWarps) {
         // ================================================================================ collector warps
         const int c = warp - kTopkDataWarps;                 // looks after the data threads 128 c .. 128 c + 127
-        int chunk = (int)(w_begin % chunks);
+        int chunk = w_begin % chunks;
         for (int j = 0; j < n_local; ++j) {
             const int st = j % kTopkStages, slot = j % kTopkSlots;
             const unsigned short* sp = reinterpret_cast<const unsigned short*>(s_stage + st * kTopkStageBytes);
@@ -428,34 +458,18 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
     }
 
     // ==================================================================================== control warp
-    const unsigned short* lg = reinterpret_cast<const unsigned short*>(logits);
-    RowCursor<COUNTS> in, cur;                               // the next item to stream, the item being finished
-    in.seek(w_begin, chunks, n_nodes, S, B);
-    cur = in;
-    // stream the next item into stage `issued` % kTopkStages (the copy is rounded up to 16 bytes, which stays inside the
-    // row because ldl is a multiple of 8 elements)
-    int issued = 0;
-    auto issue = [&]() {
-        const int base = (int)in.chunk * chunk_elems;
-        const uint32_t bytes = ((uint32_t)min(chunk_elems, V - base) * 2u + 15u) & ~15u;
-        const int st = issued % kTopkStages;
-        if (lane == 0) {
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(topk_smem_u32(&s_full[st])), "r"(bytes) : "memory");
-            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                         ::"r"(topk_smem_u32(s_stage + st * kTopkStageBytes)), "l"(lg + (size_t)in.mem * ldl + base), "r"(bytes),
-                           "r"(topk_smem_u32(&s_full[st])) : "memory");
-        }
-        in.next(chunks, n_nodes, S, B);
-        ++issued;
-    };
-    while (issued < n_local && issued < kTopkStages) issue();
-
+    RowCursor<COUNTS> cur;                                   // the item being finished
+    cur.seek(w_begin, chunks, n_nodes, S, B);
     // the current row's k best over the chunks walked so far (lane r: r-th 64-bit key value image << 32 | ~global index;
     // 0 = none) and its running log-sum-exp parts
     u64 run = 0;
     float run_m = -INFINITY, run_s = 0.f;
     bool part_starts_row = false;
 
+    // this warp does every global write of the CTA, none of them ahead of the dependency wait
+    auto wait_once = [&]() {
+        if (!waited) { pdl_wait(); waited = true; }
+    };
     // rank the candidates of item i, merge them into the row's list, write what is complete
     auto finish_item = [&](int i) {
         const int p = i % kTopkSlots;
@@ -491,8 +505,7 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
         list[lane] = 0;                                  // entries 0..31 are zero between items
         if (lane == 0) s_count[p] = 0;
 
-        const long long row = cur.row;
-        const int chunk = (int)cur.chunk, base = chunk * chunk_elems;
+        const int row = cur.row, chunk = cur.chunk, base = chunk * chunk_elems;
         const size_t out_row = (size_t)cur.mem;
         cur.next(chunks, n_nodes, S, B);
         float csum = 0.f;
@@ -507,13 +520,15 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
             for (int o = 16; o > 0; o >>= 1) csum += __shfl_xor_sync(0xFFFFFFFFu, csum, o);
         }
         if (chunks == 1) {                               // the chunk is the row: write it out
+            const float row_sum = LSE ? cmax + logf(csum) : 0.f;
+            wait_once();
             if (lane < k) {
                 const int32_t id = (int32_t)(0xFFFFu - (mine & 0xFFFFu));
                 ids[out_row * k + lane] = id;
                 if (vals) vals[out_row * k + lane] = value_of_sortable16(mine >> 16);
                 if (lane == 0) argmax[out_row] = id;
             }
-            if (LSE && lane == 0) row_lse[out_row] = cmax + logf(csum);
+            if (LSE && lane == 0) row_lse[out_row] = row_sum;
             return;
         }
         const bool part_begins = (i == 0) || (chunk == 0);
@@ -549,16 +564,11 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
             }
         }
         if (!part_ends) return;
+        wait_once();
         u64 win = run;
         float fin_m = run_m, fin_s = run_s;
         if (!(part_starts_row && chunk == chunks - 1)) {
             // the row's chunks are spread over several CTAs: CTAs c_first..c_last each hold one part
-            auto cta_of = [&](long long w) -> int {      // the CTA whose range contains item w
-                int c = (int)((w * G) / items);
-                while (c + 1 < G && items * (c + 1) / G <= w) ++c;
-                while (c > 0 && items * c / G > w) --c;
-                return c;
-            };
             const int c_first = cta_of(row * chunks), c_last = cta_of(row * chunks + chunks - 1);
             const int n_parts = c_last - c_first + 1, slot = (int)blockIdx.x - c_first;
             u64* dst = ws_cand + ((size_t)row * chunks + slot) * kMaxK;
@@ -632,9 +642,9 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, long long items_all, 
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             issue();
         }
-        if (!waited) { pdl_wait(); waited = true; }      // this warp does every global write of the CTA
         if (!have) {
             // give up: report, wait (bounded) for the copies still in flight, return
+            wait_once();
             if (lane == 0) {
                 if (status) atomicOr(status, GOOSE_ST_TIMEOUT);
                 volatile int no_abort = 0;               // draining ignores the abort flag
@@ -656,11 +666,10 @@ cudaError_t launch_topk_any(int num_sms, cudaStream_t st, const __nv_bfloat16* l
     // equal chunks (a multiple of 8 elements: every copy starts on 16 bytes), so that no item is a remainder
     const int chunks = (V + kTopkChunk - 1) / kTopkChunk;
     const int chunk_elems = ((V + chunks - 1) / chunks + 7) & ~7;
-    const long long items = (long long)rows * chunks;
+    const int items = rows * chunks;                 // (a row costs the context 1 KB of scratch a chunk: far below 2^31)
     // every CTA gets q = ceil(items / SMs) items or one fewer; using the fewest CTAs that q allows loses no time and
     // makes the ranges fall on row boundaries when q is a multiple of the chunks per row (no cross-CTA merges then)
-    const long long q = (items + num_sms - 1) / num_sms;
-    const int grid = (int)((items + q - 1) / q);
+    const int q = (items + num_sms - 1) / num_sms, grid = (items + q - 1) / q;
     auto kernel = row_lse ? (n_nodes ? node_topk_kernel<true, true> : node_topk_kernel<true, false>)
                           : (n_nodes ? node_topk_kernel<false, true> : node_topk_kernel<false, false>);
     return launch_pdl(kernel, dim3(grid), dim3(kTopkThreads), kTopkSmem, st, logits, items, V, ldl, k, chunks, chunk_elems, ws,
