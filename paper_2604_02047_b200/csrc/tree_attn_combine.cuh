@@ -24,6 +24,11 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     uint32_t r;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
@@ -35,6 +40,7 @@ struct Work {
     const int32_t* ctx_len;
     const int32_t* n_nodes;   // per-sequence node counts, or NULL (every tree has B nodes)
     int S, H, B, G;           // H = heads of the work list = M tiles x key/value heads (M-tile-major)
+    uint32_t G_magic;         // ceil(2^32 / G): division by G without the 20-instruction sequence
     long long total;          // all items
     bool small;               // total * (G + 1) fits 31 bits: 32-bit arithmetic (64-bit division is slow on the GPU)
     // ctx_len comes from device memory: a negative value is treated as 0 (the tree rows alone).  A sequence's keys are
@@ -44,15 +50,27 @@ struct Work {
         const int nn = nodes_of(n_nodes, s, B);
         return nn == 0 ? 0 : (max(ctx_len[s], 0) + nn + kTile - 1) / kTile;
     }
-    __device__ __forceinline__ void init() {
-        long long tot = 0;
-        for (int s = 0; s < S; ++s) tot += (long long)H * tiles(s);
+    __device__ __forceinline__ void set_total(long long tot) {
         total = tot;
         small = tot * (G + 1) < 0x7FFFFFFFll;
     }
+    __device__ __forceinline__ void init() {
+        long long tot = 0;
+        for (int s = 0; s < S; ++s) tot += (long long)H * tiles(s);
+        set_total(tot);
+    }
+    // the same by a whole warp, lane s loading sequence s's length; returns the tiles of sequence `lane`
+    __device__ __forceinline__ int init_warp(int lane) {
+        const int mine = lane < S ? tiles(lane) : 0;
+        long long sum = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)mine);
+        for (int s0 = 32; s0 < S; s0 += 32) sum += __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(s0 + lane < S ? tiles(s0 + lane) : 0));
+        set_total(H * sum);
+        return mine;
+    }
     __device__ __forceinline__ long long cta_start(int c) const {
-        if (small) return ((uint32_t)total * (uint32_t)c) / (uint32_t)G;
-        return total * c / G;
+        if (!small) return total * c / G;
+        const uint32_t n = (uint32_t)total * (uint32_t)c, q = __umulhi(n, G_magic);   // exact or one too large (n < 2^31)
+        return q * (uint32_t)G > n ? q - 1 : q;
     }
     __device__ __forceinline__ int cta_of(long long w) const {
         int c = small ? (int)(((uint32_t)w * (uint32_t)G) / (uint32_t)total) : (int)(w * G / total);
@@ -80,6 +98,28 @@ struct Cursor {               // walks items in order
         h = wk.small ? (int)((uint32_t)rem / (uint32_t)TT) : (int)(rem / TT);
         t = (int)(rem - (long long)h * TT);
     }
+    // the same by a whole warp for the common small batch: `mine` = tiles of sequence `lane` (Work::init_warp)
+    __device__ __forceinline__ void seek_warp(const Work& wk, long long w0, int lane, int mine) {
+        if (!wk.small || wk.S > 32) { seek(wk, w0); return; }
+        w = w0;
+        uint32_t rem = (uint32_t)w0;
+        s = 0;
+        if (wk.S > 1) {
+            uint32_t upto = (uint32_t)wk.H * (uint32_t)mine;     // items up to and with sequence `lane`
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, upto, o);
+                if (lane >= o) upto += u;
+            }
+            s = __ffs(__ballot_sync(0xFFFFFFFFu, upto > rem)) - 1;   // (w0 < total: some lane has it)
+            rem -= __shfl_sync(0xFFFFFFFFu, upto - (uint32_t)wk.H * (uint32_t)mine, s);
+        }
+        T = __shfl_sync(0xFFFFFFFFu, mine, s);
+        h = (int)__float2uint_rz(__fdividef((float)rem, (float)T));   // h < 2^16: off by one at most
+        t = (int)rem - h * T;
+        if (t < 0) { --h; t += T; }
+        if (t >= T) { ++h; t -= T; }
+    }
     __device__ __forceinline__ void next(const Work& wk) {
         ++w; ++t;
         if (t == T) {
@@ -106,6 +146,7 @@ struct CombineArgs {
     const int32_t* n_nodes;
     int S, B, H, Hkv, g, nb;
     int G;                    // CTAs of the main kernel
+    uint32_t G_magic;         // ceil(2^32 / G)
     int Hw;                   // heads of the work list
     const float* partials;
     __nv_bfloat16* out;
@@ -129,7 +170,7 @@ __device__ __forceinline__ void combine_heads(const CombineArgs& ca, int rg, int
     // kernel triggers its dependents after its own pdl_wait(), i.e. after whatever produced ctx_len[] completed.
     // So all of it runs before the wait, and the partial loads are issued the moment the main grid is done.
     Work wk;
-    wk.ctx_len = ctx_len; wk.n_nodes = n_nodes; wk.S = S; wk.H = Hw; wk.B = B; wk.G = G;
+    wk.ctx_len = ctx_len; wk.n_nodes = n_nodes; wk.S = S; wk.H = Hw; wk.B = B; wk.G = G; wk.G_magic = ca.G_magic;
     wk.init();
     long long off = 0;
     for (int ss = 0; ss < s; ++ss) off += (long long)Hw * wk.tiles(ss);

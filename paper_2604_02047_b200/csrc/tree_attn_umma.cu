@@ -198,7 +198,7 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                       const __grid_constant__ CUtensorMap tmap_v, const int64_t* __restrict__ row_off,
                       const int32_t* __restrict__ ctx_len, const int32_t* __restrict__ parent,
                       const int32_t* __restrict__ n_nodes,
-                      int S, int B, int H, int Hkv_arg, int g_arg, int nb_arg, int64_t kv_rows, float scale_log2,
+                      int S, int B, int H, int Hkv_arg, int g_arg, int nb_arg, uint32_t G_magic, int64_t kv_rows, float scale_log2,
                       float* __restrict__ partials,
                       int32_t* __restrict__ status,
                       __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
@@ -230,6 +230,7 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                      ::"r"(smem_u32(&hd->tmem_base)), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    if (threadIdx.x == 0) { prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -250,24 +251,30 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     Work wk;
     // g query heads per key/value head, nb nodes per M tile (nb * g <= 128), n_mt M tiles per sequence
     const int n_mt = kGrouped ? (B + nb - 1) / nb : 1;
-    wk.ctx_len = ctx_len; wk.n_nodes = n_nodes; wk.S = S; wk.H = n_mt * Hkv; wk.B = B; wk.G = gridDim.x;
-    wk.init();
+    wk.ctx_len = ctx_len; wk.n_nodes = n_nodes; wk.S = S; wk.H = n_mt * Hkv; wk.B = B; wk.G = gridDim.x; wk.G_magic = G_magic;
+    // where this CTA starts, found by every warp for itself with all lanes; the lengths and the rows of up to 32 sequences
+    // come in one round of loads (lane = sequence).  The first load of K waits for nothing else.
+    const int64_t my_row = lane < S ? row_off[lane] : 0;
+    const int my_tiles = wk.init_warp(lane);
     const long long w_begin = wk.cta_start(blockIdx.x), w_end = wk.cta_start(blockIdx.x + 1);
+    Cursor cu;
+    if (w_begin < w_end) cu.seek_warp(wk, w_begin, lane, my_tiles);
+    const int first_s = w_begin < w_end ? cu.s : 0;
+    const int64_t first_row = __shfl_sync(0xFFFFFFFFu, my_row, first_s & 31);
+    auto row_of = [&](int s) -> int64_t { return s == first_s && s < 32 ? first_row : row_off[s]; };
 
 
     if (w_begin < w_end) {
         if (warp == 0) {
             // =========================================================== TMA producer
             if (lane == 0) {
-                prefetch_tmap(&tmap_q); prefetch_tmap(&tmap_k); prefetch_tmap(&tmap_v);
                 // K and V are read exactly once: mark them evict-first so that the split-KV partials
                 // (written and re-read within this launch) stay resident in L2
                 const unsigned long long pol_stream = l2_policy_evict_first();
-                Cursor cu; cu.seek(wk, w_begin);
                 uint32_t ring = 0, seg = 0;
                 bool ok = true;
                 while (ok && cu.w < w_end) {
-                    const int64_t row0 = row_off[cu.s];
+                    const int64_t row0 = row_of(cu.s);
                     // Q of this segment
                     const uint32_t qb = seg & 1;           // seg = index of this segment
                     ok = mbar_wait(hd, &hd->q_empty[qb], ((seg >> 1) & 1) ^ 1, status);
@@ -307,7 +314,6 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
         } else if (warp == 1) {
             // =========================================================== MMA issuer
             if (lane == 0) {
-                Cursor cu; cu.seek(wk, w_begin);
                 uint32_t jg = 0, seg = 0;                  // CTA-global tile and segment counters
                 bool ok = true;
                 const uint32_t q_base = smem_u32(q_smem), kv_addr = smem_u32(kv_smem);
@@ -371,12 +377,11 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
             const int i_local = kGrouped ? row / g : row;  // row = (node of the M tile, head of the group)
             const int member = row - i_local * g;
             const int sm_tid = threadIdx.x - 64;           // 0..127
-            Cursor cu; cu.seek(wk, w_begin);
             uint32_t jg = 0, seg = 0, gsync = 0;
             bool ok = true;
             uint32_t v[128];
             int cur_s = -1, cur_mt = -1;
-            bool bad = false;
+            bool bad = false, anc_built = false;
             uint32_t anc[4] = {0, 0, 0, 0};
 
             while (ok && cu.w < w_end) {
@@ -402,7 +407,7 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                     }
                     // the sequence's rows must lie inside the cache (TMA would only read zeros outside, but the
                     // result would be meaningless): treated like an invalid tree, with its own status bit
-                    const int64_t r0 = row_off[s0];
+                    const int64_t r0 = row_of(s0);
                     const bool bad_rows = ctx_len[s0] < 0 || r0 < 0 || r0 + ctx + nn > kv_rows;
                     if (bad_rows && sm_tid == 0) { hd->bad_parent = 1; atomicOr(&status[s0], GOOSE_ST_BAD_ROWS); }
                     ok = group_sync(hd, gsync, status);
@@ -411,8 +416,15 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                     if (!ok) break;
                     if (sm_tid == 0 && bad) { hd->bad_parent = 0; if (!bad_rows) atomicOr(&status[s0], GOOSE_ST_BAD_PARENT); }
                 }
-                if (new_seq || mt != cur_mt) {             // hd->par[] still holds this sequence's parents
+                if (new_seq || mt != cur_mt) {
                     cur_mt = mt;
+                    anc_built = false;
+                }
+                // the ancestor set of this thread's row, for segments that reach the tree rows (hd->par[] still holds this
+                // sequence's parents)
+                const int t_last = (int)min((long long)T - 1, t_first + (w_end - cu.w) - 1);
+                if (!anc_built && (t_last + 1) * kTile > ctx) {
+                    anc_built = true;
                     anc[0] = anc[1] = anc[2] = anc[3] = 0;
                     if (row_valid) {
                         if (bad) {
@@ -441,8 +453,13 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                     ok = mbar_wait(hd, &hd->s_full[jg & 1], (jg >> 1) & 1, status);
                     if (!ok) break;
                     tc_fence_after();
-                    float m_use = 0.f;
-                    if (warp_has_rows) {
+                    // The exponentials of a tile are taken relative to the maximum known before it, while the tile's own
+                    // maximum is found beside them (the special-function units, 8 cycles an instruction and warp, take 1024
+                    // of the about 2000 cycles of a tile; the maximum's instructions hide behind them).  Only where it grew
+                    // by more than the threshold, and on a segment's first tile, the maximum comes first: O is rescaled
+                    // and the scores are read again (P replaces them only at the end).
+                    bool max_first = first;
+                    while (ok && warp_has_rows) {
                         const uint32_t s_addr = tmem + kColS + (jg & 1) * 128 + lane_sel;
                         TMEM_LD32(s_addr, v, 0); TMEM_LD32(s_addr + 32, v, 32);
                         TMEM_LD32(s_addr + 64, v, 64); TMEM_LD32(s_addr + 96, v, 96);
@@ -465,20 +482,16 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                             for (int c = 0; c < 128; ++c)
                                 v[c] = ((vw[c >> 5] >> (c & 31)) & 1u) ? v[c] : 0xFF800000u;   // -inf
                         }
-                        // one warp per scheduler: nothing hides a serial chain, so the row maximum (and the row
-                        // sum below) run as four independent chains
-                        float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                        if (max_first) {
+                            // one warp per scheduler: nothing hides a serial chain, so the row maximum (and the row
+                            // sum below) run as four independent chains
+                            float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-                        for (int c = 0; c < 128; c += 4) {
-                            mx4[0] = fmaxf(mx4[0], __uint_as_float(v[c]));     mx4[1] = fmaxf(mx4[1], __uint_as_float(v[c + 1]));
-                            mx4[2] = fmaxf(mx4[2], __uint_as_float(v[c + 2])); mx4[3] = fmaxf(mx4[3], __uint_as_float(v[c + 3]));
-                        }
-                        float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-                        mx *= scale_log2;                  // scale > 0
-                        const float m_new = fmaxf(m_run, mx);
-                        // lazy rescaling: keep the stale maximum unless it grew by more than the threshold
-                        const bool need = first ? true : (m_new > m_run + kRescaleThreshold);
-                        if (__any_sync(0xFFFFFFFFu, need)) {
+                            for (int c = 0; c < 128; c += 8)
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) mx4[e] = max3(mx4[e], __uint_as_float(v[c + 2 * e]), __uint_as_float(v[c + 2 * e + 1]));
+                            const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * scale_log2;   // scale > 0
+                            const float m_new = fmaxf(m_run, mx);
                             const float alpha = (m_run == -INFINITY) ? 0.f : ex2(m_run - m_new);
                             if (!first) {
                                 // O holds tiles < t of this segment: wait for PV(t-1), then scale the row
@@ -501,43 +514,50 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                             l_run *= alpha;
                             m_run = m_new;
                         }
-                        m_use = (m_run == -INFINITY) ? 0.f : m_run;
-                    }
-                    // P (bf16 pairs) overwrites the first 64 columns of this tile's S buffer: this thread has its whole
-                    // S row in registers, and QK^T of tile jg+2 is ordered after PV(jg) in the MMA pipe
-                    if (warp_has_rows) {
-                        float ls4[4] = {0.f, 0.f, 0.f, 0.f};
-                        const float neg_m = -m_use;
+                        const float neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
+                        const unsigned long long scale2 = pack_f32x2(scale_log2, scale_log2), neg2 = pack_f32x2(neg_m, neg_m);
+                        unsigned long long ls2[2] = {0, 0};
+                        float mx2[2] = {-INFINITY, -INFINITY};
 #pragma unroll
                         for (int e = 0; e < 64; ++e) {
-                            float p0 = ex2(fmaf(__uint_as_float(v[2 * e]), scale_log2, neg_m));
-                            float p1 = ex2(fmaf(__uint_as_float(v[2 * e + 1]), scale_log2, neg_m));
-                            ls4[e & 3] += p0 + p1;
+                            const float s0 = __uint_as_float(v[2 * e]), s1 = __uint_as_float(v[2 * e + 1]);
+                            if (!first) mx2[e & 1] = max3(mx2[e & 1], s0, s1);
+                            const float2 x2 = unpack_f32x2(fma_f32x2(pack_f32x2(s0, s1), scale2, neg2));
+                            const float p0 = ex2(x2.x), p1 = ex2(x2.y);
+                            ls2[e & 1] = add_f32x2(ls2[e & 1], pack_f32x2(p0, p1));
                             v[e] = pack_bf16x2(p0, p1);
                         }
-                        l_run += (ls4[0] + ls4[1]) + (ls4[2] + ls4[3]);
+                        if (!max_first) {
+                            const bool grew = row_valid && fmaxf(mx2[0], mx2[1]) * scale_log2 > m_run + kRescaleThreshold;
+                            max_first = __any_sync(0xFFFFFFFFu, grew);
+                            if (max_first) continue;
+                        }
+                        const float2 l2 = unpack_f32x2(add_f32x2(ls2[0], ls2[1]));
+                        l_run += l2.x + l2.y;
+                        // P (bf16 pairs) overwrites the first 64 columns of this tile's S buffer: this thread has its whole
+                        // S row in registers, and QK^T of tile jg+2 is ordered after PV(jg) in the MMA pipe
                         const uint32_t p_taddr = tmem + kColS + (jg & 1) * 128 + lane_sel;
                         TMEM_ST32(p_taddr, v, 0);
                         TMEM_ST32(p_taddr + 32, v, 32);
                         tmem_wait_st();
+                        break;
                     }
                     // observe every phase of pv_done in order (a parity wait must never lag two phases behind its
                     // barrier); by now PV(jg-1) has normally completed, so this does not stall
-                    if (jg > 0) ok = mbar_wait(hd, &hd->pv_done, (jg - 1) & 1, status);
+                    if (ok && jg > 0) ok = mbar_wait(hd, &hd->pv_done, (jg - 1) & 1, status);
                     if (!ok) break;
                     // ragged end: V rows past the sequence's last key may hold anything -> zero them
                     if ((t + 1) * kTile > n_keys) {
                         const uint32_t ring = 2 * jg + 1, st = ring % kStages;
                         ok = mbar_wait(hd, &hd->kv_full[st], (ring / kStages) & 1, status);
                         if (!ok) break;
-                        const int r_local = sm_tid;        // one V row (key) per thread
-                        if (t * kTile + r_local >= n_keys) {
-                            unsigned char* vrow = kv_smem + st * kStageBytes + r_local * 128;
-#pragma unroll
-                            for (int c = 0; c < 8; ++c) {
-                                *reinterpret_cast<uint4*>(vrow + c * 16) = make_uint4(0, 0, 0, 0);
-                                *reinterpret_cast<uint4*>(vrow + kHalfBytes + c * 16) = make_uint4(0, 0, 0, 0);
-                            }
+                        // rows n_keys - t * 128 .. 127 are one contiguous piece of each half (the swizzle stays inside a
+                        // row): consecutive threads clear consecutive 16-byte words.  (A row per thread had all lanes of
+                        // a store on the same four banks: 0.5 to 0.9 us on the last tile of every head.)
+                        const int first_off = max(n_keys - t * kTile, 0) * 128;
+                        for (int off = first_off + sm_tid * 16; off < kHalfBytes; off += 128 * 16) {
+                            *reinterpret_cast<uint4*>(kv_smem + st * kStageBytes + off) = make_uint4(0, 0, 0, 0);
+                            *reinterpret_cast<uint4*>(kv_smem + st * kStageBytes + kHalfBytes + off) = make_uint4(0, 0, 0, 0);
                         }
                         fence_proxy_async();               // generic-proxy writes -> visible to the tensor core
                     }
@@ -724,18 +744,19 @@ cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __
         return cudaErrorInvalidValue;
     int grid = c->num_sms;
     if (2 * grid > c->n_slots) grid = c->n_slots / 2;
+    const uint32_t g_magic = (uint32_t)((0x100000000ull + grid - 1) / grid);
     const bool grouped = g > 1;
     const bool counts = n_nodes != nullptr;
     auto main_kernel = grouped ? (counts ? tree_attn_umma_kernel<true, true> : tree_attn_umma_kernel<true, false>)
                                : (counts ? tree_attn_umma_kernel<false, true> : tree_attn_umma_kernel<false, false>);
     cudaError_t e = launch_pdl(main_kernel, dim3(grid),
                                dim3(kThreads), kUmmaSmem, st, mq, mk, mv, row_off, ctx_len, parent, n_nodes, S, B, H, Hkv, g, nb,
-                               kv_rows, scale * kLog2e, c->partials, c->status, out, lse);
+                               g_magic, kv_rows, scale * kLog2e, c->partials, c->status, out, lse);
     c->launches++;
     if (e != cudaSuccess) return e;
     CombineArgs ca;
     ca.ctx_len = ctx_len; ca.n_nodes = n_nodes; ca.S = S; ca.B = B; ca.H = H; ca.Hkv = Hkv; ca.g = g; ca.nb = nb;
-    ca.G = grid; ca.Hw = n_mt * Hkv; ca.partials = c->partials; ca.out = out; ca.lse = lse;
+    ca.G = grid; ca.G_magic = g_magic; ca.Hw = n_mt * Hkv; ca.partials = c->partials; ca.out = out; ca.lse = lse;
     const int row_groups = (nb * g + 31) / 32;
     if (defer_merge) {                                  // the caller runs the merge as a role of a later launch
         defer_merge->args = ca; defer_merge->row_groups = row_groups; defer_merge->grouped = grouped;
