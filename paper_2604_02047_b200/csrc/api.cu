@@ -327,6 +327,23 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
     // kernel's CTAs leave their SMs (out[] and lse[] are complete when the step is).
     goose::CombinePlan merge_plan;
     merge_plan.valid = false;
+    // The cluster form of the attention merges its heads itself and leaves SMs idle; the top-k goes onto those, beside it,
+    // where that takes each of them at most kTopkBeside items (1.5 us an item: done before the attention, which is not
+    // below 8 us).  Its CTAs all end at once, so a top-k that has to follow would start late: with more items the step
+    // keeps the persistent form, in whose ragged end the top-k starts (32 heads, 2k keys, 80 rows: persistent 19.15 us,
+    // clusters with the top-k behind them 20.7, beside them 17.5).
+    constexpr int kTopkBeside = 7;
+    int topk_ctas = 0;
+    bool may_cluster = true;
+    if (S > 0 && !attn_done) {
+        const int g = H / Hkv, nb = B * g <= 128 ? B : 128 / g;
+        const int n = goose::attn_cluster(c, S, B, H, Hkv);
+        if (n > 1) {
+            topk_ctas = c->num_sms - (B + nb - 1) / nb * Hkv * n;
+            may_cluster = topk_ctas > 0 && goose::topk_items(S * B, V) <= kTopkBeside * topk_ctas;
+            if (!may_cluster) topk_ctas = 0;
+        }
+    }
     if (!(scale > 0.f) || !(scale < 1e30f)) return GOOSE_EINVAL;
     {
         int impl = c->attn_impl;
@@ -337,9 +354,10 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
             cudaError_t ea = goose::launch_tree_attn_umma(c, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_cache,
                                                           (const __nv_bfloat16*)v_cache, kv_rows, row_off, ctx_len, parent,
                                                           n_nodes, S, B, H, Hkv, scale, (__nv_bfloat16*)out, lse,
-                                                          static_cast<cudaStream_t>(stream), &merge_plan);
+                                                          static_cast<cudaStream_t>(stream), &merge_plan, may_cluster);
             if (ea != cudaSuccess) return cuda_fail(ea);
         } else {
+            topk_ctas = 0;
             rc = goose_tree_attn_gqa(c, q, k_cache, v_cache, kv_rows, row_off, ctx_len, parent, n_nodes, S, B, H, Hkv, D, scale,
                                      out, lse, stream);
             if (rc) return rc;
@@ -354,7 +372,7 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
         if (logits_ready) GOOSE_CUDA(cudaStreamWaitEvent(static_cast<cudaStream_t>(stream), logits_ready, 0));
         cudaError_t et = goose::launch_node_topk(c, (const __nv_bfloat16*)logits, S * B, V, ldl, k, argmax, topk_ids, topk_vals,
                                                  harvest ? row_lse : nullptr, static_cast<cudaStream_t>(stream),
-                                                 /*inputs_ready=*/true, n_nodes, B);
+                                                 /*inputs_ready=*/true, n_nodes, B, topk_ctas);
         if (et != cudaSuccess) return cuda_fail(et);
     }
     // acceptance walk + compaction in one launch (same results as goose_accept followed by goose_kv_compact); with a

@@ -45,6 +45,7 @@ struct goose_ctx {
     cudaStream_t side;        // the logits are uploaded here, next to the attention kernels
     cudaStream_t side_down;   // the attention output goes down here while the logits are still going up
     cudaEvent_t ev_fork, ev_logits, ev_attn, ev_out;
+    int max_clusters[9];      // clusters of n attention CTAs that the device holds at once, by n
     long long launches;
     void* encode_tiled;       // cuTensorMapEncodeTiled entry point (driver), resolved at create
 };
@@ -120,24 +121,34 @@ __device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, un
 }
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                              Args&&... args) {
+inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem,
+                                      cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    return launch_pdl_cluster(kernel, grid, block, 1, smem, st, args...);
 }
 #endif
 
 // launchers (each returns a cudaError_t from the launch)
-// inputs_ready: the logits were complete before the kernel preceding this one in the stream started (see the kernel)
+// max_ctas (0: one per SM): the largest grid
+// inputs_ready: everything in front of the kernel that precedes this one in the stream is complete when this one can
+// start, and that kernel has nothing to do with this one's inputs and outputs (see the kernel)
 // n_nodes (may be NULL) with B: row r = s * B + i exists iff i < n_nodes[s]; other rows are neither read nor written
 cudaError_t launch_node_topk(goose_ctx* c, const __nv_bfloat16* logits, int rows, int V, int64_t ldl, int k,
                              int32_t* argmax, int32_t* ids, float* vals, float* row_lse, cudaStream_t st,
-                             bool inputs_ready = false, const int32_t* n_nodes = nullptr, int B = 0);
+                             bool inputs_ready = false, const int32_t* n_nodes = nullptr, int B = 0, int max_ctas = 0);
+// items of that kernel's work list: chunks of rows
+int topk_items(int rows, int V);
 cudaError_t launch_harvest_scatter(goose_ctx* c, const int32_t* row_tok, int rows, int table_rows, int k,
                                    const int32_t* ids, const float* vals, const float* row_lse,
                                    int32_t* adj_ids, float* adj_scores, cudaStream_t st);
@@ -163,7 +174,9 @@ cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __
                                   const __nv_bfloat16* vc, int64_t kv_rows, const int64_t* row_off,
                                   const int32_t* ctx_len, const int32_t* parent, const int32_t* n_nodes, int S, int B, int H,
                                   int Hkv, float scale, __nv_bfloat16* out, float* lse, cudaStream_t st,
-                                  struct CombinePlan* defer_merge = nullptr);
+                                  struct CombinePlan* defer_merge = nullptr, bool may_cluster = true);
+// CTAs a head of the cluster form of that kernel has for these sizes (1: the persistent form)
+int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv);
 
 cudaError_t launch_bounded_wait_selftest(goose_ctx* c, long long limit_cycles, int32_t* result, cudaStream_t st);
 
@@ -172,11 +185,12 @@ int mma_splits(const goose_ctx* c, int S, int H);
 
 // per-device kernel attributes (dynamic shared memory limits); called once from goose_create
 cudaError_t init_mma_kernel();
-cudaError_t init_umma_kernel();
+cudaError_t init_umma_kernel(goose_ctx* c);
 cudaError_t init_topk_kernel();
-inline cudaError_t init_kernels(goose_ctx*) {
+constexpr int kMaxCluster = 8;        // the portable limit
+inline cudaError_t init_kernels(goose_ctx* c) {
     cudaError_t e = init_mma_kernel();
-    if (e == cudaSuccess) e = init_umma_kernel();
+    if (e == cudaSuccess) e = init_umma_kernel(c);
     return e != cudaSuccess ? e : init_topk_kernel();
 }
 

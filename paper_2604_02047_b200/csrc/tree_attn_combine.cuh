@@ -153,6 +153,42 @@ struct CombineArgs {
     float* lse;
 };
 
+// one round: kCombineRound parts of a row, their (m, l) and 16 columns of O/l, into the running (M, L, acc)
+__device__ __forceinline__ void merge_round(const float (&mp)[kCombineRound], const float (&lp)[kCombineRound],
+                                            const uint4 (&x)[kCombineRound][2], float& M_run, float& L_run, float (&acc)[16]) {
+    float M_new = M_run;
+#pragma unroll
+    for (int q = 0; q < kCombineRound; ++q) M_new = fmaxf(M_new, mp[q]);
+    const float a_old = (M_run == -INFINITY) ? 0.f : ex2(M_run - M_new);
+    L_run *= a_old;
+#pragma unroll
+    for (int u = 0; u < 16; ++u) acc[u] *= a_old;
+#pragma unroll
+    for (int q = 0; q < kCombineRound; ++q) {
+        const float w = ((mp[q] == -INFINITY) ? 0.f : ex2(mp[q] - M_new)) * lp[q];   // un-normalise: O_p = x_p * l_p
+        L_run += w;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const uint32_t hw[4] = {x[q][u].x, x[q][u].y, x[q][u].z, x[q][u].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hw[e]));
+                acc[8 * u + 2 * e] += w * f.x;
+                acc[8 * u + 2 * e + 1] += w * f.y;
+            }
+        }
+    }
+    M_run = M_new;
+}
+__device__ __forceinline__ void store_merged(__nv_bfloat16* dst, const float (&acc)[16], float L) {
+    const float inv = 1.f / L;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+        reinterpret_cast<uint4*>(dst)[u] =
+            make_uint4(pack_bf16x2(acc[8 * u] * inv, acc[8 * u + 1] * inv), pack_bf16x2(acc[8 * u + 2] * inv, acc[8 * u + 3] * inv),
+                       pack_bf16x2(acc[8 * u + 4] * inv, acc[8 * u + 5] * inv), pack_bf16x2(acc[8 * u + 6] * inv, acc[8 * u + 7] * inv));
+}
+
 template <bool kGrouped, bool kCounts>
 __device__ __forceinline__ void combine_heads(const CombineArgs& ca, int rg, int h, int s) {
     const int32_t* __restrict__ ctx_len = ca.ctx_len;
@@ -217,36 +253,9 @@ __device__ __forceinline__ void combine_heads(const CombineArgs& ca, int rg, int
             for (int u = 0; u < 2; ++u)
                 x[q][u] = use ? __ldcg(p4 + (2 * warp + u) * 128) : make_uint4(0u, 0u, 0u, 0u);
         }
-        float M_new = M_run;
-#pragma unroll
-        for (int q = 0; q < kCombineRound; ++q) M_new = fmaxf(M_new, mp[q]);
-        const float a_old = (M_run == -INFINITY) ? 0.f : ex2(M_run - M_new);
-        L_run *= a_old;
-#pragma unroll
-        for (int u = 0; u < 16; ++u) acc[u] *= a_old;
-#pragma unroll
-        for (int q = 0; q < kCombineRound; ++q) {
-            const float w = ((mp[q] == -INFINITY) ? 0.f : ex2(mp[q] - M_new)) * lp[q];   // un-normalise: O_p = x_p * l_p
-            L_run += w;
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const uint32_t hw[4] = {x[q][u].x, x[q][u].y, x[q][u].z, x[q][u].w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hw[e]));
-                    acc[8 * u + 2 * e] += w * f.x;
-                    acc[8 * u + 2 * e + 1] += w * f.y;
-                }
-            }
-        }
-        M_run = M_new;
+        merge_round(mp, lp, x, M_run, L_run, acc);
     }
-    const float inv = 1.f / L_run;
-    uint4* dst = reinterpret_cast<uint4*>(out + (((size_t)s * B + node) * H + hq) * kHeadDim + 16 * warp);
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-        dst[u] = make_uint4(pack_bf16x2(acc[8 * u] * inv, acc[8 * u + 1] * inv), pack_bf16x2(acc[8 * u + 2] * inv, acc[8 * u + 3] * inv),
-                            pack_bf16x2(acc[8 * u + 4] * inv, acc[8 * u + 5] * inv), pack_bf16x2(acc[8 * u + 6] * inv, acc[8 * u + 7] * inv));
+    store_merged(out + (((size_t)s * B + node) * H + hq) * kHeadDim + 16 * warp, acc, L_run);
     if (lse && warp == 0) lse[((size_t)s * B + node) * H + hq] = (M_run + log2f(L_run)) * kLn2;
 }
 

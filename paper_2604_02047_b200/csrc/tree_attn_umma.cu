@@ -16,6 +16,10 @@
 //                                  mask on the tiles that reach the tree rows, exp2, P (bf16) written back
 //                                  over the first 64 columns of the S buffer it came from, lazy rescaling
 //                                  of O in TMEM, epilogue (output or partial).
+// One sequence whose heads come out near the SM count (kCluster): a thread-block cluster takes each head instead, its CTAs
+// contiguous tile ranges of it.  No CTA then works on two heads (a second segment costs its softmax, PV and epilogue in
+// turn, 2 to 3 us at the end of the slowest CTA), and the cluster merges its head itself, behind its own barrier, instead
+// of a kernel behind all of them (boundary 1 us, a cold start on every SM, 2 us, and one more launch).
 // All B <= 128 query rows ride in one M = 128 MMA; rows >= B compute on don't-care data and are
 // never written out.  Grouped-query attention (H query heads over Hkv key/value heads, g = H / Hkv) stacks the g
 // query heads of a group into the same M tile -- row r = (node r / g, group member r % g) -- so a K/V tile is
@@ -153,6 +157,11 @@ __device__ __forceinline__ void umma_commit(unsigned long long* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// the cluster's barrier: orders the partials written by its CTAs before the reads behind it
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
 #define TMEM_LD32(taddr, v, off)                                                                                      \
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "                                                            \
                  "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"                                          \
@@ -192,13 +201,14 @@ __device__ __forceinline__ bool group_sync(Header* hd, uint32_t& n, int32_t* sta
 // kGrouped = false is multi-head attention: one query head per key/value head and one M tile per sequence are
 // compile-time facts there (the per-row index arithmetic folds away); kGrouped = true takes them from the arguments.
 // kCounts = false is the instantiation for n_nodes == NULL: the counts fold away at compile time
-template <bool kGrouped, bool kCounts>
+template <bool kGrouped, bool kCounts, bool kCluster>
 __global__ void __launch_bounds__(kThreads, 1)
 tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                       const __grid_constant__ CUtensorMap tmap_v, const int64_t* __restrict__ row_off,
                       const int32_t* __restrict__ ctx_len, const int32_t* __restrict__ parent,
                       const int32_t* __restrict__ n_nodes,
-                      int S, int B, int H, int Hkv_arg, int g_arg, int nb_arg, uint32_t G_magic, int64_t kv_rows, float scale_log2,
+                      int S, int B, int H, int Hkv_arg, int g_arg, int nb_arg, uint32_t G_magic, int cluster, int64_t kv_rows,
+                      float scale_log2,
                       float* __restrict__ partials,
                       int32_t* __restrict__ status,
                       __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
@@ -256,9 +266,16 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     // come in one round of loads (lane = sequence).  The first load of K waits for nothing else.
     const int64_t my_row = lane < S ? row_off[lane] : 0;
     const int my_tiles = wk.init_warp(lane);
-    const long long w_begin = wk.cta_start(blockIdx.x), w_end = wk.cta_start(blockIdx.x + 1);
+    // cluster mode: this CTA is number `rank` of the `cluster` CTAs that share head `head` of the one sequence
+    const int head = kCluster ? blockIdx.x / cluster : 0, rank = kCluster ? blockIdx.x - head * cluster : 0;
+    const int T_all = kCluster ? __shfl_sync(0xFFFFFFFFu, my_tiles, 0) : 0;
+    // its first tile; rounded up, so that the last CTA, which has the masked tile, has no tile more than the others
+    auto rank_start = [&](int r) { return (T_all * r + cluster - 1) / cluster; };
+    const long long w_begin = kCluster ? (long long)head * T_all + rank_start(rank) : wk.cta_start(blockIdx.x);
+    const long long w_end = kCluster ? (long long)head * T_all + rank_start(rank + 1) : wk.cta_start(blockIdx.x + 1);
     Cursor cu;
-    if (w_begin < w_end) cu.seek_warp(wk, w_begin, lane, my_tiles);
+    if (kCluster) { cu.w = w_begin; cu.s = 0; cu.h = head; cu.t = rank_start(rank); cu.T = T_all; }
+    else if (w_begin < w_end) cu.seek_warp(wk, w_begin, lane, my_tiles);
     const int first_s = w_begin < w_end ? cu.s : 0;
     const int64_t first_row = __shfl_sync(0xFFFFFFFFu, my_row, first_s & 31);
     auto row_of = [&](int s) -> int64_t { return s == first_s && s < 32 ? first_row : row_off[s]; };
@@ -603,7 +620,7 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                 } else {
                     // partial -> workspace slot of this CTA (combined by tree_attn_combine_kernel): O/l in fp16
                     // (relative error 2^-11, far below the bf16 rounding of the final output), m and l in fp32
-                    const int slot = 2 * blockIdx.x + (t_first == 0 ? 1 : 0);
+                    const int slot = kCluster ? blockIdx.x : 2 * blockIdx.x + (t_first == 0 ? 1 : 0);
                     float* part = partials + (size_t)slot * kUmmaPartFloats;
                     if (row_valid) {
                         // invalid parent[]: a neutral partial (O = 0; the head's first part carries weight 1)
@@ -631,9 +648,62 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     }
 
     // ---- teardown
-    __syncwarp();
-    tc_fence_before();
-    __syncthreads();
+    if constexpr (kCluster) {
+        // merge of the cluster's partials: this CTA takes its share of the rows, a thread 16 columns of a row
+        //   M = max m_p,  L = sum l_p 2^(m_p - M),  out = sum_p 2^(m_p - M) l_p (O/l)_p / L
+        // (one warp a scheduler and some 300 dependent instructions: all arithmetic that needs no partial stands in front
+        // of the barrier, and every load is unconditional -- a part that is not there is read from the first one, which
+        // always is, and weighs nothing.  Partials in the CTAs' shared memory, read by ld.shared::cluster, were slower than
+        // through L2: 15.65 against 14.4 us a call at 32 heads and 2k keys, 24.8 against 22.5 at 40 heads and 4k.)
+        const int mt = kGrouped ? head / Hkv : 0, hk = head - mt * Hkv;
+        const int rows = min(nb, nodes_of(n_nodes, 0, B) - mt * nb) * g;
+        const bool split = T_all > 1 && rows > 0;          // (a single tile was written by the CTA that had it)
+        const int r0 = rows * rank / cluster, n_rows = split ? rows * (rank + 1) / cluster - r0 : 0;
+        int task = threadIdx.x;
+        int u = n_rows > 0 ? task / n_rows : 0, row = r0 + task - u * n_rows;   // neighbouring threads: neighbouring rows
+        const bool all_parts = T_all >= cluster;
+        __syncwarp();
+        tc_fence_before();
+        cluster_sync();                                    // the head's partials are complete in its CTAs' shared memory
+        for (; task < n_rows * 8;) {
+            const float* at_m = partials + (size_t)head * cluster * kUmmaPartFloats + kPartHalfWords + row;
+            const uint4* at_x = reinterpret_cast<const uint4*>(partials + (size_t)head * cluster * kUmmaPartFloats) + 2 * u * 128 + row;
+            float M_run = -INFINITY, L_run = 0.f, acc[16];
+#pragma unroll
+            for (int c = 0; c < 16; ++c) acc[c] = 0.f;
+            for (int pb = 0; pb < cluster; pb += kCombineRound) {
+                float mp[kCombineRound], lp[kCombineRound];
+                uint4 x[kCombineRound][2];
+                bool use[kCombineRound];
+#pragma unroll
+                for (int q = 0; q < kCombineRound; ++q) {
+                    const int p = pb + q;
+                    use[q] = p < cluster && (all_parts || rank_start(p + 1) > rank_start(p));
+                    const size_t peer = use[q] ? p : 0;
+                    const float* pm = at_m + peer * kUmmaPartFloats;
+                    const uint4* px = at_x + peer * (kUmmaPartFloats / 4);
+                    mp[q] = __ldcg(pm);
+                    lp[q] = __ldcg(pm + kMaxB);
+                    x[q][0] = __ldcg(px);
+                    x[q][1] = __ldcg(px + 128);
+                }
+#pragma unroll
+                for (int q = 0; q < kCombineRound; ++q)
+                    if (!use[q]) { mp[q] = -INFINITY; lp[q] = 0.f; }
+                merge_round(mp, lp, x, M_run, L_run, acc);
+            }
+            const int i_local = kGrouped ? row / g : row;
+            const size_t at = (size_t)(mt * nb + i_local) * H + hk * g + (row - i_local * g);
+            store_merged(out + at * kHeadDim + 16 * u, acc, L_run);
+            if (lse && u == 0) lse[at] = (M_run + log2f(L_run)) * kLn2;
+            task += kThreads;
+            u = task / n_rows; row = r0 + task - u * n_rows;
+        }
+    } else {
+        __syncwarp();
+        tc_fence_before();
+        __syncthreads();
+    }
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
@@ -708,14 +778,37 @@ cudaError_t launch_bounded_wait_selftest(goose_ctx* c, long long limit_cycles, i
     return cudaGetLastError();
 }
 
-cudaError_t init_umma_kernel() {
-    cudaError_t e = cudaFuncSetAttribute(tree_attn_umma_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(tree_attn_umma_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(tree_attn_umma_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmem);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(tree_attn_umma_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmem);
+namespace {
+typedef void (*UmmaKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const int64_t*, const int32_t*, const int32_t*,
+                           const int32_t*, int, int, int, int, int, int, uint32_t, int, int64_t, float, float*, int32_t*,
+                           __nv_bfloat16*, float*);
+UmmaKernel umma_kernel(bool grouped, bool counts, bool cluster) {
+    if (cluster) return grouped ? (counts ? tree_attn_umma_kernel<true, true, true> : tree_attn_umma_kernel<true, false, true>)
+                                : (counts ? tree_attn_umma_kernel<false, true, true> : tree_attn_umma_kernel<false, false, true>);
+    return grouped ? (counts ? tree_attn_umma_kernel<true, true, false> : tree_attn_umma_kernel<true, false, false>)
+                   : (counts ? tree_attn_umma_kernel<false, true, false> : tree_attn_umma_kernel<false, false, false>);
+}
+}  // namespace
+
+cudaError_t init_umma_kernel(goose_ctx* c) {
+    for (int i = 0; i < 8; ++i) {
+        cudaError_t e = cudaFuncSetAttribute(umma_kernel(i & 1, i & 2, i & 4), cudaFuncAttributeMaxDynamicSharedMemorySize, kUmmaSmem);
+        if (e != cudaSuccess) return e;
+    }
+    // how many clusters of each size the device holds at once (its SMs come in groups of unequal size)
+    for (int n = 2; n <= kMaxCluster; ++n) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(n * c->num_sms); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kUmmaSmem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = n; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        int m = 0;
+        cudaError_t e = cudaOccupancyMaxActiveClusters(&m, umma_kernel(true, true, true), &cfg);
+        if (e != cudaSuccess) return e;
+        c->max_clusters[n] = m;
+    }
+    return cudaSuccess;
 }
 
 int auto_attn_impl(const goose_ctx* c, int S, int B, int H) {
@@ -726,11 +819,25 @@ int auto_attn_impl(const goose_ctx* c, int S, int B, int H) {
     return c->encode_tiled ? GOOSE_ATTN_UMMA : GOOSE_ATTN_MMA;
 }
 
+// One sequence: a cluster per head where that leaves few SMs out.  The largest cluster (of at most 8 CTAs) that the device
+// holds one of per head at once; from 0.78 of the SMs on: an SM takes in 51 GB/s at most (a persistent grid on 225 MB: 68.8
+// us on 74 CTAs, 51.0 on 104, 48.2 on 120, 44.0 on 148), so 120 of 148 stream almost as fast as HBM gives and 104 do not.
+// Attention call, persistent grid and merge kernel -> clusters: 32 heads 10.4 -> 9.4 us (512 keys), 15.55 -> 13.7 (1.5k),
+// 16.25 -> 14.4 (2k); 40 heads 23.45 -> 22.5 (4k).  Several sequences may differ in length by any factor: persistent grid.
+int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv) {
+    const int g = H / Hkv, nb = B * g <= kTile ? B : kTile / g, Hw = (B + nb - 1) / nb * Hkv;
+    int cluster = 1;
+    if (S == 1)
+        for (int n = 2; n <= kMaxCluster; ++n)
+            if (c->max_clusters[n] >= Hw && 100 * Hw * n >= 78 * c->num_sms && Hw * n <= c->num_sms) cluster = n;
+    return cluster;
+}
+
 cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __nv_bfloat16* kc,
                                   const __nv_bfloat16* vc, int64_t kv_rows, const int64_t* row_off,
                                   const int32_t* ctx_len, const int32_t* parent, const int32_t* n_nodes, int S, int B, int H,
                                   int Hkv, float scale, __nv_bfloat16* out, float* lse, cudaStream_t st,
-                                  CombinePlan* defer_merge) {
+                                  CombinePlan* defer_merge, bool may_cluster) {
     if (defer_merge) defer_merge->valid = false;
     if (!c->encode_tiled) return cudaErrorNotSupported;
     if (S == 0) return cudaSuccess;
@@ -742,21 +849,21 @@ cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __
         !make_map(c->encode_tiled, &mk, kc, kv_rows, Hkv, kTile) ||
         !make_map(c->encode_tiled, &mv, vc, kv_rows, Hkv, kTile))
         return cudaErrorInvalidValue;
-    int grid = c->num_sms;
+    const int Hw = n_mt * Hkv;
+    const int cluster = may_cluster ? attn_cluster(c, S, B, H, Hkv) : 1;
+    int grid = cluster > 1 ? Hw * cluster : c->num_sms;
     if (2 * grid > c->n_slots) grid = c->n_slots / 2;
     const uint32_t g_magic = (uint32_t)((0x100000000ull + grid - 1) / grid);
     const bool grouped = g > 1;
     const bool counts = n_nodes != nullptr;
-    auto main_kernel = grouped ? (counts ? tree_attn_umma_kernel<true, true> : tree_attn_umma_kernel<true, false>)
-                               : (counts ? tree_attn_umma_kernel<false, true> : tree_attn_umma_kernel<false, false>);
-    cudaError_t e = launch_pdl(main_kernel, dim3(grid),
-                               dim3(kThreads), kUmmaSmem, st, mq, mk, mv, row_off, ctx_len, parent, n_nodes, S, B, H, Hkv, g, nb,
-                               g_magic, kv_rows, scale * kLog2e, c->partials, c->status, out, lse);
+    cudaError_t e = launch_pdl_cluster(umma_kernel(grouped, counts, cluster > 1), dim3(grid), dim3(kThreads), cluster, kUmmaSmem,
+                                       st, mq, mk, mv, row_off, ctx_len, parent, n_nodes, S, B, H, Hkv, g, nb, g_magic, cluster,
+                                       kv_rows, scale * kLog2e, c->partials, c->status, out, lse);
     c->launches++;
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || cluster > 1) return e;          // (a cluster merges its head itself)
     CombineArgs ca;
     ca.ctx_len = ctx_len; ca.n_nodes = n_nodes; ca.S = S; ca.B = B; ca.H = H; ca.Hkv = Hkv; ca.g = g; ca.nb = nb;
-    ca.G = grid; ca.G_magic = g_magic; ca.Hw = n_mt * Hkv; ca.partials = c->partials; ca.out = out; ca.lse = lse;
+    ca.G = grid; ca.G_magic = g_magic; ca.Hw = Hw; ca.partials = c->partials; ca.out = out; ca.lse = lse;
     const int row_groups = (nb * g + 31) / 32;
     if (defer_merge) {                                  // the caller runs the merge as a role of a later launch
         defer_merge->args = ca; defer_merge->row_groups = row_groups; defer_merge->grouped = grouped;
