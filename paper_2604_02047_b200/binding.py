@@ -2,7 +2,7 @@
 
 Every function takes torch CUDA tensors (or, for the ``*_host`` call, pinned CPU tensors),
 passes their ``data_ptr()`` and the current CUDA stream to ``libgoose.so`` and returns the
-output tensors.  No step of the method runs in Python or in torch ops; if the library is
+output tensors.  The stream-ordered calls go through ``_marshal.so`` (``csrc/marshal.cpp``), the others through ctypes.  No step of the method runs in Python or in torch ops; if the library is
 missing or a call fails, an exception is raised -- there is no fallback path.
 """
 from __future__ import annotations
@@ -29,6 +29,7 @@ ATTN_AUTO, ATTN_MMA, ATTN_UMMA = 0, 1, 2
 ST_BAD_PARENT, ST_BAD_PATH, ST_TIMEOUT, ST_BAD_ROWS, ST_BAD_NODES = 1, 2, 4, 8, 16
 
 _lib: Optional[ctypes.CDLL] = None
+_native = None
 
 
 class GooseError(RuntimeError):
@@ -59,6 +60,20 @@ def load_library() -> ctypes.CDLL:
     return lib
 
 
+def load_marshal():
+    """Load ``_marshal.so``: the argument marshalling of the stream-ordered calls (linked against ``libgoose.so``)."""
+    global _native
+    if _native is None:
+        load_library()
+        try:
+            from . import _marshal
+        except ImportError as e:
+            raise GooseError("_marshal.so is missing or does not load (%s): run `python -m paper_2604_02047_b200.build` "
+                             "(there is no fallback path)" % e) from e
+        _native = _marshal
+    return _native
+
+
 def _check(rc: int, what: str) -> None:
     if rc != 0:
         msg = load_library().goose_strerror(rc).decode()
@@ -77,6 +92,16 @@ def _dev(t: torch.Tensor, dtype: torch.dtype, name: str) -> torch.Tensor:
     if not t.is_cuda or t.dtype != dtype or not t.is_contiguous():
         raise GooseError("%s must be a contiguous CUDA tensor of dtype %s" % (name, dtype))
     return t
+
+
+_KINDS = {"b": torch.bfloat16, "l": torch.int64, "i": torch.int32, "f": torch.float32}
+
+
+def _all_dev(kinds: str, names: str, *tensors) -> None:
+    """``_dev`` for several tensors at once: a kind each (bf16, int64, int32, float32), names for the message."""
+    bad = _native.check(kinds, *tensors)
+    if bad >= 0:
+        _dev(tensors[bad], _KINDS[kinds[bad]], names.split()[bad])
 
 
 def _nn(n_nodes: Optional[torch.Tensor], S: int) -> Optional[torch.Tensor]:
@@ -98,9 +123,10 @@ def _host_nn(h_n_nodes: Optional[torch.Tensor], S: int) -> Optional[torch.Tensor
 
 
 def _kv_heads(k_cache: torch.Tensor, v_cache: torch.Tensor) -> int:
-    if k_cache.dim() != 3 or tuple(k_cache.shape) != tuple(v_cache.shape):
+    shape = k_cache.shape
+    if len(shape) != 3 or shape != v_cache.shape:
         raise GooseError("k_cache and v_cache must both be [rows][Hkv][D]")
-    return int(k_cache.shape[1])
+    return shape[1]
 
 
 def _same_heads(k_cache: torch.Tensor, v_cache: torch.Tensor, H: int, what: str) -> None:
@@ -115,12 +141,14 @@ class Goose:
     def __init__(self, max_S: int = 16, max_B: int = 128, max_H: int = 64, device: int = 0,
                  attn_impl: int = ATTN_AUTO):
         self.lib = load_library()
+        self.call = load_marshal()
         if not torch.cuda.is_available():
             raise GooseError("no CUDA device: the tree-verification step only runs on the GPU")
         h = ctypes.c_void_p()
         _check(self.lib.goose_create(ctypes.byref(h), ctypes.c_int(device), ctypes.c_int(max_S),
                                      ctypes.c_int(max_B), ctypes.c_int(max_H), ctypes.c_int(128)), "goose_create")
         self.h = h
+        self._h = h.value            # for the marshalled calls
         self.device = torch.device("cuda", device)
         self.max_S, self.max_B, self.max_H = max_S, max_B, max_H
         if attn_impl != ATTN_AUTO:
@@ -130,7 +158,7 @@ class Goose:
         if getattr(self, "h", None):
             torch.cuda.synchronize(self.device)
             self.lib.goose_destroy(self.h)
-            self.h = None
+            self.h = self._h = None
 
     def __del__(self):
         try:
@@ -160,18 +188,15 @@ class Goose:
                   out: Optional[torch.Tensor] = None, want_lse: bool = False,
                   lse: Optional[torch.Tensor] = None, n_nodes: Optional[torch.Tensor] = None
                   ) -> Tuple[torch.Tensor, Optional[torch.Tensor]]:
-        _dev(q, torch.bfloat16, "q"); _dev(k_cache, torch.bfloat16, "k_cache"); _dev(v_cache, torch.bfloat16, "v_cache")
-        _dev(row_off, torch.int64, "row_off"); _dev(ctx_len, torch.int32, "ctx_len"); _dev(parent, torch.int32, "parent")
+        _all_dev("bbblii", "q k_cache v_cache row_off ctx_len parent", q, k_cache, v_cache, row_off, ctx_len, parent)
         S, B, H, D = q.shape
         _same_heads(k_cache, v_cache, H, "tree_attn")
         if out is None:
             out = torch.empty_like(q)
         if want_lse and lse is None:
             lse = torch.empty((S, B, H), dtype=torch.float32, device=q.device)
-        _check(self.lib.goose_tree_attn(self.h, _p(q), _p(k_cache), _p(v_cache), ctypes.c_int64(k_cache.shape[0]),
-                                        _p(row_off), _p(ctx_len), _p(parent), _p(_nn(n_nodes, S)), ctypes.c_int(S), ctypes.c_int(B),
-                                        ctypes.c_int(H), ctypes.c_int(D), ctypes.c_float(scale), _p(out), _p(lse),
-                                        _stream()), "goose_tree_attn")
+        _check(self.call.tree_attn(self._h, q, k_cache, v_cache, k_cache.shape[0], row_off, ctx_len, parent, _nn(n_nodes, S),
+                                   S, B, H, D, scale, out, lse), "goose_tree_attn")
         return out, lse
 
     def tree_attn_gqa(self, q, k_cache, v_cache, row_off, ctx_len, parent, scale: float,
@@ -179,18 +204,15 @@ class Goose:
                       lse: Optional[torch.Tensor] = None, n_nodes: Optional[torch.Tensor] = None
                       ) -> Tuple[torch.Tensor, Optional[torch.Tensor]]:
         """Grouped-query attention: q [S][B][H][D], caches [rows][Hkv][D]; Hkv is read from the caches' shape."""
-        _dev(q, torch.bfloat16, "q"); _dev(k_cache, torch.bfloat16, "k_cache"); _dev(v_cache, torch.bfloat16, "v_cache")
-        _dev(row_off, torch.int64, "row_off"); _dev(ctx_len, torch.int32, "ctx_len"); _dev(parent, torch.int32, "parent")
+        _all_dev("bbblii", "q k_cache v_cache row_off ctx_len parent", q, k_cache, v_cache, row_off, ctx_len, parent)
         S, B, H, D = q.shape
         Hkv = _kv_heads(k_cache, v_cache)
         if out is None:
             out = torch.empty_like(q)
         if want_lse and lse is None:
             lse = torch.empty((S, B, H), dtype=torch.float32, device=q.device)
-        _check(self.lib.goose_tree_attn_gqa(self.h, _p(q), _p(k_cache), _p(v_cache), ctypes.c_int64(k_cache.shape[0]),
-                                            _p(row_off), _p(ctx_len), _p(parent), _p(_nn(n_nodes, S)), ctypes.c_int(S), ctypes.c_int(B),
-                                            ctypes.c_int(H), ctypes.c_int(Hkv), ctypes.c_int(D), ctypes.c_float(scale),
-                                            _p(out), _p(lse), _stream()), "goose_tree_attn_gqa")
+        _check(self.call.tree_attn_gqa(self._h, q, k_cache, v_cache, k_cache.shape[0], row_off, ctx_len, parent,
+                                       _nn(n_nodes, S), S, B, H, Hkv, D, scale, out, lse), "goose_tree_attn_gqa")
         return out, lse
 
     def node_topk(self, logits, k: int, V: Optional[int] = None, want_vals: bool = True,
@@ -207,15 +229,12 @@ class Goose:
             ids = torch.empty((rows, k), dtype=torch.int32, device=logits.device)
             vals = torch.empty((rows, k), dtype=torch.float32, device=logits.device) if want_vals else None
         nn = None if n_nodes is None else _nn(n_nodes, rows // max(B, 1))
-        _check(self.lib.goose_node_topk(self.h, _p(logits), ctypes.c_int(rows), ctypes.c_int(V), ctypes.c_int64(ldl),
-                                        ctypes.c_int(k), _p(nn), ctypes.c_int(B), _p(argmax), _p(ids), _p(vals), _stream()),
-               "goose_node_topk")
+        _check(self.call.node_topk(self._h, logits, rows, V, ldl, k, nn, B, argmax, ids, vals), "goose_node_topk")
         return argmax, ids, vals
 
     def harvest(self, logits, k: int, row_tok, adj_ids, adj_scores, V: Optional[int] = None):
         """Top-k + log-sum-exp of every row, then scatter into the adjacency table (updated in place)."""
-        _dev(logits, torch.bfloat16, "logits"); _dev(row_tok, torch.int32, "row_tok")
-        _dev(adj_ids, torch.int32, "adj_ids"); _dev(adj_scores, torch.float32, "adj_scores")
+        _all_dev("biif", "logits row_tok adj_ids adj_scores", logits, row_tok, adj_ids, adj_scores)
         rows, ldl = logits.shape
         V = ldl if V is None else V
         dev = logits.device
@@ -223,31 +242,26 @@ class Goose:
         ids = torch.empty((rows, k), dtype=torch.int32, device=dev)
         vals = torch.empty((rows, k), dtype=torch.float32, device=dev)
         lse = torch.empty(rows, dtype=torch.float32, device=dev)
-        _check(self.lib.goose_harvest(self.h, _p(logits), ctypes.c_int(rows), ctypes.c_int(V), ctypes.c_int64(ldl),
-                                      ctypes.c_int(k), _p(row_tok), ctypes.c_int(adj_ids.shape[0]), _p(adj_ids),
-                                      _p(adj_scores), _p(argmax), _p(ids), _p(vals), _p(lse), _stream()),
-               "goose_harvest")
+        _check(self.call.harvest(self._h, logits, rows, V, ldl, k, row_tok, adj_ids.shape[0], adj_ids, adj_scores, argmax, ids,
+                                 vals, lse), "goose_harvest")
         return argmax, ids, vals, lse
 
     def accept(self, draft_tok, parent, argmax, n_nodes: Optional[torch.Tensor] = None):
-        _dev(draft_tok, torch.int32, "draft_tok"); _dev(parent, torch.int32, "parent"); _dev(argmax, torch.int32, "argmax")
+        _all_dev("iii", "draft_tok parent argmax", draft_tok, parent, argmax)
         S, B = parent.shape
         path = torch.empty((S, B), dtype=torch.int32, device=parent.device)
         alen = torch.empty(S, dtype=torch.int32, device=parent.device)
         bonus = torch.empty(S, dtype=torch.int32, device=parent.device)
-        _check(self.lib.goose_accept(self.h, _p(draft_tok), _p(parent), _p(_nn(n_nodes, S)), _p(argmax), ctypes.c_int(S), ctypes.c_int(B),
-                                     _p(path), _p(alen), _p(bonus), _stream()), "goose_accept")
+        _check(self.call.accept(self._h, draft_tok, parent, _nn(n_nodes, S), argmax, S, B, path, alen, bonus), "goose_accept")
         return path, alen, bonus
 
     def kv_compact(self, k_cache, v_cache, row_off, ctx_len, path, accept_len, n_nodes: Optional[torch.Tensor] = None):
-        _dev(k_cache, torch.bfloat16, "k_cache"); _dev(v_cache, torch.bfloat16, "v_cache")
-        _dev(path, torch.int32, "path"); _dev(accept_len, torch.int32, "accept_len")
+        _all_dev("bbii", "k_cache v_cache path accept_len", k_cache, v_cache, path, accept_len)
         rows, H, D = k_cache.shape
         S, B = path.shape
         new_ctx = torch.empty(S, dtype=torch.int32, device=path.device)
-        _check(self.lib.goose_kv_compact(self.h, _p(k_cache), _p(v_cache), ctypes.c_int64(rows), _p(row_off),
-                                         _p(ctx_len), _p(path), _p(accept_len), _p(_nn(n_nodes, S)), ctypes.c_int(S), ctypes.c_int(B),
-                                         ctypes.c_int(H), ctypes.c_int(D), _p(new_ctx), _stream()), "goose_kv_compact")
+        _check(self.call.kv_compact(self._h, k_cache, v_cache, rows, row_off, ctx_len, path, accept_len, _nn(n_nodes, S), S, B,
+                                    H, D, new_ctx), "goose_kv_compact")
         return new_ctx
 
     # ------------------------------------------------------------------ whole step
@@ -272,13 +286,10 @@ class Goose:
         V = ldl if V is None else V
         if outs is None:
             outs = self.alloc_step_outputs(S, B, H, D, k, q.device)
-        _check(self.lib.goose_verify_step(
-            self.h, _p(q), _p(k_cache), _p(v_cache), ctypes.c_int64(k_cache.shape[0]), _p(row_off), _p(ctx_len),
-            _p(parent), _p(_nn(n_nodes, S)), _p(draft_tok), _p(logits), ctypes.c_int64(ldl), ctypes.c_int(S), ctypes.c_int(B),
-            ctypes.c_int(H), ctypes.c_int(D), ctypes.c_int(V), ctypes.c_int(k), ctypes.c_float(scale),
-            _p(outs["out"]), _p(outs.get("lse")), _p(outs["argmax"]), _p(outs["topk_ids"]), _p(outs["topk_vals"]),
-            _p(outs["path"]), _p(outs["accept_len"]), _p(outs["bonus"]), _p(outs["new_ctx_len"]), _stream()),
-            "goose_verify_step")
+        _check(self.call.verify_step(
+            self._h, q, k_cache, v_cache, k_cache.shape[0], row_off, ctx_len, parent, _nn(n_nodes, S), draft_tok, logits, ldl,
+            S, B, H, D, V, k, scale, outs["out"], outs.get("lse"), outs["argmax"], outs["topk_ids"], outs["topk_vals"],
+            outs["path"], outs["accept_len"], outs["bonus"], outs["new_ctx_len"]), "goose_verify_step")
         return outs
 
     def verify_step_gqa(self, q, k_cache, v_cache, row_off, ctx_len, parent, draft_tok, logits, k: int, scale: float,
@@ -290,13 +301,10 @@ class Goose:
         V = ldl if V is None else V
         if outs is None:
             outs = self.alloc_step_outputs(S, B, H, D, k, q.device)
-        _check(self.lib.goose_verify_step_gqa(
-            self.h, _p(q), _p(k_cache), _p(v_cache), ctypes.c_int64(k_cache.shape[0]), _p(row_off), _p(ctx_len),
-            _p(parent), _p(_nn(n_nodes, S)), _p(draft_tok), _p(logits), ctypes.c_int64(ldl), ctypes.c_int(S), ctypes.c_int(B),
-            ctypes.c_int(H), ctypes.c_int(Hkv), ctypes.c_int(D), ctypes.c_int(V), ctypes.c_int(k), ctypes.c_float(scale),
-            _p(outs["out"]), _p(outs.get("lse")), _p(outs["argmax"]), _p(outs["topk_ids"]), _p(outs["topk_vals"]),
-            _p(outs["path"]), _p(outs["accept_len"]), _p(outs["bonus"]), _p(outs["new_ctx_len"]), _stream()),
-            "goose_verify_step_gqa")
+        _check(self.call.verify_step_gqa(
+            self._h, q, k_cache, v_cache, k_cache.shape[0], row_off, ctx_len, parent, _nn(n_nodes, S), draft_tok, logits, ldl,
+            S, B, H, Hkv, D, V, k, scale, outs["out"], outs.get("lse"), outs["argmax"], outs["topk_ids"], outs["topk_vals"],
+            outs["path"], outs["accept_len"], outs["bonus"], outs["new_ctx_len"]), "goose_verify_step_gqa")
         return outs
 
     def verify_step_harvest(self, q, k_cache, v_cache, row_off, ctx_len, parent, draft_tok, logits, k: int, scale: float,
@@ -306,20 +314,18 @@ class Goose:
         grouped-query (Hkv is read from the caches' shape).  ``outs`` gains ``row_lse`` [S*B]."""
         S, B, H, D = q.shape
         Hkv = _kv_heads(k_cache, v_cache)
-        _dev(adj_ids, torch.int32, "adj_ids"); _dev(adj_scores, torch.float32, "adj_scores")
+        _all_dev("if", "adj_ids adj_scores", adj_ids, adj_scores)
         ldl = logits.shape[1]
         V = ldl if V is None else V
         if outs is None:
             outs = self.alloc_step_outputs(S, B, H, D, k, q.device)
         if "row_lse" not in outs:
             outs["row_lse"] = torch.empty(S * B, dtype=torch.float32, device=q.device)
-        _check(self.lib.goose_verify_step_harvest(
-            self.h, _p(q), _p(k_cache), _p(v_cache), ctypes.c_int64(k_cache.shape[0]), _p(row_off), _p(ctx_len),
-            _p(parent), _p(_nn(n_nodes, S)), _p(draft_tok), _p(logits), ctypes.c_int64(ldl), ctypes.c_int(S), ctypes.c_int(B),
-            ctypes.c_int(H), ctypes.c_int(Hkv), ctypes.c_int(D), ctypes.c_int(V), ctypes.c_int(k), ctypes.c_float(scale),
-            _p(outs["out"]), _p(outs.get("lse")), _p(outs["argmax"]), _p(outs["topk_ids"]), _p(outs["topk_vals"]),
-            _p(outs["path"]), _p(outs["accept_len"]), _p(outs["bonus"]), _p(outs["new_ctx_len"]), _p(outs["row_lse"]),
-            ctypes.c_int(adj_ids.shape[0]), _p(adj_ids), _p(adj_scores), _stream()), "goose_verify_step_harvest")
+        _check(self.call.verify_step_harvest(
+            self._h, q, k_cache, v_cache, k_cache.shape[0], row_off, ctx_len, parent, _nn(n_nodes, S), draft_tok, logits, ldl,
+            S, B, H, Hkv, D, V, k, scale, outs["out"], outs.get("lse"), outs["argmax"], outs["topk_ids"], outs["topk_vals"],
+            outs["path"], outs["accept_len"], outs["bonus"], outs["new_ctx_len"], outs["row_lse"], adj_ids.shape[0], adj_ids,
+            adj_scores), "goose_verify_step_harvest")
         return outs
 
     def verify_step_host_gqa(self, k_cache, v_cache, h_q, h_k_new, h_v_new, h_row_off, h_ctx_len, h_parent,

@@ -1,4 +1,5 @@
-"""Build libgoose.so (the CUDA library behind the C ABI) in-tree with nvcc for sm_100a."""
+"""Build libgoose.so (the CUDA library behind the C ABI, nvcc for sm_100a) and _marshal.so (its argument marshalling for
+Python) in-tree."""
 from __future__ import annotations
 
 import os
@@ -10,6 +11,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libgoose.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
 SOURCES = ["api.cu", "node_topk.cu", "harvest.cu", "accept.cu", "kv_compact.cu", "tree_attn_mma.cu",
            "tree_attn_umma.cu", "spine_tree.cpp"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
@@ -36,10 +38,31 @@ def _source_hash() -> str:
     return h.hexdigest()
 
 
+def _build_marshal() -> None:
+    """Host code only; the torch headers and libraries are those of the running interpreter's torch."""
+    import sysconfig
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = MARSHAL + ".tmp%d" % os.getpid()
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi())]
+    for d in (INCLUDE, os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+              os.path.join(cuda, "include"), sysconfig.get_path("include")):
+        cmd += ["-I", d]
+    cmd += [os.path.join(CSRC, "marshal.cpp"), "-o", tmp, "-L", HERE, "-l:libgoose.so", "-L", os.path.join(root, "lib"),
+            "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(r.stdout + r.stderr)
+        raise RuntimeError("building _marshal.so failed")
+    os.replace(tmp, MARSHAL)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every source for sm_100a and link libgoose.so; no-op when the library matches the sources."""
     src_hash = _source_hash()
-    if not force and os.path.exists(LIB) and os.path.exists(HASH_FILE) and open(HASH_FILE).read().strip() == src_hash:
+    if not force and os.path.exists(LIB) and os.path.exists(MARSHAL) and os.path.exists(HASH_FILE) and open(HASH_FILE).read().strip() == src_hash:
         return LIB
     objdir = os.path.join(HERE, "build")
     os.makedirs(objdir, exist_ok=True)
@@ -65,6 +88,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         sys.stderr.write(r.stdout + r.stderr)
         raise RuntimeError("link failed")
     os.replace(tmp, LIB)
+    _build_marshal()
     with open(HASH_FILE, "w") as f:
         f.write(src_hash + "\n")
     return LIB

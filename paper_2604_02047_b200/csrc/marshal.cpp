@@ -1,0 +1,95 @@
+// Argument marshalling of the stream-ordered entry points for Python: tensors to pointers, numbers to C numbers, the
+// current stream appended, nothing else.  A whole model's verification pass is 66 calls; through ctypes, with every argument
+// wrapped by Python code, a call took 13 us of host time, more than its kernels (measured at 32 heads and 1.5k keys).
+#include <torch/csrc/autograd/python_variable.h>
+#include <ATen/core/Tensor.h>
+#include <c10/cuda/CUDAStream.h>
+
+#include <tuple>
+#include <type_traits>
+#include <utility>
+
+#include "goose.h"
+
+namespace {
+
+template <typename T>
+bool convert(PyObject* o, T& v) {
+    if constexpr (std::is_pointer_v<T>) {
+        if (o == Py_None) v = nullptr;
+        else if (THPVariable_Check(o)) v = reinterpret_cast<T>(const_cast<void*>(THPVariable_Unpack(o).const_data_ptr()));
+        else v = reinterpret_cast<T>(PyLong_AsVoidPtr(o));
+    } else if constexpr (std::is_floating_point_v<T>) {
+        v = static_cast<T>(PyFloat_AsDouble(o));
+    } else {
+        v = static_cast<T>(PyLong_AsLongLong(o));
+    }
+    return !PyErr_Occurred();
+}
+
+// int f(args..., void* stream) as a Python function of args...
+template <auto F>
+struct Entry;
+template <typename... A, int (*F)(A...)>
+struct Entry<F> {
+    template <size_t... I>
+    static PyObject* run(PyObject* const* args, std::index_sequence<I...>) {
+        std::tuple<A...> v{};
+        try {
+            if (!(convert(args[I], std::get<I>(v)) && ...)) return nullptr;
+            std::get<sizeof...(A) - 1>(v) = c10::cuda::getCurrentCUDAStream().stream();
+        } catch (const std::exception& e) {
+            PyErr_SetString(PyExc_RuntimeError, e.what());
+            return nullptr;
+        }
+        int rc;
+        Py_BEGIN_ALLOW_THREADS
+        rc = std::apply(F, v);
+        Py_END_ALLOW_THREADS
+        return PyLong_FromLong(rc);
+    }
+    static PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t n) {
+        constexpr Py_ssize_t want = sizeof...(A) - 1;
+        if (n != want) return PyErr_Format(PyExc_TypeError, "%zd arguments expected, %zd given", want, n);
+        return run(args, std::make_index_sequence<want>{});
+    }
+};
+
+// check(kinds, tensors...): the index of the first one that is not a contiguous CUDA tensor of its kind, -1 if there is none
+PyObject* check(PyObject*, PyObject* const* args, Py_ssize_t n) {
+    Py_ssize_t len = 0;
+    const char* kinds = n > 0 ? PyUnicode_AsUTF8AndSize(args[0], &len) : nullptr;
+    if (!kinds) return nullptr;
+    if (len != n - 1) return PyErr_Format(PyExc_TypeError, "%zd kinds, %zd tensors", len, n - 1);
+    for (Py_ssize_t i = 0; i < len; ++i) {
+        if (!THPVariable_Check(args[i + 1])) return PyLong_FromSsize_t(i);
+        const at::Tensor& t = THPVariable_Unpack(args[i + 1]);
+        const at::ScalarType want = kinds[i] == 'b' ? at::kBFloat16 : kinds[i] == 'l' ? at::kLong : kinds[i] == 'i' ? at::kInt : at::kFloat;
+        if (!t.is_cuda() || t.scalar_type() != want || !t.is_contiguous()) return PyLong_FromSsize_t(i);
+    }
+    return PyLong_FromLong(-1);
+}
+
+template <auto F>
+constexpr PyMethodDef entry(const char* name) {
+    return {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&Entry<F>::call)), METH_FASTCALL, nullptr};
+}
+
+PyMethodDef methods[] = {
+    entry<&goose_tree_attn>("tree_attn"),
+    entry<&goose_tree_attn_gqa>("tree_attn_gqa"),
+    entry<&goose_node_topk>("node_topk"),
+    entry<&goose_harvest>("harvest"),
+    entry<&goose_accept>("accept"),
+    entry<&goose_kv_compact>("kv_compact"),
+    entry<&goose_verify_step>("verify_step"),
+    entry<&goose_verify_step_gqa>("verify_step_gqa"),
+    entry<&goose_verify_step_harvest>("verify_step_harvest"),
+    {"check", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&check)), METH_FASTCALL, nullptr},
+    {nullptr, nullptr, 0, nullptr}};
+
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__marshal() { return PyModule_Create(&module); }
