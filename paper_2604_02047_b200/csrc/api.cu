@@ -337,7 +337,7 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
     bool may_cluster = true;
     if (S > 0 && !attn_done) {
         const int g = H / Hkv, nb = B * g <= 128 ? B : 128 / g;
-        const int n = goose::attn_cluster(c, S, B, H, Hkv);
+        const int n = goose::attn_cluster(c, S, B, H, Hkv, kv_rows, true);
         if (n > 1) {
             topk_ctas = c->num_sms - (B + nb - 1) / nb * Hkv * n;
             may_cluster = topk_ctas > 0 && goose::topk_items(S * B, V) <= kTopkBeside * topk_ctas;

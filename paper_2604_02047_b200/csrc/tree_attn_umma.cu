@@ -16,7 +16,7 @@
 //                                  mask on the tiles that reach the tree rows, exp2, P (bf16) written back
 //                                  over the first 64 columns of the S buffer it came from, lazy rescaling
 //                                  of O in TMEM, epilogue (output or partial).
-// One sequence whose heads come out near the SM count (kCluster): a thread-block cluster takes each head instead, its CTAs
+// One sequence that is not too long (kCluster, see attn_cluster): a thread-block cluster takes each head instead, its CTAs
 // contiguous tile ranges of it.  No CTA then works on two heads (a second segment costs its softmax, PV and epilogue in
 // turn, 2 to 3 us at the end of the slowest CTA), and the cluster merges its head itself, behind its own barrier, instead
 // of a kernel behind all of them (boundary 1 us, a cold start on every SM, 2 us, and one more launch).
@@ -819,18 +819,27 @@ int auto_attn_impl(const goose_ctx* c, int S, int B, int H) {
     return c->encode_tiled ? GOOSE_ATTN_UMMA : GOOSE_ATTN_MMA;
 }
 
-// One sequence: a cluster per head where that leaves few SMs out.  The largest cluster (of at most 8 CTAs) that the device
-// holds one of per head at once; from 0.78 of the SMs on: an SM takes in 51 GB/s at most (a persistent grid on 225 MB: 68.8
-// us on 74 CTAs, 51.0 on 104, 48.2 on 120, 44.0 on 148), so 120 of 148 stream almost as fast as HBM gives and 104 do not.
-// Attention call, persistent grid and merge kernel -> clusters: 32 heads 10.4 -> 9.4 us (512 keys), 15.55 -> 13.7 (1.5k),
-// 16.25 -> 14.4 (2k); 40 heads 23.45 -> 22.5 (4k).  Several sequences may differ in length by any factor: persistent grid.
-int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv) {
+// One sequence: a cluster per head, the largest (of at most 8 CTAs) that the device holds one of per head at once -- where
+// the SMs that this leaves out cost less than the merge kernel and the second segments that it saves.  A tile of the longest
+// CTA takes about 1.5 us in either form; the line is drawn at `lost` = tiles / n - heads * tiles / SMs = 4.4 (3 with clusters
+// of two, and those only in a step, where the top-k runs beside them: alone they were 0.3 us slower at lost = 1.3).
+// ctx_len[] is device data: the tiles are bounded by the rows of the cache, so that a long prefix never meets the slower
+// form.  Attention call / step with harvest, persistent -> clusters (us, by lost):
+//   32 heads 512 keys (0.2) 10.4 -> 8.7 / -;   2k (0.6) 16.25 -> 14.0 / -;     16k (4.4) 50.4 -> 49.1 / 55.4 -> 52.6
+//   40 heads 4k (2.1) 23.45 -> 22.6 / -;       8k (4.1) 36.0 -> 36.0 / 41.1 -> 39.9;   16k (8.1) 61.1 -> 62.4 / 65.4 -> 66.4
+//   52 heads (n = 2) 2k (2.5) 20.3 -> 21.0 / 27.0 -> 24.1;   4k (4.9) 27.3 -> 31.1 / 33.3 -> 34.5
+//   32 over 8 heads, tree of 32 (n = 8)        4k (2.3) 15.0 -> 12.3 / 18.3 -> 15.8;   8k (4.5) 19.1 -> 17.7;   16k (8.9) 24.3 -> 27.8
+//   32 over 8, tree of 60: 16 heads (n = 6)    3k (1.4) 16.4 -> 12.9 / 25.1 -> 20.2;   8k (3.7) 21.6 -> 21.3;   16k (7.4) 30.2 -> 34.2
+//   16 over 2, tree of 16 (n = 8)              4k (3.6) 29.3 -> 11.7 (the merge kernel has 74 parts a head there)
+int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, bool in_step) {
+    if (S != 1) return 1;                               // (several may differ in length by any factor)
     const int g = H / Hkv, nb = B * g <= kTile ? B : kTile / g, Hw = (B + nb - 1) / nb * Hkv;
-    int cluster = 1;
-    if (S == 1)
-        for (int n = 2; n <= kMaxCluster; ++n)
-            if (c->max_clusters[n] >= Hw && 100 * Hw * n >= 78 * c->num_sms && Hw * n <= c->num_sms) cluster = n;
-    return cluster;
+    int n = 1;
+    for (int i = 2; i <= kMaxCluster; ++i)
+        if (c->max_clusters[i] >= Hw && Hw * i <= c->num_sms) n = i;
+    if (n == 1 || (n == 2 && !in_step)) return 1;
+    const int64_t tiles = (kv_rows + kTile - 1) / kTile;
+    return tiles * (c->num_sms - Hw * n) * 10 <= (int64_t)(n == 2 ? 30 : 44) * n * c->num_sms ? n : 1;
 }
 
 cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __nv_bfloat16* kc,
@@ -850,7 +859,8 @@ cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __
         !make_map(c->encode_tiled, &mv, vc, kv_rows, Hkv, kTile))
         return cudaErrorInvalidValue;
     const int Hw = n_mt * Hkv;
-    const int cluster = may_cluster ? attn_cluster(c, S, B, H, Hkv) : 1;
+    // (with a deferred merge the call is part of a step, which has asked attn_cluster itself and put the top-k beside)
+    const int cluster = may_cluster ? attn_cluster(c, S, B, H, Hkv, kv_rows, defer_merge != nullptr) : 1;
     int grid = cluster > 1 ? Hw * cluster : c->num_sms;
     if (2 * grid > c->n_slots) grid = c->n_slots / 2;
     const uint32_t g_magic = (uint32_t)((0x100000000ull + grid - 1) / grid);

@@ -39,8 +39,8 @@ def _attn(goose, x, n_nodes=None, parent=None):
     return out.float().cpu().numpy().astype(np.float64), lse.cpu().numpy(), int(goose.last_status(1)[0])
 
 
-# heads of the work list: 32 (clusters of 4) and 40 (clusters of 3); grouped, with one M tile or two: 32 or 64, 20 or 40
-@pytest.mark.parametrize("H,Hkv", [(32, 32), (40, 40), (64, 32), (40, 20)])
+# heads of the work list: 32 (clusters of 4) and 40 (clusters of 3); grouped, with one M tile to eight: 20 or 40, 8 to 32, 2 to 16
+@pytest.mark.parametrize("H,Hkv", [(32, 32), (40, 40), (40, 20), (32, 8), (16, 2)])
 @pytest.mark.parametrize("ctx,B", [(0, 1), (0, 128), (1, 16), (112, 16), (113, 16), (127, 1), (128, 60), (300, 64), (383, 33),
                                    (449, 60), (512, 80), (900, 128)])
 def test_cluster_shapes(goose, oracle, H, Hkv, ctx, B):
@@ -74,15 +74,16 @@ def test_cluster_invalid_tree(goose, ctx):
     assert status == 1 and np.all(out == 0.0)
 
 
-@pytest.mark.parametrize("B,V", [(16, 32000), (80, 32000), (128, 32000), (60, 70000)])
-def test_step_with_clusters(goose, oracle, B, V):
+@pytest.mark.parametrize("H,Hkv,B,V", [(32, 32, 16, 32000), (32, 32, 80, 32000), (32, 32, 128, 32000), (32, 32, 60, 70000),
+                                       (52, 52, 60, 32000), (32, 8, 60, 70000), (16, 2, 100, 32000)])
+def test_step_with_clusters(goose, oracle, H, Hkv, B, V):
     """Rows that fit beside the clusters (all, or several a CTA) and rows that do not: integers exact, caches exact."""
     from paper_2604_02047_b200 import binding
     rng = np.random.default_rng([B, V])
-    x = _inputs(rng, 32, 32, B, 600, V=V, k=8)
+    x = _inputs(rng, H, Hkv, B, 600, V=V, k=8)
     d = binding.to_device(x)
-    got = goose.verify_step(d["q"], d["k_cache"], d["v_cache"], d["row_off"], d["ctx_len"], d["parent"], d["draft_tok"],
-                            d["logits"], 8, x.scale)
+    got = goose.verify_step_gqa(d["q"], d["k_cache"], d["v_cache"], d["row_off"], d["ctx_len"], d["parent"], d["draft_tok"],
+                                d["logits"], 8, x.scale)
     torch.cuda.synchronize()
     am, ids, vals = oracle.node_topk(x.logits, 8)
     path, alen, bonus = oracle.accept(x.draft_tok, x.parent, am.reshape(1, B))
