@@ -3,8 +3,8 @@
 //
 // Row ctx+j <- row ctx+path[j].  path is increasing with path[j] >= j, so a thread that owns one
 // 16-byte column of the row and walks j upwards never overwrites a row it still has to read:
-// sources of later moves are > j.  Moves are issued in batches of 8 (all loads of a batch before its
-// stores; a batch's destinations are below every later source), which keeps 8 loads in flight per
+// sources of later moves are > j.  Moves are issued in batches of 16 (all loads of a batch before its
+// stores; a batch's destinations are below every later source), which keeps 16 loads in flight per
 // thread without any barrier.
 #include "goose_internal.cuh"
 #include "tree_attn_combine.cuh"
@@ -12,7 +12,7 @@
 namespace goose {
 
 constexpr int kCompactThreads = 128;
-constexpr int kCompactBatch = 8;
+constexpr int kCompactBatch = 16;
 
 // kCounts = false is the instantiation for n_nodes == NULL
 template <bool kCounts>
@@ -32,7 +32,13 @@ kv_compact_kernel(__nv_bfloat16* kc, __nv_bfloat16* vc,
     const int col = blockIdx.x * kCompactThreads + threadIdx.x;
     pdl_wait();
     pdl_trigger();
+    // one round of loads for everything that says what moves (path[] beyond accept_len is loaded and not looked at): a
+    // call is three dependent trips to L2 and HBM -- these, the rows, the stores -- and little else
+    static_assert(kCompactThreads >= kMaxB, "a thread a path entry");
+    const int pj = threadIdx.x < B ? path[(size_t)s * B + threadIdx.x] : -1;
     const int ctx = ctx_len[s];
+    const int64_t r0 = row_off[s];
+    int L = accept_len[s];
     const int nn = nodes_of(n_nodes, s, B);              // nodes of this sequence's tree; 0: it has left the batch
     if (nn == 0) {                                       // nothing moves, nothing is appended
         if (blockIdx.x == 0 && which == 0 && threadIdx.x == 0) {
@@ -41,20 +47,15 @@ kv_compact_kernel(__nv_bfloat16* kc, __nv_bfloat16* vc,
         }
         return;
     }
-    int L = accept_len[s];
+    if (threadIdx.x < kMaxB) s_path[threadIdx.x] = pj;
     if (threadIdx.x == 0) s_bad = 0;
     __syncthreads();
     // rows this sequence owns must lie inside the cache: never form an address from unchecked device data
-    const int64_t r0 = row_off[s];
     const bool bad_rows = ctx < 0 || r0 < 0 || r0 + ctx + nn > kv_rows;
     bool bad = (L < 0 || L >= nn) || bad_rows;
-    if (!bad) {
-        for (int j = threadIdx.x; j <= L; j += kCompactThreads) {
-            int pj = path[(size_t)s * B + j];
-            s_path[j] = pj;
-            int prev = (j == 0) ? -1 : path[(size_t)s * B + j - 1];
-            if (pj < j || pj >= nn || pj <= prev || (j == 0 && pj != 0)) s_bad = 1;
-        }
+    if (!bad && (int)threadIdx.x <= L) {
+        const int j = threadIdx.x, prev = j == 0 ? -1 : s_path[j - 1];
+        if (pj < j || pj >= nn || pj <= prev || (j == 0 && pj != 0)) s_bad = 1;
     }
     __syncthreads();
     bad = bad || s_bad;
@@ -65,7 +66,7 @@ kv_compact_kernel(__nv_bfloat16* kc, __nv_bfloat16* vc,
     }
     if (bad || col >= row_vec) return;
 
-    uint4* base = reinterpret_cast<uint4*>(which ? vc : kc) + ((size_t)(row_off[s] + ctx)) * row_vec + col;
+    uint4* base = reinterpret_cast<uint4*>(which ? vc : kc) + ((size_t)(r0 + ctx)) * row_vec + col;
     for (int j0 = 1; j0 <= L; j0 += kCompactBatch) {
         uint4 r[kCompactBatch];
 #pragma unroll
