@@ -42,6 +42,7 @@ struct Work {
     int S, H, B, G;           // H = heads of the work list = M tiles x key/value heads (M-tile-major)
     uint32_t G_magic;         // ceil(2^32 / G): division by G without the 20-instruction sequence
     long long total;          // all items
+    int pad;                  // idle items in front of every head, see set_total
     bool small;               // total * (G + 1) fits 31 bits: 32-bit arithmetic (64-bit division is slow on the GPU)
     // ctx_len comes from device memory: a negative value is treated as 0 (the tree rows alone).  A sequence's keys are
     // its prefix and the nodes its tree really has; a sequence without nodes (it has left the batch) has no items.
@@ -50,21 +51,40 @@ struct Work {
         const int nn = nodes_of(n_nodes, s, B);
         return nn == 0 ? 0 : (max(ctx_len[s], 0) + nn + kTile - 1) / kTile;
     }
-    __device__ __forceinline__ void set_total(long long tot) {
-        total = tot;
-        small = tot * (G + 1) < 0x7FFFFFFFll;
+    // items of a head of T tiles
+    __device__ __forceinline__ int width(int T) const { return T > 0 ? T + pad : 0; }
+    // A CTA that goes over from one head to the next pays for it (its epilogue and the next head's first softmax stand in
+    // turn: 2 to 3 us), so a head starts with idle items that take as much of the CTA's range.  Two tiles' worth, from two tiles a CTA on
+    // (below, a CTA could hold idle items alone).  Attention call without -> 1 / 2 / 3 idle items: 8 x 32 heads, 333 to 6000
+    // keys 81.5 -> 75.3 / 75.0 / 75.4 us; 2 x 32 over 8, tree of 61, 1000 to 5000 18.4 -> 17.2 / 16.4 / -; 4 x 32 over 8, 4k
+    // to 16k 31.0 -> 29.7 / 28.75 / -; 52 heads, 8k 43.5 -> 43.4 / 43.5 / 43.5.  (The partition is found by whole warps: the
+    // longer arithmetic, which once cost what the padding gained, is not seen: 43.55 with none and the code for it.)
+    __device__ __forceinline__ void set_total(long long tile_count, int live) {
+        pad = tile_count >= 2 * (long long)G ? 2 : 0;
+        total = tile_count + (long long)pad * H * live;
+        small = total * (G + 1) < 0x7FFFFFFFll;
     }
     __device__ __forceinline__ void init() {
         long long tot = 0;
-        for (int s = 0; s < S; ++s) tot += (long long)H * tiles(s);
-        set_total(tot);
+        int live = 0;
+        for (int s = 0; s < S; ++s) {
+            const int T = tiles(s);
+            tot += (long long)H * T;
+            live += T > 0;
+        }
+        set_total(tot, live);
     }
     // the same by a whole warp, lane s loading sequence s's length; returns the tiles of sequence `lane`
     __device__ __forceinline__ int init_warp(int lane) {
         const int mine = lane < S ? tiles(lane) : 0;
         long long sum = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)mine);
-        for (int s0 = 32; s0 < S; s0 += 32) sum += __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(s0 + lane < S ? tiles(s0 + lane) : 0));
-        set_total(H * sum);
+        int live = n_nodes ? __popc(__ballot_sync(0xFFFFFFFFu, mine > 0)) : S;
+        for (int s0 = 32; s0 < S; s0 += 32) {
+            const int more = s0 + lane < S ? tiles(s0 + lane) : 0;
+            sum += __reduce_add_sync(0xFFFFFFFFu, (uint32_t)more);
+            if (n_nodes) live += __popc(__ballot_sync(0xFFFFFFFFu, more > 0));
+        }
+        set_total(H * sum, live);
         return mine;
     }
     __device__ __forceinline__ long long cta_start(int c) const {
@@ -88,15 +108,21 @@ struct Cursor {               // walks items in order
         long long off = 0;
         int ss = 0;
         int TT = wk.tiles(0);
-        while (ss + 1 < wk.S && off + (long long)wk.H * TT <= w0) {
-            off += (long long)wk.H * TT;
+        while (ss + 1 < wk.S && off + (long long)wk.H * wk.width(TT) <= w0) {
+            off += (long long)wk.H * wk.width(TT);
             ++ss;
             TT = wk.tiles(ss);
         }
         s = ss; T = TT; w = w0;
         const long long rem = w0 - off;
-        h = wk.small ? (int)((uint32_t)rem / (uint32_t)TT) : (int)(rem / TT);
-        t = (int)(rem - (long long)h * TT);
+        const int W = wk.width(TT);
+        h = wk.small ? (int)((uint32_t)rem / (uint32_t)W) : (int)(rem / W);
+        enter(wk, (int)(rem - (long long)h * W));
+    }
+    // at item v of the head: past the idle ones
+    __device__ __forceinline__ void enter(const Work& wk, int v) {
+        t = v - wk.pad;
+        if (t < 0) { w -= t; t = 0; }
     }
     // the same by a whole warp for the common small batch: `mine` = tiles of sequence `lane` (Work::init_warp)
     __device__ __forceinline__ void seek_warp(const Work& wk, long long w0, int lane, int mine) {
@@ -105,25 +131,28 @@ struct Cursor {               // walks items in order
         uint32_t rem = (uint32_t)w0;
         s = 0;
         if (wk.S > 1) {
-            uint32_t upto = (uint32_t)wk.H * (uint32_t)mine;     // items up to and with sequence `lane`
+            const uint32_t own = (uint32_t)wk.H * (uint32_t)wk.width(mine);
+            uint32_t upto = own;                                 // items up to and with sequence `lane`
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, upto, o);
                 if (lane >= o) upto += u;
             }
             s = __ffs(__ballot_sync(0xFFFFFFFFu, upto > rem)) - 1;   // (w0 < total: some lane has it)
-            rem -= __shfl_sync(0xFFFFFFFFu, upto - (uint32_t)wk.H * (uint32_t)mine, s);
+            rem -= __shfl_sync(0xFFFFFFFFu, upto - own, s);
         }
         T = __shfl_sync(0xFFFFFFFFu, mine, s);
-        h = (int)__float2uint_rz(__fdividef((float)rem, (float)T));   // h < 2^16: off by one at most
-        t = (int)rem - h * T;
-        if (t < 0) { --h; t += T; }
-        if (t >= T) { ++h; t -= T; }
+        const int W = wk.width(T);
+        h = (int)__float2uint_rz(__fdividef((float)rem, (float)W));   // h < 2^16: off by one at most
+        int v = (int)rem - h * W;
+        if (v < 0) { --h; v += W; }
+        if (v >= W) { ++h; v -= W; }
+        enter(wk, v);
     }
     __device__ __forceinline__ void next(const Work& wk) {
         ++w; ++t;
         if (t == T) {
-            t = 0; ++h;
+            t = 0; ++h; w += wk.pad;
             if (h == wk.H) {                              // next sequence that has any items
                 h = 0; ++s;
                 if (!wk.n_nodes) { if (s < wk.S) T = wk.tiles(s); }
@@ -209,9 +238,9 @@ __device__ __forceinline__ void combine_heads(const CombineArgs& ca, int rg, int
     wk.ctx_len = ctx_len; wk.n_nodes = n_nodes; wk.S = S; wk.H = Hw; wk.B = B; wk.G = G; wk.G_magic = ca.G_magic;
     wk.init();
     long long off = 0;
-    for (int ss = 0; ss < s; ++ss) off += (long long)Hw * wk.tiles(ss);
+    for (int ss = 0; ss < s; ++ss) off += (long long)Hw * wk.width(wk.tiles(ss));
     const int T = wk.tiles(s);                             // 0: the sequence has no nodes, hence no items and no output
-    const long long head_first = off + (long long)h * T;
+    const long long head_first = off + (long long)h * wk.width(T) + wk.pad;
     const bool any = !kCounts || T > 0;                    // (without counts every sequence has tiles)
     const int c_lo = any ? wk.cta_of(head_first) : 0, c_hi = any ? wk.cta_of(head_first + T - 1) : 0;
     const bool whole = c_lo == c_hi;                       // written directly by the main kernel (or nothing to write)
