@@ -201,8 +201,8 @@ int goose_kv_compact(goose_ctx* ctx, void* k_cache, void* v_cache, int64_t kv_ro
                      int32_t* new_ctx_len, void* stream);
 
 /* The whole step on one stream, in data-flow order: tree attention, node top-k (rows = S*B),
- * acceptance walk, KV compaction (the last two share one launch, which with the tensor-core attention
- * kernel also finishes the attention: the merge of its split heads runs there, beside the walk).  All
+ * acceptance walk, KV compaction (the last two share one launch, which where the attention's heads
+ * are split over its whole grid also finishes the attention: their merge runs there, beside the walk).  All
  * results, out and lse included, are complete in stream order when the call's last kernel is.  Arguments
  * and results as in the four calls above (new_ctx_len must not overlap ctx_len).  q, the caches' tree rows, parent, draft_tok,
  * logits, ctx_len and row_off are INPUTS of the step: they must be complete in stream order before the
