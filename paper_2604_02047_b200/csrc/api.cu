@@ -337,9 +337,11 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
     bool may_cluster = true;
     if (S > 0 && !attn_done) {
         const int g = H / Hkv, nb = B * g <= 128 ? B : 128 / g;
-        const int n = goose::attn_cluster(c, S, B, H, Hkv, kv_rows, true);
+        const int n = goose::attn_cluster(c, S, B, H, Hkv, kv_rows, harvest ? 2 : 1);
         if (n > 1) {
-            topk_ctas = c->num_sms - (B + nb - 1) / nb * Hkv * n;
+            // a few SMs stay free for the step's last launch: its CTAs fit beside neither kernel, and its loads ahead of
+            // the wait would start only when the attention ends
+            topk_ctas = c->num_sms - (B + nb - 1) / nb * Hkv * n - 4;
             may_cluster = topk_ctas > 0 && goose::topk_items(S * B, V) <= kTopkBeside * topk_ctas;
             if (!may_cluster) topk_ctas = 0;
         }
@@ -354,7 +356,7 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
             cudaError_t ea = goose::launch_tree_attn_umma(c, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_cache,
                                                           (const __nv_bfloat16*)v_cache, kv_rows, row_off, ctx_len, parent,
                                                           n_nodes, S, B, H, Hkv, scale, (__nv_bfloat16*)out, lse,
-                                                          static_cast<cudaStream_t>(stream), &merge_plan, may_cluster);
+                                                          static_cast<cudaStream_t>(stream), &merge_plan, may_cluster, harvest ? 2 : 1);
             if (ea != cudaSuccess) return cuda_fail(ea);
         } else {
             topk_ctas = 0;

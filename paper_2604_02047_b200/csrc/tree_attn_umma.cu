@@ -830,23 +830,27 @@ int auto_attn_impl(const goose_ctx* c, int S, int B, int H) {
 //   52 heads (n = 2) 2k (2.5) 20.3 -> 21.0 / 27.0 -> 24.1;   4k (4.9) 27.3 -> 31.1 / 33.3 -> 34.5
 //   32 over 8 heads, tree of 32 (n = 8)        4k (2.3) 15.0 -> 12.3 / 18.3 -> 15.8;   8k (4.5) 19.1 -> 17.7;   16k (8.9) 24.3 -> 27.8
 //   32 over 8, tree of 60: 16 heads (n = 6)    3k (1.4) 16.4 -> 12.9 / 25.1 -> 20.2;   8k (3.7) 21.6 -> 21.3;   16k (7.4) 30.2 -> 34.2
+// A step without a harvest has a shorter top-k to hide, and on most of the SMs the line is 1.5 for it: 32 heads 2k (0.6)
+// 19.1 -> 18.3, 40 heads 4k (2.1) 26.7 -> 26.9 (and 27.8 -> 29.1 with longer accepted paths on cold inputs).
 //   16 over 2, tree of 16 (n = 8)              4k (3.6) 29.3 -> 11.7 (the merge kernel has 74 parts a head there)
-int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, bool in_step) {
+int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int step) {
     if (S != 1) return 1;                               // (several may differ in length by any factor)
     const int g = H / Hkv, nb = B * g <= kTile ? B : kTile / g, Hw = (B + nb - 1) / nb * Hkv;
     int n = 1;
     for (int i = 2; i <= kMaxCluster; ++i)
         if (c->max_clusters[i] >= Hw && Hw * i <= c->num_sms) n = i;
-    if (n == 1 || (n == 2 && !in_step)) return 1;
+    if (n == 1 || (n == 2 && step == 0)) return 1;
     const int64_t tiles = (kv_rows + kTile - 1) / kTile;
-    return tiles * (c->num_sms - Hw * n) * 10 <= (int64_t)(n == 2 ? 30 : 44) * n * c->num_sms ? n : 1;
+    const bool many = 10 * Hw * n >= 7 * c->num_sms;
+    const int line = step == 1 && many ? 15 : n == 2 ? 30 : 44;
+    return tiles * (c->num_sms - Hw * n) * 10 <= (int64_t)line * n * c->num_sms ? n : 1;
 }
 
 cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __nv_bfloat16* kc,
                                   const __nv_bfloat16* vc, int64_t kv_rows, const int64_t* row_off,
                                   const int32_t* ctx_len, const int32_t* parent, const int32_t* n_nodes, int S, int B, int H,
                                   int Hkv, float scale, __nv_bfloat16* out, float* lse, cudaStream_t st,
-                                  CombinePlan* defer_merge, bool may_cluster) {
+                                  CombinePlan* defer_merge, bool may_cluster, int step) {
     if (defer_merge) defer_merge->valid = false;
     if (!c->encode_tiled) return cudaErrorNotSupported;
     if (S == 0) return cudaSuccess;
@@ -859,8 +863,7 @@ cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __
         !make_map(c->encode_tiled, &mv, vc, kv_rows, Hkv, kTile))
         return cudaErrorInvalidValue;
     const int Hw = n_mt * Hkv;
-    // (with a deferred merge the call is part of a step, which has asked attn_cluster itself and put the top-k beside)
-    const int cluster = may_cluster ? attn_cluster(c, S, B, H, Hkv, kv_rows, defer_merge != nullptr) : 1;
+    const int cluster = may_cluster ? attn_cluster(c, S, B, H, Hkv, kv_rows, step) : 1;
     int grid = cluster > 1 ? Hw * cluster : c->num_sms;
     if (2 * grid > c->n_slots) grid = c->n_slots / 2;
     const uint32_t g_magic = (uint32_t)((0x100000000ull + grid - 1) / grid);
