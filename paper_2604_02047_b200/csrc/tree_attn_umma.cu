@@ -470,13 +470,12 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                     ok = mbar_wait(hd, &hd->s_full[jg & 1], (jg >> 1) & 1, status);
                     if (!ok) break;
                     tc_fence_after();
-                    // The exponentials of a tile are taken relative to the maximum known before it, while the tile's own
-                    // maximum is found beside them (the special-function units, 8 cycles an instruction and warp, take 1024
-                    // of the about 2000 cycles of a tile; the maximum's instructions hide behind them).  Only where it grew
-                    // by more than the threshold, and on a segment's first tile, the maximum comes first: O is rescaled
-                    // and the scores are read again (P replaces them only at the end).
-                    bool max_first = first;
-                    while (ok && warp_has_rows) {
+                    // The maximum stands in front of the exponentials.  Taken beside them, relative to the older maximum and with
+                    // a second pass over a tile whose maximum grew by more than the threshold, the tile's registers did not
+                    // fit (20 to 112 bytes of spill loads in every instantiation) and such a tile cost twice.  Attention call
+                    // beside -> in front, us: 32 heads 4k 20.4 -> 18.9, 52 heads 8k 44.1 -> 43.5, 8 x 32 heads 16k 336 -> 328,
+                    // 32 over 8 heads 16k 30.0 -> 28.6; scores that rise by 2^9 a tile, 4 x 32 heads 2k to 8k 66.9 -> 48.9.
+                    if (warp_has_rows) {
                         const uint32_t s_addr = tmem + kColS + (jg & 1) * 128 + lane_sel;
                         TMEM_LD32(s_addr, v, 0); TMEM_LD32(s_addr + 32, v, 32);
                         TMEM_LD32(s_addr + 64, v, 64); TMEM_LD32(s_addr + 96, v, 96);
@@ -499,16 +498,18 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                             for (int c = 0; c < 128; ++c)
                                 v[c] = ((vw[c >> 5] >> (c & 31)) & 1u) ? v[c] : 0xFF800000u;   // -inf
                         }
-                        if (max_first) {
-                            // one warp per scheduler: nothing hides a serial chain, so the row maximum (and the row
-                            // sum below) run as four independent chains
-                            float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                        // one warp per scheduler: nothing hides a serial chain, so the row maximum (and the row sum below)
+                        // run as four independent chains
+                        float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-                            for (int c = 0; c < 128; c += 8)
+                        for (int c = 0; c < 128; c += 8)
 #pragma unroll
-                                for (int e = 0; e < 4; ++e) mx4[e] = max3(mx4[e], __uint_as_float(v[c + 2 * e]), __uint_as_float(v[c + 2 * e + 1]));
-                            const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * scale_log2;   // scale > 0
-                            const float m_new = fmaxf(m_run, mx);
+                            for (int e = 0; e < 4; ++e) mx4[e] = max3(mx4[e], __uint_as_float(v[c + 2 * e]), __uint_as_float(v[c + 2 * e + 1]));
+                        const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * scale_log2;   // scale > 0
+                        const float m_new = fmaxf(m_run, mx);
+                        // lazy rescaling: keep the stale maximum unless it grew by more than the threshold (in a row that
+                        // exists: the others hold whatever shared memory held, and results may not depend on that)
+                        if (__any_sync(0xFFFFFFFFu, first || (row_valid && m_new > m_run + kRescaleThreshold))) {
                             const float alpha = (m_run == -INFINITY) ? 0.f : ex2(m_run - m_new);
                             if (!first) {
                                 // O holds tiles < t of this segment: wait for PV(t-1), then scale the row
@@ -534,20 +535,12 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                         const float neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
                         const unsigned long long scale2 = pack_f32x2(scale_log2, scale_log2), neg2 = pack_f32x2(neg_m, neg_m);
                         unsigned long long ls2[2] = {0, 0};
-                        float mx2[2] = {-INFINITY, -INFINITY};
 #pragma unroll
                         for (int e = 0; e < 64; ++e) {
-                            const float s0 = __uint_as_float(v[2 * e]), s1 = __uint_as_float(v[2 * e + 1]);
-                            if (!first) mx2[e & 1] = max3(mx2[e & 1], s0, s1);
-                            const float2 x2 = unpack_f32x2(fma_f32x2(pack_f32x2(s0, s1), scale2, neg2));
+                            const float2 x2 = unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1])), scale2, neg2));
                             const float p0 = ex2(x2.x), p1 = ex2(x2.y);
                             ls2[e & 1] = add_f32x2(ls2[e & 1], pack_f32x2(p0, p1));
                             v[e] = pack_bf16x2(p0, p1);
-                        }
-                        if (!max_first) {
-                            const bool grew = row_valid && fmaxf(mx2[0], mx2[1]) * scale_log2 > m_run + kRescaleThreshold;
-                            max_first = __any_sync(0xFFFFFFFFu, grew);
-                            if (max_first) continue;
                         }
                         const float2 l2 = unpack_f32x2(add_f32x2(ls2[0], ls2[1]));
                         l_run += l2.x + l2.y;
@@ -557,7 +550,6 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                         TMEM_ST32(p_taddr, v, 0);
                         TMEM_ST32(p_taddr + 32, v, 32);
                         tmem_wait_st();
-                        break;
                     }
                     // observe every phase of pv_done in order (a parity wait must never lag two phases behind its
                     // barrier); by now PV(jg-1) has normally completed, so this does not stall
