@@ -1,6 +1,7 @@
 // Argument marshalling of the stream-ordered entry points for Python: tensors to pointers, numbers to C numbers, the
 // current stream appended, nothing else.  A whole model's verification pass is 66 calls; through ctypes, with every argument
 // wrapped by Python code, a call took 13 us of host time, more than its kernels (measured at 32 heads and 1.5k keys).
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <ATen/core/Tensor.h>
 #include <c10/cuda/CUDAStream.h>
@@ -27,6 +28,21 @@ bool convert(PyObject* o, T& v) {
     return !PyErr_Occurred();
 }
 
+// f(), its C++ exceptions as Python ones: none may leave an entry (a tensor subclass answers in Python, and may raise)
+template <typename Fn>
+PyObject* guarded(Fn f) {
+    try {
+        return f();
+    } catch (python_error& e) {
+        e.restore();
+    } catch (const c10::Error& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what_without_backtrace());
+    } catch (const std::exception& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+    }
+    return nullptr;
+}
+
 // int f(args..., void* stream) as a Python function of args...
 template <auto F>
 struct Entry;
@@ -34,19 +50,16 @@ template <typename... A, int (*F)(A...)>
 struct Entry<F> {
     template <size_t... I>
     static PyObject* run(PyObject* const* args, std::index_sequence<I...>) {
-        std::tuple<A...> v{};
-        try {
+        return guarded([&]() -> PyObject* {
+            std::tuple<A...> v{};
             if (!(convert(args[I], std::get<I>(v)) && ...)) return nullptr;
             std::get<sizeof...(A) - 1>(v) = c10::cuda::getCurrentCUDAStream().stream();
-        } catch (const std::exception& e) {
-            PyErr_SetString(PyExc_RuntimeError, e.what());
-            return nullptr;
-        }
-        int rc;
-        Py_BEGIN_ALLOW_THREADS
-        rc = std::apply(F, v);
-        Py_END_ALLOW_THREADS
-        return PyLong_FromLong(rc);
+            int rc;
+            Py_BEGIN_ALLOW_THREADS
+            rc = std::apply(F, v);
+            Py_END_ALLOW_THREADS
+            return PyLong_FromLong(rc);
+        });
     }
     static PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t n) {
         constexpr Py_ssize_t want = sizeof...(A) - 1;
@@ -61,13 +74,15 @@ PyObject* check(PyObject*, PyObject* const* args, Py_ssize_t n) {
     const char* kinds = n > 0 ? PyUnicode_AsUTF8AndSize(args[0], &len) : nullptr;
     if (!kinds) return nullptr;
     if (len != n - 1) return PyErr_Format(PyExc_TypeError, "%zd kinds, %zd tensors", len, n - 1);
-    for (Py_ssize_t i = 0; i < len; ++i) {
-        if (!THPVariable_Check(args[i + 1])) return PyLong_FromSsize_t(i);
-        const at::Tensor& t = THPVariable_Unpack(args[i + 1]);
-        const at::ScalarType want = kinds[i] == 'b' ? at::kBFloat16 : kinds[i] == 'l' ? at::kLong : kinds[i] == 'i' ? at::kInt : at::kFloat;
-        if (!t.is_cuda() || t.scalar_type() != want || !t.is_contiguous()) return PyLong_FromSsize_t(i);
-    }
-    return PyLong_FromLong(-1);
+    return guarded([&]() -> PyObject* {
+        for (Py_ssize_t i = 0; i < len; ++i) {
+            if (!THPVariable_Check(args[i + 1])) return PyLong_FromSsize_t(i);
+            const at::Tensor& t = THPVariable_Unpack(args[i + 1]);
+            const at::ScalarType want = kinds[i] == 'b' ? at::kBFloat16 : kinds[i] == 'l' ? at::kLong : kinds[i] == 'i' ? at::kInt : at::kFloat;
+            if (!t.is_cuda() || t.scalar_type() != want || !t.is_contiguous()) return PyLong_FromSsize_t(i);
+        }
+        return PyLong_FromLong(-1);
+    });
 }
 
 template <auto F>

@@ -1,0 +1,43 @@
+"""The argument marshalling of the stream-ordered calls, as far as it goes without a GPU: what it does with tensors happens
+before the first CUDA call."""
+import os
+import subprocess
+import sys
+
+import pytest
+import torch
+
+from paper_2604_02047_b200 import binding, build
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def marshal():
+    build.build()
+    return binding.load_marshal()
+
+
+def test_a_tensor_that_raises_is_an_exception():
+    """A subclass that answers is_contiguous() in Python and raises there (in a process of its own: as a C++ exception that
+    leaves the entry it ends the interpreter)."""
+    code = '''
+import torch
+from paper_2604_02047_b200 import binding
+
+class Raises(torch.Tensor):
+    @staticmethod
+    def __new__(cls):
+        return torch.Tensor._make_wrapper_subclass(cls, (4,), dtype=torch.float32, device="cuda", dispatch_sizes_strides_policy="strides")
+    @classmethod
+    def __torch_dispatch__(cls, func, types, args=(), kwargs=None):
+        raise KeyError("not here")
+
+try:
+    binding.load_marshal().check("f", Raises())
+except KeyError as e:
+    print("raised", e)
+'''
+    build.build()
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0 and "raised 'not here'" in r.stdout, (r.returncode, r.stdout, r.stderr[-500:])
