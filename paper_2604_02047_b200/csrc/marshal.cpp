@@ -18,7 +18,12 @@ template <typename T>
 bool convert(PyObject* o, T& v) {
     if constexpr (std::is_pointer_v<T>) {
         if (o == Py_None) v = nullptr;
-        else if (THPVariable_Check(o)) v = reinterpret_cast<T>(const_cast<void*>(THPVariable_Unpack(o).const_data_ptr()));
+        else if (THPVariable_Check(o)) {
+            // what the library writes is asked for as such: a copy-on-write tensor gets memory of its own then
+            const at::Tensor& t = THPVariable_Unpack(o);
+            if constexpr (std::is_const_v<std::remove_pointer_t<T>>) v = static_cast<T>(t.const_data_ptr());
+            else v = static_cast<T>(t.mutable_data_ptr());
+        }
         else v = reinterpret_cast<T>(PyLong_AsVoidPtr(o));
     } else if constexpr (std::is_floating_point_v<T>) {
         v = static_cast<T>(PyFloat_AsDouble(o));

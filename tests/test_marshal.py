@@ -41,3 +41,19 @@ except KeyError as e:
     build.build()
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
     assert r.returncode == 0 and "raised 'not here'" in r.stdout, (r.returncode, r.stdout, r.stderr[-500:])
+
+
+def test_what_is_written_is_not_shared(marshal):
+    """A copy-on-write clone among the outputs gets memory of its own; one among the inputs need not."""
+    def accept(tok, path):
+        x = torch.zeros(4, dtype=torch.int32)
+        try:
+            marshal.accept(None, tok, x, None, x, 1, 4, path, x, x)   # no context: an error code where there is a GPU
+        except RuntimeError:
+            pass                                                      # no current stream without one
+
+    base = torch.zeros(4, dtype=torch.int32)
+    read, written = torch._lazy_clone(base), torch._lazy_clone(base)
+    accept(read, written)
+    assert torch._C._is_cow_tensor(read) and not torch._C._is_cow_tensor(written)
+    assert written.data_ptr() != torch._C._data_address(base) and written.tolist() == [0, 0, 0, 0]
