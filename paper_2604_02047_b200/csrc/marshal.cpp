@@ -16,15 +16,22 @@ namespace {
 
 template <typename T>
 bool convert(PyObject* o, T& v) {
-    if constexpr (std::is_pointer_v<T>) {
+    if constexpr (std::is_same_v<T, goose_ctx*>) {
+        v = o == Py_None ? nullptr : static_cast<T>(PyLong_AsVoidPtr(o));
+    } else if constexpr (std::is_pointer_v<T>) {
         if (o == Py_None) v = nullptr;
         else if (THPVariable_Check(o)) {
             // what the library writes is asked for as such: a copy-on-write tensor gets memory of its own then
             const at::Tensor& t = THPVariable_Unpack(o);
             if constexpr (std::is_const_v<std::remove_pointer_t<T>>) v = static_cast<T>(t.const_data_ptr());
             else v = static_cast<T>(t.mutable_data_ptr());
+        } else {
+            // any other object has to say itself where its memory is (a number is not an address)
+            PyObject* at = PyObject_CallMethod(o, "data_ptr", nullptr);
+            if (!at) return false;
+            v = static_cast<T>(PyLong_AsVoidPtr(at));
+            Py_DECREF(at);
         }
-        else v = reinterpret_cast<T>(PyLong_AsVoidPtr(o));
     } else if constexpr (std::is_floating_point_v<T>) {
         v = static_cast<T>(PyFloat_AsDouble(o));
     } else {

@@ -57,3 +57,13 @@ def test_what_is_written_is_not_shared(marshal):
     accept(read, written)
     assert torch._C._is_cow_tensor(read) and not torch._C._is_cow_tensor(written)
     assert written.data_ptr() != torch._C._data_address(base) and written.tolist() == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("number", [0, 1, 4096, True])
+def test_a_number_is_not_an_address(marshal, number):
+    x = torch.zeros(4, dtype=torch.int32)
+    for at in (1, 2, 4, 7, 9):                                        # each tensor of the call, read or written
+        args = [None, x, x, None, x, 1, 4, x, x, x]
+        args[at] = number
+        with pytest.raises(AttributeError):
+            marshal.accept(*args)
