@@ -2,8 +2,8 @@
 
 Every function takes torch CUDA tensors (or, for the ``*_host`` call, pinned CPU tensors),
 passes their ``data_ptr()`` and the current CUDA stream to ``libgoose.so`` and returns the
-output tensors.  The stream-ordered calls go through ``_marshal.so`` (``csrc/marshal.cpp``), the others through ctypes.  No step of the method runs in Python or in torch ops; if the library is
-missing or a call fails, an exception is raised -- there is no fallback path.
+output tensors.  The stream-ordered calls go through the extension module ``_marshal`` (``csrc/marshal.cpp``), the others
+through ctypes.  No step of the method runs in Python or in torch ops; if the library is missing or a call fails, an exception is raised -- there is no fallback path.
 """
 from __future__ import annotations
 
@@ -61,15 +61,18 @@ def load_library() -> ctypes.CDLL:
 
 
 def load_marshal():
-    """Load ``_marshal.so``: the argument marshalling of the stream-ordered calls (linked against ``libgoose.so``)."""
+    """Load the extension module ``_marshal``: the argument marshalling of the stream-ordered calls (linked against ``libgoose.so``)."""
     global _native
     if _native is None:
         load_library()
         try:
             from . import _marshal
         except ImportError as e:
-            raise GooseError("_marshal.so is missing or does not load (%s): run `python -m paper_2604_02047_b200.build` "
-                             "(there is no fallback path)" % e) from e
+            raise GooseError("the extension module _marshal is missing or does not load (%s): run "
+                             "`python -m paper_2604_02047_b200.build` (there is no fallback path)" % e) from e
+        if _marshal.built_for != torch.__version__:           # it reads tensors by the layout of that version's headers
+            raise GooseError("the extension module _marshal was built for torch %s, this is %s: run "
+                             "`python -m paper_2604_02047_b200.build`" % (_marshal.built_for, torch.__version__))
         _native = _marshal
     return _native
 
