@@ -554,8 +554,8 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
             run = lane < k ? s_run[lane] : 0ull;
             __syncwarp();
             if (LSE) {
-                const float M = fmaxf(run_m, cmax);
-                run_s = run_s * expf(run_m - M) + csum * expf(cmax - M);
+                const float M = fmaxf(run_m, cmax);          // -inf: nothing but -inf so far, both sums are 0
+                if (M != -INFINITY) run_s = run_s * expf(run_m - M) + csum * expf(cmax - M);
                 run_m = M;
             }
         }
@@ -617,7 +617,7 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
                 float sum = 0.f;
                 for (int c = 0; c < n_parts; ++c) {
                     const float2 ms = __ldcg(&ws_lse[(size_t)row * chunks + c]);
-                    sum += ms.y * expf(ms.x - M);
+                    if (ms.x != -INFINITY) sum += ms.y * expf(ms.x - M);
                 }
                 fin_m = M; fin_s = sum;
             }

@@ -72,3 +72,42 @@ def test_candidates_of_odd_rows(goose, oracle, V, k):
     got = lse.cpu().numpy().astype(np.float64)
     assert np.all(np.abs(got - ref) <= 6e-6 + np.abs(ref) * 2.0 ** -23), (got - ref)
     assert goose.last_status(2).tolist() == [0, 0]
+
+
+@pytest.fixture(scope="module")
+def goose_many():
+    from paper_2604_02047_b200 import binding, build
+    build.build()
+    g = binding.Goose(max_S=8, max_B=128, max_H=4)
+    yield g
+    g.close()
+
+
+@pytest.mark.parametrize("k", [8, 16])
+@pytest.mark.parametrize("V,repeats", [(4104, 62), (32768, 62), (70008, 21), (128256, 16), (262144, 8)])
+def test_odd_rows_many_a_cta(goose_many, oracle, V, repeats, k):
+    """The same rows repeated and shuffled: six items and more for every CTA, so that stages and slots come back into use
+    behind odd rows, and several chunks of a masked row meet in one CTA or in two."""
+    rng = np.random.default_rng([V, k])
+    kinds = _rows(V, rng)
+    n, sms = len(kinds), torch.cuda.get_device_properties(0).multi_processor_count
+    assert n * repeats * -(-V // 32768) > 6 * sms
+    which = rng.permutation(np.repeat(np.arange(n), repeats))
+    x = torch.from_numpy(kinds.view(np.int16)).view(torch.bfloat16).cuda()[torch.from_numpy(which).cuda()].contiguous()
+    ref_am, ref_ids, ref_vals = (a[which] for a in oracle.node_topk(kinds, k))
+    rows = len(which)
+    wide = torch.from_numpy(kinds.view(np.int16)).view(torch.bfloat16).double().numpy()
+    top = wide.max(axis=1)
+    ref = (top + np.log(np.exp(wide - top[:, None]).sum(axis=1)))[which]
+    for _ in range(3):
+        am, ids, vals = goose_many.node_topk(x, k)
+        adj_ids = torch.zeros((rows, k), dtype=torch.int32, device="cuda")
+        adj_sc = torch.zeros((rows, k), dtype=torch.float32, device="cuda")
+        am2, ids2, vals2, lse = goose_many.harvest(x, k, torch.arange(rows, dtype=torch.int32, device="cuda"), adj_ids, adj_sc)
+        torch.cuda.synchronize()
+        for a, i, v in ((am, ids, vals), (am2, ids2, vals2)):
+            assert np.array_equal(i.cpu().numpy(), ref_ids) and np.array_equal(a.cpu().numpy(), ref_am)
+            assert np.array_equal(v.cpu().numpy().astype(np.float64), ref_vals)
+        got = lse.cpu().numpy().astype(np.float64)
+        assert np.all(np.abs(got - ref) <= 6e-6 + np.abs(ref) * 2.0 ** -23), (got - ref)
+    assert goose_many.last_status(8).tolist() == [0] * 8
