@@ -55,6 +55,7 @@ constexpr int kTopkListCap = kMaxK * kTopkPerThread + kTopkCollectWarps * kMaxK 
 constexpr int kTopkSmem = kTopkStages * kTopkStageBytes + kTopkSlots * kTopkListCap * 4;   // dynamic shared memory
 constexpr long long kTopkWaitCycles = 2000000000ll;          // bound of every wait: about one second of SM clock
 constexpr float kTopkLog2e = 1.4426950408889634f;
+constexpr float kTopkLateMax = 11.f;                         // see the sums of exponentials: 11 log2(e) < 16
 constexpr uint32_t kImageNegInf = 0x007Fu;                   // sortable16 of -inf
 
 typedef unsigned long long u64;
@@ -287,9 +288,12 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
             __nv_bfloat162 m2;
             if (LSE) {
                 // sum of exp(x - c), c = the largest value of the warp's first sweep; the control warp weights the sum with
-                // the c it was taken with.  Elements past the end: 0.  Later sweeps may hold larger values: only where one
-                // is above c by more than 44 (2^64) is the sum taken again.  (Two lanes of packed fp32 arithmetic an
-                // instruction: the issue slots, not the special-function units, would be the limit otherwise.)
+                // the c it was taken with.  Elements past the end: 0.  Later sweeps may hold larger values: where one
+                // is above c by more than 11 the sum is taken again, so that the exponents' arguments stay below 16 and their
+                // rounding (2^-21) below that of the other steps.  (With a bound of 44 rows whose largest values come late were
+                // off by up to 1.6e-6 instead of 0.8e-6; one warp that sums twice costs 2.4 us of 24 with 1500 x 32000 logits
+                // that have one token 15 above the field each.)  Two lanes of packed fp32 arithmetic an instruction: the
+                // issue slots, not the special-function units, would be the limit otherwise.
                 auto add8 = [&](const uint4& w, u64 (&es)[2], float c) {
                     const u64 l2 = pack_f32x2(kTopkLog2e, kTopkLog2e), c2 = pack_f32x2(-c, -c);
                     const uint32_t y[4] = {w.x, w.y, w.z, w.w};
@@ -312,7 +316,7 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
                     add8(w, es, c);
                 }
                 const uint32_t wmax = __reduce_max_sync(0xFFFFFFFFu, image_max(m2));
-                if (wmax != kImageNegInf && (sum_max == kImageNegInf || float_of_sortable16(wmax) - c > 44.f)) {
+                if (wmax != kImageNegInf && (sum_max == kImageNegInf || float_of_sortable16(wmax) - c > kTopkLateMax)) {
                     sum_max = wmax;
                     c = float_of_sortable16(wmax);
                     es[0] = es[1] = 0;

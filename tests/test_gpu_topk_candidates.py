@@ -2,7 +2,8 @@
 threshold, chunk lengths at the edges of a thread's, a sweep's and a chunk's share, masked rows, and row log-sum-exps whose
 largest value comes late, far above the first sweep's, or not at all.  Identifiers and values bit-exact against the oracle;
 the log-sum-exp against numpy in 64 bits: fp32 sums of at most 2^18 terms in chains of at most 64, then trees, hence
-|error| <= (64 + 20) 2^-24 + 2 ulp of ex2.approx (2^-22) = 6e-6, plus half an ulp of the largest |lse| here (2^-17)."""
+|error| <= (64 + 20) 2^-24 + 2 ulp of ex2.approx (2^-22) + the rounding of two arguments below 16 (2^-20 ln 2) = 6e-6, plus
+half an ulp of the largest |lse| here (2^-17)."""
 import numpy as np
 import pytest
 import torch
@@ -111,3 +112,20 @@ def test_odd_rows_many_a_cta(goose_many, oracle, V, repeats, k):
         got = lse.cpu().numpy().astype(np.float64)
         assert np.all(np.abs(got - ref) <= 6e-6 + np.abs(ref) * 2.0 ** -23), (got - ref)
     assert goose_many.last_status(8).tolist() == [0] * 8
+
+
+@pytest.mark.parametrize("V", [32000, 128256])
+@pytest.mark.parametrize("below", [0, 8, 12, 24, 43])
+def test_log_sum_exp_of_late_values(goose_many, V, below):
+    """Rows of which the first eighth of every chunk (what the warps see first) lies `below` the rest.  28000 and more terms of
+    one size: their own roundings average out, what is left is half an ulp of a result in [8, 16) (2^-21), the two arguments'
+    roundings while they are below 16 (2^-21 ln 2 each) and an ulp of the logarithm (2^-22 of at most 3): 1.9e-6 at worst,
+    and 1.2e-6 without the logarithm's, which is rarely a whole one.  With arguments up to 64 it was 1.6e-6."""
+    g = torch.Generator(device="cuda").manual_seed(below)
+    x = torch.randn((300, V), generator=g, device="cuda")
+    x[:, torch.arange(V, device="cuda") % (V // -(-V // 32768)) < 4096] -= below
+    x = x.bfloat16()
+    adj_ids = torch.zeros((300, 8), dtype=torch.int32, device="cuda")
+    adj_sc = torch.zeros((300, 8), dtype=torch.float32, device="cuda")
+    lse = goose_many.harvest(x, 8, torch.arange(300, dtype=torch.int32, device="cuda"), adj_ids, adj_sc)[3]
+    assert (lse.double() - torch.logsumexp(x.double(), 1)).abs().max().item() <= 1.2e-6
