@@ -637,6 +637,8 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
 
     for (int j = 0; j < n_local; ++j) {
         const bool have = slot_wait(s_list_done, j);     // (implies the maxima and sums: the collectors waited for them)
+        __syncwarp();                                    // every lane's clears of item j - 1's list stand before the copy that
+                                                         // lets the slot's next user in (lane 0 alone issues it)
         if (have && issued < n_local) {                  // nobody reads item j's stage any more
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             issue();
