@@ -328,21 +328,29 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
     goose::CombinePlan merge_plan;
     merge_plan.valid = false;
     // The cluster form of the attention merges its heads itself and leaves SMs idle; the top-k goes onto those, beside it,
-    // where that takes each of them at most kTopkBeside items (1.5 us an item: done before the attention, which is not
-    // below 8 us).  Its CTAs all end at once, so a top-k that has to follow would start late: with more items the step
-    // keeps the persistent form, in whose ragged end the top-k starts (32 heads, 2k keys, 80 rows: persistent 19.15 us,
-    // clusters with the top-k behind them 20.7, beside them 17.5).
-    constexpr int kTopkBeside = 7;
+    // where it is done about when the attention is: at most 7 items an SM, and with the log-sum-exp, whose items take 2.2 us
+    // instead of 1.5, 3 and one for every tile of a CTA (7 too where behind the persistent form it would take more than an item
+    // an SM).  The clusters' CTAs all end at once, so a top-k that has to follow would start late: with more items the step
+    // keeps the persistent form, in whose ragged end the top-k starts.  us, persistent ->
+    // clusters (items an SM, tiles a CTA):  32 heads, 128 rows 512 keys (8, 2) 16.6 -> 17.5, 1k (8, 3) 18.3 -> 18.4;   40 heads, 128
+    // rows 256 (6, 1) 15.6 -> 15.2.   With the log-sum-exp:  32 heads, 80 rows 256 (5, 1) 16.1 -> 15.8, 512 (5, 2) 17.8 -> 16.4;
+    // 40 heads, 128 rows 256 (6, 1) 18.1 -> 18.8, 512 (6, 2) 19.3 -> 19.8, 768 (6, 3) 20.5 -> 20.4, 1k (6, 3) 21.2 -> 20.3;
+    // 32 heads, 128 rows 2k (8, 5) 22.7 -> 23.3;   16 heads, 64 rows of 128256 329 (6, 1) 22.8 -> 21.8.
     int topk_ctas = 0;
     bool may_cluster = true;
+    const int topk_items = goose::topk_items(S * B, V);
+    const int kind = harvest || topk_items > c->num_sms ? 2 : 1;
     if (S > 0 && !attn_done) {
         const int g = H / Hkv, nb = B * g <= 128 ? B : 128 / g;
-        const int n = goose::attn_cluster(c, S, B, H, Hkv, kv_rows, harvest ? 2 : 1);
+        const int n = goose::attn_cluster(c, S, B, H, Hkv, kv_rows, kind);
         if (n > 1) {
+            const int64_t tiles = ((kv_rows + 127) / 128 + n - 1) / n;       // of a CTA
+            const int beside = harvest && topk_items <= c->num_sms && tiles < 4 ? 3 + (int)tiles : 7;
             // a few SMs stay free for the step's last launch: its CTAs fit beside neither kernel, and its loads ahead of
-            // the wait would start only when the attention ends
+            // the wait would start only when the attention ends (none, 2, 4, 8 free SMs, us: 32 heads, 80 rows 2k 18.3, 18.0, 17.9,
+            // 18.0 and with the harvest 18.1, 17.8, 17.8, 20.1;  52 heads 2k with the harvest 24.9, 24.0, 23.9, 24.0)
             topk_ctas = c->num_sms - (B + nb - 1) / nb * Hkv * n - 4;
-            may_cluster = topk_ctas > 0 && goose::topk_items(S * B, V) <= kTopkBeside * topk_ctas;
+            may_cluster = topk_ctas > 0 && topk_items <= beside * topk_ctas;
             if (!may_cluster) topk_ctas = 0;
         }
     }
@@ -356,7 +364,7 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
             cudaError_t ea = goose::launch_tree_attn_umma(c, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_cache,
                                                           (const __nv_bfloat16*)v_cache, kv_rows, row_off, ctx_len, parent,
                                                           n_nodes, S, B, H, Hkv, scale, (__nv_bfloat16*)out, lse,
-                                                          static_cast<cudaStream_t>(stream), &merge_plan, may_cluster, harvest ? 2 : 1);
+                                                          static_cast<cudaStream_t>(stream), &merge_plan, may_cluster, kind);
             if (ea != cudaSuccess) return cuda_fail(ea);
         } else {
             topk_ctas = 0;

@@ -176,7 +176,7 @@ cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __
                                   int Hkv, float scale, __nv_bfloat16* out, float* lse, cudaStream_t st,
                                   struct CombinePlan* defer_merge = nullptr, bool may_cluster = true, int step = 0);
 // CTAs a head of the cluster form of that kernel has for these sizes (1: the persistent form); step: 0 = the attention
-// alone, 1 = in a step, 2 = in a step with a harvest
+// alone, 1 = in a step, 2 = in a step whose top-k is long (more than an item an SM, or with the log-sum-exp)
 int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int step);
 
 cudaError_t launch_bounded_wait_selftest(goose_ctx* c, long long limit_cycles, int32_t* result, cudaStream_t st);

@@ -812,29 +812,37 @@ int auto_attn_impl(const goose_ctx* c, int S, int B, int H) {
 }
 
 // One sequence: a cluster per head, the largest (of at most 8 CTAs) that the device holds one of per head at once -- where
-// the SMs that this leaves out cost less than the merge kernel and the second segments that it saves.  A tile of the longest
-// CTA takes about 1.5 us in either form; the line is drawn at `lost` = tiles / n - heads * tiles / SMs = 4.4 (3 with clusters
-// of two, and those only in a step, where the top-k runs beside them: alone they were 0.3 us slower at lost = 1.3).
-// ctx_len[] is device data: the tiles are bounded by the rows of the cache, so that a long prefix never meets the slower
-// form.  Attention call / step with harvest, persistent -> clusters (us, by lost):
-//   32 heads 512 keys (0.2) 10.4 -> 8.7 / -;   2k (0.6) 16.25 -> 14.0 / -;     16k (4.4) 50.4 -> 49.1 / 55.4 -> 52.6
-//   40 heads 4k (2.1) 23.45 -> 22.6 / -;       8k (4.1) 36.0 -> 36.0 / 41.1 -> 39.9;   16k (8.1) 61.1 -> 62.4 / 65.4 -> 66.4
-//   52 heads (n = 2) 2k (2.5) 20.3 -> 21.0 / 27.0 -> 24.1;   4k (4.9) 27.3 -> 31.1 / 33.3 -> 34.5
-//   32 over 8 heads, tree of 32 (n = 8)        4k (2.3) 15.0 -> 12.3 / 18.3 -> 15.8;   8k (4.5) 19.1 -> 17.7;   16k (8.9) 24.3 -> 27.8
-//   32 over 8, tree of 60: 16 heads (n = 6)    3k (1.4) 16.4 -> 12.9 / 25.1 -> 20.2;   8k (3.7) 21.6 -> 21.3;   16k (7.4) 30.2 -> 34.2
-// A step without a harvest has a shorter top-k to hide, and on most of the SMs the line is 1.5 for it: 32 heads 2k (0.6)
-// 19.1 -> 18.3, 40 heads 4k (2.1) 26.7 -> 26.9 (and 27.8 -> 29.1 with longer accepted paths on cold inputs).
-//   16 over 2, tree of 16 (n = 8)              4k (3.6) 29.3 -> 11.7 (the merge kernel has 74 parts a head there)
+// the SMs that this leaves out cost less than the merge kernel and the second segments that it saves.  What they cost grows
+// with lost = tiles / n - heads * tiles / SMs, the tiles that the longest CTA has more than an equal share; what is saved
+// depends on what else the launches do, so there are three kinds of call.  ctx_len[] is device data: the tiles are bounded
+// by the rows of the cache, so that a long prefix never meets the slower form -- and a short one in a cache with many spare
+// rows does not meet the faster one.  us, persistent -> clusters, (lost):
+// the attention alone saves the merge kernel: 4.4, and no clusters of two
+//   32 heads (n = 4) 2k (0.6) 16.1 -> 13.8, 16k (4.4) 51.5 -> 49.0;     40 heads (n = 3) 4k (2.1) 23.6 -> 22.7, 8k (4.1) 36.2 -> 35.2
+//   52 heads (n = 2) 1k (1.3) 14.7 -> 15.5, 2k (2.5) 18.9 -> 20.4;      8 heads (n = 8) 4k (2.3) 15.8 -> 12.6, 12k (6.9) 21.7 -> 22.0
+//   2 heads (n = 8) 4k (3.6) 25.5 -> 11.8;   two to four M tiles a key/value head, 3.5:  16 heads (n = 6) 3k (1.4) 14.5 -> 12.5,
+//   6k (2.8) 18.5 -> 17.6, 8k (3.8) 20.5 -> 20.4, 12k (5.7) 24.4 -> 27.2;   32 heads over 8 (n = 4) 16k (4.4) 43.5 -> 45.9
+// a step whose top-k takes more than an item an SM, or the log-sum-exp too, has that beside the clusters: 4.4, and 3 for two
+//   32 heads, 80 rows 16k (4.4) 55.3 -> 51.2;   40 heads 8k (4.1) 40.8 -> 39.2;   52 heads 2k (2.5) 25.9 -> 23.9, 3k (3.7) 29.7 -> 29.4,
+//   4k (4.9) 33.5 -> 34.0;   8 heads, 32 rows 6k (3.5) 20.6 -> 19.3, 12k (6.9) 24.2 -> 26.0;   16 heads, 60 rows of 128256 8k (3.8) 31.7 -> 25.6
+// any other step hides its top-k in the persistent form's ragged end and has the merge in its last launch: less is saved, by
+// number of CTAs and of parts a head (the merge of 74 parts is slow)
+//   52 heads 512 (0.7) 17.1 -> 18.9: no clusters of two;   40 heads 512 (0.3) 16.0 -> 15.0, 768 (0.4) 17.0 -> 16.7, 1k (0.6) 16.9 -> 17.7,
+//   4k (2.1) 26.6 -> 27.2: 0.5 with three;   32 heads 2k (0.6) 18.7 -> 17.9, 8k (2.2) 33.1 -> 32.5, 14 heads (n = 8) 2k (0.5) 16.6 -> 15.7,
+//   4k (1.0) 18.2 -> 18.1, 8k (2.0) 22.5 -> 22.5, 12k (3.0) 26.3 -> 26.9: 1.5 on 70 % of the SMs or more;   8 heads 4k (2.3) 17.7 -> 16.9,
+//   6k (3.5) 19.0 -> 19.4 (19.7 -> 18.6 where no draft token is accepted), 16 heads 2k (1.0) 16.1 -> 15.0, 4k (1.9) 18.0 -> 18.3,
+//   8k (3.8) 22.7 -> 23.8: 3.5;   2 heads 8k (7.2) 33.0 -> 20.3
 int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int step) {
     if (S != 1) return 1;                               // (several may differ in length by any factor)
     const int g = H / Hkv, nb = B * g <= kTile ? B : kTile / g, Hw = (B + nb - 1) / nb * Hkv;
     int n = 1;
     for (int i = 2; i <= kMaxCluster; ++i)
         if (c->max_clusters[i] >= Hw && Hw * i <= c->num_sms) n = i;
-    if (n == 1 || (n == 2 && step == 0)) return 1;
+    if (n == 1 || (n == 2 && step != 2)) return 1;
     const int64_t tiles = (kv_rows + kTile - 1) / kTile;
-    const bool many = 10 * Hw * n >= 7 * c->num_sms;
-    const int line = step == 1 && many ? 15 : n == 2 ? 30 : 44;
+    int line = n == 2 ? 30 : 44;                        // tenths of a tile
+    if (Hw > Hkv && step == 0) line = 35;               // several M tiles a head: K/V come from L2, idle SMs cost their share
+    if (step == 1 && Hw > 4) line = n == 3 ? 5 : 10 * Hw * n >= 7 * c->num_sms ? 15 : 35;
     return tiles * (c->num_sms - Hw * n) * 10 <= (int64_t)line * n * c->num_sms ? n : 1;
 }
 

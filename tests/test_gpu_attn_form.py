@@ -1,0 +1,79 @@
+"""One sequence: the form of the attention kernel that the library takes is never clearly the slower one.  The same step in a
+cache with very many spare rows gets the persistent form (the rule sees the rows of the cache, not the lengths on the device),
+so the two forms can be timed side by side."""
+import time
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2604_02047_b200 import synth
+
+pytestmark = pytest.mark.gpu
+SPARE = 40000                  # 300 and more tiles: above every line of the rule
+
+
+@pytest.fixture(scope="module")
+def goose():
+    from paper_2604_02047_b200 import binding, build
+    build.build()
+    g = binding.Goose(max_S=1, max_B=128, max_H=64)
+    yield g
+    g.close()
+
+
+@pytest.mark.parametrize("op,H,Hkv,B,ctx", [
+    ("step", 52, 52, 128, 512), ("step", 52, 52, 128, 1024), ("step", 40, 40, 80, 1024), ("step", 40, 40, 16, 1024),
+    ("step", 32, 32, 80, 2048), ("step", 32, 8, 32, 6144), ("cycle", 40, 40, 128, 256), ("cycle", 32, 32, 128, 512),
+    ("cycle", 52, 52, 128, 2048), ("call", 52, 52, 128, 2048), ("call", 32, 8, 60, 8192), ("call", 32, 8, 128, 16384)])
+def test_form(goose, op, H, Hkv, B, ctx):
+    """Not above 1.05 times the persistent form (medians of nine; two equal forms differ by up to 1.02 here)."""
+    D, V, k = 128, 32000, 8
+    gen = torch.Generator(device="cuda").manual_seed(0)
+    rand = lambda *shape: torch.randn(shape, generator=gen, device="cuda", dtype=torch.bfloat16)  # noqa: E731
+    dev = lambda a, t: torch.from_numpy(np.ascontiguousarray(a, dtype=t)).cuda()  # noqa: E731
+    rng = np.random.default_rng(0)
+    parent = synth.spine_tree(rng, B, min(B, 16), 3)[0]
+    n = int(np.clip(300e6 / (2 * (ctx + B) * Hkv * D * 2), 3, 12))          # states: more than L2 holds
+    tree = dev(parent[None], np.int32), dev(synth.distinct_sibling_tokens(rng, parent, V)[None], np.int32)
+    row_off, ctx_len = dev([0], np.int64), dev([ctx], np.int32)
+    ids, scores = torch.zeros((V, k), dtype=torch.int32, device="cuda"), torch.zeros((V, k), device="cuda")
+    states = []
+    for _ in range(n):
+        kv = rand(2, ctx + B, Hkv, D)
+        roomy = torch.empty(2, ctx + B + SPARE, Hkv, D, dtype=torch.bfloat16, device="cuda")
+        roomy[:, :ctx + B] = kv
+        states.append((rand(1, B, H, D), kv, roomy, rand(B, V), goose.alloc_step_outputs(1, B, H, D, k)))
+
+    def run(which):
+        for q, kv, roomy, logits, outs in states:
+            kc, vc = (kv, roomy)[which]
+            if op == "call":
+                goose.tree_attn_gqa(q, kc, vc, row_off, ctx_len, tree[0], D ** -0.5, out=outs["out"])
+            elif op == "step":
+                goose.verify_step_gqa(q, kc, vc, row_off, ctx_len, *tree, logits, k, D ** -0.5, outs=outs)
+            else:
+                goose.verify_step_harvest(q, kc, vc, row_off, ctx_len, *tree, logits, k, D ** -0.5, ids, scores, outs=outs)
+
+    graphs = []
+    for which in (0, 1):
+        run(which)
+        torch.cuda.synchronize()
+        graphs.append(torch.cuda.CUDAGraph())
+        with torch.cuda.graph(graphs[-1]):
+            run(which)
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    t = [[], []]
+    for _ in range(9):
+        for which, graph in enumerate(graphs):
+            time.sleep(0.02)
+            graph.replay()
+            ev[0].record()
+            for _ in range(20):
+                graph.replay()
+            ev[1].record()
+            torch.cuda.synchronize()
+            t[which].append(ev[0].elapsed_time(ev[1]) / 20 / n * 1e3)
+    chosen, persistent = (float(np.median(x)) for x in t)
+    print("%s %d/%d heads, %d rows, %d keys: %.2f us, persistent %.2f" % (op, H, Hkv, B, ctx, chosen, persistent))
+    assert chosen <= 1.05 * persistent
