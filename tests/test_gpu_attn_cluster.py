@@ -6,6 +6,7 @@ import pytest
 import torch
 
 from paper_2604_02047_b200 import synth
+from test_gpu_chained_steps import _run_chain
 from test_gpu_parity import ATTN_TOL, LSE_TOL, attn_row_err
 
 pytestmark = pytest.mark.gpu
@@ -97,4 +98,51 @@ def test_step_with_clusters(goose, oracle, H, Hkv, B, V):
         rows = binding.bf16_to_bits(cache)
         for j in range(int(alen[0]) + 1):
             assert np.array_equal(rows[r0 + j], before[r0 + int(path[0, j])])
+    assert int(goose.last_status(1)[0]) == 0
+
+
+@pytest.mark.parametrize("H,B", [(32, 16), (40, 24)])
+def test_steps_back_to_back(goose, oracle, H, B):
+    """Three steps of one sequence without synchronisation in between, chains accepted whole and random trees: the top-k
+    beside the clusters writes its results before it waits for the attention."""
+    _run_chain(goose, oracle, 1, H, B, 4096, 4, [500], lambda t, s: synth.chain_tree(B), seed=70, full_accept=True, prewrite=True)
+    rng = np.random.default_rng(H)
+    _run_chain(goose, oracle, 1, H, B, 32000, 8, [300], lambda t, s: synth.spine_tree(rng, B, 8, 3)[0], seed=80, full_accept=False,
+               prewrite=False)
+
+
+@pytest.mark.parametrize("H,Hkv,B,ctx,V", [(32, 32, 80, 600, 32000), (40, 40, 80, 900, 32000), (52, 52, 60, 300, 32000), (32, 8, 60, 900, 70000)])
+def test_cycles_back_to_back(goose, oracle, H, Hkv, B, ctx, V):
+    """Four steps with harvest into one table, on clusters that take 64 to 86 % of the SMs: each against the oracle when waited
+    for, and the same four enqueued at once leave the same bits everywhere."""
+    from paper_2604_02047_b200 import binding
+    rng = np.random.default_rng([H, Hkv, B])
+    xs = [_inputs(rng, H, Hkv, B, ctx, V=V, k=8) for _ in range(4)]
+
+    def run(wait):
+        ids, scores = torch.full((V, 8), -1, dtype=torch.int32, device="cuda"), torch.zeros((V, 8), device="cuda")
+        ds = [binding.to_device(x) for x in xs]
+        outs = [goose.alloc_step_outputs(1, B, H, 128, 8) for _ in xs]
+        torch.cuda.synchronize()
+        for d, o in zip(ds, outs):
+            goose.verify_step_harvest(d["q"], d["k_cache"], d["v_cache"], d["row_off"], d["ctx_len"], d["parent"], d["draft_tok"],
+                                      d["logits"], 8, xs[0].scale, ids, scores, outs=o)
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return outs, [d[n] for d in ds for n in ("k_cache", "v_cache")] + [ids, scores]
+
+    outs, kept = run(True)
+    for x, o in zip(xs, outs):
+        am, top, _ = oracle.node_topk(x.logits, 8)
+        path, alen, bonus = oracle.accept(x.draft_tok, x.parent, am.reshape(1, B))
+        assert np.array_equal(o["topk_ids"].cpu().numpy(), top) and np.array_equal(o["path"].cpu().numpy(), path)
+        assert o["accept_len"].tolist() == alen.tolist() and o["bonus"].tolist() == bonus.tolist()
+        ref, _ = oracle.tree_attn(x.q, x.k_cache, x.v_cache, x.row_off, x.ctx_len, x.parent, x.scale)
+        assert attn_row_err(o["out"].float().cpu().numpy().astype(np.float64), ref).max() <= ATTN_TOL
+    for _ in range(3):
+        again, kept2 = run(False)
+        for o, p in zip(outs, again):
+            assert all(torch.equal(o[n], p[n]) for n in ("out", "argmax", "topk_ids", "topk_vals", "path", "accept_len", "bonus", "new_ctx_len", "row_lse"))
+        assert all(torch.equal(a, b) for a, b in zip(kept, kept2))
     assert int(goose.last_status(1)[0]) == 0

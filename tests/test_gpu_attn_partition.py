@@ -41,3 +41,22 @@ def test_partition(goose, oracle, H, Hkv, B, ctxs, counts):
         assert np.all(out[s, n:] == 7.0) and np.all(lse[s, n:] == 7.0)
         if n:
             assert attn_row_err(out[s, :n], ref[s, :n]).max() <= ATTN_TOL and np.abs(lse[s, :n] - ref_lse[s, :n]).max() <= LSE_TOL
+
+
+@pytest.mark.parametrize("H,Hkv,B,ctx", [(8, 8, 20, 4700), (8, 8, 20, 4716), (16, 2, 16, 4096), (40, 40, 16, 1000), (32, 32, 33, 300), (4, 4, 1, 0)])
+def test_one_sequence_in_a_large_cache(goose, oracle, H, Hkv, B, ctx):
+    """One sequence whose cache has 60000 spare rows: the persistent form, which the exact caches of these sizes do not meet.  The
+    first two lists have CTAs with idle items alone (8 heads of 37 tiles: 2.1 items a CTA, two idle ones first)."""
+    from paper_2604_02047_b200 import binding
+    rng = np.random.default_rng([H, Hkv, B, ctx])
+    x = synth.make_inputs(1, H, B, [ctx], [synth.random_tree(rng, B)], Hkv=Hkv, seed=H + ctx, V=8, with_logits=False)
+    ref, ref_lse = oracle.tree_attn(x.q, x.k_cache, x.v_cache, x.row_off, x.ctx_len, x.parent, x.scale)
+    d = binding.to_device(x)
+    roomy = [torch.cat([d[n], torch.full((60000, Hkv, 128), float("nan"), dtype=torch.bfloat16, device="cuda")]) for n in ("k_cache", "v_cache")]
+    before = goose.launch_count()
+    out, lse = goose.tree_attn_gqa(d["q"], *roomy, d["row_off"], d["ctx_len"], d["parent"], x.scale, want_lse=True)
+    torch.cuda.synchronize()
+    assert goose.launch_count() == before + 2, "main kernel and merge"
+    assert not goose.last_status(1).any()
+    assert attn_row_err(out.float().cpu().numpy().astype(np.float64), ref).max() <= ATTN_TOL
+    assert np.abs(lse.cpu().numpy() - ref_lse).max() <= LSE_TOL

@@ -129,3 +129,20 @@ def test_log_sum_exp_of_late_values(goose_many, V, below):
     adj_sc = torch.zeros((300, 8), dtype=torch.float32, device="cuda")
     lse = goose_many.harvest(x, 8, torch.arange(300, dtype=torch.int32, device="cuda"), adj_ids, adj_sc)[3]
     assert (lse.double() - torch.logsumexp(x.double(), 1)).abs().max().item() <= 1.2e-6
+
+
+@pytest.mark.parametrize("V,k", [(70008, 8), (128256, 10), (262144, 16)])
+def test_calls_after_node_counts(goose_many, oracle, V, k):
+    """Rows whose chunks meet in several CTAs count arrivals in memory that calls share: a call that leaves rows out (node
+    counts) must leave every counter as it found it, for calls with and without counts behind it."""
+    S, B = 4, 15
+    bits = _rows(V, np.random.default_rng([V, k]))[:B]
+    ref_am, ref_ids, _ = oracle.node_topk(bits, k)
+    x = torch.from_numpy(bits.view(np.int16)).view(torch.bfloat16).cuda().repeat(S, 1).contiguous()
+    for counts in ([15, 0, 7, 1], None, [1, 1, 1, 15], [0, 15, 15, 3], None):
+        nn = None if counts is None else torch.tensor(counts, dtype=torch.int32, device="cuda")
+        am, ids, _ = goose_many.node_topk(x, k, n_nodes=nn, B=B)
+        torch.cuda.synchronize()
+        am, ids = am.cpu().numpy().reshape(S, B), ids.cpu().numpy().reshape(S, B, k)
+        for s, n in enumerate(counts or [B] * S):
+            assert np.array_equal(ids[s, :n], ref_ids[:n]) and np.array_equal(am[s, :n], ref_am[:n]), (counts, s)
