@@ -656,7 +656,7 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
         const bool all_parts = T_all >= cluster;
         __syncwarp();
         tc_fence_before();
-        cluster_sync();                                    // the head's partials are complete in its CTAs' shared memory
+        cluster_sync();                                    // the head's partials are complete in the workspace (L2)
         for (; task < n_rows * 8;) {
             const float* at_m = partials + (size_t)head * cluster * kUmmaPartFloats + kPartHalfWords + row;
             const uint4* at_x = reinterpret_cast<const uint4*>(partials + (size_t)head * cluster * kUmmaPartFloats) + 2 * u * 128 + row;
@@ -820,7 +820,7 @@ int auto_attn_impl(const goose_ctx* c, int S, int B, int H) {
 // the attention alone saves the merge kernel: 4.4, and no clusters of two
 //   32 heads (n = 4) 2k (0.6) 16.1 -> 13.8, 16k (4.4) 51.5 -> 49.0;     40 heads (n = 3) 4k (2.1) 23.6 -> 22.7, 8k (4.1) 36.2 -> 35.2
 //   52 heads (n = 2) 1k (1.3) 14.7 -> 15.5, 2k (2.5) 18.9 -> 20.4;      8 heads (n = 8) 4k (2.3) 15.8 -> 12.6, 12k (6.9) 21.7 -> 22.0
-//   2 heads (n = 8) 4k (3.6) 25.5 -> 11.8;   two to four M tiles a key/value head, 3.5:  16 heads (n = 6) 3k (1.4) 14.5 -> 12.5,
+//   two to four M tiles a key/value head, 3.5:  16 heads (n = 6) 3k (1.4) 14.5 -> 12.5,
 //   6k (2.8) 18.5 -> 17.6, 8k (3.8) 20.5 -> 20.4, 12k (5.7) 24.4 -> 27.2;   32 heads over 8 (n = 4) 16k (4.4) 43.5 -> 45.9
 // a step whose top-k takes more than an item an SM, or the log-sum-exp too, has that beside the clusters: 4.4, and 3 for two
 //   32 heads, 80 rows 16k (4.4) 55.3 -> 51.2;   40 heads 8k (4.1) 40.8 -> 39.2;   52 heads 2k (2.5) 25.9 -> 23.9, 3k (3.7) 29.7 -> 29.4,
@@ -831,7 +831,12 @@ int auto_attn_impl(const goose_ctx* c, int S, int B, int H) {
 //   4k (2.1) 26.6 -> 27.2: 0.5 with three;   32 heads 2k (0.6) 18.7 -> 17.9, 8k (2.2) 33.1 -> 32.5, 14 heads (n = 8) 2k (0.5) 16.6 -> 15.7,
 //   4k (1.0) 18.2 -> 18.1, 8k (2.0) 22.5 -> 22.5, 12k (3.0) 26.3 -> 26.9: 1.5 on 70 % of the SMs or more;   8 heads 4k (2.3) 17.7 -> 16.9,
 //   6k (3.5) 19.0 -> 19.4 (19.7 -> 18.6 where no draft token is accepted), 16 heads 2k (1.0) 16.1 -> 15.0, 4k (1.9) 18.0 -> 18.3,
-//   8k (3.8) 22.7 -> 23.8: 3.5;   2 heads 8k (7.2) 33.0 -> 20.3
+//   8k (3.8) 22.7 -> 23.8: 3.5
+// up to four heads, whatever the call: the merge of 37 parts a head and more is slow
+//   2 heads, call / step / with harvest 2k (1.9) 26.0 -> 9.6 / 24.0 -> 13.5 / 24.1 -> 13.8, 8k (7.2) 30.3 -> 16.5 / 32.9 -> 20.5 / 33.0 -> 20.6,
+//   12k (10.8) 28.4 -> 20.9 / 26.8 -> 25.0 / 28.4 -> 24.8, 16k (14.4) 28.7 -> 25.3 / 27.8 -> 29.4 / 29.1 -> 29.6: 10, and one head has more to win
+//   4 heads, tree of 60  2k (1.7) 17.3 -> 10.3 / 18.6 -> 13.9 / 21.6 -> 14.0, 6k (4.8) 19.7 -> 14.9 / 20.8 -> 18.5 / 22.2 -> 18.7,
+//   8k (6.4) 19.8 -> 17.1 / 21.8 -> 20.8 / 23.0 -> 21.0, 10k (7.7) 20.6 -> 18.8 / 21.7 -> 22.4 / 23.0 -> 22.4: 6
 int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int step) {
     if (S != 1) return 1;                               // (several may differ in length by any factor)
     const int g = H / Hkv, nb = B * g <= kTile ? B : kTile / g, Hw = (B + nb - 1) / nb * Hkv;
@@ -840,8 +845,8 @@ int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_ro
         if (c->max_clusters[i] >= Hw && Hw * i <= c->num_sms) n = i;
     if (n == 1 || (n == 2 && step != 2)) return 1;
     const int64_t tiles = (kv_rows + kTile - 1) / kTile;
-    int line = n == 2 ? 30 : 44;                        // tenths of a tile
-    if (Hw > Hkv && step == 0) line = 35;               // several M tiles a head: K/V come from L2, idle SMs cost their share
+    int line = n == 2 ? 30 : Hw <= 2 ? 100 : Hw <= 4 ? 60 : 44;   // tenths of a tile
+    if (Hw > Hkv && Hw > 4 && step == 0) line = 35;               // several M tiles a head: K/V come from L2, idle SMs cost their share
     if (step == 1 && Hw > 4) line = n == 3 ? 5 : 10 * Hw * n >= 7 * c->num_sms ? 15 : 35;
     return tiles * (c->num_sms - Hw * n) * 10 <= (int64_t)line * n * c->num_sms ? n : 1;
 }
