@@ -79,7 +79,7 @@ extern "C" {
 /* attention kernel selection (goose_set_attn_impl) */
 #define GOOSE_ATTN_AUTO  0
 #define GOOSE_ATTN_MMA   1    /* warp-level mma.sync flash-decode kernel (any B <= 128)            */
-#define GOOSE_ATTN_UMMA  2    /* tcgen05 + TMEM + TMA persistent kernel                            */
+#define GOOSE_ATTN_UMMA  2    /* tcgen05 + TMEM + TMA kernel, persistent or a cluster per head     */
 
 typedef struct goose_ctx goose_ctx;
 
@@ -103,7 +103,9 @@ int goose_set_attn_impl(goose_ctx* ctx, int impl);
  * over the visible keys j = prefix rows 0..ctx_len[s]-1 and tree rows ctx_len[s]+a for every
  * ancestor a of i, i included.  bf16 inputs, fp32 accumulation, bf16 output (round to nearest even).
  *   q        bf16 [S][B][H][D]                       16-byte aligned
- *   k_cache, v_cache  bf16 [kv_rows][H][D]           16-byte aligned; kv_rows = rows allocated
+ *   k_cache, v_cache  bf16 [kv_rows][H][D]           16-byte aligned; kv_rows = rows allocated, or fewer: no row beyond
+ *            them is touched.  With S = 1 the tensor-core kernel's form is chosen by kv_rows (the lengths are on the
+ *            device): a bound near row_off + ctx_len + B gets a short prefix its faster form in a large cache too.
  *   row_off  int64 [S], ctx_len int32 [S], parent int32 [S][B], n_nodes int32 [S] or NULL   (device arrays)
  *   out      bf16 [S][B][H][D]; lse fp32 [S][B][H] = log-sum-exp of the scaled scores, or NULL
  * Rows row_off[s]+ctx_len[s]+B .. are never read as values (their contents may be anything).

@@ -10,9 +10,9 @@
 //   control warp (1)     streams the items into a ring of three 64 KB shared-memory stages with bulk asynchronous copies
 //                        (cp.async.bulk), ranks an item's candidates, merges the chunks of a row, writes the results
 //   data warps (16)      64 values per thread into registers: thread maxima with packed-bf16 max, half-warp maxima with
-//                        redux.sync.  With the log-sum-exp they also sum the exponentials relative to the warp's largest
-//                        value so far, eight elements at a time behind their load, so that one warp's exponentials cover
-//                        another's loads and maxima
+//                        redux.sync.  With the log-sum-exp they also sum the exponentials relative to the largest value
+//                        of the warp's first sweep, eight elements at a time behind their load, so that one warp's
+//                        exponentials cover another's loads and maxima
 //   collector warps (4)  T by rank counting (every lane counts the keys above its own: independent compares instead of k
 //                        dependent reduction rounds); the threads whose maximum is >= T; keys of their elements >= T
 // What bounds it: the stream (64 KB an item and SM: 1.47 us at the copy peak) and, with the log-sum-exp, the 32768

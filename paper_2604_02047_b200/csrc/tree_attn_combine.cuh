@@ -54,11 +54,12 @@ struct Work {
     // items of a head of T tiles
     __device__ __forceinline__ int width(int T) const { return T > 0 ? T + pad : 0; }
     // A CTA that goes over from one head to the next pays for it (its epilogue and the next head's first softmax stand in
-    // turn: 2 to 3 us), so a head starts with idle items that take as much of the CTA's range.  Two tiles' worth, from two tiles a CTA on
-    // (below, a CTA could hold idle items alone).  Attention call without -> 1 / 2 / 3 idle items: 8 x 32 heads, 333 to 6000
-    // keys 81.5 -> 75.3 / 75.0 / 75.4 us; 2 x 32 over 8, tree of 61, 1000 to 5000 18.4 -> 17.2 / 16.4 / -; 4 x 32 over 8, 4k
-    // to 16k 31.0 -> 29.7 / 28.75 / -; 52 heads, 8k 43.5 -> 43.4 / 43.5 / 43.5.  (The partition is found by whole warps: the
-    // longer arithmetic, which once cost what the padding gained, is not seen: 43.55 with none and the code for it.)
+    // turn: 2 to 3 us), so a head starts with idle items that take as much of the CTA's range.  Two tiles' worth, from two tiles
+    // a CTA on (a CTA whose whole share is idle items has no work, as one without a share).  Attention call with none / 1 / 2, us:
+    // 8 x 32 heads, 333 to 6000 keys 69.7 / 61.5 / 57.7;  16 x 32 over 8, 1k to 8k 63.8 / 60.8 / 59.4;  4 x 16 over 2, 8k 29.5 / 28.4 / 27.9;
+    // 2 x 32, 4k to 8k 42.5 / 40.3 / 40.0;  2 x 32 over 8, tree of 61, 1k to 5k 19.9 / 20.0 / 20.4;  52 heads 4k 27.4 / 26.4 / 27.2, 8k
+    // 43.9 / 43.4 / 43.4.  In long streams a head switch hides behind the other CTAs' loads and the idle items cost as little:
+    // 8 x 32, 16k 329.5 / 329.7 / 329.6, 16 x 32, 1k to 16k 389.2 / 389.7 / 389.1 (sustained 438 / 438 / 436).
     __device__ __forceinline__ void set_total(long long tile_count, int live) {
         pad = tile_count >= 2 * (long long)G ? 2 : 0;
         total = tile_count + (long long)pad * H * live;
