@@ -40,11 +40,11 @@ MIN_REGIONS = 5                 # the K-step timed region is repeated at least t
 BURST_GAP_S = 0.2               # idle time in front of every burst region (the part cools back to its full clocks)
 BURST_MS = 10.0                 # length of a burst region of the per-kernel legs
 SUSTAIN_SECONDS = 1.5           # further regions keep the GPU under the same load until the clock sampler has >= 10 samples
-# DRAM traffic per attention call (main + merge kernels) from the ncu captures summarised under profiles/ (bytes); these
+# DRAM traffic per attention call (the merge kernel, where there is one, reads from L2) from the ncu captures summarised under profiles/ (bytes); these
 # are NOT measured by the run that prints them: `roofline.traffic_source` names the capture.  None = not captured.
-NCU_TRAFFIC_BYTES = {"33b": (227_200_000, "profiles/tree_attn_umma_33b.md"),      # 223.29 MB read + 3.89-3.95 MB written
-                     "13b": (89_230_000, "profiles/tree_attn_umma_13b.md"),       # 86.42 MB read + 2.65-2.98 MB written
-                     "gqa8b": (169_570_000, "profiles/tree_attn_umma_gqa8b.md")}  # 165.0 MB read + 3.2-5.8 MB written
+NCU_TRAFFIC_BYTES = {"33b": (227_890_000, "profiles/tree_attn_umma_33b.md"),      # 223.29 MB read + 4.13-5.07 MB written
+                     "13b": (88_760_000, "profiles/tree_attn_umma_13b.md"),       # 86.46 MB read + 2.30 MB written
+                     "gqa8b": (171_380_000, "profiles/tree_attn_umma_gqa8b.md")}  # 164.99 MB read + 5.75-7.02 MB written
 
 
 def _peaks():
@@ -590,9 +590,10 @@ def run_ours(args, x, cfg, rank, world, local_rank):
                     "step_with_harvest_us": sh_ms * 1e3,
                     "four_calls_us": legs["four"][0] * 1e3,
                     "four_calls_note": "goose_tree_attn, goose_node_topk, goose_accept, goose_kv_compact one after the other "
-                                       "(5 launches, every kernel waits for its predecessor before it reads anything); the "
-                                       "metric is goose_verify_step, whose 3 launches overlap the top-k with the attention "
-                                       "kernel's tail and run the merge of the split heads beside the walk and the compaction",
+                                       "(5 launches, 4 where the attention's clusters merge their heads themselves; every kernel "
+                                       "waits for its predecessor before it reads anything); the metric is goose_verify_step, "
+                                       "whose 3 launches overlap the top-k with the attention and run the merge of the split "
+                                       "heads beside the walk and the compaction",
                     "step_l2_warm_us": legs["warm"][0] * 1e3,
                     "step_l2_warm_note": "the same input replica every replay, so whatever of its footprint fits stays in L2; "
                                          "context only, the metric is the L2-cold rotation",
