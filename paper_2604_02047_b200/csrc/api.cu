@@ -348,7 +348,9 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
             const int beside = harvest && topk_items <= c->num_sms && tiles < 4 ? 3 + (int)tiles : 7;
             // a few SMs stay free for the step's last launch: its CTAs fit beside neither kernel, and its loads ahead of
             // the wait would start only when the attention ends (none, 2, 4, 8 free SMs, us: 32 heads, 80 rows 2k 18.3, 18.0, 17.9,
-            // 18.0 and with the harvest 18.1, 17.8, 17.8, 20.1;  52 heads 2k with the harvest 24.9, 24.0, 23.9, 24.0)
+            // 18.0 and with the harvest 18.1, 17.8, 17.8, 20.1;  52 heads 2k with the harvest 24.9, 24.0, 23.9, 24.0; beside a
+            // shorter attention the round of items that they cost the top-k shows: 32 heads, 80 rows 512 keys with the harvest 15.0,
+            // 16.4, 16.4, 19.8)
             topk_ctas = c->num_sms - (B + nb - 1) / nb * Hkv * n - 4;
             may_cluster = topk_ctas > 0 && topk_items <= beside * topk_ctas;
             if (!may_cluster) topk_ctas = 0;

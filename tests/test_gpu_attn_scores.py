@@ -68,4 +68,4 @@ def test_price_of_rising_scores(goose):
 
     once(level), once(rising)
     t = [(once(level), once(rising)) for _ in range(9)]
-    assert np.median([r for _, r in t]) <= 1.3 * np.median([l for l, _ in t])
+    assert min(r for _, r in t) <= 1.3 * min(l for l, _ in t)
