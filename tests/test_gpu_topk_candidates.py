@@ -132,17 +132,22 @@ def test_log_sum_exp_of_late_values(goose_many, V, below):
 
 
 @pytest.mark.parametrize("V,k", [(70008, 8), (128256, 10), (262144, 16)])
-def test_calls_after_node_counts(goose_many, oracle, V, k):
-    """Rows whose chunks meet in several CTAs count arrivals in memory that calls share: a call that leaves rows out (node
-    counts) must leave every counter as it found it, for calls with and without counts behind it."""
+def test_long_rows_with_node_counts(goose_many, oracle, V, k):
+    """Rows of several chunks, most of them left out by node counts: fewer items than CTAs, and a row's parts are counted over
+    the CTAs that have one.  (Counted over empty CTAs between them too, such a row waits for arrivals that never come: nothing
+    is written, and the counter in memory, which calls share, spoils the calls behind.)  Outputs hold a mark before each call."""
     S, B = 4, 15
     bits = _rows(V, np.random.default_rng([V, k]))[:B]
-    ref_am, ref_ids, _ = oracle.node_topk(bits, k)
+    ref_am, ref_ids, ref_vals = oracle.node_topk(bits, k)
     x = torch.from_numpy(bits.view(np.int16)).view(torch.bfloat16).cuda().repeat(S, 1).contiguous()
     for counts in ([15, 0, 7, 1], None, [1, 1, 1, 15], [0, 15, 15, 3], None):
         nn = None if counts is None else torch.tensor(counts, dtype=torch.int32, device="cuda")
-        am, ids, _ = goose_many.node_topk(x, k, n_nodes=nn, B=B)
+        outs = (torch.full((S * B,), -7, dtype=torch.int32, device="cuda"), torch.full((S * B, k), -7, dtype=torch.int32, device="cuda"),
+                torch.full((S * B, k), -7.0, device="cuda"))
+        goose_many.node_topk(x, k, n_nodes=nn, B=B, outs=outs)
         torch.cuda.synchronize()
-        am, ids = am.cpu().numpy().reshape(S, B), ids.cpu().numpy().reshape(S, B, k)
+        am, ids, vals = (o.cpu().numpy().reshape(S, B, -1) for o in outs)
         for s, n in enumerate(counts or [B] * S):
-            assert np.array_equal(ids[s, :n], ref_ids[:n]) and np.array_equal(am[s, :n], ref_am[:n]), (counts, s)
+            assert np.array_equal(ids[s, :n], ref_ids[:n]) and np.array_equal(am[s, :n, 0], ref_am[:n]), (counts, s)
+            assert np.array_equal(vals[s, :n].astype(np.float64), ref_vals[:n])
+            assert np.all(am[s, n:] == -7) and np.all(ids[s, n:] == -7) and np.all(vals[s, n:] == -7.0)
