@@ -75,6 +75,10 @@ struct Work {
         }
         set_total(tot, live);
     }
+    // the same by a whole warp from the tiles of up to 32 sequences, one a lane (has: the lane's sequence has any)
+    __device__ __forceinline__ void init_lanes(int tiles, bool has) {
+        set_total(H * (long long)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)tiles), __popc(__ballot_sync(0xFFFFFFFFu, has)));
+    }
     // the same by a whole warp, lane s loading sequence s's length; returns the tiles of sequence `lane`
     __device__ __forceinline__ int init_warp(int lane) {
         const int mine = lane < S ? tiles(lane) : 0;

@@ -124,6 +124,21 @@ __device__ __forceinline__ void tma_load_3d_hint(void* dst, const CUtensorMap* m
                  "[%0], [%1, {%3, %4, %5}], [%2], %6;"
                  ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "l"(policy) : "memory");
 }
+// brings a box of a tensor map into L2: a hint; nothing reaches the SM, and a box outside the tensor touches nothing
+__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int c0, int c1, int c2) {
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global [%0, {%1, %2, %3}];" ::"l"(map), "r"(c0), "r"(c1), "r"(c2) : "memory");
+}
+// a load that may run beside the kernel that writes the word (it returns the old or the new value)
+__device__ __forceinline__ int32_t load_early(const int32_t* p) {
+    int32_t v;
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int64_t load_early(const int64_t* p) {
+    int64_t v;
+    asm volatile("ld.relaxed.gpu.global.s64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ unsigned long long l2_policy_evict_first() {
     unsigned long long pol;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
@@ -251,31 +266,59 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
         asm volatile("prefetch.global.L2 [%0];" ::"l"(row_off));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(parent));
     }
-    // everything above touched no global memory: now wait for the preceding kernel, then let the next
+    Work wk;
+    // g query heads per key/value head, nb nodes per M tile (nb * g <= 128), n_mt M tiles per sequence
+    const int n_mt = kGrouped ? (B + nb - 1) / nb : 1;
+    wk.ctx_len = ctx_len; wk.n_nodes = n_nodes; wk.S = S; wk.H = n_mt * Hkv; wk.B = B; wk.G = gridDim.x; wk.G_magic = G_magic;
+    // cluster mode: this CTA is number `rank` of the `cluster` CTAs that share head `head` of the one sequence
+    const int head = kCluster ? blockIdx.x / cluster : 0, rank = kCluster ? blockIdx.x - head * cluster : 0;
+    int T_all = 0;                                      // tiles of that sequence
+    // its first tile; rounded up, so that the last CTA, which has the masked tile, has no tile more than the others
+    auto rank_start = [&](int r) { return (T_all * r + cluster - 1) / cluster; };
+    // this CTA's items, found by a whole warp (lane = sequence, `tiles` its tiles); a list of more than 32 sequences is read again
+    long long w_begin = 0, w_end = 0;
+    Cursor cu;
+    auto locate = [&](int tiles, int lane) {
+        if (kCluster) {
+            T_all = __shfl_sync(0xFFFFFFFFu, tiles, 0);
+            w_begin = (long long)head * T_all + rank_start(rank); w_end = (long long)head * T_all + rank_start(rank + 1);
+            cu.w = w_begin; cu.s = 0; cu.h = head; cu.t = rank_start(rank); cu.T = T_all;
+        } else {
+            w_begin = wk.cta_start(blockIdx.x); w_end = wk.cta_start(blockIdx.x + 1);
+            if (w_begin < w_end) cu.seek_warp(wk, w_begin, lane, tiles);
+        }
+    };
+    // The CTA is up 0.7 to 1 us before the kernel in front has ended, and the first load of K after that used to take 1.8 us.
+    // One warp brings the CTA's first tile into L2 meanwhile: where it lies is worked out from lengths that the kernel in front
+    // may still be writing, so all of it is a hint, worked out again below.  Attention call without -> with, us: 32 heads 512 keys
+    // 9.2 -> 8.6, 1531 12.4 -> 11.6, 2k 13.6 -> 12.9, 8k 29.2 -> 28.3; 52 heads 8k 43.7 -> 42.0; 4 x 32 over 8, 4k to 16k 41.1 -> 39.8.
+    // (Two tiles and more, or by CTAs on idle SMs all of the next call's tiles: slower, 2k 14.1 and more.  The copies in flight
+    // are then so many that HBM delivers less.)
+    if (warp == 2 && S <= 32) {
+        const bool mine = lane < S;
+        const int nn = !mine ? 0 : kCounts ? load_early(n_nodes + lane) : B;
+        const int ctx = mine ? max(load_early(ctx_len + lane), 0) : 0;
+        const int64_t row0 = mine ? load_early(row_off + lane) : 0;
+        const int tiles = nn > 0 && nn <= B && ctx <= kv_rows ? (ctx + nn + kTile - 1) / kTile : 0;
+        wk.init_lanes(tiles, tiles > 0);
+        locate(tiles, lane);
+        if (w_begin < w_end && (kCluster || wk.small)) {
+            const int64_t row = __shfl_sync(0xFFFFFFFFu, row0, cu.s) + (int64_t)cu.t * kTile;
+            if (lane < 4 && row >= 0 && row < kv_rows)
+                tma_prefetch_3d(lane & 2 ? &tmap_v : &tmap_k, (lane & 1) * 64, kGrouped ? cu.h % Hkv : cu.h, (int)row);
+        }
+    }
+    // everything above only looked: now wait for the preceding kernel, then let the next
     // one (the combine kernel) get resident early -- it waits for this grid before reading the partials
     pdl_wait();
     pdl_trigger();
     if (n_nodes && blockIdx.x == 0 && threadIdx.x == 33)   // an idle lane reports node counts outside [0, B] (read as 0)
         for (int s = 0; s < S; ++s)
             if (nodes_bad(n_nodes, s, B)) atomicOr(&status[s], GOOSE_ST_BAD_NODES);
-    Work wk;
-    // g query heads per key/value head, nb nodes per M tile (nb * g <= 128), n_mt M tiles per sequence
-    const int n_mt = kGrouped ? (B + nb - 1) / nb : 1;
-    wk.ctx_len = ctx_len; wk.n_nodes = n_nodes; wk.S = S; wk.H = n_mt * Hkv; wk.B = B; wk.G = gridDim.x; wk.G_magic = G_magic;
     // where this CTA starts, found by every warp for itself with all lanes; the lengths and the rows of up to 32 sequences
     // come in one round of loads (lane = sequence).  The first load of K waits for nothing else.
     const int64_t my_row = lane < S ? row_off[lane] : 0;
-    const int my_tiles = wk.init_warp(lane);
-    // cluster mode: this CTA is number `rank` of the `cluster` CTAs that share head `head` of the one sequence
-    const int head = kCluster ? blockIdx.x / cluster : 0, rank = kCluster ? blockIdx.x - head * cluster : 0;
-    const int T_all = kCluster ? __shfl_sync(0xFFFFFFFFu, my_tiles, 0) : 0;
-    // its first tile; rounded up, so that the last CTA, which has the masked tile, has no tile more than the others
-    auto rank_start = [&](int r) { return (T_all * r + cluster - 1) / cluster; };
-    const long long w_begin = kCluster ? (long long)head * T_all + rank_start(rank) : wk.cta_start(blockIdx.x);
-    const long long w_end = kCluster ? (long long)head * T_all + rank_start(rank + 1) : wk.cta_start(blockIdx.x + 1);
-    Cursor cu;
-    if (kCluster) { cu.w = w_begin; cu.s = 0; cu.h = head; cu.t = rank_start(rank); cu.T = T_all; }
-    else if (w_begin < w_end) cu.seek_warp(wk, w_begin, lane, my_tiles);
+    locate(wk.init_warp(lane), lane);
     const int first_s = w_begin < w_end ? cu.s : 0;
     const int64_t first_row = __shfl_sync(0xFFFFFFFFu, my_row, first_s & 31);
     auto row_of = [&](int s) -> int64_t { return s == first_s && s < 32 ? first_row : row_off[s]; };
