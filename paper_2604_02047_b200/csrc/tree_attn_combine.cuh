@@ -154,8 +154,10 @@ struct Cursor {               // walks items in order
         if (v >= W) { ++h; v -= W; }
         enter(wk, v);
     }
-    __device__ __forceinline__ void next(const Work& wk) {
-        ++w; ++t;
+    // items of this head from here to its end, at most up to item `w_end` of the list; and past n of them
+    __device__ __forceinline__ int run(long long w_end) const { return (int)min((long long)(T - t), w_end - w); }
+    __device__ __forceinline__ void skip(const Work& wk, int n) {
+        w += n; t += n;
         if (t == T) {
             t = 0; ++h; w += wk.pad;
             if (h == wk.H) {                              // next sequence that has any items
