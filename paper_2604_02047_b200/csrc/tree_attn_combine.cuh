@@ -36,6 +36,10 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 }
 
 // ---------------------------------------------------------------- work partition (same code in every role)
+// 64-bit division out of line.  The merge finds CTAs and their starts in a dozen places, each with such a division for lists of
+// 2^31 / SMs items and more: a third of its code, fetched by every launch and reached by hardly any (step of 40 heads at 4k, with
+// the merge beside walk and compaction: 25.8 -> 25.1 us; 52 heads at 8k 45.8 -> 45.3).
+static __device__ __noinline__ long long div64(long long a, long long b) { return a / b; }
 struct Work {
     const int32_t* ctx_len;
     const int32_t* n_nodes;   // per-sequence node counts, or NULL (every tree has B nodes)
@@ -68,11 +72,16 @@ struct Work {
     __device__ __forceinline__ void init() {
         long long tot = 0;
         int live = 0;
-        for (int s = 0; s < S; ++s) {
+        auto add = [&](int s) {
             const int T = tiles(s);
             tot += (long long)H * T;
             live += T > 0;
-        }
+        };
+        // (small without counts; with them unrolled, since two dependent loads a sequence would follow one another)
+        if (n_nodes) for (int s = 0; s < S; ++s) add(s);
+        else
+#pragma unroll 1
+            for (int s = 0; s < S; ++s) add(s);
         set_total(tot, live);
     }
     // the same by a whole warp from the tiles of up to 32 sequences, one a lane (has: the lane's sequence has any)
@@ -92,16 +101,19 @@ struct Work {
         set_total(H * sum, live);
         return mine;
     }
+    template <bool kCall = false>
     __device__ __forceinline__ long long cta_start(int c) const {
-        if (!small) return total * c / G;
+        if (!small) return kCall ? div64(total * c, G) : total * c / G;
         const uint32_t n = (uint32_t)total * (uint32_t)c, q = __umulhi(n, G_magic);   // exact or one too large (n < 2^31)
         return q * (uint32_t)G > n ? q - 1 : q;
     }
     __device__ __forceinline__ int cta_of(long long w) const {
-        int c = small ? (int)(((uint32_t)w * (uint32_t)G) / (uint32_t)total) : (int)(w * G / total);
+        int c = small ? (int)(((uint32_t)w * (uint32_t)G) / (uint32_t)total) : (int)div64(w * G, total);
         if (c >= G) c = G - 1;
-        while (c + 1 < G && cta_start(c + 1) <= w) ++c;
-        while (c > 0 && cta_start(c) > w) --c;
+#pragma unroll 1
+        while (c + 1 < G && cta_start<true>(c + 1) <= w) ++c;
+#pragma unroll 1
+        while (c > 0 && cta_start<true>(c) > w) --c;
         return c;
     }
 };
@@ -245,7 +257,10 @@ __device__ __forceinline__ void combine_heads(const CombineArgs& ca, int rg, int
     wk.ctx_len = ctx_len; wk.n_nodes = n_nodes; wk.S = S; wk.H = Hw; wk.B = B; wk.G = G; wk.G_magic = ca.G_magic;
     wk.init();
     long long off = 0;
-    for (int ss = 0; ss < s; ++ss) off += (long long)Hw * wk.width(wk.tiles(ss));
+    if (kCounts) for (int ss = 0; ss < s; ++ss) off += (long long)Hw * wk.width(wk.tiles(ss));
+    else
+#pragma unroll 1
+        for (int ss = 0; ss < s; ++ss) off += (long long)Hw * wk.width(wk.tiles(ss));
     const int T = wk.tiles(s);                             // 0: the sequence has no nodes, hence no items and no output
     const long long head_first = off + (long long)h * wk.width(T) + wk.pad;
     const bool any = !kCounts || T > 0;                    // (without counts every sequence has tiles)
@@ -258,7 +273,7 @@ __device__ __forceinline__ void combine_heads(const CombineArgs& ca, int rg, int
     const bool row_valid = i_local < nb && node < nodes_of(n_nodes, s, B);
     // CTA c's partial for this head sits in slot 2c, or 2c+1 when its segment starts at the head's first tile,
     // which only the first CTA can do.  With fewer items than CTAs some CTAs in [c_lo, c_hi] are empty.
-    const int flag_lo = wk.cta_start(c_lo) <= head_first ? 1 : 0;
+    const int flag_lo = wk.cta_start<true>(c_lo) <= head_first ? 1 : 0;
     const bool sparse = wk.total < G;
     // every CTA waits, also those with nothing to do: the next kernel in the stream relies on "this grid is
     // complete" implying "the main grid is complete"
@@ -272,6 +287,7 @@ __device__ __forceinline__ void combine_heads(const CombineArgs& ca, int rg, int
 
     // kCombineRound parts per round: their (m, l) and their two 16-byte pieces of O/l are loaded together
     // (16 independent loads in flight per thread); a running (M, L) with rescaling merges the rounds
+#pragma unroll 1
     for (int cb = c_lo; cb <= c_hi; cb += kCombineRound) {
         float mp[kCombineRound], lp[kCombineRound];
         uint4 x[kCombineRound][2];
@@ -279,7 +295,7 @@ __device__ __forceinline__ void combine_heads(const CombineArgs& ca, int rg, int
         for (int q = 0; q < kCombineRound; ++q) {
             const int c = cb + q;
             bool use = c <= c_hi;
-            if (use && sparse) use = wk.cta_start(c + 1) > wk.cta_start(c);
+            if (use && sparse) use = wk.cta_start<true>(c + 1) > wk.cta_start<true>(c);
             const int sl = use ? 2 * c + (c == c_lo ? flag_lo : 0) : 0;
             const float* pp = partials + (size_t)sl * kUmmaPartFloats;
             mp[q] = use ? __ldcg(pp + kPartHalfWords + row) : -INFINITY;
