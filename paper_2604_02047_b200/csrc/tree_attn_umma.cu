@@ -303,15 +303,21 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     // 9.2 -> 8.6, 1531 12.4 -> 11.6, 2k 13.6 -> 12.9, 8k 29.2 -> 28.3; 52 heads 8k 43.7 -> 42.0; 4 x 32 over 8, 4k to 16k 41.1 -> 39.8.
     // (Two tiles and more, or by CTAs on idle SMs all of the next call's tiles: slower, 2k 14.1 and more.  The copies in flight
     // are then so many that HBM delivers less.)
-    if (warp == 2 && S <= 32) {
+    // Multi-head: all warps work their place out here, and where the lengths behind the wait are the same (they are, unless the kernel
+    // in front writes them) it stands: step of 32 heads at 2k 17.0 -> 16.7, 40 heads 4k 25.3 -> 24.9, 52 heads 8k 45.5 -> 45.2, 8 ragged
+    // sequences 85.5 -> 84.5.  (Grouped-query heads gained nothing: two sequences, 32 layers 593 -> 596.)
+    int early_ctx = 0, early_nn = 0;
+    bool placed = false;
+    if (S <= 32 && (!kGrouped || warp == 2)) {
         const bool mine = lane < S;
-        const int nn = !mine ? 0 : kCounts ? load_early(n_nodes + lane) : B;
-        const int ctx = mine ? max(load_early(ctx_len + lane), 0) : 0;
-        const int64_t row0 = mine ? load_early(row_off + lane) : 0;
-        const int tiles = nn > 0 && nn <= B && ctx <= kv_rows ? (ctx + nn + kTile - 1) / kTile : 0;
+        early_nn = !mine ? 0 : kCounts ? load_early(n_nodes + lane) : B;
+        early_ctx = mine ? load_early(ctx_len + lane) : 0;
+        const int64_t row0 = warp == 2 && mine ? load_early(row_off + lane) : 0;
+        const int ctx = max(early_ctx, 0), tiles = early_nn > 0 && early_nn <= B && ctx <= kv_rows ? (ctx + early_nn + kTile - 1) / kTile : 0;
         wk.init_lanes(tiles, tiles > 0);
-        locate(tiles, lane);
-        if (w_begin < w_end && (kCluster || wk.small)) {
+        placed = kCluster || wk.small;                  // (a longer list is walked through lengths in memory: not yet)
+        if (placed) locate(tiles, lane);
+        if (warp == 2 && placed && w_begin < w_end) {
             const int64_t row = __shfl_sync(0xFFFFFFFFu, row0, cu.s) + (int64_t)cu.t * kTile;
             if (lane < 4 && row >= 0 && row < kv_rows)
                 tma_prefetch_3d(lane & 2 ? &tmap_v : &tmap_k, (lane & 1) * 64, kGrouped ? cu.h % Hkv : cu.h, (int)row);
@@ -327,7 +333,12 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     // where this CTA starts, found by every warp for itself with all lanes; the lengths and the rows of up to 32 sequences
     // come in one round of loads (lane = sequence).  The first load of K waits for nothing else.
     const int64_t my_row = lane < S ? row_off[lane] : 0;
-    locate(wk.init_warp(lane), lane);
+    if (kGrouped) {
+        locate(wk.init_warp(lane), lane);
+    } else {
+        const bool same = placed && (lane >= S || (ctx_len[lane] == early_ctx && early_ctx <= kv_rows && (!kCounts || n_nodes[lane] == early_nn)));
+        if (!__all_sync(0xFFFFFFFFu, same)) locate(wk.init_warp(lane), lane);
+    }
     const int first_s = w_begin < w_end ? cu.s : 0;
     const int64_t first_row = __shfl_sync(0xFFFFFFFFu, my_row, first_s & 31);
     auto row_of = [&](int s) -> int64_t { return s == first_s && s < 32 ? first_row : row_off[s]; };
