@@ -64,7 +64,7 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 
 // Nodes of sequence s: n_nodes[s] when the array is given, else B.  The array is device data: a value outside [0, B]
 // reads as 0 (the sequence is skipped like one that has left the batch) and is reported as GOOSE_ST_BAD_NODES.
-__device__ __forceinline__ int nodes_of(const int32_t* __restrict__ n_nodes, int s, int B) {
+__host__ __device__ __forceinline__ int nodes_of(const int32_t* __restrict__ n_nodes, int s, int B) {
     if (!n_nodes) return B;
     const int n = n_nodes[s];
     return (n < 0 || n > B) ? 0 : n;

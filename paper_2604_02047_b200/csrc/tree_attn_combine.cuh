@@ -36,27 +36,43 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 }
 
 // ---------------------------------------------------------------- work partition (same code in every role)
+// The arithmetic compiles for the host as well, where a test walks it over lengths that no kernel should meet.
 // 64-bit division out of line.  The merge finds CTAs and their starts in a dozen places, each with such a division for lists of
 // 2^31 / SMs items and more: a third of its code, fetched by every launch and reached by hardly any (step of 40 heads at 4k, with
 // the merge beside walk and compaction: 25.8 -> 25.1 us; 52 heads at 8k 45.8 -> 45.3).
-static __device__ __noinline__ long long div64(long long a, long long b) { return a / b; }
+static __host__ __device__ __noinline__ long long div64(long long a, long long b) { return a / b; }
+__host__ __device__ __forceinline__ uint32_t mul_hi(uint32_t a, uint32_t b) {
+#ifdef __CUDA_ARCH__
+    return __umulhi(a, b);
+#else
+    return (uint32_t)(((uint64_t)a * b) >> 32);
+#endif
+}
 struct Work {
     const int32_t* ctx_len;
     const int32_t* n_nodes;   // per-sequence node counts, or NULL (every tree has B nodes)
     int S, H, B, G;           // H = heads of the work list = M tiles x key/value heads (M-tile-major)
+    int kv_rows;              // rows of the cache, see prefix()
     uint32_t G_magic;         // ceil(2^32 / G): division by G without the 20-instruction sequence
     long long total;          // all items
     int pad;                  // idle items in front of every head, see set_total
     bool small;               // total * (G + 1) fits 31 bits: 32-bit arithmetic (64-bit division is slow on the GPU)
-    // ctx_len comes from device memory: a negative value is treated as 0 (the tree rows alone).  A sequence's keys are
-    // its prefix and the nodes its tree really has; a sequence without nodes (it has left the batch) has no items.
-    __device__ __forceinline__ int tiles(int s) const {
-        if (!n_nodes) return (max(ctx_len[s], 0) + B + kTile - 1) / kTile;
+    // ctx_len comes from device memory.  A negative value is treated as 0 (the tree rows alone), a prefix longer than the cache
+    // as one of the whole cache: such a sequence is flagged and zero-filled, and its list stays one that every range, count and
+    // division below is right for.
+    __host__ __device__ __forceinline__ int prefix(int ctx) const { return min(max(ctx, 0), kv_rows); }
+    // A sequence's keys are its prefix and the nodes its tree really has; a sequence without nodes (it has left the batch) has
+    // no items.
+    __host__ __device__ __forceinline__ int tiles_of(int ctx, int nn) const {
+        return (int)(((uint32_t)prefix(ctx) + (uint32_t)nn + kTile - 1) / kTile);
+    }
+    __host__ __device__ __forceinline__ int tiles(int s) const {
+        if (!n_nodes) return tiles_of(ctx_len[s], B);
         const int nn = nodes_of(n_nodes, s, B);
-        return nn == 0 ? 0 : (max(ctx_len[s], 0) + nn + kTile - 1) / kTile;
+        return nn == 0 ? 0 : tiles_of(ctx_len[s], nn);
     }
     // items of a head of T tiles
-    __device__ __forceinline__ int width(int T) const { return T > 0 ? T + pad : 0; }
+    __host__ __device__ __forceinline__ int width(int T) const { return T > 0 ? T + pad : 0; }
     // A CTA that goes over from one head to the next pays for it (its epilogue and the next head's first softmax stand in
     // turn: 2 to 3 us), so a head starts with idle items that take as much of the CTA's range.  Two tiles' worth, from two tiles
     // a CTA on (a CTA whose whole share is idle items has no work, as one without a share).  Attention call with none / 1 / 2, us:
@@ -64,12 +80,12 @@ struct Work {
     // 2 x 32, 4k to 8k 42.5 / 40.3 / 40.0;  2 x 32 over 8, tree of 61, 1k to 5k 19.9 / 20.0 / 20.4;  52 heads 4k 27.4 / 26.4 / 27.2, 8k
     // 43.9 / 43.4 / 43.4.  In long streams a head switch hides behind the other CTAs' loads and the idle items cost as little:
     // 8 x 32, 16k 329.5 / 329.7 / 329.6, 16 x 32, 1k to 16k 389.2 / 389.7 / 389.1 (sustained 438 / 438 / 436).
-    __device__ __forceinline__ void set_total(long long tile_count, int live) {
+    __host__ __device__ __forceinline__ void set_total(long long tile_count, int live) {
         pad = tile_count >= 2 * (long long)G ? 2 : 0;
         total = tile_count + (long long)pad * H * live;
         small = total * (G + 1) < 0x7FFFFFFFll;
     }
-    __device__ __forceinline__ void init() {
+    __host__ __device__ __forceinline__ void init() {
         long long tot = 0;
         int live = 0;
         auto add = [&](int s) {
@@ -102,12 +118,12 @@ struct Work {
         return mine;
     }
     template <bool kCall = false>
-    __device__ __forceinline__ long long cta_start(int c) const {
+    __host__ __device__ __forceinline__ long long cta_start(int c) const {
         if (!small) return kCall ? div64(total * c, G) : total * c / G;
-        const uint32_t n = (uint32_t)total * (uint32_t)c, q = __umulhi(n, G_magic);   // exact or one too large (n < 2^31)
+        const uint32_t n = (uint32_t)total * (uint32_t)c, q = mul_hi(n, G_magic);   // exact or one too large (n < 2^31)
         return q * (uint32_t)G > n ? q - 1 : q;
     }
-    __device__ __forceinline__ int cta_of(long long w) const {
+    __host__ __device__ __forceinline__ int cta_of(long long w) const {
         int c = small ? (int)(((uint32_t)w * (uint32_t)G) / (uint32_t)total) : (int)div64(w * G, total);
         if (c >= G) c = G - 1;
 #pragma unroll 1
@@ -118,10 +134,17 @@ struct Work {
     }
 };
 
+// first tile of CTA r of the n CTAs (a cluster) that share a head of T tiles; rounded up, so that the last CTA, which has the
+// masked tile, has no tile more than the others.  n_magic = ceil(2^32 / n): a division by a multiplication, exact for the
+// T * 8 < 2^28 that Work::tiles_of() can give
+__host__ __device__ __forceinline__ int cluster_start(int T, int r, int n, uint32_t n_magic) {
+    return (int)mul_hi((uint32_t)(T * r + n - 1), n_magic);
+}
+
 struct Cursor {               // walks items in order
     long long w;              // item index
     int s, h, t, T;
-    __device__ __forceinline__ void seek(const Work& wk, long long w0) {
+    __host__ __device__ __forceinline__ void seek(const Work& wk, long long w0) {
         long long off = 0;
         int ss = 0;
         int TT = wk.tiles(0);
@@ -137,7 +160,7 @@ struct Cursor {               // walks items in order
         enter(wk, (int)(rem - (long long)h * W));
     }
     // at item v of the head: past the idle ones
-    __device__ __forceinline__ void enter(const Work& wk, int v) {
+    __host__ __device__ __forceinline__ void enter(const Work& wk, int v) {
         t = v - wk.pad;
         if (t < 0) { w -= t; t = 0; }
     }
@@ -167,8 +190,8 @@ struct Cursor {               // walks items in order
         enter(wk, v);
     }
     // items of this head from here to its end, at most up to item `w_end` of the list; and past n of them
-    __device__ __forceinline__ int run(long long w_end) const { return (int)min((long long)(T - t), w_end - w); }
-    __device__ __forceinline__ void skip(const Work& wk, int n) {
+    __host__ __device__ __forceinline__ int run(long long w_end) const { return (int)min((long long)(T - t), w_end - w); }
+    __host__ __device__ __forceinline__ void skip(const Work& wk, int n) {
         w += n; t += n;
         if (t == T) {
             t = 0; ++h; w += wk.pad;
@@ -196,6 +219,7 @@ struct CombineArgs {
     int G;                    // CTAs of the main kernel
     uint32_t G_magic;         // ceil(2^32 / G)
     int Hw;                   // heads of the work list
+    int kv_rows;
     const float* partials;
     __nv_bfloat16* out;
     float* lse;
@@ -254,7 +278,7 @@ __device__ __forceinline__ void combine_heads(const CombineArgs& ca, int rg, int
     // kernel triggers its dependents after its own pdl_wait(), i.e. after whatever produced ctx_len[] completed.
     // So all of it runs before the wait, and the partial loads are issued the moment the main grid is done.
     Work wk;
-    wk.ctx_len = ctx_len; wk.n_nodes = n_nodes; wk.S = S; wk.H = Hw; wk.B = B; wk.G = G; wk.G_magic = ca.G_magic;
+    wk.ctx_len = ctx_len; wk.n_nodes = n_nodes; wk.S = S; wk.H = Hw; wk.B = B; wk.G = G; wk.G_magic = ca.G_magic; wk.kv_rows = ca.kv_rows;
     wk.init();
     long long off = 0;
     if (kCounts) for (int ss = 0; ss < s; ++ss) off += (long long)Hw * wk.width(wk.tiles(ss));

@@ -278,12 +278,11 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     // g query heads per key/value head, nb nodes per M tile (nb * g <= 128), n_mt M tiles per sequence
     const int n_mt = kGrouped ? (B + nb - 1) / nb : 1;
     wk.ctx_len = ctx_len; wk.n_nodes = n_nodes; wk.S = S; wk.H = n_mt * Hkv; wk.B = B; wk.G = gridDim.x; wk.G_magic = G_magic;
+    wk.kv_rows = (int)kv_rows;                          // (the entry points take no more than 2^31 - 1)
     // cluster mode: this CTA is number `rank` of the `cluster` CTAs that share head `head` of the one sequence
     const int head = kCluster ? (int)__umulhi(blockIdx.x, G_magic) : 0, rank = kCluster ? blockIdx.x - head * cluster : 0;
     int T_all = 0;                                      // tiles of that sequence
-    // its first tile; rounded up, so that the last CTA, which has the masked tile, has no tile more than the others
-    // (a division by a multiplication, exact below 2^29: T_all * 8 < 2^28)
-    auto rank_start = [&](int r) { return (int)__umulhi((uint32_t)(T_all * r + cluster - 1), G_magic); };
+    auto rank_start = [&](int r) { return cluster_start(T_all, r, cluster, G_magic); };
     // this CTA's items, found by a whole warp (lane = sequence, `tiles` its tiles); a list of more than 32 sequences is read again
     long long w_begin = 0, w_end = 0;
     Cursor cu;
@@ -313,7 +312,7 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
         early_nn = !mine ? 0 : kCounts ? load_early(n_nodes + lane) : B;
         early_ctx = mine ? load_early(ctx_len + lane) : 0;
         const int64_t row0 = warp == 2 && mine ? load_early(row_off + lane) : 0;
-        const int ctx = max(early_ctx, 0), tiles = early_nn > 0 && early_nn <= B && ctx <= kv_rows ? (ctx + early_nn + kTile - 1) / kTile : 0;
+        const int tiles = early_nn > 0 && early_nn <= B ? wk.tiles_of(early_ctx, early_nn) : 0;
         wk.init_lanes(tiles, tiles > 0);
         placed = kCluster || wk.small;                  // (a longer list is walked through lengths in memory: not yet)
         if (placed) locate(tiles, lane);
@@ -336,7 +335,7 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     if (kGrouped) {
         locate(wk.init_warp(lane), lane);
     } else {
-        const bool same = placed && (lane >= S || (ctx_len[lane] == early_ctx && early_ctx <= kv_rows && (!kCounts || n_nodes[lane] == early_nn)));
+        const bool same = placed && (lane >= S || (ctx_len[lane] == early_ctx && (!kCounts || n_nodes[lane] == early_nn)));
         if (!__all_sync(0xFFFFFFFFu, same)) locate(wk.init_warp(lane), lane);
     }
     const int first_s = w_begin < w_end ? cu.s : 0;
@@ -475,7 +474,7 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                 const int nn = nodes_of(n_nodes, s0, B);   // nodes this sequence's tree really has (> 0: it has items)
                 const bool row_valid = i_local < nb && node < nn;
                 const bool warp_has_rows = 32 * (warp & 3) < min(nb, nn - mt * nb) * g;
-                const int ctx = max(ctx_len[s0], 0);
+                const int ctx = wk.prefix(ctx_len[s0]);
                 const int n_keys = ctx + nn;               // rows behind may hold anything: masked, and zeroed in V
                 const int32_t* par = parent + (size_t)s0 * B;
                 const int t_first = cu.t;
@@ -945,7 +944,7 @@ cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __
     if (e != cudaSuccess || cluster > 1) return e;          // (a cluster merges its head itself)
     CombineArgs ca;
     ca.ctx_len = ctx_len; ca.n_nodes = n_nodes; ca.S = S; ca.B = B; ca.H = H; ca.Hkv = Hkv; ca.g = g; ca.nb = nb;
-    ca.G = grid; ca.G_magic = g_magic; ca.Hw = Hw; ca.partials = c->partials; ca.out = out; ca.lse = lse;
+    ca.G = grid; ca.G_magic = g_magic; ca.Hw = Hw; ca.kv_rows = (int)kv_rows; ca.partials = c->partials; ca.out = out; ca.lse = lse;
     const int row_groups = (nb * g + 31) / 32;
     if (defer_merge) {                                  // the caller runs the merge as a role of a later launch
         defer_merge->args = ca; defer_merge->row_groups = row_groups; defer_merge->grouped = grouped;
