@@ -436,7 +436,7 @@ int goose_verify_step_host_gqa(goose_ctx* c, void* k_cache, void* v_cache, int64
     for (int s = 0; s < S; ++s) {
         const int nn = h_n_nodes ? h_n_nodes[s] : B;        // host data: validated here, before anything is enqueued
         if (nn < 0 || nn > B) return GOOSE_EINVAL;
-        if (nn > 0 && (h_row_off[s] < 0 || h_ctx_len[s] < 0 || h_row_off[s] + h_ctx_len[s] + nn > kv_rows)) return GOOSE_EINVAL;
+        if (nn > 0 && goose::rows_outside(h_row_off[s], h_ctx_len[s], nn, kv_rows)) return GOOSE_EINVAL;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 

@@ -73,6 +73,12 @@ __device__ __forceinline__ bool nodes_bad(const int32_t* __restrict__ n_nodes, i
     return n_nodes != nullptr && (n_nodes[s] < 0 || n_nodes[s] > B);
 }
 
+// Do a sequence's rows row .. row + ctx + nn - 1 leave the cache?  row and ctx are device data: the sum would wrap for a row
+// near 2^63, the differences cannot.
+__host__ __device__ __forceinline__ bool rows_outside(int64_t row, int ctx, int nn, int64_t kv_rows) {
+    return ctx < 0 || row < 0 || row > kv_rows - nn - ctx;
+}
+
 // Bounded mbarrier wait, shared by every kernel that waits on asynchronous copies or tensor-core commits.
 // Returns 0 when the barrier phase completed, 1 when `*abort_flag` was raised by another thread of the CTA meanwhile,
 // 2 when `limit_cycles` SM cycles passed (the caller raises the flag, records GOOSE_ST_TIMEOUT and unwinds).

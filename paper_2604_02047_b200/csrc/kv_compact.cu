@@ -51,7 +51,7 @@ kv_compact_kernel(__nv_bfloat16* kc, __nv_bfloat16* vc,
     if (threadIdx.x == 0) s_bad = 0;
     __syncthreads();
     // rows this sequence owns must lie inside the cache: never form an address from unchecked device data
-    const bool bad_rows = ctx < 0 || r0 < 0 || r0 + ctx + nn > kv_rows;
+    const bool bad_rows = rows_outside(r0, ctx, nn, kv_rows);
     bool bad = (L < 0 || L >= nn) || bad_rows;
     if (!bad && (int)threadIdx.x <= L) {
         const int j = threadIdx.x, prev = j == 0 ? -1 : s_path[j - 1];
@@ -179,7 +179,7 @@ accept_compact_kernel(__nv_bfloat16* kc, __nv_bfloat16* vc, const int64_t* __res
     // rows this sequence owns must lie inside the cache: never form an address from unchecked device data
     const int ctx0 = ctx_len[s];
     const int64_t r0 = row_off[s];
-    const bool bad_rows = live && (ctx0 < 0 || r0 < 0 || r0 + ctx0 + nn > kv_rows);
+    const bool bad_rows = live && rows_outside(r0, ctx0, nn, kv_rows);
     constexpr int kPer = kMaxB / 32;
     int my_par[kPer], my_tok[kPer];
     bool bad = false;

@@ -123,7 +123,7 @@ tree_attn_mma_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* _
         bad |= (i == 0) ? (p != -1) : (p < 0 || p >= i);
     }
     // the sequence's rows must lie inside the cache: never form an address from unchecked device data
-    const bool bad_rows = ctx_len[s] < 0 || row0 < 0 || row0 + ctx + B > kv_rows;
+    const bool bad_rows = rows_outside(row0, ctx_len[s], B, kv_rows);
     bad = __syncthreads_or(bad | (bad_rows ? 1 : 0));
 
     const int rowA = warp * 16 + g, rowB = rowA + 8;       // this thread's two query rows

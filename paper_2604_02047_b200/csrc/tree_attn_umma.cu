@@ -317,8 +317,8 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
         placed = kCluster || wk.small;                  // (a longer list is walked through lengths in memory: not yet)
         if (placed) locate(tiles, lane);
         if (warp == 2 && placed && w_begin < w_end) {
-            const int64_t row = __shfl_sync(0xFFFFFFFFu, row0, cu.s) + (int64_t)cu.t * kTile;
-            if (lane < 4 && row >= 0 && row < kv_rows)
+            const int64_t first = __shfl_sync(0xFFFFFFFFu, row0, cu.s), row = min(first, kv_rows) + (int64_t)cu.t * kTile;
+            if (lane < 4 && first >= 0 && row < kv_rows)
                 tma_prefetch_3d(lane & 2 ? &tmap_v : &tmap_k, (lane & 1) * 64, kGrouped ? cu.h % Hkv : cu.h, (int)row);
         }
     }
@@ -490,8 +490,7 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                     }
                     // the sequence's rows must lie inside the cache (TMA would only read zeros outside, but the
                     // result would be meaningless): treated like an invalid tree, with its own status bit
-                    const int64_t r0 = row_of(s0);
-                    const bool bad_rows = ctx_len[s0] < 0 || r0 < 0 || r0 + ctx + nn > kv_rows;
+                    const bool bad_rows = rows_outside(row_of(s0), ctx_len[s0], nn, kv_rows);
                     if (bad_rows && sm_tid == 0) { hd->bad_parent = 1; atomicOr(&status[s0], GOOSE_ST_BAD_ROWS); }
                     ok = group_sync(hd, gsync, status);
                     bad = hd->bad_parent != 0;

@@ -1,6 +1,7 @@
 """The attention's work partition, compiled for the host from the kernels' own header and walked as the roles walk it: every tile of
 every head dealt exactly once, in order, within the arrays -- for lengths that no kernel should meet as well (they are device data),
-where a sequence counts as one of the whole cache.  The merge's idea of which CTAs have a part of a head agrees."""
+where a sequence counts as one of the whole cache.  The merge's idea of which CTAs have a part of a head agrees.  And the check that
+every kernel makes of a sequence's rows."""
 import ctypes
 import os
 import subprocess
@@ -58,26 +59,30 @@ extern "C" int walk(int S, int B, int Hw, int G, int cluster, int kv_rows, const
     }
     return 0;
 }
+extern "C" int outside(int64_t row, int ctx, int nn, int64_t kv_rows) { return rows_outside(row, ctx, nn, kv_rows); }
 """
 
 
 @pytest.fixture(scope="module")
-def walk(tmp_path_factory):
+def lib(tmp_path_factory):
     d = tmp_path_factory.mktemp("partition")
     src, lib = str(d / "walk.cu"), str(d / "walk.so")
     with open(src, "w") as f:
         f.write(SOURCE)
     r = subprocess.run([build._nvcc()] + build.NVCC_FLAGS + ["-shared", src, "-o", lib], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
-    fn = ctypes.CDLL(lib).walk
+    return ctypes.CDLL(lib)
 
+
+@pytest.fixture(scope="module")
+def walk(lib):
     def call(B, Hw, G, cluster, kv_rows, ctx, counts):
         S = len(ctx)
         c = np.asarray(ctx, np.int32)
         nn = None if counts is None else np.asarray(counts, np.int32)
         first, last, dealt = (np.full((S, Hw), v, np.int32) for v in (-1, -1, 0))
         p = lambda a: None if a is None else a.ctypes.data_as(ctypes.c_void_p)
-        return fn(S, B, Hw, G, cluster, kv_rows, p(c), p(nn), p(first), p(last), p(dealt)), dealt
+        return lib.walk(S, B, Hw, G, cluster, kv_rows, p(c), p(nn), p(first), p(last), p(dealt)), dealt
 
     return call
 
@@ -106,3 +111,14 @@ def test_every_tile_is_dealt_once(walk, form, B, counts):
                 for s, c in enumerate(ctx):
                     n = B if nn is None else nn[s] if 0 <= nn[s] <= B else 0
                     assert (dealt[s] == (0 if n == 0 else -(-(min(max(c, 0), kv_rows) + n) // 128))).all()
+
+
+@pytest.mark.parametrize("kv_rows", [1, 900, BIG, 2 ** 40])
+def test_rows_outside_the_cache(lib, kv_rows):
+    """Row offsets up to the ends of 64 bits, against integers without an end."""
+    ends = [0, 1, 5, kv_rows - 17, kv_rows - 16, kv_rows, kv_rows + 1, 2 ** 62, 2 ** 63 - 2 ** 31 - 200, 2 ** 63 - 300, 2 ** 63 - 16, 2 ** 63 - 1, -1, -2 ** 63]
+    for row in ends:
+        for ctx in (0, 1, 16, 883, 899, 900, BIG - 200, BIG, -1, -2 ** 31):
+            for n in (1, 16, 128):
+                want = ctx < 0 or row < 0 or row + ctx + n > kv_rows
+                assert lib.outside(ctypes.c_int64(row), ctx, n, ctypes.c_int64(kv_rows)) == want, (row, ctx, n)

@@ -1,4 +1,4 @@
-"""Lengths on the device that put a sequence outside the cache, up to the largest an int holds: the sequence gets its status bit, zeros
+"""Lengths and row offsets on the device that put a sequence outside the cache, up to the largest that their types hold: the sequence gets its status bit, zeros
 and an untouched cache, the others in the batch their usual results, and nothing is written around the outputs."""
 import numpy as np
 import pytest
@@ -65,3 +65,41 @@ def test_length_outside_the_cache(goose, oracle, H, Hkv, B, ctxs, counts, length
     r0, r1 = int(x.row_off[bad]), int(x.row_off[bad]) + ctxs[bad] + B
     for name, was in zip(("k_cache", "v_cache"), before):
         assert torch.equal(d[name][r0:r1], was[r0:r1])
+
+
+@pytest.mark.parametrize("row", [2 ** 63 - 1, 2 ** 63 - 130, 2 ** 62, -2 ** 63])
+def test_row_offset_outside_the_cache(goose, oracle, row):
+    from paper_2604_02047_b200 import binding
+    S, H, B, V = 2, 8, 16, 512
+    x = synth.make_inputs(S, H, B, [130, 140], [synth.chain_tree(B)] * S, seed=3, V=V, k=4)
+    d = binding.to_device(x)
+    off = x.row_off.copy()
+    off[1] = row
+    d_off = torch.from_numpy(off).cuda()
+    ref, _ = oracle.tree_attn(x.q, x.k_cache, x.v_cache, x.row_off, x.ctx_len, x.parent, x.scale)
+
+    def check(out):
+        torch.cuda.synchronize()
+        assert goose.last_status(S).tolist() == [0, 8]
+        assert (out[1] == 0).all() and attn_row_err(out[:1].float().cpu().numpy().astype(np.float64), ref[:1]).max() <= ATTN_TOL
+
+    for impl in (binding.ATTN_MMA, binding.ATTN_UMMA):
+        goose.set_attn_impl(impl)
+        try:
+            check(goose.tree_attn(d["q"], d["k_cache"], d["v_cache"], d_off, d["ctx_len"], d["parent"], x.scale)[0])
+        finally:
+            goose.set_attn_impl(binding.ATTN_AUTO)
+    check(goose.verify_step(d["q"], d["k_cache"], d["v_cache"], d_off, d["ctx_len"], d["parent"], d["draft_tok"], d["logits"], 4, x.scale)["out"])
+    before = [d[n].clone() for n in ("k_cache", "v_cache")]
+    path = torch.tensor([[0, 2, 3] + [-1] * (B - 3)] * S, dtype=torch.int32).cuda()
+    goose.kv_compact(d["k_cache"], d["v_cache"], d_off, d["ctx_len"], path, torch.tensor([2, 2], dtype=torch.int32).cuda())
+    assert goose.last_status(S).tolist() == [0, 8]
+    for name, was in zip(("k_cache", "v_cache"), before):
+        assert torch.equal(d[name][146:], was[146:])
+    if row > 0:                                               # on host buffers: refused before anything is enqueued
+        h = {n: t.cpu().pin_memory() for n, t in d.items() if isinstance(t, torch.Tensor)}
+        new = torch.zeros((S, B, H, 128), dtype=torch.bfloat16).pin_memory()
+        outs = goose.alloc_step_outputs(S, B, H, 128, 4, device="cpu")
+        with pytest.raises(binding.GooseError, match="invalid argument"):
+            goose.verify_step_host(d["k_cache"], d["v_cache"], h["q"], new, new, torch.from_numpy(off), h["ctx_len"], h["parent"],
+                                   h["draft_tok"], h["logits"], 4, x.scale, outs)
