@@ -189,6 +189,8 @@ struct Cursor {               // walks items in order
         if (v >= W) { ++h; v -= W; }
         enter(wk, v);
     }
+    // is any of the items from here to `w_end` a tile?  (where a head's idle items were skipped there may be none)
+    __host__ __device__ __forceinline__ bool any(long long w_end) const { return w < w_end; }
     // items of this head from here to its end, at most up to item `w_end` of the list; and past n of them
     __host__ __device__ __forceinline__ int run(long long w_end) const { return (int)min((long long)(T - t), w_end - w); }
     __host__ __device__ __forceinline__ void skip(const Work& wk, int n) {

@@ -293,7 +293,10 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
             cu.w = w_begin; cu.s = 0; cu.h = head; cu.t = rank_start(rank); cu.T = T_all;
         } else {
             w_begin = wk.cta_start(blockIdx.x); w_end = wk.cta_start(blockIdx.x + 1);
-            if (w_begin < w_end) cu.seek_warp(wk, w_begin, lane, tiles);
+            if (w_begin < w_end) {
+                cu.seek_warp(wk, w_begin, lane, tiles);
+                if (!cu.any(w_end)) w_end = w_begin;    // idle items alone: no work, and no tile to look at ahead of the wait
+            }
         }
     };
     // The CTA is up 0.7 to 1 us before the kernel in front has ended, and the first load of K after that used to take 1.8 us.

@@ -15,9 +15,9 @@ SOURCE = r"""
 #include "tree_attn_combine.cuh"
 using namespace goose;
 static uint32_t magic(int n) { return (uint32_t)((0x100000000ull + n - 1) / n); }
-// 0, or what is wrong.  first / last [S][Hw]: the CTAs that have a part of the head; dealt [S][Hw]: its tiles so far
+// 0, or what is wrong.  idle: CTAs whose range is idle items alone.  first / last [S][Hw]: the CTAs that have a part of the head; dealt [S][Hw]: its tiles so far
 extern "C" int walk(int S, int B, int Hw, int G, int cluster, int kv_rows, const int32_t* ctx_len, const int32_t* n_nodes,
-                    int32_t* first, int32_t* last, int32_t* dealt) {
+                    int32_t* first, int32_t* last, int32_t* dealt, int32_t* idle) {
     const int grid = cluster > 1 ? Hw * cluster : G;
     Work wk;
     wk.ctx_len = ctx_len; wk.n_nodes = n_nodes; wk.S = S; wk.H = Hw; wk.B = B; wk.G = grid; wk.kv_rows = kv_rows;
@@ -37,6 +37,7 @@ extern "C" int walk(int S, int B, int Hw, int G, int cluster, int kv_rows, const
         }
         if (w_begin > w_end) return 1;
         if (w_begin == w_end) continue;
+        if (!cu.any(w_end)) { ++*idle; continue; }
         while (cu.w < w_end) {
             if (cu.s < 0 || cu.s >= S || cu.h < 0 || cu.h >= Hw) return 2;
             const int at = cu.s * Hw + cu.h, n = cu.run(w_end);
@@ -81,8 +82,9 @@ def walk(lib):
         c = np.asarray(ctx, np.int32)
         nn = None if counts is None else np.asarray(counts, np.int32)
         first, last, dealt = (np.full((S, Hw), v, np.int32) for v in (-1, -1, 0))
+        call.idle = ctypes.c_int32(0)
         p = lambda a: None if a is None else a.ctypes.data_as(ctypes.c_void_p)
-        return lib.walk(S, B, Hw, G, cluster, kv_rows, p(c), p(nn), p(first), p(last), p(dealt)), dealt
+        return lib.walk(S, B, Hw, G, cluster, kv_rows, p(c), p(nn), p(first), p(last), p(dealt), ctypes.byref(call.idle)), dealt
 
     return call
 
@@ -111,6 +113,13 @@ def test_every_tile_is_dealt_once(walk, form, B, counts):
                 for s, c in enumerate(ctx):
                     n = B if nn is None else nn[s] if 0 <= nn[s] <= B else 0
                     assert (dealt[s] == (0 if n == 0 else -(-(min(max(c, 0), kv_rows) + n) // 128))).all()
+
+
+@pytest.mark.parametrize("Hw,B,ctx,idle", [(8, 20, 4700, True), (8, 20, 4716, True), (32, 16, 9000, False)])
+def test_ranges_of_idle_items_alone(walk, Hw, B, ctx, idle):
+    """Two idle items stand in front of a head: with about two items a CTA some CTAs have nothing else, and count as without work."""
+    rc, dealt = walk(B, Hw, 148, 1, ctx + B, [ctx], None)
+    assert rc == 0 and (dealt == -(-(ctx + B) // 128)).all() and (walk.idle.value > 0) == idle
 
 
 @pytest.mark.parametrize("kv_rows", [1, 900, BIG, 2 ** 40])
