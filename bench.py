@@ -42,9 +42,9 @@ BURST_MS = 10.0                 # length of a burst region of the per-kernel leg
 SUSTAIN_SECONDS = 1.5           # further regions keep the GPU under the same load until the clock sampler has >= 10 samples
 # DRAM traffic per attention call (the merge kernel, where there is one, reads from L2) from the ncu captures summarised under profiles/ (bytes); these
 # are NOT measured by the run that prints them: `roofline.traffic_source` names the capture.  None = not captured.
-NCU_TRAFFIC_BYTES = {"33b": (227_890_000, "profiles/tree_attn_umma_33b.md"),      # 223.29 MB read + 4.13-5.07 MB written
-                     "13b": (88_760_000, "profiles/tree_attn_umma_13b.md"),       # 86.46 MB read + 2.30 MB written
-                     "gqa8b": (171_380_000, "profiles/tree_attn_umma_gqa8b.md")}  # 164.99 MB read + 5.75-7.02 MB written
+NCU_TRAFFIC_BYTES = {"33b": (227_140_000, "profiles/tree_attn_umma_33b.md"),      # 223.29 MB read + 3.65-4.07 MB written
+                     "13b": (89_340_000, "profiles/tree_attn_umma_13b.md"),       # 86.46 MB read + 2.73-3.04 MB written
+                     "gqa8b": (169_310_000, "profiles/tree_attn_umma_gqa8b.md")}  # 164.99 MB read + 4.12-4.51 MB written
 
 
 def _peaks():
@@ -591,7 +591,7 @@ def run_ours(args, x, cfg, rank, world, local_rank):
                     "four_calls_us": legs["four"][0] * 1e3,
                     "four_calls_note": "goose_tree_attn, goose_node_topk, goose_accept, goose_kv_compact one after the other "
                                        "(5 launches, 4 where the attention's clusters merge their heads themselves; every kernel "
-                                       "waits for its predecessor before it reads anything); the metric is goose_verify_step, "
+                                       "waits for its predecessor before it reads what it works on); the metric is goose_verify_step, "
                                        "whose 3 launches overlap the top-k with the attention and run the merge of the split "
                                        "heads beside the walk and the compaction",
                     "step_l2_warm_us": legs["warm"][0] * 1e3,

@@ -53,8 +53,10 @@ struct goose_ctx {
 namespace goose {
 
 // Programmatic dependent launch.  Every kernel of the library is launched with the
-// programmatic-stream-serialisation attribute and runs  prologue (no global memory access) ->
-// pdl_wait() -> pdl_trigger() -> body.  pdl_wait() returns once the preceding kernel in the stream has
+// programmatic-stream-serialisation attribute and runs  prologue -> pdl_wait() -> pdl_trigger() -> body.
+// The prologue takes no result from global memory: it touches none, or only what is final already (inputs of the
+// step, ahead of the wait on the step's earlier kernels), or it looks and works out again behind the wait what it saw
+// (the tensor-core attention kernel: lengths, counts, rows, its first tile).  pdl_wait() returns once the preceding kernel in the stream has
 // completed and its writes are visible; because that kernel passed its own pdl_wait() before it
 // triggered, completion is transitive over the whole stream.  The overlap gained is the launch latency
 // and the prologue of the next kernel.

@@ -37,6 +37,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 
 // ---------------------------------------------------------------- work partition (same code in every role)
 // The arithmetic compiles for the host as well, where a test walks it over lengths that no kernel should meet.
+//
 // 64-bit division out of line.  The merge finds CTAs and their starts in a dozen places, each with such a division for lists of
 // 2^31 / SMs items and more: a third of its code, fetched by every launch and reached by hardly any (step of 40 heads at 4k, with
 // the merge beside walk and compaction: 25.8 -> 25.1 us; 52 heads at 8k 45.8 -> 45.3).
@@ -136,7 +137,8 @@ struct Work {
 
 // first tile of CTA r of the n CTAs (a cluster) that share a head of T tiles; rounded up, so that the last CTA, which has the
 // masked tile, has no tile more than the others.  n_magic = ceil(2^32 / n): a division by a multiplication, exact for the
-// T * 8 < 2^28 that Work::tiles_of() can give
+// T * 8 < 2^28 that Work::tiles_of() can give (the division itself stood in front of the first load: attention call 512 keys
+// 8.51 -> 8.15, 1531 11.78 -> 11.42, 32 over 8 heads 3k 12.50 -> 12.10 us)
 __host__ __device__ __forceinline__ int cluster_start(int T, int r, int n, uint32_t n_magic) {
     return (int)mul_hi((uint32_t)(T * r + n - 1), n_magic);
 }

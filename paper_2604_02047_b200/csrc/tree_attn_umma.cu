@@ -153,7 +153,8 @@ __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
 // memory, and the other half, the same for all.  One descriptor a tile and additions instead of sixteen built from scratch by
 // the issuing thread, and tile counts and stages carried along instead of worked out tile by tile (with 64-bit list positions
 // and divisions by five), stood between a tile's arrival and its scores: attention call 512 keys 8.5 -> 8.1, 1531 11.4 -> 11.0,
-// 2k 12.7 -> 12.4, 8k 28.0 -> 27.4 (32 heads), 32 over 8 heads 3k 12.2 -> 11.9, 2 x 32 over 8 16.7 -> 16.4 us.
+// 2k 12.7 -> 12.4, 8k 28.0 -> 27.4 (32 heads), 32 over 8 heads 3k 12.2 -> 11.9, 2 x 32 over 8 16.7 -> 16.4 us, with the
+// multiplication of cluster_start(), to which the clusters owe most of it.
 __device__ __forceinline__ uint32_t smem_desc_lo(uint32_t addr, uint32_t lbo) { return ((addr >> 4) & 0x3FFF) | ((lbo >> 4) << 16); }
 __device__ __forceinline__ uint64_t smem_desc(uint32_t lo) {
     constexpr uint32_t hi = (1024u >> 4) /*SBO: the next eight rows*/ | (1u << 14) /*descriptor version*/ | (2u << 29) /*SWIZZLE_128B*/;
@@ -303,11 +304,15 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     // One warp brings the CTA's first tile into L2 meanwhile: where it lies is worked out from lengths that the kernel in front
     // may still be writing, so all of it is a hint, worked out again below.  Attention call without -> with, us: 32 heads 512 keys
     // 9.2 -> 8.6, 1531 12.4 -> 11.6, 2k 13.6 -> 12.9, 8k 29.2 -> 28.3; 52 heads 8k 43.7 -> 42.0; 4 x 32 over 8, 4k to 16k 41.1 -> 39.8.
+    // That is behind a kernel of this library, which lets its dependents in as soon as its own wait is over.  Behind one that does
+    // not, the CTA comes up when the lengths are final and there is little time to gain (a small element-wise kernel, then the call;
+    // both, without -> with the look and the places below): 512 10.9 to 11.4 -> 10.9, 1531 14.1 to 14.6 -> 13.9 to 14.7.
     // (Two tiles and more, or by CTAs on idle SMs all of the next call's tiles: slower, 2k 14.1 and more.  The copies in flight
     // are then so many that HBM delivers less.)
     // Multi-head: all warps work their place out here, and where the lengths behind the wait are the same (they are, unless the kernel
     // in front writes them) it stands: step of 32 heads at 2k 17.0 -> 16.7, 40 heads 4k 25.3 -> 24.9, 52 heads 8k 45.5 -> 45.2, 8 ragged
-    // sequences 85.5 -> 84.5.  (Grouped-query heads gained nothing: two sequences, 32 layers 593 -> 596.)
+    // sequences 85.5 -> 84.5.  Grouped-query heads look again: with the place kept, call of 4 x 32 over 8 35.4 -> 35.7, 2 x 32 over 8
+    // 17.0 -> 17.6, one sequence in clusters 12.10 -> 12.01 and its cycle 20.6 -> 20.7.
     int early_ctx = 0, early_nn = 0;
     bool placed = false;
     if (S <= 32 && (!kGrouped || warp == 2)) {
