@@ -210,10 +210,8 @@ int goose_harvest(goose_ctx* c, const void* logits, int rows, int V, int64_t ldl
     if (k < 1 || k > GOOSE_MAX_K || k > V) return GOOSE_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = goose::launch_node_topk(c, (const __nv_bfloat16*)logits, rows, V, ldl, k, argmax, topk_ids,
-                                            topk_vals, row_lse, st);
-    if (e != cudaSuccess) return cuda_fail(e);
-    e = goose::launch_harvest_scatter(c, row_tok, rows, table_rows, k, topk_ids, topk_vals, row_lse, adj_ids,
-                                      adj_scores, st);
+                                            topk_vals, row_lse, st, false, nullptr, 0, 0,
+                                            goose::HarvestTable{row_tok, table_rows, adj_ids, adj_scores});
     if (e != cudaSuccess) return cuda_fail(e);
     return GOOSE_OK;
 }

@@ -147,19 +147,28 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 #endif
 
+// Where a harvest puts what it finds: logits row r predicts the successors of token row_tok[r], whose row of the dense tables
+// [table_rows][k] gets the k ids and their softmax probabilities (a token outside the table: nothing).  Of several rows with one token
+// the last one stands.  adj_ids == NULL: no harvest.
+struct HarvestTable {
+    const int32_t* row_tok;
+    int table_rows;
+    int32_t* adj_ids;
+    float* adj_scores;
+};
+
 // launchers (each returns a cudaError_t from the launch)
 // max_ctas (0: one per SM): the largest grid
 // inputs_ready: everything in front of the kernel that precedes this one in the stream is complete when this one can
 // start, and that kernel has nothing to do with this one's inputs and outputs (see the kernel)
+// table (with row_lse, without n_nodes): the harvest of every row
 // n_nodes (may be NULL) with B: row r = s * B + i exists iff i < n_nodes[s]; other rows are neither read nor written
 cudaError_t launch_node_topk(goose_ctx* c, const __nv_bfloat16* logits, int rows, int V, int64_t ldl, int k,
                              int32_t* argmax, int32_t* ids, float* vals, float* row_lse, cudaStream_t st,
-                             bool inputs_ready = false, const int32_t* n_nodes = nullptr, int B = 0, int max_ctas = 0);
+                             bool inputs_ready = false, const int32_t* n_nodes = nullptr, int B = 0, int max_ctas = 0,
+                             HarvestTable table = {});
 // items of that kernel's work list: chunks of rows
 int topk_items(int rows, int V);
-cudaError_t launch_harvest_scatter(goose_ctx* c, const int32_t* row_tok, int rows, int table_rows, int k,
-                                   const int32_t* ids, const float* vals, const float* row_lse,
-                                   int32_t* adj_ids, float* adj_scores, cudaStream_t st);
 cudaError_t launch_accept(goose_ctx* c, const int32_t* draft_tok, const int32_t* parent, const int32_t* n_nodes,
                           const int32_t* argmax, int S, int B, int32_t* path, int32_t* accept_len, int32_t* bonus,
                           cudaStream_t st);

@@ -102,7 +102,7 @@ cudaError_t launch_kv_compact(goose_ctx* c, __nv_bfloat16* kc, __nv_bfloat16* vc
 // they are read before the dependency wait; argmax[] (the top-k kernel's result) and the cache rows are read after it.
 // With a harvest (adj_ids != NULL) the launch carries a third block role, blockIdx.y == 2: one warp per logits row of the
 // sequence writes that row's top-k ids and softmax scores to adjacency-table row draft_tok[row] unless a later row of the
-// call carries the same token -- the rule of harvest_scatter_kernel, decided here before the wait (tokens are inputs).
+// call carries the same token -- the rule of HarvestTable, decided here before the wait (tokens are inputs).
 // With the persistent form of the tensor-core attention kernel the launch also carries the merge of that kernel's split heads (kMerge: 0 = no
 // merge role, 1 = multi-head, 2 = grouped-query attention; 256 threads per CTA then): blockIdx.y >= base_roles is head
 // blockIdx.y - base_roles of the attention work list, blockIdx.x its group of 32 rows.  The merge needs the main kernel
