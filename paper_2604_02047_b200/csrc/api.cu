@@ -334,25 +334,42 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
     // rows 256 (6, 1) 15.6 -> 15.2.   With the log-sum-exp:  32 heads, 80 rows 256 (5, 1) 16.1 -> 15.8, 512 (5, 2) 17.8 -> 16.4;
     // 40 heads, 128 rows 256 (6, 1) 18.1 -> 18.8, 512 (6, 2) 19.3 -> 19.8, 768 (6, 3) 20.5 -> 20.4, 1k (6, 3) 21.2 -> 20.3;
     // 32 heads, 128 rows 2k (8, 5) 22.7 -> 23.3;   16 heads, 64 rows of 128256 329 (6, 1) 22.8 -> 21.8.
-    int topk_ctas = 0;
-    bool may_cluster = true;
-    const int topk_items = goose::topk_items(S * B, V);
+    int topk_ctas = 0, cluster = 1;
+    const int topk_items = goose::topk_items(S * B, V), chunks = goose::topk_chunks(V);
     const int kind = harvest || topk_items > c->num_sms ? 2 : 1;
     if (S > 0 && !attn_done) {
-        const int g = H / Hkv, nb = B * g <= 128 ? B : 128 / g;
-        const int n = goose::attn_cluster(c, S, B, H, Hkv, kv_rows, kind);
-        if (n > 1) {
-            const int64_t tiles = ((kv_rows + 127) / 128 + n - 1) / n;       // of a CTA
-            const int beside = harvest && topk_items <= c->num_sms && tiles < 4 ? 3 + (int)tiles : 7;
-            // a few SMs stay free for the step's last launch: its CTAs fit beside neither kernel, and its loads ahead of
-            // the wait would start only when the attention ends (none, 2, 4, 8 free SMs, us: 32 heads, 80 rows 2k 18.3, 18.0, 17.9,
-            // 18.0 and with the harvest 18.1, 17.8, 17.8, 20.1;  52 heads 2k with the harvest 24.9, 24.0, 23.9, 24.0; beside a
-            // shorter attention the round of items that they cost the top-k shows: 32 heads, 80 rows 512 keys with the harvest 15.0,
-            // 16.4, 16.4, 19.8)
-            topk_ctas = c->num_sms - (B + nb - 1) / nb * Hkv * n - 4;
-            may_cluster = topk_ctas > 0 && topk_items <= beside * topk_ctas;
-            if (!may_cluster) topk_ctas = 0;
+        // a few SMs stay free for the step's last launch: its CTAs fit beside neither kernel, and its loads ahead of
+        // the wait would start only when the attention ends (none, 2, 4, 8 free SMs, us: 32 heads, 80 rows 2k 18.3, 18.0, 17.9,
+        // 18.0 and with the harvest 18.1, 17.8, 17.8, 20.1;  52 heads 2k with the harvest 24.9, 24.0, 23.9, 24.0; beside a
+        // shorter attention the round of items that they cost the top-k shows: 32 heads, 80 rows 512 keys with the harvest 15.0,
+        // 16.4, 16.4, 19.8)
+        auto left = [&](int n) { return c->num_sms - goose::attn_heads(B, H, Hkv) * n - 4; };
+        auto tiles = [&](int n) { return (int)(((kv_rows + 127) / 128 + n - 1) / n); };      // of a CTA
+        auto beside = [&](int n) {
+            const int most = harvest && topk_items <= c->num_sms && tiles(n) < 4 ? 3 + tiles(n) : 7;
+            return left(n) > 0 && topk_items <= most * left(n);
+        };
+        if (kind == 1) {
+            const int n = goose::attn_cluster(c, S, B, H, Hkv, kv_rows, kind);
+            if (n > 1 && beside(n)) cluster = n;
+        } else {
+            // Larger clusters end the attention earlier and the top-k later.  The step's end, by either, in us (fitted to the steps
+            // below; 3.7 and 1.5: rows spread over CTAs), decides.  Largest cluster that the device holds -> this, us:  32 over 8
+            // heads, 60 rows of 128256 with the harvest 1k 20.1 -> 14.8, 3k 20.6 -> 18.1 (6 -> 5 CTAs a head), 6k 21.4 (6 stays), without
+            // 1k 15.8 -> 14.0, 3k 16.7 (6 stays);  80 rows of 32000 with the harvest 3k 19.5 (persistent) -> 18.5;  16 over 2, 128
+            // rows of 128256 3k 26.5 (persistent) -> 22.9;  32 heads, 128 rows of 32000 2k 21.2 (persistent) -> 19.8.
+            double best = 1e30;
+            for (int n = 2; n <= goose::kMaxCluster; ++n) {
+                if (!goose::attn_cluster_fits(c, n, S, B, H, Hkv, kv_rows, kind) || !beside(n)) continue;
+                const int q = goose::topk_share(topk_items, chunks, left(n), harvest);
+                const bool spread = q % chunks != 0;
+                const double attn_end = 11.0 + 1.25 * tiles(n);
+                const double topk_end = harvest ? 7.3 + 1.8 * q + (spread ? 3.7 : 0) : 11.0 + 0.75 * q + (spread ? 1.5 : 0);
+                const double end = attn_end > topk_end ? attn_end : topk_end;
+                if (end <= best) { best = end; cluster = n; }
+            }
         }
+        if (cluster > 1) topk_ctas = left(cluster);
     }
     if (!(scale > 0.f) || !(scale < 1e30f)) return GOOSE_EINVAL;
     {
@@ -364,7 +381,7 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
             cudaError_t ea = goose::launch_tree_attn_umma(c, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_cache,
                                                           (const __nv_bfloat16*)v_cache, kv_rows, row_off, ctx_len, parent,
                                                           n_nodes, S, B, H, Hkv, scale, (__nv_bfloat16*)out, lse,
-                                                          static_cast<cudaStream_t>(stream), &merge_plan, may_cluster, kind);
+                                                          static_cast<cudaStream_t>(stream), &merge_plan, cluster, kind);
             if (ea != cudaSuccess) return cuda_fail(ea);
         } else {
             topk_ctas = 0;

@@ -157,6 +157,8 @@ struct HarvestTable {
     float* adj_scores;
 };
 
+constexpr int kMaxCluster = 8;        // the portable limit
+
 // launchers (each returns a cudaError_t from the launch)
 // max_ctas (0: one per SM): the largest grid
 // inputs_ready: everything in front of the kernel that precedes this one in the stream is complete when this one can
@@ -169,6 +171,8 @@ cudaError_t launch_node_topk(goose_ctx* c, const __nv_bfloat16* logits, int rows
                              HarvestTable table = {});
 // items of that kernel's work list: chunks of rows
 int topk_items(int rows, int V);
+int topk_chunks(int V);                                    // of a row
+int topk_share(int items, int chunks, int ctas, bool lse);   // items a CTA gets
 cudaError_t launch_accept(goose_ctx* c, const int32_t* draft_tok, const int32_t* parent, const int32_t* n_nodes,
                           const int32_t* argmax, int S, int B, int32_t* path, int32_t* accept_len, int32_t* bonus,
                           cudaStream_t st);
@@ -191,9 +195,12 @@ cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __
                                   const __nv_bfloat16* vc, int64_t kv_rows, const int64_t* row_off,
                                   const int32_t* ctx_len, const int32_t* parent, const int32_t* n_nodes, int S, int B, int H,
                                   int Hkv, float scale, __nv_bfloat16* out, float* lse, cudaStream_t st,
-                                  struct CombinePlan* defer_merge = nullptr, bool may_cluster = true, int step = 0);
-// CTAs a head of the cluster form of that kernel has for these sizes (1: the persistent form); step: 0 = the attention
-// alone, 1 = in a step, 2 = in a step whose top-k is long (more than an item an SM, or with the log-sum-exp)
+                                  struct CombinePlan* defer_merge = nullptr, int cluster = 0, int step = 0);
+// cluster: CTAs a head, 1: the persistent form, 0: the kernel's own choice, which is
+// attn_cluster(): step: 0 = the attention alone, 1 = in a step, 2 = in a step whose top-k is long (more than an item an SM, or with
+// the log-sum-exp).  There the caller weighs the sizes that attn_cluster_fits() allows against the SMs they leave to the top-k.
+int attn_heads(int B, int H, int Hkv);                     // heads of the work list of a sequence
+bool attn_cluster_fits(const goose_ctx* c, int n, int S, int B, int H, int Hkv, int64_t kv_rows, int step);
 int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int step);
 
 cudaError_t launch_bounded_wait_selftest(goose_ctx* c, long long limit_cycles, int32_t* result, cudaStream_t st);
@@ -205,7 +212,6 @@ int mma_splits(const goose_ctx* c, int S, int H);
 cudaError_t init_mma_kernel();
 cudaError_t init_umma_kernel(goose_ctx* c);
 cudaError_t init_topk_kernel();
-constexpr int kMaxCluster = 8;        // the portable limit
 inline cudaError_t init_kernels(goose_ctx* c) {
     cudaError_t e = init_mma_kernel();
     if (e == cudaSuccess) e = init_umma_kernel(c);

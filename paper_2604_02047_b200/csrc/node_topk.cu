@@ -30,6 +30,7 @@
 // spinning).  Every mbarrier wait is bounded: when one runs out the CTA reports GOOSE_ST_TIMEOUT, drains its own copies in
 // flight (bounded again) and returns.
 #include <mutex>
+#include <type_traits>
 
 #include "goose_internal.cuh"
 
@@ -145,18 +146,20 @@ struct RowCursor {
 }  // namespace
 
 // LSE = true additionally returns the row's log-sum-exp (for the softmax scores of the harvest): the data warps sum
-// exp(x - chunk max) over every element, chunks are merged like split softmax partials.  With a table (TABLE: LSE without counts) the
+// exp(x - chunk max) over every element, chunks are merged like split softmax partials.  With a table (LSE without counts) the
 // control warp also writes the row's ids and scores there, unless a later row has the same token: a scan of the later tokens, no
 // atomics, by a warp of its own beside the item's stream.  1500 x 32000, a kernel behind this one -> here 26.1 -> 25.4 us (in the control
 // warp, whose time the next copy waits for: 28.7).
 // COUNTS = false is the instantiation for n_nodes == NULL (the item list is known before the dependency wait)
-template <bool LSE, bool COUNTS, bool TABLE>
-__global__ void __launch_bounds__(kTopkThreads + (TABLE ? 32 : 0), 1)
+struct NoTable {};
+template <bool LSE, bool COUNTS, class Table>
+__global__ void __launch_bounds__(kTopkThreads + (std::is_same_v<Table, NoTable> ? 0 : 32), 1)
 node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V, int64_t ldl, int k, int chunks,
                  int chunk_elems, u64* __restrict__ ws_cand, int32_t* __restrict__ row_counters,
                  int32_t* __restrict__ argmax, int32_t* __restrict__ ids, float* __restrict__ vals,
                  float* __restrict__ row_lse, float2* __restrict__ ws_lse, int32_t* __restrict__ status,
-                 int inputs_ready, const int32_t* __restrict__ n_nodes, int S, int B, const HarvestTable table) {
+                 int inputs_ready, const int32_t* __restrict__ n_nodes, int S, int B, const Table table) {
+    constexpr bool TABLE = !std::is_same_v<Table, NoTable>;
     extern __shared__ __align__(128) unsigned char s_stage[];   // kTopkStages x 64 KB, then the candidate lists
     __shared__ u64 s_full[kTopkStages];                  // the stage holds its item
     __shared__ u64 s_max_done[kTopkSlots], s_list_done[kTopkSlots];
@@ -469,7 +472,7 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
         return;
     }
 
-    if (TABLE && warp > kTopkControlWarp) {
+    if constexpr (TABLE) if (warp > kTopkControlWarp) {
         // ================================================================================ table warp
         // which row of the table each item's logits row writes: a scan of the later rows' tokens beside the item's stream (an item's
         // arrival implies that its slot's last user is finished)
@@ -504,11 +507,13 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
     float run_m = -INFINITY, run_s = 0.f;
     bool part_starts_row = false;
 
-    auto write_table = [&](int p, int32_t id, float val, float lse) {   // of the item in slot p
-        if (!TABLE || lane >= k || s_table_row[p] < 0) return;
-        const int table_row = s_table_row[p];
-        table.adj_ids[(size_t)table_row * k + lane] = id;
-        table.adj_scores[(size_t)table_row * k + lane] = expf(val - lse);
+    auto write_table = [&](int p, int32_t id, float val, float lse) {   // of the item in slot p, by the lanes below k
+        if constexpr (TABLE) {
+            const int at = s_table_row[p];
+            if (at < 0) return;
+            table.adj_ids[(size_t)at * k + lane] = id;
+            table.adj_scores[(size_t)at * k + lane] = expf(val - lse);
+        }
     };
 
     // rank the candidates of item i, merge them into the row's list, write what is complete
@@ -561,17 +566,14 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
             for (int o = 16; o > 0; o >>= 1) csum += __shfl_xor_sync(0xFFFFFFFFu, csum, o);
         }
         if (chunks == 1) {                               // the chunk is the row: write it out
-            const int32_t id = (int32_t)(0xFFFFu - (mine & 0xFFFFu));
             if (lane < k) {
+                const int32_t id = (int32_t)(0xFFFFu - (mine & 0xFFFFu));
                 ids[out_row * k + lane] = id;
                 if (vals) vals[out_row * k + lane] = value_of_sortable16(mine >> 16);
                 if (lane == 0) argmax[out_row] = id;
+                if constexpr (TABLE) write_table(p, id, value_of_sortable16(mine >> 16), cmax + logf(csum));
             }
-            if (LSE && (TABLE || lane == 0)) {
-                const float lse = cmax + logf(csum);
-                if (lane == 0) row_lse[out_row] = lse;
-                write_table(p, id, value_of_sortable16(mine >> 16), lse);
-            }
+            if (LSE && lane == 0) row_lse[out_row] = cmax + logf(csum);
             return;
         }
         const bool part_begins = (i == 0) || (chunk == 0);
@@ -669,16 +671,16 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
                 fin_m = M; fin_s = sum;
             }
         }
-        const int32_t id = (int32_t)(0xFFFFFFFFu - (uint32_t)(win & 0xFFFFFFFFull));
         if (lane < k) {
+            const int32_t id = (int32_t)(0xFFFFFFFFu - (uint32_t)(win & 0xFFFFFFFFull));
             ids[out_row * k + lane] = id;
             if (vals) vals[out_row * k + lane] = value_of_sortable16((uint32_t)(win >> 32));
             if (lane == 0) argmax[out_row] = id;
         }
         if (LSE && lane == 0) row_lse[out_row] = fin_m + logf(fin_s);
-        if (TABLE) {                                     // (parts of several CTAs: lane 0 merged them)
+        if constexpr (TABLE) {                           // (parts of several CTAs: lane 0 merged them)
             const float lse = __shfl_sync(0xFFFFFFFFu, fin_m + logf(fin_s), 0);
-            write_table(p, id, value_of_sortable16((uint32_t)(win >> 32)), lse);
+            if (lane < k) write_table(p, (int32_t)(0xFFFFFFFFu - (uint32_t)(win & 0xFFFFFFFFull)), value_of_sortable16((uint32_t)(win >> 32)), lse);
         }
     };
 
@@ -705,6 +707,17 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
     if (wait_at_end) pdl_wait();
 }
 
+// A row that is spread over CTAs costs a merge behind its last part, more than an item does: where one item more a CTA gives every
+// row to one CTA, that is the better share.  Top-k / harvest, us, without -> with:  4 chunks (V = 128256): 100 rows (q = 3 -> 4) 9.8 ->
+// 8.6 / 13.5 -> 12.1, 250 rows (7 -> 8) 16.6 -> 15.1 / 22.2 -> 20.8;  2 chunks (65536): 60 rows (1 -> 2) 6.0 -> 5.1, 150 rows (3 -> 4)
+// 8.6 -> 7.9, 900 rows (13 -> 14) 23.9 -> 22.7 / 33.5 -> 31.8;  7 chunks (200000): 122 rows (6 -> 7) 15.5 -> 13.8 / 20.7 -> 19.1.  Two
+// items more are even (4 chunks: 60 rows, 200 rows) or worse (30 rows 6.3 -> 7.7, 150 rows (5 -> 8) 18.2 -> 19.7), and so is a second
+// item with the log-sum-exp (cycle of 32 over 8 heads, 32 rows of 65536 12.4 -> 12.8).
+int topk_share(int items, int chunks, int ctas, bool lse) {
+    const int q = (items + ctas - 1) / ctas;
+    return chunks > 1 && (q + 1) % chunks == 0 && (q > 1 || !lse) ? q + 1 : q;
+}
+int topk_chunks(int V) { return (V + kTopkChunk - 1) / kTopkChunk; }
 int topk_items(int rows, int V) { return rows * ((V + kTopkChunk - 1) / kTopkChunk); }
 
 namespace {
@@ -719,12 +732,14 @@ cudaError_t launch_topk_any(int num_sms, cudaStream_t st, const __nv_bfloat16* l
     const int items = rows * chunks;                 // (a row costs the context 1 KB of scratch a chunk: far below 2^31)
     // every CTA gets q = ceil(items / SMs) items or one fewer; using the fewest CTAs that q allows loses no time and
     // makes the ranges fall on row boundaries when q is a multiple of the chunks per row (no cross-CTA merges then)
-    const int q = (items + num_sms - 1) / num_sms, grid = (items + q - 1) / q;
-    auto kernel = table.adj_ids ? node_topk_kernel<true, false, true>
-                : row_lse ? (n_nodes ? node_topk_kernel<true, true, false> : node_topk_kernel<true, false, false>)
-                          : (n_nodes ? node_topk_kernel<false, true, false> : node_topk_kernel<false, false, false>);
-    return launch_pdl(kernel, dim3(grid), dim3(kTopkThreads + (table.adj_ids ? 32 : 0)), kTopkSmem, st, logits, items, V, ldl, k, chunks, chunk_elems, ws,
-                      counters, argmax, ids, vals, row_lse, ws_lse, status, inputs_ready, n_nodes, S, B, table);
+    const int q = topk_share(items, chunks, num_sms, row_lse != nullptr), grid = (items + q - 1) / q;
+    auto launch = [&](auto kernel, int threads, auto with) {
+        return launch_pdl(kernel, dim3(grid), dim3(threads), kTopkSmem, st, logits, items, V, ldl, k, chunks, chunk_elems, ws, counters,
+                          argmax, ids, vals, row_lse, ws_lse, status, inputs_ready, n_nodes, S, B, with);
+    };
+    if (table.adj_ids) return launch(node_topk_kernel<true, false, HarvestTable>, kTopkThreads + 32, table);
+    return launch(row_lse ? (n_nodes ? node_topk_kernel<true, true, NoTable> : node_topk_kernel<true, false, NoTable>)
+                          : (n_nodes ? node_topk_kernel<false, true, NoTable> : node_topk_kernel<false, false, NoTable>), kTopkThreads, NoTable{});
 }
 }  // namespace
 
@@ -735,9 +750,9 @@ cudaError_t init_topk_kernel() {
     auto opt_in = [&](const void* fn) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopkSmem);
     };
-    opt_in((const void*)node_topk_kernel<false, false, false>);  opt_in((const void*)node_topk_kernel<false, true, false>);
-    opt_in((const void*)node_topk_kernel<true, false, false>);   opt_in((const void*)node_topk_kernel<true, true, false>);
-    opt_in((const void*)node_topk_kernel<true, false, true>);
+    opt_in((const void*)node_topk_kernel<false, false, NoTable>);  opt_in((const void*)node_topk_kernel<false, true, NoTable>);
+    opt_in((const void*)node_topk_kernel<true, false, NoTable>);   opt_in((const void*)node_topk_kernel<true, true, NoTable>);
+    opt_in((const void*)node_topk_kernel<true, false, HarvestTable>);
     return e;
 }
 

@@ -891,7 +891,8 @@ int auto_attn_impl(const goose_ctx* c, int S, int B, int H) {
     return c->encode_tiled ? GOOSE_ATTN_UMMA : GOOSE_ATTN_MMA;
 }
 
-// One sequence: a cluster per head, the largest (of at most 8 CTAs) that the device holds one of per head at once -- where
+// One sequence: a cluster per head, the largest (of at most 8 CTAs) that the device holds one of per head at once (in a step with a
+// long top-k a smaller one where that ends both earlier: see enqueue_step()) -- where
 // the SMs that this leaves out cost less than the merge kernel and the second segments that it saves.  What they cost grows
 // with lost = tiles / n - heads * tiles / SMs, the tiles that the longest CTA has more than an equal share; what is saved
 // depends on what else the launches do, so there are three kinds of call.  ctx_len[] is device data: the tiles are bounded
@@ -917,25 +918,33 @@ int auto_attn_impl(const goose_ctx* c, int S, int B, int H) {
 //   12k (10.8) 28.4 -> 20.9 / 26.8 -> 25.0 / 28.4 -> 24.8, 16k (14.4) 28.7 -> 25.3 / 27.8 -> 29.4 / 29.1 -> 29.6: 10, and one head has more to win
 //   4 heads, tree of 60  2k (1.7) 17.3 -> 10.3 / 18.6 -> 13.9 / 21.6 -> 14.0, 6k (4.8) 19.7 -> 14.9 / 20.8 -> 18.5 / 22.2 -> 18.7,
 //   8k (6.4) 19.8 -> 17.1 / 21.8 -> 20.8 / 23.0 -> 21.0, 10k (7.7) 20.6 -> 18.8 / 21.7 -> 22.4 / 23.0 -> 22.4: 6
-int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int step) {
-    if (S != 1) return 1;                               // (several may differ in length by any factor)
-    const int g = H / Hkv, nb = B * g <= kTile ? B : kTile / g, Hw = (B + nb - 1) / nb * Hkv;
-    int n = 1;
-    for (int i = 2; i <= kMaxCluster; ++i)
-        if (c->max_clusters[i] >= Hw && Hw * i <= c->num_sms) n = i;
-    if (n == 1 || (n == 2 && step != 2)) return 1;
+int attn_heads(int B, int H, int Hkv) {
+    const int g = H / Hkv, nb = B * g <= kTile ? B : kTile / g;
+    return (B + nb - 1) / nb * Hkv;
+}
+bool attn_cluster_fits(const goose_ctx* c, int n, int S, int B, int H, int Hkv, int64_t kv_rows, int step) {
+    const int Hw = attn_heads(B, H, Hkv);
+    if (S != 1 || n < 2 || n > kMaxCluster) return false;   // (several may differ in length by any factor)
+    if (c->max_clusters[n] < Hw || Hw * n > c->num_sms || (n == 2 && step != 2)) return false;
     const int64_t tiles = (kv_rows + kTile - 1) / kTile;
     int line = n == 2 ? 30 : Hw <= 2 ? 100 : Hw <= 4 ? 60 : 44;   // tenths of a tile
     if (Hw > Hkv && Hw > 4 && step == 0) line = 35;               // several M tiles a head: K/V come from L2, idle SMs cost their share
     if (step == 1 && Hw > 4) line = n == 3 ? 5 : 10 * Hw * n >= 7 * c->num_sms ? 15 : 35;
-    return tiles * (c->num_sms - Hw * n) * 10 <= (int64_t)line * n * c->num_sms ? n : 1;
+    return tiles * (c->num_sms - Hw * n) * 10 <= (int64_t)line * n * c->num_sms;
+}
+int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int step) {
+    const int Hw = attn_heads(B, H, Hkv);
+    int n = 1;
+    for (int i = 2; i <= kMaxCluster; ++i)
+        if (c->max_clusters[i] >= Hw && Hw * i <= c->num_sms) n = i;
+    return attn_cluster_fits(c, n, S, B, H, Hkv, kv_rows, step) ? n : 1;
 }
 
 cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __nv_bfloat16* kc,
                                   const __nv_bfloat16* vc, int64_t kv_rows, const int64_t* row_off,
                                   const int32_t* ctx_len, const int32_t* parent, const int32_t* n_nodes, int S, int B, int H,
                                   int Hkv, float scale, __nv_bfloat16* out, float* lse, cudaStream_t st,
-                                  CombinePlan* defer_merge, bool may_cluster, int step) {
+                                  CombinePlan* defer_merge, int cluster, int step) {
     if (defer_merge) defer_merge->valid = false;
     if (!c->encode_tiled) return cudaErrorNotSupported;
     if (S == 0) return cudaSuccess;
@@ -948,7 +957,7 @@ cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __
         !make_map(c->encode_tiled, &mv, vc, kv_rows, Hkv, kTile))
         return cudaErrorInvalidValue;
     const int Hw = n_mt * Hkv;
-    const int cluster = may_cluster ? attn_cluster(c, S, B, H, Hkv, kv_rows, step) : 1;
+    if (cluster == 0) cluster = attn_cluster(c, S, B, H, Hkv, kv_rows, step);
     int grid = cluster > 1 ? Hw * cluster : c->num_sms;
     if (2 * grid > c->n_slots) grid = c->n_slots / 2;
     const int divisor = cluster > 1 ? cluster : grid;   // the one that the form needs on the device
