@@ -360,9 +360,9 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     const int64_t my_row = lane < S ? row_off[lane] : 0;
     // The first copies leave at once, for the place that was found ahead of the wait: what they read is final now, only the place may
     // not be.  The lengths, counts and rows come in meanwhile; where one differs, the copies are waited for and their barriers set up
-    // again, as if nothing had been asked for.  The multi-head persistent form alone: step of 40 heads 4k 24.8 -> 24.3, 2 x 32 heads
-    // 30.8 -> 30.2, 52 heads 8k 51.6 -> 50.7 us.  In clusters the call gains (1531 keys 11.45 -> 11.1) but the step loses (512 11.4 ->
-    // 11.6, 2k 16.65 -> 16.85), grouped heads lose 0.3 a call.
+    // again, as if nothing had been asked for.  The multi-head persistent form alone: step of 40 heads 4k 24.8 -> 24.3, 2 x 32 heads 30.8 -> 30.2, 52 heads 8k 51.6 ->
+    // 50.7 us.  In clusters the call gains (1531 keys 11.45 -> 11.1) but the step loses (512 11.4 -> 11.6, 2k 16.65 -> 16.85), grouped
+    // heads lose 0.3 a call.
     if (kAhead && warp == 0) {
         const bool ahead = placed && first >= 0;
         const int ctx_now = ahead && lane < S ? ctx_len[lane] : 0, nn_now = kCounts && ahead && lane < S ? n_nodes[lane] : 0;
