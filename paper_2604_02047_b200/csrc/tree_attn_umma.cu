@@ -62,7 +62,6 @@ struct Header {                                  // lives at the start of dynami
     unsigned long long group_bar;                // barrier of the 128 softmax threads (bounded, unlike bar.sync)
     uint32_t tmem_base;
     volatile int abort_flag;
-    int early;                                   // first copies ahead of the lengths: 0 = none, 1 = they stand, 2 = they were wrong
     int bad_parent;
     int par[kMaxB];                              // parent[] of the current segment's sequence
 };
@@ -238,7 +237,6 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                       int32_t* __restrict__ status,
                       __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
     if (!kCounts) n_nodes = nullptr;
-    constexpr bool kAhead = !kGrouped && !kCluster;     // first copies ahead of the lengths: see there
 
     const int Hkv = kGrouped ? Hkv_arg : H, g = kGrouped ? g_arg : 1, nb = kGrouped ? nb_arg : B;
     extern __shared__ unsigned char smem_raw[];
@@ -316,38 +314,22 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     // sequences 85.5 -> 84.5.  Grouped-query heads look again: with the place kept, call of 4 x 32 over 8 35.4 -> 35.7, 2 x 32 over 8
     // 17.0 -> 17.6, one sequence in clusters 12.10 -> 12.01 and its cycle 20.6 -> 20.7.
     int early_ctx = 0, early_nn = 0;
-    int64_t early_row = 0, first = -1;                  // of sequence `lane`; of the CTA's first, -1: outside the cache
     bool placed = false;
     if (S <= 32 && (!kGrouped || warp == 2)) {
         const bool mine = lane < S;
         early_nn = !mine ? 0 : kCounts ? load_early(n_nodes + lane) : B;
         early_ctx = mine ? load_early(ctx_len + lane) : 0;
-        if (mine && (warp == 2 || (kAhead && warp == 0))) early_row = load_early(row_off + lane);
+        const int64_t row0 = warp == 2 && mine ? load_early(row_off + lane) : 0;
         const int tiles = early_nn > 0 && early_nn <= B ? wk.tiles_of(early_ctx, early_nn) : 0;
         wk.init_lanes(tiles, tiles > 0);
         placed = kCluster || wk.small;                  // (a longer list is walked through lengths in memory: not yet)
         if (placed) locate(tiles, lane);
-        if ((warp == 2 || (kAhead && warp == 0)) && placed && w_begin < w_end) {
-            first = __shfl_sync(0xFFFFFFFFu, early_row, cu.s);
-            const int64_t row = min(first, kv_rows) + (int64_t)cu.t * kTile;
-            if (first < 0 || row >= kv_rows) first = -1;
-            if (warp == 2 && lane < 4 && first >= 0)
+        if (warp == 2 && placed && w_begin < w_end) {
+            const int64_t first = __shfl_sync(0xFFFFFFFFu, row0, cu.s), row = min(first, kv_rows) + (int64_t)cu.t * kTile;
+            if (lane < 4 && first >= 0 && row < kv_rows)
                 tma_prefetch_3d(lane & 2 ? &tmap_v : &tmap_k, (lane & 1) * 64, kGrouped ? cu.h % Hkv : cu.h, (int)row);
         }
     }
-    // Q of a segment.  box = nb nodes x g heads x 64 dims: lands as rows r = node * g + member (rows past the sequence's last node
-    // hold the next sequence's queries or the zero fill: never written out)
-    auto load_q = [&](int hk, int row, uint32_t qb) {
-        mbar_expect_tx(&hd->q_full[qb], (uint32_t)(nb * g) * 256u);
-        tma_load_4d(q_smem + qb * kQBytes, &tmap_q, &hd->q_full[qb], 0, 0, hk, row);
-        tma_load_4d(q_smem + qb * kQBytes + kHalfBytes, &tmap_q, &hd->q_full[qb], 64, 0, hk, row);
-    };
-    auto load_kv = [&](const CUtensorMap* mp, uint32_t st, int hk, int krow, unsigned long long pol_stream) {
-        unsigned char* dst = kv_smem + st * kStageBytes;
-        mbar_expect_tx(&hd->kv_full[st], kStageBytes);
-        tma_load_3d_hint(dst, mp, &hd->kv_full[st], 0, hk, krow, pol_stream);
-        tma_load_3d_hint(dst + kHalfBytes, mp, &hd->kv_full[st], 64, hk, krow, pol_stream);
-    };
     // everything above only looked: now wait for the preceding kernel, then let the next
     // one (the combine kernel) get resident early -- it waits for this grid before reading the partials
     pdl_wait();
@@ -356,28 +338,8 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
         for (int s = 0; s < S; ++s)
             if (nodes_bad(n_nodes, s, B)) atomicOr(&status[s], GOOSE_ST_BAD_NODES);
     // where this CTA starts, found by every warp for itself with all lanes; the lengths and the rows of up to 32 sequences
-    // come in one round of loads (lane = sequence)
+    // come in one round of loads (lane = sequence).  The first load of K waits for nothing else.
     const int64_t my_row = lane < S ? row_off[lane] : 0;
-    // The first copies leave at once, for the place that was found ahead of the wait: what they read is final now, only the place may
-    // not be.  The lengths, counts and rows come in meanwhile; where one differs, the copies are waited for and their barriers set up
-    // again, as if nothing had been asked for.  The multi-head persistent form alone: step of 40 heads 4k 24.8 -> 24.3, 2 x 32 heads 30.8 -> 30.2, 52 heads 8k 51.6 ->
-    // 50.7 us.  In clusters the call gains (1531 keys 11.45 -> 11.1) but the step loses (512 11.4 -> 11.6, 2k 16.65 -> 16.85), grouped
-    // heads lose 0.3 a call.
-    if (kAhead && warp == 0) {
-        const bool ahead = placed && first >= 0;
-        const int ctx_now = ahead && lane < S ? ctx_len[lane] : 0, nn_now = kCounts && ahead && lane < S ? n_nodes[lane] : 0;
-        if (ahead && lane == 0) {
-            const int hk = cu.h, krow = (int)(first + (int64_t)cu.t * kTile);
-            const unsigned long long pol_stream = l2_policy_evict_first();
-            load_kv(&tmap_k, 0, hk, krow, pol_stream);
-            load_q(hk, cu.s * B, 0);
-            load_kv(&tmap_v, 1, hk, krow, pol_stream);
-        }
-        __syncwarp();
-        const bool stands = ahead && (lane >= S || (ctx_now == early_ctx && my_row == early_row && (!kCounts || nn_now == early_nn)));
-        const bool all = __all_sync(0xFFFFFFFFu, stands);
-        if (lane == 0) hd->early = !ahead ? 0 : all ? 1 : 2;
-    }
     if (kGrouped) {
         locate(wk.init_warp(lane), lane);
     } else {
@@ -387,26 +349,6 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
     const int first_s = w_begin < w_end ? cu.s : 0;
     const int64_t first_row = __shfl_sync(0xFFFFFFFFu, my_row, first_s & 31);
     auto row_of = [&](int s) -> int64_t { return s == first_s && s < 32 ? first_row : row_off[s]; };
-    if (kAhead) __syncthreads();
-    const int early = kAhead ? hd->early : 0;
-    if (early == 2) {
-        if (threadIdx.x == 0) {
-            mbar_drain(&hd->kv_full[0], 0); mbar_drain(&hd->q_full[0], 0); mbar_drain(&hd->kv_full[1], 0);
-            if (!mbar_try_wait(&hd->kv_full[0], 0) || !mbar_try_wait(&hd->q_full[0], 0) || !mbar_try_wait(&hd->kv_full[1], 0)) {
-                hd->abort_flag = 1;                     // (a copy that never came: nothing else is started)
-                atomicOr(status, GOOSE_ST_TIMEOUT);
-            } else {
-                unsigned long long* bars[3] = {&hd->kv_full[0], &hd->kv_full[1], &hd->q_full[0]};
-                for (int i = 0; i < 3; ++i) {
-                    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bars[i])) : "memory");
-                    mbar_init(bars[i], 1);
-                }
-                asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            }
-        }
-        __syncthreads();
-        if (hd->abort_flag) w_end = w_begin;
-    }
 
 
     if (w_begin < w_end) {
@@ -416,26 +358,32 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
                 // K and V are read exactly once: mark them evict-first so that the split-KV partials
                 // (written and re-read within this launch) stay resident in L2
                 const unsigned long long pol_stream = l2_policy_evict_first();
-                uint32_t ring = early == 1 ? 2 : 0, st = ring, phase = 0, seg = 0;   // copies issued; the stage of the next and its phase
+                uint32_t ring = 0, st = 0, phase = 0, seg = 0;   // copies issued; the stage of the next and its phase
                 bool ok = true;
                 while (ok && cu.w < w_end) {
                     const int64_t row0 = row_of(cu.s);
-                    const bool begun = kAhead && seg == 0 && early == 1;   // Q and the first tile are on their way
+                    // Q of this segment
                     const uint32_t qb = seg & 1;           // seg = index of this segment
+                    ok = mbar_wait(hd, &hd->q_empty[qb], ((seg >> 1) & 1) ^ 1, status);
+                    if (!ok) break;
+                    // box = nb nodes x g heads x 64 dims: lands as rows r = node * g + member (rows past the
+                    // sequence's last node hold the next sequence's queries or the zero fill: never written out)
                     const int mt = kGrouped ? cu.h / Hkv : 0, hk = cu.h - mt * Hkv;
-                    if (!begun) {
-                        ok = mbar_wait(hd, &hd->q_empty[qb], ((seg >> 1) & 1) ^ 1, status);
-                        if (!ok) break;
-                        load_q(hk, cu.s * B + mt * nb, qb);
-                    }
+                    mbar_expect_tx(&hd->q_full[qb], (uint32_t)(nb * g) * 256u);
+                    tma_load_4d(q_smem + qb * kQBytes, &tmap_q, &hd->q_full[qb], 0, 0, hk, cu.s * B + mt * nb);
+                    tma_load_4d(q_smem + qb * kQBytes + kHalfBytes, &tmap_q, &hd->q_full[qb], 64, 0, hk, cu.s * B + mt * nb);
                     ++seg;                                 // segments whose Q load has been issued
                     const int n = cu.run(w_end);
-                    int krow = (int)(row0 + (int64_t)(cu.t + begun) * kTile);
-                    for (int i = begun; i < n && ok; ++i, krow += kTile) {
+                    int krow = (int)(row0 + (int64_t)cu.t * kTile);
+                    for (int i = 0; i < n && ok; ++i, krow += kTile) {
                         for (int kv = 0; kv < 2 && ok; ++kv) {
                             ok = mbar_wait(hd, &hd->kv_empty[st], phase ^ 1, status);
                             if (!ok) break;
-                            load_kv(kv ? &tmap_v : &tmap_k, st, hk, krow, pol_stream);
+                            unsigned char* dst = kv_smem + st * kStageBytes;
+                            mbar_expect_tx(&hd->kv_full[st], kStageBytes);
+                            const CUtensorMap* mp = kv ? &tmap_v : &tmap_k;
+                            tma_load_3d_hint(dst, mp, &hd->kv_full[st], 0, hk, krow, pol_stream);
+                            tma_load_3d_hint(dst + kHalfBytes, mp, &hd->kv_full[st], 64, hk, krow, pol_stream);
                             ++ring;
                             if (++st == kStages) { st = 0; phase ^= 1; }
                         }
