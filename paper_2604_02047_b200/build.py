@@ -15,7 +15,7 @@ LIB = os.path.join(HERE, "libgoose.so")
 # named for the interpreter whose ABI it has: another one does not import it
 MARSHAL = os.path.join(HERE, "_marshal" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 MARSHAL_SOURCE = "marshal.cpp"
-SOURCES = ["api.cu", "node_topk.cu", "accept.cu", "kv_compact.cu", "tree_attn_mma.cu",
+SOURCES = ["api.cu", "node_topk.cu", "harvest.cu", "accept.cu", "kv_compact.cu", "tree_attn_mma.cu",
            "tree_attn_umma.cu", "spine_tree.cpp"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
               "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]

@@ -209,9 +209,11 @@ int goose_harvest(goose_ctx* c, const void* logits, int rows, int V, int64_t ldl
     if (V < 1 || V > GOOSE_MAX_V || ldl < V || (ldl & 7) != 0 || !aligned16(logits)) return GOOSE_EINVAL;
     if (k < 1 || k > GOOSE_MAX_K || k > V) return GOOSE_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const goose::HarvestTable table{row_tok, table_rows, adj_ids, adj_scores};
+    const bool scatter = rows > goose::kTableRows;
     cudaError_t e = goose::launch_node_topk(c, (const __nv_bfloat16*)logits, rows, V, ldl, k, argmax, topk_ids,
-                                            topk_vals, row_lse, st, false, nullptr, 0, 0,
-                                            goose::HarvestTable{row_tok, table_rows, adj_ids, adj_scores});
+                                            topk_vals, row_lse, st, false, nullptr, 0, 0, scatter ? goose::HarvestTable{} : table);
+    if (e == cudaSuccess && scatter) e = goose::launch_harvest_scatter(c, table, rows, k, topk_ids, topk_vals, row_lse, st);
     if (e != cudaSuccess) return cuda_fail(e);
     return GOOSE_OK;
 }

@@ -157,13 +157,21 @@ struct HarvestTable {
     float* adj_scores;
 };
 
+// Up to this many rows the top-k kernel writes the table, above it a scatter kernel behind it: the scan for later rows with a row's
+// token grows with the rows, and in the top-k kernel one warp of an SM has it for all of the SM's rows, one after the other.  Beyond what
+// hides beside the stream of a row the whole kernel waits for it.  Harvest, us, scatter kernel -> here (distinct tokens, the longest
+// scans):  V = 32000: 600 rows 15.5 -> 14.4, 1500 26.0 -> 25.4, 2048 31.3 -> 31.6, 2500 36.8 -> 39.3, 4000 57 -> 83, 8000 108 -> 470;
+// V = 65536: 1000 34.2 -> 31.8, 1500 48.5 -> 46.1, 2048 57.8 -> 57.5, 6000 159 -> 282;  V = 128256: 1500 82.3 -> 82.5, 2048 105.3 ->
+// 106.3, 8000 407 -> 642.
+constexpr int kTableRows = 1536;
+
 constexpr int kMaxCluster = 8;        // the portable limit
 
 // launchers (each returns a cudaError_t from the launch)
 // max_ctas (0: one per SM): the largest grid
 // inputs_ready: everything in front of the kernel that precedes this one in the stream is complete when this one can
 // start, and that kernel has nothing to do with this one's inputs and outputs (see the kernel)
-// table (with row_lse, without n_nodes): the harvest of every row
+// table (with row_lse, without n_nodes, at most kTableRows rows): the harvest of every row
 // n_nodes (may be NULL) with B: row r = s * B + i exists iff i < n_nodes[s]; other rows are neither read nor written
 cudaError_t launch_node_topk(goose_ctx* c, const __nv_bfloat16* logits, int rows, int V, int64_t ldl, int k,
                              int32_t* argmax, int32_t* ids, float* vals, float* row_lse, cudaStream_t st,
@@ -173,6 +181,9 @@ cudaError_t launch_node_topk(goose_ctx* c, const __nv_bfloat16* logits, int rows
 int topk_items(int rows, int V);
 int topk_chunks(int V);                                    // of a row
 int topk_share(int items, int chunks, int ctas, bool lse);   // items a CTA gets
+// a harvest of more than kTableRows rows: the table, out of the top-k kernel's results
+cudaError_t launch_harvest_scatter(goose_ctx* c, const HarvestTable& table, int rows, int k, const int32_t* ids, const float* vals,
+                                   const float* row_lse, cudaStream_t st);
 cudaError_t launch_accept(goose_ctx* c, const int32_t* draft_tok, const int32_t* parent, const int32_t* n_nodes,
                           const int32_t* argmax, int S, int B, int32_t* path, int32_t* accept_len, int32_t* bonus,
                           cudaStream_t st);

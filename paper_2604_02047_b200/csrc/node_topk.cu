@@ -54,6 +54,7 @@ constexpr int kTopkSlots = 4;
 // elements > T', 64 each, and of the elements equal to T' every collector takes at most k
 constexpr int kTopkQuickList = 128;
 constexpr int kTopkListCap = kMaxK * kTopkPerThread + kTopkCollectWarps * kMaxK + (kTopkCollectWarps - 1) * kTopkQuickList;
+constexpr int kTableLoads = 8;                               // tokens a lane has in flight while it looks for a later row
 constexpr int kTopkSmem = kTopkStages * kTopkStageBytes + kTopkSlots * kTopkListCap * 4;   // dynamic shared memory
 constexpr long long kTopkWaitCycles = 2000000000ll;          // bound of every wait: about one second of SM clock
 constexpr float kTopkLog2e = 1.4426950408889634f;
@@ -148,8 +149,9 @@ struct RowCursor {
 // LSE = true additionally returns the row's log-sum-exp (for the softmax scores of the harvest): the data warps sum
 // exp(x - chunk max) over every element, chunks are merged like split softmax partials.  With a table (LSE without counts) the
 // control warp also writes the row's ids and scores there, unless a later row has the same token: a scan of the later tokens, no
-// atomics, by a warp of its own beside the item's stream.  1500 x 32000, a kernel behind this one -> here 26.1 -> 25.4 us (in the control
-// warp, whose time the next copy waits for: 28.7).
+// atomics, by a warp of its own beside the item's stream.  1500 x 32000, a kernel behind this one -> here 26.0 -> 25.4 us (in the control
+// warp, whose time the next copy waits for: 28.7); 16 tokens a lane in flight instead of 8: 2048 x 32000 31.5 -> 31.3, but
+// 1500 x 128256 82.5 -> 84.8.
 // COUNTS = false is the instantiation for n_nodes == NULL (the item list is known before the dependency wait)
 struct NoTable {};
 template <bool LSE, bool COUNTS, class Table>
@@ -474,25 +476,33 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
 
     if constexpr (TABLE) if (warp > kTopkControlWarp) {
         // ================================================================================ table warp
-        // which row of the table each item's logits row writes: a scan of the later rows' tokens beside the item's stream (an item's
-        // arrival implies that its slot's last user is finished)
+        // which row of the table an item's logits row writes: a scan of the later rows' tokens beside the item's stream (an item's
+        // arrival implies that its slot's last user is finished), for the items that end this CTA's part of a row alone -- nobody
+        // reads the others' answer -- and up to the first later row with the token
         const int rows = items_all / chunks;
+        int row = w_begin / chunks, chunk = w_begin - row * chunks;
         for (int j = 0; j < n_local; ++j) {
             if (mbar_wait_bounded(&s_full[j % kTopkStages], (uint32_t)(j / kTopkStages) & 1u, kTopkWaitCycles, &s_abort) != 0) {
                 s_abort = 1;
                 break;
             }
-            const int row = (w_begin + j) / chunks, tok = table.row_tok[row];
-            bool later = tok < 0 || tok >= table.table_rows;
-            if (!later) {
-#pragma unroll 8
-                for (int r = row + 1 + lane; r < rows; r += 32) later |= table.row_tok[r] == tok;
+            int to = -1;
+            if (chunk == chunks - 1 || j == n_local - 1) {
+                const int tok = table.row_tok[row];
+                bool stands = tok >= 0 && tok < table.table_rows;
+                for (int r = row + 1; stands && r < rows; r += 32 * kTableLoads) {
+                    bool later = false;
+#pragma unroll
+                    for (int u = 0; u < kTableLoads; ++u) later |= table.row_tok[min(r + u * 32 + lane, rows - 1)] == tok;
+                    stands = !__any_sync(0xFFFFFFFFu, later);
+                }
+                if (stands) to = tok;
             }
-            later = __any_sync(0xFFFFFFFFu, later);
             if (lane == 0) {
-                s_table_row[j % kTopkSlots] = later ? -1 : tok;
+                s_table_row[j % kTopkSlots] = to;
                 topk_mbar_arrive(&s_list_done[j % kTopkSlots]);
             }
+            if (++chunk == chunks) { chunk = 0; ++row; }
         }
         if (wait_at_end) pdl_wait();
         return;
