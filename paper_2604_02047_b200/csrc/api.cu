@@ -4,6 +4,7 @@
 #include <new>
 
 #include "goose_internal.cuh"
+#include "topk_deal.cuh"
 #include "tree_attn_combine.cuh"
 
 namespace {
@@ -46,9 +47,6 @@ int check_shape(const goose_ctx* c, int S, int B, int H, int D) {
     if (D != GOOSE_HEAD_DIM) return GOOSE_EINVAL;
     return GOOSE_OK;
 }
-
-constexpr int kTopkChunkElems = 32768;
-constexpr int kTopkMaxChunks = GOOSE_MAX_V / kTopkChunkElems;   // 8
 
 }  // namespace
 
@@ -94,7 +92,7 @@ int goose_create(goose_ctx** out, int device, int max_S, int max_B, int max_H, i
     if (slots < 4LL * c->num_sms) slots = 4LL * c->num_sms;
     c->n_slots = (int)slots;
     c->topk_rows_cap = max_S * max_B;
-    c->topk_cand_cap = (int64_t)c->topk_rows_cap * kTopkMaxChunks * GOOSE_MAX_K;
+    c->topk_cand_cap = (int64_t)c->topk_rows_cap * goose::kTopkMaxChunks * GOOSE_MAX_K;
 
     bool ok = true;
     cudaError_t setup_err = cudaSuccess;               // a failure that is not an allocation keeps its own code
@@ -102,7 +100,7 @@ int goose_create(goose_ctx** out, int device, int max_S, int max_B, int max_H, i
     ok = ok && cudaMalloc(&c->head_counters, sizeof(int32_t) * (size_t)heads) == cudaSuccess;
     ok = ok && cudaMalloc(&c->topk_cand, sizeof(unsigned long long) * (size_t)c->topk_cand_cap) == cudaSuccess;
     ok = ok && cudaMalloc(&c->row_counters, sizeof(int32_t) * (size_t)c->topk_rows_cap) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->topk_lse_ws, sizeof(float) * 2 * (size_t)c->topk_rows_cap * kTopkMaxChunks) == cudaSuccess;
+    ok = ok && cudaMalloc(&c->topk_lse_ws, sizeof(float) * 2 * (size_t)c->topk_rows_cap * goose::kTopkMaxChunks) == cudaSuccess;
     ok = ok && cudaMalloc(&c->status, sizeof(int32_t) * (size_t)max_S) == cudaSuccess;
     ok = ok && cudaMalloc(&c->selftest_word, sizeof(int32_t)) == cudaSuccess;
     if (ok) {
@@ -363,8 +361,8 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
             double best = 1e30;
             for (int n = 2; n <= goose::kMaxCluster; ++n) {
                 if (!goose::attn_cluster_fits(c, n, S, B, H, Hkv, kv_rows, kind) || !beside(n)) continue;
-                const int q = goose::topk_share(topk_items, chunks, left(n), harvest);
-                const bool spread = q % chunks != 0;
+                const int q = n_nodes ? (topk_items + left(n) - 1) / left(n) : goose::topk_share(topk_items, chunks, left(n), harvest);
+                const bool spread = n_nodes ? chunks > 1 : q % chunks != 0;
                 const double attn_end = 11.0 + 1.25 * tiles(n);
                 const double topk_end = harvest ? 7.3 + 1.8 * q + (spread ? 3.7 : 0) : 11.0 + 0.75 * q + (spread ? 1.5 : 0);
                 const double end = attn_end > topk_end ? attn_end : topk_end;

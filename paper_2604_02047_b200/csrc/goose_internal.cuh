@@ -177,10 +177,6 @@ cudaError_t launch_node_topk(goose_ctx* c, const __nv_bfloat16* logits, int rows
                              int32_t* argmax, int32_t* ids, float* vals, float* row_lse, cudaStream_t st,
                              bool inputs_ready = false, const int32_t* n_nodes = nullptr, int B = 0, int max_ctas = 0,
                              HarvestTable table = {});
-// items of that kernel's work list: chunks of rows
-int topk_items(int rows, int V);
-int topk_chunks(int V);                                    // of a row
-int topk_share(int items, int chunks, int ctas, bool lse);   // items a CTA gets
 // a harvest of more than kTableRows rows: the table, out of the top-k kernel's results
 cudaError_t launch_harvest_scatter(goose_ctx* c, const HarvestTable& table, int rows, int k, const int32_t* ids, const float* vals,
                                    const float* row_lse, cudaStream_t st);

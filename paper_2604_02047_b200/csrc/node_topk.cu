@@ -33,6 +33,7 @@
 #include <type_traits>
 
 #include "goose_internal.cuh"
+#include "topk_deal.cuh"
 
 namespace goose {
 
@@ -42,9 +43,8 @@ constexpr int kTopkDataThreads = kTopkDataWarps * 32;
 constexpr int kTopkControlWarp = kTopkDataWarps + kTopkCollectWarps;
 constexpr int kTopkThreads = (kTopkControlWarp + 1) * 32;    // 16 + 4 + 1 warps, and with a table one more
 constexpr int kTopkPerThread = 64;                           // of a data thread: 8 x 128-bit shared-memory loads
-constexpr int kTopkChunk = kTopkDataThreads * kTopkPerThread;   // 32768 elements
+static_assert(kTopkChunk == kTopkDataThreads * kTopkPerThread);
 constexpr int kTopkSweep = kTopkDataThreads * 8;             // elements that the data threads load at once
-constexpr int kTopkMaxChunks = GOOSE_MAX_V / kTopkChunk;     // 8
 constexpr int kTopkStages = 3;
 constexpr int kTopkStageBytes = kTopkChunk * 2;              // 64 KB
 // what an item hands from role to role lives in slot (item & 3): a slot comes back into use only after the control warp
@@ -160,7 +160,7 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
                  int chunk_elems, u64* __restrict__ ws_cand, int32_t* __restrict__ row_counters,
                  int32_t* __restrict__ argmax, int32_t* __restrict__ ids, float* __restrict__ vals,
                  float* __restrict__ row_lse, float2* __restrict__ ws_lse, int32_t* __restrict__ status,
-                 int inputs_ready, const int32_t* __restrict__ n_nodes, int S, int B, const Table table) {
+                 int inputs_ready, const int32_t* __restrict__ n_nodes, int S, int B, const TopkDeal deal, const Table table) {
     constexpr bool TABLE = !std::is_same_v<Table, NoTable>;
     extern __shared__ __align__(128) unsigned char s_stage[];   // kTopkStages x 64 KB, then the candidate lists
     __shared__ u64 s_full[kTopkStages];                  // the stage holds its item
@@ -182,7 +182,6 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
                                                          // entries 0..31 of a list are zero between items
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int G = gridDim.x;
     if (!COUNTS) n_nodes = nullptr;
     const bool control = warp == kTopkControlWarp;
 
@@ -200,11 +199,15 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
     }
     if (warp == 1)
         for (int i = 0; i < kTopkSlots; ++i) s_lists[i * kTopkListCap + lane] = 0;
-    // CTA c's items: the first `more` CTAs have per + 1 of them, the others per (32-bit arithmetic throughout: 64-bit
-    // divisions in front of the first copy and barrier set-up by one thread had cost 0.5 us a call)
-    int items = items_all, per = items_all / G, more = items_all - per * G;   // final when !COUNTS
-    auto cta_start = [&](int c) { return c * per + min(c, more); };
-    auto cta_of = [&](int w) { return w < more * (per + 1) ? w / (per + 1) : more + (w - more * (per + 1)) / per; };
+    // CTA c's items: the first `more` CTAs have `unit` more of them than the `per` that all have (32-bit arithmetic throughout: 64-bit
+    // divisions in front of the first copy and barrier set-up by one thread had cost 0.5 us a call).  With node counts the rows
+    // that exist are dealt below, item by item: whole rows where their share allows it were up to 15 % faster (121 of 240
+    // rows of 128256 13.0 -> 11.4 us) and, by the divisions in front of the first copy, up to 4 % slower (176 of 200 rows of 262144 21.9 ->
+    // 22.8, 359 of 480 rows of 32000 8.8 -> 9.1).
+    const int G = gridDim.x, unit = COUNTS ? 1 : deal.unit;
+    int items = items_all, per = COUNTS ? items / G : deal.per, more = COUNTS ? items - per * G : deal.more;
+    auto cta_start = [&](int c) { return c * per + min(c, more) * unit; };
+    auto cta_of = [&](int w) { return w < more * (per + unit) ? w / (per + unit) : more + (w - more * (per + unit)) / per; };
     // inputs_ready: the caller guarantees that everything in front of the preceding kernel in the stream was complete when
     // this one could start, and that the preceding kernel touches neither the logits nor what this kernel writes (the
     // whole-step call: that kernel is the attention kernel, which lets its dependents start behind its own wait).  The
@@ -221,8 +224,7 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
     if (COUNTS && n_nodes) {
         int live = 0;
         for (int s = 0; s < S; ++s) live += nodes_of(n_nodes, s, B);
-        items = live * chunks;
-        per = items / G; more = items - per * G;
+        items = live * chunks; per = items / G; more = items - per * G;
     }
     const int w_begin = cta_start(blockIdx.x), n_local = cta_start(blockIdx.x + 1) - w_begin;
 
@@ -717,19 +719,6 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
     if (wait_at_end) pdl_wait();
 }
 
-// A row that is spread over CTAs costs a merge behind its last part, more than an item does: where one item more a CTA gives every
-// row to one CTA, that is the better share.  Top-k / harvest, us, without -> with:  4 chunks (V = 128256): 100 rows (q = 3 -> 4) 9.8 ->
-// 8.6 / 13.5 -> 12.1, 250 rows (7 -> 8) 16.6 -> 15.1 / 22.2 -> 20.8;  2 chunks (65536): 60 rows (1 -> 2) 6.0 -> 5.1, 150 rows (3 -> 4)
-// 8.6 -> 7.9, 900 rows (13 -> 14) 23.9 -> 22.7 / 33.5 -> 31.8;  7 chunks (200000): 122 rows (6 -> 7) 15.5 -> 13.8 / 20.7 -> 19.1.  Two
-// items more are even (4 chunks: 60 rows, 200 rows) or worse (30 rows 6.3 -> 7.7, 150 rows (5 -> 8) 18.2 -> 19.7), and so is a second
-// item with the log-sum-exp (cycle of 32 over 8 heads, 32 rows of 65536 12.4 -> 12.8).
-int topk_share(int items, int chunks, int ctas, bool lse) {
-    const int q = (items + ctas - 1) / ctas;
-    return chunks > 1 && (q + 1) % chunks == 0 && (q > 1 || !lse) ? q + 1 : q;
-}
-int topk_chunks(int V) { return (V + kTopkChunk - 1) / kTopkChunk; }
-int topk_items(int rows, int V) { return rows * ((V + kTopkChunk - 1) / kTopkChunk); }
-
 namespace {
 cudaError_t launch_topk_any(int num_sms, cudaStream_t st, const __nv_bfloat16* logits, int rows, int V, int64_t ldl, int k,
                             u64* ws, int32_t* counters, int32_t* argmax, int32_t* ids, float* vals, float* row_lse,
@@ -737,15 +726,13 @@ cudaError_t launch_topk_any(int num_sms, cudaStream_t st, const __nv_bfloat16* l
                             HarvestTable table = {}) {
     const int S = (n_nodes && B > 0) ? rows / B : 0;
     // equal chunks (a multiple of 8 elements: every copy starts on 16 bytes), so that no item is a remainder
-    const int chunks = (V + kTopkChunk - 1) / kTopkChunk;
+    const int chunks = topk_chunks(V);
     const int chunk_elems = ((V + chunks - 1) / chunks + 7) & ~7;
-    const int items = rows * chunks;                 // (a row costs the context 1 KB of scratch a chunk: far below 2^31)
-    // every CTA gets q = ceil(items / SMs) items or one fewer; using the fewest CTAs that q allows loses no time and
-    // makes the ranges fall on row boundaries when q is a multiple of the chunks per row (no cross-CTA merges then)
-    const int q = topk_share(items, chunks, num_sms, row_lse != nullptr), grid = (items + q - 1) / q;
+    const TopkDeal deal = topk_deal(rows, chunks, num_sms, row_lse != nullptr, n_nodes != nullptr);   // (a row costs the context 1 KB of
+                                                     // scratch a chunk: its items are far below 2^31)
     auto launch = [&](auto kernel, int threads, auto with) {
-        return launch_pdl(kernel, dim3(grid), dim3(threads), kTopkSmem, st, logits, items, V, ldl, k, chunks, chunk_elems, ws, counters,
-                          argmax, ids, vals, row_lse, ws_lse, status, inputs_ready, n_nodes, S, B, with);
+        return launch_pdl(kernel, dim3(deal.grid), dim3(threads), kTopkSmem, st, logits, rows * chunks, V, ldl, k, chunks, chunk_elems, ws, counters,
+                          argmax, ids, vals, row_lse, ws_lse, status, inputs_ready, n_nodes, S, B, deal, with);
     };
     if (table.adj_ids) return launch(node_topk_kernel<true, false, HarvestTable>, kTopkThreads + 32, table);
     return launch(row_lse ? (n_nodes ? node_topk_kernel<true, true, NoTable> : node_topk_kernel<true, false, NoTable>)
@@ -827,7 +814,7 @@ extern "C" int goose_node_topk_static(const void* logits, int rows, int V, int64
         num_sms = g_static_sms[dev];
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int chunks = (V + kTopkChunk - 1) / kTopkChunk;
+    const int chunks = topk_chunks(V);
     // the counters must start at zero; the array keeps whatever an earlier (possibly interrupted) call left
     int32_t* counters = reinterpret_cast<int32_t*>(scratch + kStaticCandWords);
     if (chunks > 1 && cudaMemsetAsync(counters, 0, sizeof(int32_t) * (size_t)rows, st) != cudaSuccess)
