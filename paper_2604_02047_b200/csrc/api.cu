@@ -50,6 +50,70 @@ int check_shape(const goose_ctx* c, int S, int B, int H, int D) {
 
 }  // namespace
 
+// The step's split of the SMs: how many CTAs a head the attention gets (1: its persistent form) and, beside clusters, how many the top-k.
+// The cluster form of the attention merges its heads itself and leaves SMs idle; the top-k goes onto those, beside it,
+// where it is done about when the attention is: at most 7 items an SM, and with the log-sum-exp, whose items take 2.2 us
+// instead of 1.5, 3 and one for every tile of a CTA (7 too where behind the persistent form it would take more than an item
+// an SM).  The clusters' CTAs all end at once, so a top-k that has to follow would start late: with more items the step
+// keeps the persistent form, in whose ragged end the top-k starts.  us, persistent ->
+// clusters (items an SM, tiles a CTA):  32 heads, 128 rows 512 keys (8, 2) 16.6 -> 17.5, 1k (8, 3) 18.3 -> 18.4;   40 heads, 128
+// rows 256 (6, 1) 15.6 -> 15.2.   With the log-sum-exp:  32 heads, 80 rows 256 (5, 1) 16.1 -> 15.8, 512 (5, 2) 17.8 -> 16.4;
+// 40 heads, 128 rows 256 (6, 1) 18.1 -> 18.8, 512 (6, 2) 19.3 -> 19.8, 768 (6, 3) 20.5 -> 20.4, 1k (6, 3) 21.2 -> 20.3;
+// 32 heads, 128 rows 2k (8, 5) 22.7 -> 23.3;   16 heads, 64 rows of 128256 329 (6, 1) 22.8 -> 21.8.
+namespace goose {
+StepSplit step_split(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int V, bool harvest, bool counts) {
+    const int items = topk_items(S * B, V), chunks = topk_chunks(V), Hw = attn_heads(B, H, Hkv);
+    const int kind = harvest || items > c->num_sms ? 2 : 1;
+    const int all_tiles = (int)((kv_rows + 127) / 128);
+    // a few SMs stay free for the step's last launch: its CTAs fit beside neither kernel, and its loads ahead of
+    // the wait would start only when the attention ends (none, 2, 4, 8 free SMs, us: 32 heads, 80 rows 2k 18.3, 18.0, 17.9,
+    // 18.0 and with the harvest 18.1, 17.8, 17.8, 20.1;  52 heads 2k with the harvest 24.9, 24.0, 23.9, 24.0; beside a
+    // shorter attention the round of items that they cost the top-k shows: 32 heads, 80 rows 512 keys with the harvest 15.0,
+    // 16.4, 16.4, 19.8)
+    auto left = [&](int n) { return c->num_sms - Hw * n - 4; };
+    auto tiles = [&](int n, int of) { return (of + n - 1) / n; };                            // of a CTA
+    auto beside = [&](int n) {
+        const int most = harvest && items <= c->num_sms && tiles(n, all_tiles) < 4 ? 3 + tiles(n, all_tiles) : 7;
+        return left(n) > 0 && items <= most * left(n);
+    };
+    const int largest = attn_cluster(c, S, B, H, Hkv, kv_rows, kind);
+    int cluster = largest > 1 && beside(largest) ? largest : 1;
+    if (kind == 2) {
+        // A long top-k.  Smaller clusters end the attention later and the top-k earlier; where a smaller one ends the step earlier than the
+        // above does, it takes it.  The ends, in us, as medians of 558 steps and cycles of one sequence, each with every size that the
+        // device holds (14 head layouts, 5 to 128 rows, 200 to 14000 keys, eight vocabularies, half of them in caches with spare rows):
+        // the attention's end by the tiles of a CTA, the top-k's by the items of a CTA, whatever their length (a chain of
+        // dependent steps bounds an item), and 3.3 or 2.4 more where rows are merged over CTAs; the persistent form ends with
+        // its top-k behind it.  The fit is within 8 to 10 % in nine of ten steps, so a gain has to be 1 us; and since ctx_len[] is device data and a
+        // cache may have spare rows, it has to be half of one with a quarter of the cache's rows too.  Rows of nodes that do not
+        // exist count: the host does not know them.  558 steps, the largest cluster -> this: geometric mean 1.049, 0.993 to 1.57.  32 over 8
+        // heads, 60 rows of 128256 with the harvest 1k 19.7 -> 15.5 (6 -> 5 CTAs a head), 3k 20.1 -> 18.9, 6k 21.5 (6 stays);  16 over
+        // 2, 128 rows of 128256 with the harvest 3k 26.2 (persistent) -> 22.4 (4).
+        const bool grouped = H != Hkv;
+        auto end = [&](int n, int of) {
+            const int ctas = n > 1 ? left(n) : c->num_sms;
+            const int q = counts ? (items + ctas - 1) / ctas : topk_share(items, chunks, ctas, harvest);
+            const bool cut = counts ? chunks > 1 : q % chunks != 0;
+            if (n == 1) {
+                const double w = (double)of * Hw / c->num_sms;                              // tiles of a CTA
+                return harvest ? 12.5 + 1.3 * w + 2.5 * q + 3.6 * cut : 11.0 + 1.35 * w + 1.85 * q + 3.4 * cut;
+            }
+            const double attn = (grouped ? 11.8 : 10.2) + 1.15 * tiles(n, of);
+            const double topk = harvest ? 7.5 + 1.9 * q + 3.3 * cut : 7.1 + 1.35 * q + 2.4 * cut;
+            return attn > topk ? attn : topk;
+        };
+        const int few = all_tiles / 4 > 1 ? all_tiles / 4 : 1, without = cluster;
+        double gain = 1.0;
+        for (int n = kMaxCluster; n > 1; --n) {
+            if (n == without || !attn_cluster_fits(c, n, S, B, H, Hkv, kv_rows, kind) || !beside(n)) continue;
+            const double g = end(without, all_tiles) - end(n, all_tiles);
+            if (g > gain && end(without, few) - end(n, few) >= 0.5) { gain = g; cluster = n; }
+        }
+    }
+    return {cluster, cluster > 1 ? left(cluster) : 0};
+}
+}  // namespace goose
+
 extern "C" {
 
 const char* goose_strerror(int rc) {
@@ -325,52 +389,10 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
     // kernel's CTAs leave their SMs (out[] and lse[] are complete when the step is).
     goose::CombinePlan merge_plan;
     merge_plan.valid = false;
-    // The cluster form of the attention merges its heads itself and leaves SMs idle; the top-k goes onto those, beside it,
-    // where it is done about when the attention is: at most 7 items an SM, and with the log-sum-exp, whose items take 2.2 us
-    // instead of 1.5, 3 and one for every tile of a CTA (7 too where behind the persistent form it would take more than an item
-    // an SM).  The clusters' CTAs all end at once, so a top-k that has to follow would start late: with more items the step
-    // keeps the persistent form, in whose ragged end the top-k starts.  us, persistent ->
-    // clusters (items an SM, tiles a CTA):  32 heads, 128 rows 512 keys (8, 2) 16.6 -> 17.5, 1k (8, 3) 18.3 -> 18.4;   40 heads, 128
-    // rows 256 (6, 1) 15.6 -> 15.2.   With the log-sum-exp:  32 heads, 80 rows 256 (5, 1) 16.1 -> 15.8, 512 (5, 2) 17.8 -> 16.4;
-    // 40 heads, 128 rows 256 (6, 1) 18.1 -> 18.8, 512 (6, 2) 19.3 -> 19.8, 768 (6, 3) 20.5 -> 20.4, 1k (6, 3) 21.2 -> 20.3;
-    // 32 heads, 128 rows 2k (8, 5) 22.7 -> 23.3;   16 heads, 64 rows of 128256 329 (6, 1) 22.8 -> 21.8.
-    int topk_ctas = 0, cluster = 1;
-    const int topk_items = goose::topk_items(S * B, V), chunks = goose::topk_chunks(V);
-    const int kind = harvest || topk_items > c->num_sms ? 2 : 1;
-    if (S > 0 && !attn_done) {
-        // a few SMs stay free for the step's last launch: its CTAs fit beside neither kernel, and its loads ahead of
-        // the wait would start only when the attention ends (none, 2, 4, 8 free SMs, us: 32 heads, 80 rows 2k 18.3, 18.0, 17.9,
-        // 18.0 and with the harvest 18.1, 17.8, 17.8, 20.1;  52 heads 2k with the harvest 24.9, 24.0, 23.9, 24.0; beside a
-        // shorter attention the round of items that they cost the top-k shows: 32 heads, 80 rows 512 keys with the harvest 15.0,
-        // 16.4, 16.4, 19.8)
-        auto left = [&](int n) { return c->num_sms - goose::attn_heads(B, H, Hkv) * n - 4; };
-        auto tiles = [&](int n) { return (int)(((kv_rows + 127) / 128 + n - 1) / n); };      // of a CTA
-        auto beside = [&](int n) {
-            const int most = harvest && topk_items <= c->num_sms && tiles(n) < 4 ? 3 + tiles(n) : 7;
-            return left(n) > 0 && topk_items <= most * left(n);
-        };
-        if (kind == 1) {
-            const int n = goose::attn_cluster(c, S, B, H, Hkv, kv_rows, kind);
-            if (n > 1 && beside(n)) cluster = n;
-        } else {
-            // Larger clusters end the attention earlier and the top-k later.  The step's end, by either, in us (fitted to the steps
-            // below; 3.7 and 1.5: rows spread over CTAs), decides.  Largest cluster that the device holds -> this, us:  32 over 8
-            // heads, 60 rows of 128256 with the harvest 1k 20.1 -> 14.8, 3k 20.6 -> 18.1 (6 -> 5 CTAs a head), 6k 21.4 (6 stays), without
-            // 1k 15.8 -> 14.0, 3k 16.7 (6 stays);  80 rows of 32000 with the harvest 3k 19.5 (persistent) -> 18.5;  16 over 2, 128
-            // rows of 128256 3k 26.5 (persistent) -> 22.9;  32 heads, 128 rows of 32000 2k 21.2 (persistent) -> 19.8.
-            double best = 1e30;
-            for (int n = 2; n <= goose::kMaxCluster; ++n) {
-                if (!goose::attn_cluster_fits(c, n, S, B, H, Hkv, kv_rows, kind) || !beside(n)) continue;
-                const int q = n_nodes ? (topk_items + left(n) - 1) / left(n) : goose::topk_share(topk_items, chunks, left(n), harvest);
-                const bool spread = n_nodes ? chunks > 1 : q % chunks != 0;
-                const double attn_end = 11.0 + 1.25 * tiles(n);
-                const double topk_end = harvest ? 7.3 + 1.8 * q + (spread ? 3.7 : 0) : 11.0 + 0.75 * q + (spread ? 1.5 : 0);
-                const double end = attn_end > topk_end ? attn_end : topk_end;
-                if (end <= best) { best = end; cluster = n; }
-            }
-        }
-        if (cluster > 1) topk_ctas = left(cluster);
-    }
+    // SMs of the top-k beside a cluster form of the attention (the host-buffer call waits for its logits, and the attention's end is its own)
+    const goose::StepSplit split = S > 0 && !attn_done ? goose::step_split(c, S, B, H, Hkv, kv_rows, V, harvest, n_nodes != nullptr)
+                                                       : goose::StepSplit{1, 0};
+    int topk_ctas = split.topk_ctas;
     if (!(scale > 0.f) || !(scale < 1e30f)) return GOOSE_EINVAL;
     {
         int impl = c->attn_impl;
@@ -381,7 +403,7 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
             cudaError_t ea = goose::launch_tree_attn_umma(c, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_cache,
                                                           (const __nv_bfloat16*)v_cache, kv_rows, row_off, ctx_len, parent,
                                                           n_nodes, S, B, H, Hkv, scale, (__nv_bfloat16*)out, lse,
-                                                          static_cast<cudaStream_t>(stream), &merge_plan, cluster, kind);
+                                                          static_cast<cudaStream_t>(stream), &merge_plan, split.cluster);
             if (ea != cudaSuccess) return cuda_fail(ea);
         } else {
             topk_ctas = 0;

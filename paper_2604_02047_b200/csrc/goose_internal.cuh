@@ -202,13 +202,16 @@ cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __
                                   const __nv_bfloat16* vc, int64_t kv_rows, const int64_t* row_off,
                                   const int32_t* ctx_len, const int32_t* parent, const int32_t* n_nodes, int S, int B, int H,
                                   int Hkv, float scale, __nv_bfloat16* out, float* lse, cudaStream_t st,
-                                  struct CombinePlan* defer_merge = nullptr, int cluster = 0, int step = 0);
-// cluster: CTAs a head, 1: the persistent form, 0: the kernel's own choice, which is
-// attn_cluster(): step: 0 = the attention alone, 1 = in a step, 2 = in a step whose top-k is long (more than an item an SM, or with
-// the log-sum-exp).  There the caller weighs the sizes that attn_cluster_fits() allows against the SMs they leave to the top-k.
+                                  struct CombinePlan* defer_merge = nullptr, int cluster = 0);
+// cluster: CTAs a head, 1: the persistent form, 0: the kernel's own choice for a call of its own.
+// attn_cluster(): the largest cluster that the device holds, where it pays, else 1;  step: 0 = the attention alone, 1 = in a step, 2 = in a
+// step whose top-k is long (more than an item an SM, or with the log-sum-exp).
 int attn_heads(int B, int H, int Hkv);                     // heads of the work list of a sequence
 bool attn_cluster_fits(const goose_ctx* c, int n, int S, int B, int H, int Hkv, int64_t kv_rows, int step);
 int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int step);
+// a step on device buffers: the attention's cluster size and the top-k's CTAs beside it (0: all SMs, behind the attention)
+struct StepSplit { int cluster, topk_ctas; };
+StepSplit step_split(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int V, bool harvest, bool counts);
 
 cudaError_t launch_bounded_wait_selftest(goose_ctx* c, long long limit_cycles, int32_t* result, cudaStream_t st);
 

@@ -892,7 +892,7 @@ int auto_attn_impl(const goose_ctx* c, int S, int B, int H) {
 }
 
 // One sequence: a cluster per head, the largest (of at most 8 CTAs) that the device holds one of per head at once (in a step with a
-// long top-k a smaller one where that ends both earlier: see enqueue_step()) -- where
+// long top-k a smaller one where that ends both earlier: see step_split()) -- where
 // the SMs that this leaves out cost less than the merge kernel and the second segments that it saves.  What they cost grows
 // with lost = tiles / n - heads * tiles / SMs, the tiles that the longest CTA has more than an equal share; what is saved
 // depends on what else the launches do, so there are three kinds of call.  ctx_len[] is device data: the tiles are bounded
@@ -944,7 +944,7 @@ cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __
                                   const __nv_bfloat16* vc, int64_t kv_rows, const int64_t* row_off,
                                   const int32_t* ctx_len, const int32_t* parent, const int32_t* n_nodes, int S, int B, int H,
                                   int Hkv, float scale, __nv_bfloat16* out, float* lse, cudaStream_t st,
-                                  CombinePlan* defer_merge, int cluster, int step) {
+                                  CombinePlan* defer_merge, int cluster) {
     if (defer_merge) defer_merge->valid = false;
     if (!c->encode_tiled) return cudaErrorNotSupported;
     if (S == 0) return cudaSuccess;
@@ -957,7 +957,7 @@ cudaError_t launch_tree_attn_umma(goose_ctx* c, const __nv_bfloat16* q, const __
         !make_map(c->encode_tiled, &mv, vc, kv_rows, Hkv, kTile))
         return cudaErrorInvalidValue;
     const int Hw = n_mt * Hkv;
-    if (cluster == 0) cluster = attn_cluster(c, S, B, H, Hkv, kv_rows, step);
+    if (cluster == 0) cluster = attn_cluster(c, S, B, H, Hkv, kv_rows, 0);
     int grid = cluster > 1 ? Hw * cluster : c->num_sms;
     if (2 * grid > c->n_slots) grid = c->n_slots / 2;
     const int divisor = cluster > 1 ? cluster : grid;   // the one that the form needs on the device
