@@ -92,7 +92,7 @@ StepSplit step_split(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t k
         const bool grouped = H != Hkv;
         auto end = [&](int n, int of) {
             const int ctas = n > 1 ? left(n) : c->num_sms;
-            const int q = counts ? (items + ctas - 1) / ctas : topk_share(items, chunks, ctas, harvest);
+            const int q = counts ? (items + ctas - 1) / ctas : topk_share(items, chunks, ctas, harvest || n > 1);
             const bool cut = counts ? chunks > 1 : q % chunks != 0;
             if (n == 1) {
                 const double w = (double)of * Hw / c->num_sms;                              // tiles of a CTA

@@ -168,7 +168,7 @@ constexpr int kTableRows = 1536;
 constexpr int kMaxCluster = 8;        // the portable limit
 
 // launchers (each returns a cudaError_t from the launch)
-// max_ctas (0: one per SM): the largest grid
+// max_ctas (0: one per SM): the largest grid, beside the attention of a step
 // inputs_ready: everything in front of the kernel that precedes this one in the stream is complete when this one can
 // start, and that kernel has nothing to do with this one's inputs and outputs (see the kernel)
 // table (with row_lse, without n_nodes, at most kTableRows rows): the harvest of every row

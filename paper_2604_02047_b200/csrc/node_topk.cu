@@ -723,12 +723,12 @@ namespace {
 cudaError_t launch_topk_any(int num_sms, cudaStream_t st, const __nv_bfloat16* logits, int rows, int V, int64_t ldl, int k,
                             u64* ws, int32_t* counters, int32_t* argmax, int32_t* ids, float* vals, float* row_lse,
                             float2* ws_lse, int32_t* status, int inputs_ready, const int32_t* n_nodes = nullptr, int B = 0,
-                            HarvestTable table = {}) {
+                            HarvestTable table = {}, bool beside = false) {
     const int S = (n_nodes && B > 0) ? rows / B : 0;
     // equal chunks (a multiple of 8 elements: every copy starts on 16 bytes), so that no item is a remainder
     const int chunks = topk_chunks(V);
     const int chunk_elems = ((V + chunks - 1) / chunks + 7) & ~7;
-    const TopkDeal deal = topk_deal(rows, chunks, num_sms, row_lse != nullptr, n_nodes != nullptr);   // (a row costs the context 1 KB of
+    const TopkDeal deal = topk_deal(rows, chunks, num_sms, row_lse || beside, n_nodes != nullptr);   // (a row costs the context 1 KB of
                                                      // scratch a chunk: its items are far below 2^31)
     auto launch = [&](auto kernel, int threads, auto with) {
         return launch_pdl(kernel, dim3(deal.grid), dim3(threads), kTopkSmem, st, logits, rows * chunks, V, ldl, k, chunks, chunk_elems, ws, counters,
@@ -759,7 +759,7 @@ cudaError_t launch_node_topk(goose_ctx* c, const __nv_bfloat16* logits, int rows
     if (rows == 0) return cudaSuccess;
     cudaError_t e = launch_topk_any(max_ctas > 0 ? max_ctas : c->num_sms, st, logits, rows, V, ldl, k, c->topk_cand, c->row_counters, argmax, ids, vals,
                                     row_lse, reinterpret_cast<float2*>(c->topk_lse_ws), c->status, inputs_ready ? 1 : 0,
-                                    n_nodes, B, table);
+                                    n_nodes, B, table, max_ctas > 0);
     c->launches++;
     return e;
 }
