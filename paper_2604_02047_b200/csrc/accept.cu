@@ -92,4 +92,6 @@ cudaError_t launch_accept(goose_ctx* c, const int32_t* draft_tok, const int32_t*
     return e;
 }
 
+cudaError_t init_accept_kernel() { return load_kernels({(const void*)accept_kernel}); }
+
 }  // namespace goose

@@ -300,4 +300,10 @@ cudaError_t launch_accept_compact(goose_ctx* c, __nv_bfloat16* kc, __nv_bfloat16
     return e;
 }
 
+cudaError_t init_compact_kernel() {
+    return load_kernels({(const void*)accept_compact_kernel<false, 0>, (const void*)accept_compact_kernel<true, 0>, (const void*)accept_compact_kernel<false, 1>,
+                         (const void*)accept_compact_kernel<true, 1>, (const void*)accept_compact_kernel<false, 2>, (const void*)accept_compact_kernel<true, 2>,
+                         (const void*)kv_compact_kernel<false>, (const void*)kv_compact_kernel<true>});
+}
+
 }  // namespace goose

@@ -749,8 +749,10 @@ cudaError_t init_topk_kernel() {
     };
     opt_in((const void*)node_topk_kernel<false, false, NoTable>);  opt_in((const void*)node_topk_kernel<false, true, NoTable>);
     opt_in((const void*)node_topk_kernel<true, false, NoTable>);   opt_in((const void*)node_topk_kernel<true, true, NoTable>);
-    opt_in((const void*)node_topk_kernel<true, false, HarvestTable>);
     return e;
+}
+cudaError_t init_table_kernel() {
+    return cudaFuncSetAttribute(node_topk_kernel<true, false, HarvestTable>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopkSmem);
 }
 
 cudaError_t launch_node_topk(goose_ctx* c, const __nv_bfloat16* logits, int rows, int V, int64_t ldl, int k,

@@ -883,6 +883,11 @@ cudaError_t init_umma_kernel(goose_ctx* c) {
     return cudaSuccess;
 }
 
+cudaError_t init_merge_kernel() {
+    return load_kernels({(const void*)tree_attn_combine_kernel<false, false>, (const void*)tree_attn_combine_kernel<false, true>,
+                         (const void*)tree_attn_combine_kernel<true, false>, (const void*)tree_attn_combine_kernel<true, true>});
+}
+
 int auto_attn_impl(const goose_ctx* c, int S, int B, int H) {
     (void)S; (void)H;
     (void)B;
