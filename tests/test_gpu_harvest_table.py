@@ -38,6 +38,14 @@ def test_table_matches_the_oracle(oracle, rows, V, k, tokens):
     goose.close()
 
 
+@pytest.mark.parametrize("rows, V, k, tokens", [(60, 128256, 10, 20), (149, 128256, 8, 149)])
+def test_table_of_rows_that_are_merged_over_ctas(oracle, rows, V, k, tokens):
+    chunks, sms = -(-V // 32768), torch.cuda.get_device_properties(0).multi_processor_count
+    share = -(-rows * chunks // sms)                          # items of a CTA: ranges of them start inside rows
+    assert share > 1 and share % chunks and (share + 1) % chunks
+    test_table_matches_the_oracle(oracle, rows, V, k, tokens)
+
+
 @pytest.mark.parametrize("rows, V", [(8192, 4096), (5000, 32000)])
 def test_many_rows_cost_what_their_logits_cost(rows, V):
     """The look for a later row with a row's token grows with the rows; the call may not.  The log-sum-exp and the table take 1.3 to 1.55
