@@ -476,8 +476,8 @@ tree_attn_umma_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
             uint32_t anc[4] = {0, 0, 0, 0};
             // Rows of the M tile that no query fills: zeros instead of what shared memory held.  No result depends on them (and so
             // nothing waits for these stores), but a long stream is held back by the power that the card may draw, and products of
-            // zeros draw less: steps under continuous load, 16 x 32 heads 1k to 16k with 64 rows 450 -> 429 us, 7 ragged sequences of
-            // 32 heads with at most 60 rows 92.8 -> 90.9, 40 heads 4k with 80 rows 25.3 -> 24.8.  By the softmax threads, which wait
+            // zeros draw less: steps under continuous load, 16 x 32 heads 1k to 16k with 64 rows 445 -> 426 us, 7 ragged sequences of
+            // 32 heads with at most 60 rows 92.4 -> 90.0; 40 heads 4k with 80 rows even.  By the softmax threads, which wait
             // for the first scores here; in the set-up, ahead of the dependency wait, it cost short calls 0.3 to 0.4 us.
             if (!kCluster) {
                 for (int off = nb * g * 128 + sm_tid * 16; off < kHalfBytes; off += 128 * 16) {
