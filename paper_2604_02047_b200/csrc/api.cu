@@ -61,7 +61,7 @@ int check_shape(const goose_ctx* c, int S, int B, int H, int D) {
 // 40 heads, 128 rows 256 (6, 1) 18.1 -> 18.8, 512 (6, 2) 19.3 -> 19.8, 768 (6, 3) 20.5 -> 20.4, 1k (6, 3) 21.2 -> 20.3;
 // 32 heads, 128 rows 2k (8, 5) 22.7 -> 23.3;   16 heads, 64 rows of 128256 329 (6, 1) 22.8 -> 21.8.
 namespace goose {
-StepSplit step_split(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int V, bool harvest, bool counts) {
+StepSplit step_split(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int V, int k, bool harvest, bool counts) {
     const int items = topk_items(S * B, V), chunks = topk_chunks(V), Hw = attn_heads(B, H, Hkv);
     const int kind = harvest || items > c->num_sms ? 2 : 1;
     const int all_tiles = (int)((kv_rows + 127) / 128);
@@ -84,22 +84,28 @@ StepSplit step_split(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t k
         // device holds (14 head layouts, 5 to 128 rows, 200 to 14000 keys, eight vocabularies, half of them in caches with spare rows):
         // the attention's end by the tiles of a CTA, the top-k's by the items of a CTA, whatever their length (a chain of
         // dependent steps bounds an item), and 3.3 or 2.4 more where rows are merged over CTAs; the persistent form ends with
-        // its top-k behind it.  The fit is within 8 to 10 % in nine of ten steps, so a gain has to be 1 us; and since ctx_len[] is device data and a
-        // cache may have spare rows, it has to be half of one with a quarter of the cache's rows too.  Rows of nodes that do not
-        // exist count: the host does not know them.  558 steps, the largest cluster -> this: geometric mean 1.049, 0.993 to 1.57.  32 over 8
-        // heads, 60 rows of 128256 with the harvest 1k 19.7 -> 15.5 (6 -> 5 CTAs a head), 3k 20.1 -> 18.9, 6k 21.5 (6 stays);  16 over
-        // 2, 128 rows of 128256 with the harvest 3k 26.2 (persistent) -> 22.4 (4).
+        // its top-k behind it.  A merge of more than 32 candidates takes k passes of a warp (harvest, a row of four chunks over four CTAs,
+        // k = 8, 10, 16: steps of 11.5, 15.2, 17.3; seven over four 13.5, 17.5, 21.2).  The fit is within 8 to 10 % in nine of ten
+        // steps, so a gain has to be 1 us; and since ctx_len[] is device data and a cache may have spare rows, it has to be half of
+        // one with a quarter of the cache's rows too.  Rows of nodes that do not exist count: the host does not know them.  1200 other
+        // steps and cycles (k of 8, 10 and 16), the largest cluster or the persistent form -> this: geometric mean 1.095, 0.915 to 2.04, seven
+        // below 0.99 (1820 without the merge's passes: 37, down to 0.79).  32 over 8 heads, 60 rows of 128256 with the harvest 1k 19.7 -> 15.5
+        // (6 -> 5 CTAs a head), 3k 20.1 -> 18.9, 6k 21.5 (6 stays);  16 over 2, 128 rows of 128256 with the harvest 3k 26.2
+        // (persistent) -> 22.4 (4).
         const bool grouped = H != Hkv;
         auto end = [&](int n, int of) {
             const int ctas = n > 1 ? left(n) : c->num_sms;
             const int q = counts ? (items + ctas - 1) / ctas : topk_share(items, chunks, ctas, harvest || n > 1);
             const bool cut = counts ? chunks > 1 : q % chunks != 0;
+            // CTAs that a row is cut over, and their lists' merge: up to a warp's lanes it is one pass, above that k of them
+            const int parts = !cut ? 1 : chunks % q == 0 ? chunks / q : (chunks - 2) / q + 2;
+            const double merge = parts * k > 32 ? 0.3 * k : 0;
             if (n == 1) {
                 const double w = (double)of * Hw / c->num_sms;                              // tiles of a CTA
-                return harvest ? 12.5 + 1.3 * w + 2.5 * q + 3.6 * cut : 11.0 + 1.35 * w + 1.85 * q + 3.4 * cut;
+                return merge + (harvest ? 12.5 + 1.3 * w + 2.5 * q + 3.6 * cut : 11.0 + 1.35 * w + 1.85 * q + 3.4 * cut);
             }
             const double attn = (grouped ? 11.8 : 10.2) + 1.15 * tiles(n, of);
-            const double topk = harvest ? 7.5 + 1.9 * q + 3.3 * cut : 7.1 + 1.35 * q + 2.4 * cut;
+            const double topk = merge + (harvest ? 7.5 + 1.9 * q + 3.3 * cut : 7.1 + 1.35 * q + 2.4 * cut);
             return attn > topk ? attn : topk;
         };
         const int few = all_tiles / 4 > 1 ? all_tiles / 4 : 1, without = cluster;
@@ -390,7 +396,7 @@ int enqueue_step(goose_ctx* c, const void* q, void* k_cache, void* v_cache, int6
     goose::CombinePlan merge_plan;
     merge_plan.valid = false;
     // SMs of the top-k beside a cluster form of the attention (the host-buffer call waits for its logits, and the attention's end is its own)
-    const goose::StepSplit split = S > 0 && !attn_done ? goose::step_split(c, S, B, H, Hkv, kv_rows, V, harvest, n_nodes != nullptr)
+    const goose::StepSplit split = S > 0 && !attn_done ? goose::step_split(c, S, B, H, Hkv, kv_rows, V, k, harvest, n_nodes != nullptr)
                                                        : goose::StepSplit{1, 0};
     int topk_ctas = split.topk_ctas;
     if (!(scale > 0.f) || !(scale < 1e30f)) return GOOSE_EINVAL;

@@ -212,7 +212,7 @@ bool attn_cluster_fits(const goose_ctx* c, int n, int S, int B, int H, int Hkv, 
 int attn_cluster(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int step);
 // a step on device buffers: the attention's cluster size and the top-k's CTAs beside it (0: all SMs, behind the attention)
 struct StepSplit { int cluster, topk_ctas; };
-StepSplit step_split(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int V, bool harvest, bool counts);
+StepSplit step_split(const goose_ctx* c, int S, int B, int H, int Hkv, int64_t kv_rows, int V, int k, bool harvest, bool counts);
 
 cudaError_t launch_bounded_wait_selftest(goose_ctx* c, long long limit_cycles, int32_t* result, cudaStream_t st);
 

@@ -10,11 +10,11 @@ from paper_2604_02047_b200 import build
 SOURCE = r"""
 #include "goose_internal.cuh"
 #include "topk_deal.cuh"
-extern "C" void split(const int* max_clusters, int sms, int S, int B, int H, int Hkv, long long kv_rows, int V, int harvest, int counts, int* out) {
+extern "C" void split(const int* max_clusters, int sms, int S, int B, int H, int Hkv, long long kv_rows, int V, int k, int harvest, int counts, int* out) {
     goose_ctx c = {};
     c.num_sms = sms;
     for (int n = 2; n <= 8; ++n) c.max_clusters[n] = max_clusters[n];
-    const goose::StepSplit s = goose::step_split(&c, S, B, H, Hkv, kv_rows, V, harvest, counts);
+    const goose::StepSplit s = goose::step_split(&c, S, B, H, Hkv, kv_rows, V, k, harvest, counts);
     const bool long_topk = harvest || goose::topk_items(S * B, V) > sms;
     out[0] = s.cluster; out[1] = s.topk_ctas;
     out[2] = goose::attn_cluster(&c, S, B, H, Hkv, kv_rows, long_topk ? 2 : 1); out[3] = goose::attn_heads(B, H, Hkv);
@@ -38,9 +38,9 @@ def split(tmp_path_factory):
     lib = ctypes.CDLL(so)
     most = (ctypes.c_int * 9)(*MAX_CLUSTERS)
 
-    def call(S, B, H, Hkv, kv_rows, V, harvest, counts=False):
+    def call(S, B, H, Hkv, kv_rows, V, harvest, counts=False, k=8):
         out = (ctypes.c_int * 6)()
-        lib.split(most, SMS, S, B, H, Hkv, ctypes.c_longlong(kv_rows), V, int(harvest), int(counts), out)
+        lib.split(most, SMS, S, B, H, Hkv, ctypes.c_longlong(kv_rows), V, k, int(harvest), int(counts), out)
         return list(out)
 
     return call
@@ -68,6 +68,18 @@ def test_choice(split, H, Hkv, B, ctx, spare, V, harvest, cluster):
     got, ctas, largest, heads, fits, items = split(1, B, H, Hkv, ctx + B + spare, V, harvest)
     assert got == cluster
     assert ctas == (SMS - heads * got - 4 if got > 1 else 0)
+
+
+# a row that is cut over so many CTAs that their lists have more than 32 candidates is dear to merge
+MERGES = [  # heads, rows, keys, vocabulary, k -> CTAs a head
+    (32, 8, 21, 586, 128256, 8, 7), (32, 8, 21, 586, 128256, 10, 8), (40, 8, 16, 488, 200000, 8, 8), (16, 16, 31, 1535, 152064, 16, 6),
+    (40, 40, 16, 479, 152064, 16, 3), (32, 8, 60, 3001, 128256, 10, 5),
+]
+
+
+@pytest.mark.parametrize("H, Hkv, B, ctx, V, k, cluster", MERGES)
+def test_choice_knows_what_a_merge_costs(split, H, Hkv, B, ctx, V, k, cluster):
+    assert split(1, B, H, Hkv, ctx + B, V, True, k=k)[0] == cluster
 
 
 def test_every_choice_is_one_that_the_device_holds(split):
