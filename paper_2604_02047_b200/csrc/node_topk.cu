@@ -215,6 +215,10 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
     // this grid implies that kernel's.  (Waiting in front of the first result instead: CTAs with several items stood
     // still until the attention had ended, 1.6 us a step at 32 heads, 2k keys and 80 rows on 20 CTAs.)
     const bool wait_at_end = inputs_ready != 0;
+    // the range is worked out ahead of the wait, while the kernel in front runs: behind it its arguments' first reads stood before the
+    // first copy (rows of 32000: 128 rows 3.84 -> 3.75 us, harvest of 16 rows 4.90 -> 4.75)
+    int w_begin = cta_start(blockIdx.x), n_local = cta_start(blockIdx.x + 1) - w_begin;
+    asm volatile("" : "+r"(w_begin), "+r"(n_local));
     if (!wait_at_end) pdl_wait();
     pdl_trigger();
     // Per-sequence node counts (n_nodes != NULL; rows = S * B, row s * B + i belongs to node i of sequence s): rows of
@@ -225,8 +229,8 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
         int live = 0;
         for (int s = 0; s < S; ++s) live += nodes_of(n_nodes, s, B);
         items = live * chunks; per = items / G; more = items - per * G;
+        w_begin = cta_start(blockIdx.x); n_local = cta_start(blockIdx.x + 1) - w_begin;
     }
-    const int w_begin = cta_start(blockIdx.x), n_local = cta_start(blockIdx.x + 1) - w_begin;
 
     // control warp: the next item to stream; its first copies leave before the rest of the CTA is set up
     const unsigned short* lg = reinterpret_cast<const unsigned short*>(logits);
