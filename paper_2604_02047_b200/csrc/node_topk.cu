@@ -153,14 +153,15 @@ struct RowCursor {
 // warp, whose time the next copy waits for: 28.7); 16 tokens a lane in flight instead of 8: 2048 x 32000 31.5 -> 31.3, but
 // 1500 x 128256 82.5 -> 84.8.
 // COUNTS = false is the instantiation for n_nodes == NULL (the item list is known before the dependency wait)
+// per, more, unit: TopkDeal.  The arguments with a table are 160 bytes: with 176 a launch took the host 0.4 us more (harvest calls 12.1 -> 12.6)
 struct NoTable {};
 template <bool LSE, bool COUNTS, class Table>
 __global__ void __launch_bounds__(kTopkThreads + (std::is_same_v<Table, NoTable> ? 0 : 32), 1)
-node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V, int64_t ldl, int k, int chunks,
-                 int chunk_elems, u64* __restrict__ ws_cand, int32_t* __restrict__ row_counters,
+node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int per, int more, int unit, int V, int64_t ldl, int k, int chunks,
+                 int chunk_elems, int inputs_ready, u64* __restrict__ ws_cand, int32_t* __restrict__ row_counters,
                  int32_t* __restrict__ argmax, int32_t* __restrict__ ids, float* __restrict__ vals,
                  float* __restrict__ row_lse, float2* __restrict__ ws_lse, int32_t* __restrict__ status,
-                 int inputs_ready, const int32_t* __restrict__ n_nodes, int S, int B, const TopkDeal deal, const Table table) {
+                 const int32_t* __restrict__ n_nodes, int S, int B, const Table table) {
     constexpr bool TABLE = !std::is_same_v<Table, NoTable>;
     extern __shared__ __align__(128) unsigned char s_stage[];   // kTopkStages x 64 KB, then the candidate lists
     __shared__ u64 s_full[kTopkStages];                  // the stage holds its item
@@ -204,8 +205,8 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
     // that exist are dealt below, item by item: whole rows where their share allows it were up to 15 % faster (121 of 240
     // rows of 128256 13.0 -> 11.4 us) and, by the divisions in front of the first copy, up to 4 % slower (176 of 200 rows of 262144 21.9 ->
     // 22.8, 359 of 480 rows of 32000 8.8 -> 9.1).
-    const int G = gridDim.x, unit = COUNTS ? 1 : deal.unit;
-    int items = items_all, per = COUNTS ? items / G : deal.per, more = COUNTS ? items - per * G : deal.more;
+    const int G = gridDim.x;
+    if (COUNTS) unit = 1;
     auto cta_start = [&](int c) { return c * per + min(c, more) * unit; };
     auto cta_of = [&](int w) { return w < more * (per + unit) ? w / (per + unit) : more + (w - more * (per + unit)) / per; };
     // inputs_ready: the caller guarantees that everything in front of the preceding kernel in the stream was complete when
@@ -228,7 +229,8 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
     if (COUNTS && n_nodes) {
         int live = 0;
         for (int s = 0; s < S; ++s) live += nodes_of(n_nodes, s, B);
-        items = live * chunks; per = items / G; more = items - per * G;
+        const int items = live * chunks;
+        per = items / G; more = items - per * G;
         w_begin = cta_start(blockIdx.x); n_local = cta_start(blockIdx.x + 1) - w_begin;
     }
 
@@ -485,7 +487,7 @@ node_topk_kernel(const __nv_bfloat16* __restrict__ logits, int items_all, int V,
         // which row of the table an item's logits row writes: a scan of the later rows' tokens beside the item's stream (an item's
         // arrival implies that its slot's last user is finished), for the items that end this CTA's part of a row alone -- nobody
         // reads the others' answer -- and up to the first later row with the token
-        const int rows = items_all / chunks;
+        const int rows = cta_start(G) / chunks;
         int row = w_begin / chunks, chunk = w_begin - row * chunks;
         for (int j = 0; j < n_local; ++j) {
             if (mbar_wait_bounded(&s_full[j % kTopkStages], (uint32_t)(j / kTopkStages) & 1u, kTopkWaitCycles, &s_abort) != 0) {
@@ -735,8 +737,8 @@ cudaError_t launch_topk_any(int num_sms, cudaStream_t st, const __nv_bfloat16* l
     const TopkDeal deal = topk_deal(rows, chunks, num_sms, row_lse || beside, n_nodes != nullptr);   // (a row costs the context 1 KB of
                                                      // scratch a chunk: its items are far below 2^31)
     auto launch = [&](auto kernel, int threads, auto with) {
-        return launch_pdl(kernel, dim3(deal.grid), dim3(threads), kTopkSmem, st, logits, rows * chunks, V, ldl, k, chunks, chunk_elems, ws, counters,
-                          argmax, ids, vals, row_lse, ws_lse, status, inputs_ready, n_nodes, S, B, deal, with);
+        return launch_pdl(kernel, dim3(deal.grid), dim3(threads), kTopkSmem, st, logits, deal.per, deal.more, deal.unit, V, ldl, k, chunks, chunk_elems,
+                          inputs_ready, ws, counters, argmax, ids, vals, row_lse, ws_lse, status, n_nodes, S, B, with);
     };
     if (table.adj_ids) return launch(node_topk_kernel<true, false, HarvestTable>, kTopkThreads + 32, table);
     return launch(row_lse ? (n_nodes ? node_topk_kernel<true, true, NoTable> : node_topk_kernel<true, false, NoTable>)

@@ -34,7 +34,7 @@ struct TopkDeal {
 // The fewest CTAs that the share allows: that loses no time.  Where the share is whole rows, rows are dealt and none is cut: items dealt one
 // by one would leave a CTA with one item fewer in the middle of a row wherever they do not come out even (900 rows of 2 chunks: 123 CTAs
 // with 14 and 6 with 13).  With node counts the rows that exist are known on the device alone: fewer CTAs for all rows would not get whole
-// ones (per, more and unit are the kernel's affair then).
+// ones (the kernel works out per, more and unit for the rows that exist).
 inline TopkDeal topk_deal(int rows, int chunks, int ctas, bool no_second, bool counts) {
     const int items = rows * chunks, q = counts ? (items + ctas - 1) / ctas : topk_share(items, chunks, ctas, no_second);
     const int unit = !counts && q % chunks == 0 ? chunks : 1, units = items / unit, grid = (units + q / unit - 1) / (q / unit);
